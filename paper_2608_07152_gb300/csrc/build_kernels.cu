@@ -1,36 +1,183 @@
 // PVS index build and query encoding (Sec. 2.3.1; norms for App. A.1).
 //
-// One warp quantizes one vector: float32 loads, warp max of |v_j|, IEEE
-// division for the scale and the codes, and the order-independent integer
-// accumulation of the norm bounds (quantize_row_warp).  The raw float32 row
-// is copied next to the codes for authoritative scoring.
+// One warp quantizes one vector: float32 loads, warp max of |v_j|, the scale
+// by IEEE division, the codes, and the order-independent integer
+// accumulation of the norm bounds (the arithmetic quantize_row_warp states).
+// The raw float32 row is copied next to the codes for authoritative scoring.
+#include <algorithm>
+
 #include "kernels.h"
 #include "pvs_common.cuh"
 
 namespace pvs {
 
-__global__ void __launch_bounds__(256) build_kernel(const float* __restrict__ vecs, int64_t n,
+// Rows the integer arithmetic below does not cover (all-subnormal rows or
+// residuals, scales under 2^-100, a residual past the float32 grid): the
+// binary64 quantizer.  Out of line: never taken on ordinary data.
+static __device__ __noinline__ RowQuant quantize_row_slow(const float* v, int m, int m_pad, int8_t* z,
+                                                   float fixed_s) {
+    return quantize_row_warp(v, m, m_pad, z, fixed_s);
+}
+
+// One warp per row, `per_warp` (<= 32) rows of a warp in turn.  Everything per
+// element is float32 and integer work:
+//   - the code comes from the product with 1 / s (code_of);
+//   - the residual v - s c is exact in one FMA: v and s c are multiples of
+//     u = max(ulp(s) / 2, 2^-149) (v >= s / 2 where c != 0) and
+//     |v - s c| < 2^floor(log2 s) <= 2^24 u, checked per row;
+//   - the norm bounds sum norm_term_bits.
+// Lane r keeps the sums of the batch's r-th row, and the binary64 square
+// roots run once for the batch, one row per lane.
+//
+// Bound by: HBM (4m bytes read, 5m + 12 written per row); the element work is
+// about 30 instructions.  With binary64 norm terms and four passes over the row the
+// kernel was bound by the FP64 pipe: 213 ms at 8.8M x 768 (0.29 TB/s).
+// NV4: float4 of the row per lane, in registers (m_pad <= 128 NV4); 0: wider
+// rows are read again (from L1 / L2) in each of the three steps.
+
+template <int NV4>
+__global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 3) build_kernel(const float* __restrict__ vecs, int64_t n,
                                                     int m, int m_pad, int m_raw,
                                                     int8_t* __restrict__ codes,
                                                     float* __restrict__ scale,
                                                     float* __restrict__ vnorm,
                                                     float* __restrict__ enorm,
                                                     float* __restrict__ raw, int* status,
-                                                    const float* fixed_scale) {
+                                                    const float* fixed_scale, int aligned,
+                                                    int per_warp) {
+    constexpr int kKeep = NV4 > 0 ? NV4 : 1;
     const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t stride = (int64_t)gridDim.x * (blockDim.x >> 5) * per_warp;
     const float fs = fixed_scale ? *fixed_scale : 0.0f;
-    for (int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < n;
-         row += warps) {
-        const float* v = vecs + row * (int64_t)m;
-        RowQuant r = quantize_row_warp(v, m, m_pad, codes + row * (int64_t)m_pad, fs);
-        float* dst = raw + row * (int64_t)m_raw;
-        for (int j = lane; j < m_raw; j += kWarp) dst[j] = j < m ? v[j] : 0.0f;
-        if (lane == 0) {
-            scale[row] = r.s;
-            vnorm[row] = r.vnorm;
-            enorm[row] = r.enorm;
-            if (r.status) set_status(status, r.status);
+    const int steps = NV4 > 0 ? NV4 : (m_pad + 127) / 128;
+    for (int64_t row0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) *
+                        per_warp;
+         row0 < n; row0 += stride) {
+        const int batch = (int)(n - row0 < per_warp ? n - row0 : per_warp);
+        // this lane's row of the batch
+        unsigned long long tv = 0, te = 0;
+        int ev = 0, ee = 0;
+        float s_of = 0.0f, vn = 0.0f, en = 0.0f;
+        bool done = false;
+        for (int b = 0; b < batch; ++b) {
+            const int64_t row = row0 + b;
+            const float* v = vecs + row * (int64_t)m;
+            auto load = [&](int i) {
+                const int j = 4 * (lane + 32 * i);
+                float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (aligned) {
+                    if (j < m) x = __ldcs(reinterpret_cast<const float4*>(v + j));
+                } else {
+                    if (j < m) x.x = v[j];
+                    if (j + 1 < m) x.y = v[j + 1];
+                    if (j + 2 < m) x.z = v[j + 2];
+                    if (j + 3 < m) x.w = v[j + 3];
+                }
+                return x;
+            };
+            float4 keep[kKeep];
+            uint32_t mx = 0;
+#pragma unroll
+            for (int i = 0; i < steps; ++i) {
+                const float4 x = load(i);
+                if constexpr (NV4 > 0) keep[i] = x;
+                const int j = 4 * (lane + 32 * i);
+                if (j < m_raw) *reinterpret_cast<float4*>(raw + row * (int64_t)m_raw + j) = x;
+                mx = max(max(mx, __float_as_uint(fabsf(x.x))), __float_as_uint(fabsf(x.y)));
+                mx = max(max(mx, __float_as_uint(fabsf(x.z))), __float_as_uint(fabsf(x.w)));
+            }
+            mx = __reduce_max_sync(0xffffffffu, mx);
+            if (mx >= 0x7f800000u) {   // an infinity or a NaN
+                if (lane == 0) set_status(status, PVS_ERR_NONFINITE);
+                done |= lane == b;
+                continue;
+            }
+            float s = fs;
+            if (!(fs > 0.0f)) s = mx == 0 ? 1.0f : __fdiv_rn(__uint_as_float(mx), 127.0f);
+            const float rs = __frcp_rn(s);
+            uint32_t emx = 0;
+            bool out_of_range = false;
+            uint32_t* zrow = reinterpret_cast<uint32_t*>(codes + row * (int64_t)m_pad);
+            bool slow = mx != 0 && (mx < 0x00800000u || s < kFastScaleMin);
+            const int Ev = max((int)(mx >> 23), 1);   // (0: sums of 0)
+            unsigned long long a = 0, c2 = 0;
+            if (!slow) {
+#pragma unroll
+                for (int i = 0; i < steps; ++i) {
+                    const float4 x = NV4 > 0 ? keep[NV4 > 0 ? i : 0] : load(i);
+                    uint32_t y[4];
+                    const float xs[4] = {x.x, x.y, x.z, x.w};
+                    float e[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float c = code_of(xs[k], s, rs, y[k]);
+                        if (fs > 0.0f && fabsf(c) > 127.0f) out_of_range = true;
+                        e[k] = __fmaf_rn(-s, c, xs[k]);
+                        emx = max(emx, __float_as_uint(fabsf(e[k])));
+                        a += norm_term_bits(__float_as_uint(fabsf(xs[k])), Ev);
+                    }
+                    const int j4 = lane + 32 * i;
+                    if (4 * j4 < m_pad)
+                        zrow[j4] = __byte_perm(__byte_perm(y[0], y[1], 0x0040),
+                                               __byte_perm(y[2], y[3], 0x0040), 0x5410);
+                    if constexpr (NV4 > 0) keep[i] = make_float4(e[0], e[1], e[2], e[3]);
+                }
+                emx = __reduce_max_sync(0xffffffffu, emx);
+                // not on the residual's float32 grid, or a subnormal maximum
+                slow = emx >= (__float_as_uint(s) & 0x7f800000u) || (emx != 0 && emx < 0x00800000u);
+                if (fs > 0.0f && __any_sync(0xffffffffu, out_of_range)) slow = true;
+            }
+            if (slow) {   // the same for the whole warp
+                __syncwarp();
+                const RowQuant r =
+                    quantize_row_slow(v, m, m_pad, codes + row * (int64_t)m_pad, fs);
+                if (lane == b) {
+                    s_of = r.s;
+                    vn = r.vnorm;
+                    en = r.enorm;
+                    done = true;
+                }
+                if (r.status && lane == 0) set_status(status, r.status);
+                continue;
+            }
+            const int Ee = max((int)(emx >> 23), 1);
+#pragma unroll
+            for (int i = 0; i < steps; ++i) {
+                if constexpr (NV4 > 0) {
+                    c2 += norm_term_bits(__float_as_uint(fabsf(keep[i].x)), Ee);
+                    c2 += norm_term_bits(__float_as_uint(fabsf(keep[i].y)), Ee);
+                    c2 += norm_term_bits(__float_as_uint(fabsf(keep[i].z)), Ee);
+                    c2 += norm_term_bits(__float_as_uint(fabsf(keep[i].w)), Ee);
+                } else {
+                    const float4 x = load(i);
+                    const float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        uint32_t y;
+                        const float e = __fmaf_rn(-s, code_of(xs[k], s, rs, y), xs[k]);
+                        c2 += norm_term_bits(__float_as_uint(fabsf(e)), Ee);
+                    }
+                }
+            }
+            a = warp_sum(a);
+            c2 = warp_sum(c2);
+            if (lane == b) {
+                s_of = s;
+                tv = a;
+                te = c2;
+                ev = Ev - 126;
+                ee = Ee - 126;
+            }
+        }
+        if (lane < batch) {
+            if (!done) {
+                vn = norm_finish((long long)tv, ev);
+                en = norm_finish((long long)te, ee);
+                if (isinf(vn) || isinf(en)) set_status(status, PVS_ERR_OVERFLOW);
+            }
+            scale[row0 + lane] = s_of;
+            vnorm[row0 + lane] = vn;
+            enorm[row0 + lane] = en;
         }
     }
 }
@@ -39,12 +186,30 @@ cudaError_t launch_build(const float* vecs, int64_t n, int m, int m_pad, int m_r
                          int8_t* codes, float* scale, float* vnorm, float* enorm, float* raw,
                          int* status, cudaStream_t st, const float* fixed_scale) {
     if (n <= 0) return cudaSuccess;
-    int64_t blocks = (n + 7) / 8;
+    // the binary64 roots cost a warp the same for 1 row or 32: long batches
+    // once there are rows enough for every warp of the chip
+    const int per_warp = (int)std::min<int64_t>(32, std::max<int64_t>(1, n / (152 * 32)));
+    int64_t blocks = (n + 8 * per_warp - 1) / (8 * per_warp);
     if (blocks > 152 * 64) blocks = 152 * 64;
-    count_launches(1);
-    build_kernel<<<(unsigned)blocks, 256, 0, st>>>(vecs, n, m, m_pad, m_raw, codes, scale, vnorm,
-                                                   enorm, raw, status, fixed_scale);
-    return cudaGetLastError();
+    const int aligned =
+        m % 4 == 0 && (reinterpret_cast<uintptr_t>(vecs) & 15u) == 0 ? 1 : 0;
+    auto run = [&](auto kernel) {
+        count_launches(1);
+        kernel<<<(unsigned)blocks, 256, 0, st>>>(vecs, n, m, m_pad, m_raw, codes, scale, vnorm,
+                                                 enorm, raw, status, fixed_scale, aligned, per_warp);
+        return cudaGetLastError();
+    };
+    switch ((m_pad + 127) / 128) {
+        case 1: return run(build_kernel<1>);
+        case 2: return run(build_kernel<2>);
+        case 3: return run(build_kernel<3>);
+        case 4: return run(build_kernel<4>);
+        case 5: return run(build_kernel<5>);
+        case 6: return run(build_kernel<6>);
+        case 7: return run(build_kernel<7>);
+        case 8: return run(build_kernel<8>);
+        default: return run(build_kernel<0>);
+    }
 }
 
 // Largest |v_j| over count floats, as float bits (nonnegative floats order
@@ -86,135 +251,171 @@ cudaError_t launch_scale_from_maxabs(const unsigned int* maxabs_bits, float* s, 
     return cudaGetLastError();
 }
 
-// Queries: one block of kEncThreads per query, the quantizer of
-// quantize_row_warp spread over its warps (maxima and exact integer sums do
-// not depend on the order, so the results are bit-identical), plus the
-// query-side scalars of App. A.1: ||s_q z_q|| rounded up and
-// gamma_m = RU(a / RD(1 - a)), a = (8m + 64) 2^-23.
+// Queries: one block of kEncThreads per query, the quantizer of the rows
+// spread over its warps (maxima and exact integer sums do not depend on the
+// order, so the results are bit-identical), plus the query-side scalars of
+// App. A.1: ||s_q z_q|| rounded up and gamma_m = RU(a / RD(1 - a)),
+// a = (8m + 64) 2^-23.
 // q and qraw may be the same buffer (a host query staged in qraw): the raw
-// copy, after every read of the first pass, rewrites the values it read.
+// copy rewrites the values that the first loop read.
+// Bound by latency (one block, a few values per thread): float32 and integer
+// terms as in build_kernel, three block barriers, and the three square roots
+// on three warps side by side.
 constexpr int kEncThreads = 256;
 constexpr int kEncWarps = kEncThreads / kWarp;
+
+struct EncShared {
+    uint32_t u[kEncWarps][2];
+    unsigned long long t[kEncWarps][3];
+    float root[3];
+};
+
+// The scalars of a query outside the fast path (see build_kernel), in
+// binary64 by one warp; codes to z.
+static __device__ __noinline__ QueryScalars encode_query_slow(const float* v, int m, int m_pad,
+                                                              int8_t* z) {
+    const int lane = threadIdx.x & 31;
+    const RowQuant r = quantize_row_warp(v, m, m_pad, z);
+    QueryScalars out{};
+    out.status = r.status;
+    out.s = r.s;
+    out.qnorm = r.vnorm;
+    out.enorm = r.enorm;
+    // ||q_hat||: the values s z_j are exact in binary64
+    double M = 0.0;
+    for (int j = lane; j < m; j += kWarp) M = fmax(M, fabs(__dmul_rn((double)r.s, (double)z[j])));
+    M = warp_max(M);
+    long long T = 0;
+    const int e = M > 0.0 ? norm_exponent(M) : 0;
+    if (M > 0.0)
+        for (int j = lane; j < m; j += kWarp) T += norm_term(__dmul_rn((double)r.s, (double)z[j]), e);
+    out.qhat = norm_finish(warp_sum(T), e);
+    if (out.status == 0 && isinf(out.qhat)) out.status = PVS_ERR_OVERFLOW;
+    return out;
+}
 
 __global__ void __launch_bounds__(kEncThreads) encode_kernel(const float* q, int nq, int m,
                                                             int m_pad, int m_raw,
                                                             int8_t* __restrict__ zq, float* qraw,
                                                             QueryScalars* __restrict__ qs) {
-    __shared__ float s_f[kEncWarps];
-    __shared__ double s_d[kEncWarps];
-    __shared__ long long s_a[kEncWarps], s_b[kEncWarps];
-    __shared__ int s_i[kEncWarps];
+    __shared__ EncShared sh;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int qi = blockIdx.x;
     if (qi >= nq) return;
     const float* v = q + (int64_t)qi * m;
+    float* raw = qraw + (int64_t)qi * m_raw;
     int8_t* z = zq + (int64_t)qi * m_pad;
-    auto block_max_f = [&](float x) {
-        x = warp_max(x);
-        if (lane == 0) s_f[warp] = x;
-        __syncthreads();
-        float r = s_f[0];
-        for (int w = 1; w < kEncWarps; ++w) r = fmaxf(r, s_f[w]);
-        __syncthreads();
-        return r;
+    constexpr int kKeep = 4;   // values per thread held in registers (1,024 dimensions)
+    float keep[kKeep];
+    // f(j, q_j) for this thread's j < limit (q_j = 0 from m on)
+    auto each = [&](int limit, auto f) {
+#pragma unroll
+        for (int i = 0; i < kKeep; ++i)
+            if (t + i * kEncThreads < limit) f(t + i * kEncThreads, keep[i]);
+        for (int j = t + kKeep * kEncThreads; j < limit; j += kEncThreads)
+            f(j, j < m ? v[j] : 0.0f);
     };
-    auto block_max_d = [&](double x) {
-        x = warp_max(x);
-        if (lane == 0) s_d[warp] = x;
-        __syncthreads();
-        double r = s_d[0];
-        for (int w = 1; w < kEncWarps; ++w) r = fmax(r, s_d[w]);
-        __syncthreads();
-        return r;
-    };
-    auto block_sum2 = [&](long long& x, long long& y) {
-        x = warp_sum(x);
-        y = warp_sum(y);
-        if (lane == 0) {
-            s_a[warp] = x;
-            s_b[warp] = y;
-        }
-        __syncthreads();
-        x = 0;
-        y = 0;
-        for (int w = 0; w < kEncWarps; ++w) {
-            x += s_a[w];
-            y += s_b[w];
-        }
-        __syncthreads();
-    };
+    const float a = (float)((8.0 * (double)m + 64.0) * 0x1p-23);   // exact
+    const float gamma = __fdiv_ru(a, __fsub_rd(1.0f, a));
     // finiteness and max |q_j|
-    float maxabs = 0.0f;
-    bool finite = true;
-    for (int j = t; j < m; j += kEncThreads) {
-        const float x = v[j];
-        finite &= isfinite(x);
-        maxabs = fmaxf(maxabs, fabsf(x));
+    uint32_t mx = 0;
+#pragma unroll
+    for (int i = 0; i < kKeep; ++i) {
+        const int j = t + i * kEncThreads;
+        keep[i] = j < m ? v[j] : 0.0f;
     }
-    finite = __all_sync(0xffffffffu, finite);
-    if (lane == 0) s_i[warp] = finite;
-    maxabs = block_max_f(maxabs);   // (its barrier publishes s_i)
-    for (int w = 0; w < kEncWarps; ++w) finite &= s_i[w] != 0;
-    for (int j = t; j < m_raw; j += kEncThreads) qraw[(int64_t)qi * m_raw + j] = j < m ? v[j] : 0.0f;
-    QueryScalars out{};
-    out.status = 0;
-    if (finite) {
-        float s;
-        if (maxabs == 0.0f) {
-            s = 1.0f;
-        } else {
-            s = __fdiv_rn(maxabs, 127.0f);
-            if (s == 0.0f) s = __uint_as_float(1u);  // 2^-149
+    each(m_raw, [&](int j, float x) {
+        mx = max(mx, __float_as_uint(fabsf(x)));
+        raw[j] = x;
+    });
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) sh.u[warp][0] = mx;
+    __syncthreads();
+    for (int w = 0; w < kEncWarps; ++w) mx = max(mx, sh.u[w][0]);
+    if (mx >= 0x7f800000u) {   // an infinity or a NaN
+        if (t == 0) {
+            QueryScalars out{};
+            out.status = PVS_ERR_NONFINITE;
+            out.gamma = gamma;
+            qs[qi] = out;
         }
-        // codes and residual maximum (each thread later reads only its own codes)
-        double emax = 0.0;
-        for (int j = t; j < m_pad; j += kEncThreads) {
-            int c = 0;
-            if (j < m && maxabs != 0.0f) {
-                const float tq = __fdiv_rn(v[j], s);
-                float rt = roundf(tq);                     // half away from zero
-                rt = fminf(fmaxf(rt, -127.0f), 127.0f);
-                c = (int)rt;
-                const double e = __dsub_rn((double)v[j], __dmul_rn((double)s, (double)c));  // exact
-                emax = fmax(emax, fabs(e));
-            }
-            z[j] = (int8_t)c;
-        }
-        emax = block_max_d(emax);
-        // norm bounds of q and of its residual
-        long long Tv = 0, Te = 0;
-        const int ev = maxabs > 0.0f ? norm_exponent((double)maxabs) : 0;
-        const int ee = emax > 0.0 ? norm_exponent(emax) : 0;
-        for (int j = t; j < m; j += kEncThreads) {
-            const double x = (double)v[j];
-            if (maxabs > 0.0f) Tv += norm_term(x, ev);
-            if (emax > 0.0) {
-                const int c = z[j];
-                Te += norm_term(__dsub_rn(x, __dmul_rn((double)s, (double)c)), ee);
-            }
-        }
-        block_sum2(Tv, Te);
-        out.s = s;
-        out.qnorm = norm_finish(Tv, ev);
-        out.enorm = norm_finish(Te, ee);
-        if (isinf(out.qnorm) || isinf(out.enorm)) out.status = PVS_ERR_OVERFLOW;
-        // ||q_hat||: the values s z_j are exact in binary64
-        double M = 0.0;
-        for (int j = t; j < m; j += kEncThreads) M = fmax(M, fabs(__dmul_rn((double)s, (double)z[j])));
-        M = block_max_d(M);
-        long long T = 0, unused = 0;
-        const int e = M > 0.0 ? norm_exponent(M) : 0;
-        if (M > 0.0)
-            for (int j = t; j < m; j += kEncThreads) T += norm_term(__dmul_rn((double)s, (double)z[j]), e);
-        block_sum2(T, unused);
-        out.qhat = norm_finish(T, e);
-        if (out.status == 0 && isinf(out.qhat)) out.status = PVS_ERR_OVERFLOW;
-    } else {
-        out.status = PVS_ERR_NONFINITE;
+        return;
     }
+    const float s = mx == 0 ? 1.0f : __fdiv_rn(__uint_as_float(mx), 127.0f);
+    bool slow = mx != 0 && (mx < 0x00800000u || s < kFastScaleMin);
+    __syncthreads();   // sh.u is written again
+    // codes, residual maximum, largest code
+    const float rs = __frcp_rn(s);
+    uint32_t emx = 0, zmx = 0;
+    if (!slow) {
+        each(m_pad, [&](int j, float x) {
+            uint32_t y;
+            const float c = code_of(x, s, rs, y);
+            z[j] = (int8_t)(y & 0xffu);
+            emx = max(emx, __float_as_uint(fabsf(__fmaf_rn(-s, c, x))));
+            zmx = max(zmx, (uint32_t)fabsf(c));
+        });
+        emx = __reduce_max_sync(0xffffffffu, emx);
+        zmx = __reduce_max_sync(0xffffffffu, zmx);
+        if (lane == 0) {
+            sh.u[warp][0] = emx;
+            sh.u[warp][1] = zmx;
+        }
+        __syncthreads();
+        for (int w = 0; w < kEncWarps; ++w) {
+            emx = max(emx, sh.u[w][0]);
+            zmx = max(zmx, sh.u[w][1]);
+        }
+        slow = emx >= (__float_as_uint(s) & 0x7f800000u) || (emx != 0 && emx < 0x00800000u);
+    }
+    if (slow) {
+        __syncthreads();   // the codes above are rewritten
+        if (warp == 0) {
+            QueryScalars out = encode_query_slow(raw, m, m_pad, z);
+            out.gamma = gamma;
+            if (lane == 0) qs[qi] = out;
+        }
+        return;
+    }
+    // norm bounds of q, of its residual and of q_hat = s z: with s = S 2^p
+    // (S < 2^24), (s z)^2 = (S |z|)^2 2^(2p), and the largest S |z| has
+    // `bits` bits, so t = ceil((S |z|)^2 / 2^(2 bits - 48))
+    const int Ev = max((int)(mx >> 23), 1), Ee = max((int)(emx >> 23), 1);
+    const uint32_t S = (__float_as_uint(s) & 0x7fffffu) | 0x800000u;
+    const int bits = 32 - __clz((int)(S * zmx));
+    const int dh = max(2 * bits - 48, 0);   // (bits >= 24 unless every code is 0)
+    unsigned long long T[3] = {0, 0, 0};
+    each(m, [&](int, float x) {
+        uint32_t y;
+        const float c = code_of(x, s, rs, y);
+        T[0] += norm_term_bits(__float_as_uint(fabsf(x)), Ev);
+        T[1] += norm_term_bits(__float_as_uint(fabsf(__fmaf_rn(-s, c, x))), Ee);
+        const unsigned long long P = (unsigned long long)S * (uint32_t)fabsf(c);
+        T[2] += (P * P + ((1ull << dh) - 1ull)) >> dh;
+    });
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        T[k] = warp_sum(T[k]);
+        if (lane == 0) sh.t[warp][k] = T[k];
+    }
+    __syncthreads();
+    if (lane == 0 && warp < 3) {
+        unsigned long long sum = 0;
+        for (int w = 0; w < kEncWarps; ++w) sum += sh.t[w][warp];
+        // exponent of the maximum: M = f 2^e with f in [0.5, 1)
+        const int es = (int)(__float_as_uint(s) >> 23) - 150 + bits;
+        const int e = warp == 0 ? Ev - 126 : warp == 1 ? Ee - 126 : es;
+        sh.root[warp] = norm_finish((long long)sum, e);
+    }
+    __syncthreads();
     if (t == 0) {
-        const float a = (float)((8.0 * (double)m + 64.0) * 0x1p-23);   // exact
-        out.gamma = __fdiv_ru(a, __fsub_rd(1.0f, a));
+        QueryScalars out{};
+        out.s = s;
+        out.qnorm = sh.root[0];
+        out.enorm = sh.root[1];
+        out.qhat = sh.root[2];
+        out.gamma = gamma;
+        if (isinf(out.qnorm) || isinf(out.enorm) || isinf(out.qhat)) out.status = PVS_ERR_OVERFLOW;
         qs[qi] = out;
     }
 }

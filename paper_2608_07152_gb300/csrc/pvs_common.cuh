@@ -138,6 +138,39 @@ __device__ inline float norm_finish(long long T, int e) {
     return __double2float_ru(root);
 }
 
+// The terms t_j of a norm bound in integers.  A float32 x = M 2^p (M < 2^24)
+// has x^2 = M^2 2^(2p) exactly, so with E the biased exponent field of the
+// largest |x_j| (a normal number: e = E - 126) and F that of x (1 for a
+// subnormal), t = ceil(M^2 / 2^(2 (E - F))); a shift of 48 or more leaves 1
+// for every x != 0.  Equal to norm_term bit for bit (its RU64 product is
+// exact here), without binary64, which GB300 runs at 1/64 of the float32
+// rate.  bits: those of |x|.
+__device__ __forceinline__ unsigned long long norm_term_bits(uint32_t bits, int E) {
+    const int F = (int)(bits >> 23);
+    const uint32_t M = (bits & 0x7fffffu) | (F ? 0x800000u : 0u);
+    const int d = min(2 * (E - max(F, 1)), 48);
+    return ((unsigned long long)M * M + ((1ull << d) - 1ull)) >> d;
+}
+
+// The code of v against scale s (r = RN(1 / s), s >= 2^-100): its value
+// round_half_away(RN(v / s)) as a float, and in y the low byte of the code.
+// |v r - v / s| < 2^-15 for |v / s| < 128, so a product further than 2^-14
+// from every half-integer rounds as the quotient does; the others divide.
+__device__ __forceinline__ float code_of(float v, float s, float r, uint32_t& y) {
+    const float kRound = 12582912.0f;   // 1.5 2^23: the sum's last bit is an integer
+    const float t = __fmul_rn(v, r);
+    float f = __fadd_rn(t, kRound);
+    float c = __fsub_rn(f, kRound);
+    if (!(fabsf(__fsub_rn(t, c)) < 0.5f - 0x1p-14f)) {
+        c = roundf(__fdiv_rn(v, s));   // half away from zero
+        f = __fadd_rn(c, kRound);
+    }
+    y = __float_as_uint(f);
+    return c;
+}
+
+constexpr float kFastScaleMin = 0x1p-100f;   // smaller scales: the binary64 quantizer
+
 // ---------------------------------------------------------------------------
 // One warp quantizes one row of m float32 values (Sec. 2.3.1):
 //   s = RN(maxabs / 127) (zero vector: 1; underflow: smallest subnormal),
