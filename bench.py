@@ -1488,19 +1488,24 @@ def main_passage(args, pvs, synth, torch, np, rank, world, local, dev, pg):
     e2e_elapsed = slowest(pg, e2e_elapsed, dev)
     e2e_value = ranks_total / e2e_elapsed
 
-    # ---- roofline of the grouped interval pass ----
+    # ---- roofline of the pass over the codes that the executor used ----
     m_pad = ((DIM + 63) // 64) * 64
     passes = st1["interval_passes"] - st0["interval_passes"]
     pass_ms = (st1["interval_ms"] - st0["interval_ms"]) / max(passes, 1)
+    per_pass = n_timed / max(passes, 1)
+    blocks = per_pass > group   # blocks on the tensor cores: working sets only, no bounds
     read_bytes = n * (m_pad + 12)
     # bounds (lo, hi) of every row per query, and with groups the largest
     # upper bound of each 16-row block per query
-    write_bytes = 8 * n * group + (4 * ((n + 15) // 16) * group if group > 1 else 0)
+    write_bytes = 0 if blocks else (
+        8 * n * group + (4 * ((n + 15) // 16) * group if group > 1 else 0))
     alg_bytes = read_bytes + write_bytes
     achieved = alg_bytes / (pass_ms / 1e3) / 1e9
     peak, peak_kind = measured_peaks()
-    kernel = "interval_group_kernel" if group > 1 else "interval_pass_kernel"
-    traffic = (interval_traffic(n, "interval_group_kernel_passage_traffic.json") if group > 1
+    kernel = ("batch_stream_kernel" if blocks else
+              "interval_group_kernel" if group > 1 else "interval_pass_kernel")
+    traffic = (None if blocks else
+               interval_traffic(n, "interval_group_kernel_passage_traffic.json") if group > 1
                else interval_traffic(n))
 
     line = {
@@ -1510,13 +1515,13 @@ def main_passage(args, pvs, synth, torch, np, rank, world, local, dev, pg):
         "scaling": "weak", "vs_baseline": None, "dtype": "int8", "data": "synthetic",
         "config": {"workload": WORKLOAD, "N": n, "d": DIM, "queries_per_step": nq,
                    "ranks_per_query": RANKS_PER_QUERY, "chunk": CHUNK,
-                   "queries_per_pass": group, "executor_workers": PIPELINE,
+                   "queries_per_pass": per_pass, "executor_workers": PIPELINE,
                    "l2": "no flush: each interval pass streams 6.9 GB of codes (> 129 MB L2)",
                    "parallelism": f"replicas x{world} (queries sharded, no collective)"},
         "e2e": {"value": e2e_value, "unit": UNIT,
                 "h2d_bytes_per_step": nq * DIM * 4,
                 "d2h_bytes_per_step": nq * RANKS_PER_QUERY * (8 + 4),
-                "path": f"pvs_executor_run: {PIPELINE} native workers, {group} queries per "
+                "path": f"pvs_executor_run: {PIPELINE} native workers, {per_pass:.0f} queries per "
                         f"pass, pages of {CHUNK} through batched pulls, pinned host queries and "
                         "outputs",
                 "same_ranks_as_value_leg": same},
@@ -1531,8 +1536,8 @@ def main_passage(args, pvs, synth, torch, np, rank, world, local, dev, pg):
                        "first_1000_p50": statistics.median(lat1000),
                        "first_1000_p95": sorted(lat1000)[int(0.95 * (len(lat1000) - 1))],
                        "note": "a lone query with its own cursor and single-query pass"},
-        "interval_pass": {"ms": pass_ms, "GBps": achieved, "queries_per_pass": group,
-                          "ms_per_query": pass_ms / group, "passes_timed": passes},
+        "interval_pass": {"ms": pass_ms, "GBps": achieved, "queries_per_pass": per_pass,
+                          "ms_per_query": pass_ms / max(per_pass, 1), "passes_timed": passes},
         "single_query_pass": single_pass_record(lone, n, m_pad, peak),
         "per_query": {"refined_mean": (st1["refined"] - st0["refined"]) / n_timed},
         "build_s": build_s,

@@ -19,6 +19,14 @@
  * codes for all G queries) and each page of the G cursors is one batched
  * pull; every request still receives its own pages.
  *
+ * A run of more than G >= 2 requests, of at most 1,024 ranks each, over a
+ * corpus of at least 65,536 vectors of 65 .. 1,024 dimensions is served in
+ * blocks of up to 128 requests (96 above 768 dimensions): one tensor-core pass over the codes
+ * (as pvs_cursor_open_batch) opens a block's cursors, one pull computes all
+ * their ranks, and a request's pages are handed over together.  The ranks
+ * delivered are the same.  A block in which anything fails is served again
+ * in groups, so that each request gets its own status.
+ *
  * Conventions as pvs.h: the caller owns every buffer; the index must
  * outlive the executor and must not be changed (append, delete) while a run
  * is in progress.
@@ -39,12 +47,12 @@ typedef struct pvs_executor pvs_executor;
 typedef struct pvs_executor_stats {
     int64_t requests;    /* requests served (all runs)                       */
     int64_t failed;      /* of those, requests that ended in an error         */
-    int64_t pages;       /* pvs_next calls                                    */
+    int64_t pages;       /* pages delivered                                   */
     int64_t ranks;       /* ranks delivered                                   */
     int32_t workers;     /* worker threads (and streams)                      */
     int32_t group;       /* requests per grouped open (1: none)               */
-    int64_t interval_passes; /* passes over the Int8 codes (a grouped pass
-                                counts once)                                 */
+    int64_t interval_passes; /* passes over the Int8 codes (a grouped pass,
+                                or a block's, counts once)                   */
     double interval_ms;  /* their device time, CUDA events, summed           */
     int64_t refined;     /* authoritative float32 evaluations                 */
 } pvs_executor_stats;
@@ -88,7 +96,8 @@ pvs_status pvs_executor_run_ex(pvs_executor* ex, const pvs_snapshot* snap, const
 
 /*
  * Serve requests in groups of `group` (1 .. PVS_GROUP_MAX; default 1): the
- * queries of a group share one pass over the codes.  Must not be called
+ * queries of a group share one pass over the codes (from 2 on, a run of more
+ * requests than one group may be served in larger blocks, see above).  Must not be called
  * during a run.  Errors: PVS_ERR_INVALID.
  */
 pvs_status pvs_executor_set_group(pvs_executor* ex, int32_t group);

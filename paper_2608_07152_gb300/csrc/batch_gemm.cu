@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
                         const uint64_t ad = tc::smem_desc_sw128_kmajor(sa + k * 32);
                         const uint64_t bd = tc::smem_desc_sw128_kmajor(sb + k * 32);
                         if (kCta == 2)
-                            tc::mma_bf16_pair(d, ad, bd, idesc, (kc | k) != 0 ? 1u : 0u);
+                            tc::mma_f16_pair(d, ad, bd, idesc, (kc | k) != 0 ? 1u : 0u);
                         else
                             tc::mma_bf16(d, ad, bd, idesc, (kc | k) != 0 ? 1u : 0u);
                     }
@@ -471,6 +471,22 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
 }
 
 // ---- host side ---------------------------------------------------------------
+void* tensor_map_encoder() {
+    static std::once_flag once;
+    static void* fn = nullptr;
+    std::call_once(once, [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000,
+                                             cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = p;
+        else
+            cudaGetLastError();
+    });
+    return fn;
+}
+
 namespace {
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -478,21 +494,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-EncodeTiledFn encode_fn() {
-    static std::once_flag once;
-    static EncodeTiledFn fn = nullptr;
-    std::call_once(once, [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000,
-                                             cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-        else
-            cudaGetLastError();
-    });
-    return fn;
-}
+EncodeTiledFn encode_fn() { return reinterpret_cast<EncodeTiledFn>(tensor_map_encoder()); }
 
 // bf16 matrix [rows][cols] (row stride cols), box = [64 cols x box_rows], 128B swizzle.
 bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {

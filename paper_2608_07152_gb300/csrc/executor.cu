@@ -10,8 +10,11 @@
 // caller's buffers, and closes the cursor.  With a group size G >= 2 a
 // worker takes G requests at a time: one grouped open (one pass over the
 // codes for all G queries, pvs_cursor_open_group), then every page of the G
-// cursors in one batched pull.  No lock is held across a device wait; the
-// job lock is taken only at the start and end of a run.
+// cursors in one batched pull.  A run of more requests than one group, over a
+// corpus of some size, takes blocks of requests instead (batch_block):
+// their cursors come from one tensor-core pass (cursor_open_serving) and all
+// their pages from one deep batched pull.  No lock is held across a device
+// wait; the job lock is taken only at the start and end of a run.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -37,6 +40,7 @@ struct Job {
     float* scores = nullptr;
     int32_t* n_out = nullptr;
     int32_t* status = nullptr;
+    int32_t block = 0;                  // requests per batched open (0: groups of ex->group)
 };
 
 }  // namespace
@@ -216,6 +220,104 @@ void serve_group(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first,
     if (j.on_device) cudaStreamSynchronize(st);
 }
 
+// Requests per batched open for a run, or 0 to serve in groups.  A group of 8
+// costs one read of the codes and their bounds written out (8.8M x 768: 1.24
+// ms); a batched pass of up to 128 requests reads the codes once and keeps
+// only working sets (1.2 ms + 0.5 ms for its thresholds and sorting), so it
+// wins from the second group on.  Small corpora, where a pass takes
+// microseconds, and requests deeper than one batched pull stay in groups.
+constexpr int64_t kBlockRows = 65536;
+
+int32_t batch_block(const pvs_executor* ex, const Job& j) {
+    const pvs_index* x = ex->index;
+    const int64_t rows = j.snap ? j.snap->data->rows : x->size;
+    if (ex->group < 2 || j.nq <= ex->group || j.ranks > pvs::kPullBatchMax || rows < kBlockRows ||
+        !pvs::batch_stream_supported(x->m_pad, x->num_sms))
+        return 0;
+    const int32_t most = pvs::batch_stream_queries(x->m_pad);
+    const int32_t blocks = (j.nq + most - 1) / most;
+    return (j.nq + blocks - 1) / blocks;   // equal shares
+}
+
+// Device rows of a block's host outputs, freed in stream order.
+struct BlockOut {
+    cudaStream_t st = nullptr;
+    int64_t* ids = nullptr;
+    float* scores = nullptr;
+    cudaError_t get(const pvs_index* x, size_t ranks, cudaStream_t stream) {
+        st = stream;
+        void* p = nullptr;
+        cudaError_t e = cudaMallocFromPoolAsync(&p, ranks * sizeof(int64_t), x->scratch_pool, st);
+        if (e != cudaSuccess) return e;
+        ids = static_cast<int64_t*>(p);
+        e = cudaMallocFromPoolAsync(&p, ranks * sizeof(float), x->scratch_pool, st);
+        if (e == cudaSuccess) scores = static_cast<float*>(p);
+        return e;
+    }
+    ~BlockOut() {
+        if (ids) cudaFreeAsync(ids, st);
+        if (scores) cudaFreeAsync(scores, st);
+    }
+};
+
+// Requests first .. first+count-1 from one batched open and one pull of all
+// their ranks.  Returns false, with nothing delivered, when any of it failed
+// (a non-finite query, an error of one cursor): the caller serves them in
+// groups, which gives each request its own status.
+bool serve_block(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first, int32_t count) {
+    const pvs_index* x = ex->index;
+    std::vector<pvs_cursor*> cs((size_t)count, nullptr);
+    int64_t passes = 0;
+    double pass_ms = 0.0;
+    if (pvs::cursor_open_serving(ex->index, j.snap, j.queries + (size_t)first * x->m, count,
+                                 j.on_device, j.ranks, st, cs.data(), &passes, &pass_ms) != PVS_OK)
+        return false;
+    const size_t at = (size_t)first * j.ranks, total = (size_t)count * j.ranks;
+    BlockOut buf;
+    bool ok = j.on_device || buf.get(x, total, st) == cudaSuccess;
+    std::vector<int32_t> n_out((size_t)count, 0), states((size_t)count, 0);
+    if (ok) {
+        std::vector<int64_t*> id_rows((size_t)count);
+        std::vector<float*> sc_rows((size_t)count);
+        for (int32_t i = 0; i < count; ++i) {
+            id_rows[(size_t)i] = (j.on_device ? j.ids + at : buf.ids) + (size_t)i * j.ranks;
+            sc_rows[(size_t)i] = (j.on_device ? j.scores + at : buf.scores) + (size_t)i * j.ranks;
+        }
+        ok = pvs::next_batch_rows(cs.data(), count, j.ranks, 1, id_rows.data(), sc_rows.data(),
+                                  n_out.data()) >= 0;
+    }
+    if (ok && !j.on_device)   // the block's rows are consecutive on both sides
+        ok = cudaMemcpyAsync(j.ids + at, buf.ids, total * sizeof(int64_t), cudaMemcpyDeviceToHost,
+                             st) == cudaSuccess &&
+             cudaMemcpyAsync(j.scores + at, buf.scores, total * sizeof(float),
+                             cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    std::vector<pvs_stats> stats((size_t)count);
+    if (ok) ok = pvs_cursor_stats_batch(cs.data(), count, stats.data()) == PVS_OK;   // (waits)
+    for (int32_t i = 0; ok && i < count; ++i) ok = stats[(size_t)i].state >= 0;
+    if (ok) {
+        int64_t refined = 0;
+        for (int32_t i = 0; i < count; ++i) {
+            const pvs_stats& c = stats[(size_t)i];
+            refined += c.refined;
+            // passes of the queries that the batched one left: grouped (counted
+            // by the open) or their own
+            if (cs[(size_t)i]->group_size == 1) passes += c.interval_passes;
+            pass_ms += c.interval_ms / cs[(size_t)i]->group_size;
+            const int32_t r = first + i, got = n_out[(size_t)i];
+            fill_rest(j, st, r, got);
+            j.n_out[r] = got;
+            j.status[r] = got < j.ranks ? PVS_EXHAUSTED : PVS_OK;
+            count_request(ex, PVS_OK, std::max(1, (got + j.page - 1) / j.page), got);
+        }
+        ex->passes.fetch_add(passes, std::memory_order_relaxed);
+        ex->refined.fetch_add(refined, std::memory_order_relaxed);
+        std::lock_guard<std::mutex> lk(ex->ms_mutex);
+        ex->interval_ms += pass_ms;
+    }
+    pvs_cursor_close_batch(cs.data(), count);   // (waits for the stream)
+    return ok;
+}
+
 void worker_main(pvs_executor* ex, int w) {
     cudaSetDevice(ex->index->device);
     const cudaStream_t st = ex->streams[(size_t)w];
@@ -230,14 +332,19 @@ void worker_main(pvs_executor* ex, int w) {
             j = ex->job;
         }
         const int32_t G = ex->group;
-        for (;;) {
-            const int32_t i = ex->next.fetch_add(G, std::memory_order_relaxed);
-            if (i >= j.nq) break;
-            const int32_t count = std::min(G, j.nq - i);
+        auto serve = [&](int32_t i, int32_t count) {
             if (count == 1)
                 j.status[i] = serve_one(ex, j, st, i, nullptr, 0);
             else
                 serve_group(ex, j, st, i, count);
+        };
+        const int32_t step = j.block ? j.block : G;
+        for (;;) {
+            const int32_t i = ex->next.fetch_add(step, std::memory_order_relaxed);
+            if (i >= j.nq) break;
+            const int32_t count = std::min(step, j.nq - i);
+            if (j.block && count > G && serve_block(ex, j, st, i, count)) continue;
+            for (int32_t k = 0; k < count; k += G) serve(i + k, std::min(G, count - k));
         }
         std::lock_guard<std::mutex> lk(ex->m);
         if (--ex->busy == 0) ex->done_cv.notify_all();
@@ -325,7 +432,8 @@ pvs_status pvs_executor_run_ex(pvs_executor* ex, const pvs_snapshot* snap, const
     {
         std::lock_guard<std::mutex> lk(ex->m);
         ex->job = Job{snap, queries, nq, ranks, page, buffers_on_device ? 1 : 0, ids, scores,
-                      n_out, status};
+                      n_out, status, 0};
+        ex->job.block = batch_block(ex, ex->job);
         ex->next.store(0, std::memory_order_relaxed);
         ex->busy = (int)ex->threads.size();
         ++ex->generation;

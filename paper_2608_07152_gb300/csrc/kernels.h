@@ -57,6 +57,7 @@ struct CursorRef {
 
 // ---- fused single-CTA pull (pull_kernel.cu) ----------------------------------
 constexpr int kPullFusedMax = 256;   // largest pull served by one fused launch
+constexpr int kPullBatchMax = 1024;  // largest pull of the three-launch batch form
 struct PullArgs {
     int32_t* w_id;
     float* w_lo;
@@ -67,7 +68,7 @@ struct PullArgs {
     const float* qraw;
     const float* raw;
     int m_raw;
-    int n;                    // ranks to emit, 1 .. kPullFusedMax
+    int n;                    // ranks to emit, 1 .. kPullFusedMax (batch form: kPullBatchMax)
     int32_t* cand;            // scratch, >= working-set capacity
     unsigned long long* keys; // scratch, >= working-set capacity
     int64_t* out_ids;         // device
@@ -94,7 +95,7 @@ cudaError_t launch_pull_cluster(const PullArgs& a, cudaStream_t st);
 cudaError_t launch_pull_cluster_batch(const PullArgs* host_args, int ncursors, cudaStream_t st);
 // Ranks computed ahead, handed to the callers' buffers: for every entry,
 // count ids and scores from src to dst (device or pinned host memory), in
-// stream order, one launch per 64 entries (the entries are read at launch).
+// stream order, one launch per 512 entries (the entries are read at launch).
 struct RankCopy {
     const int64_t* src_ids;
     const float* src_scores;
@@ -110,7 +111,7 @@ cudaError_t launch_refine_batch(const PullArgsPack& p, int ncursors, int blocks_
                                 int m_raw, cudaStream_t st);
 
 // ---- batched open support (pull_kernel.cu, batch_support.cu) ----------------
-constexpr int kWsSortMax = 8192;     // largest per-query working set of a batched open
+constexpr int kWsSortMax = 16384;    // largest per-query working set of a batched open
 constexpr int kFrontCap = 4096;      // frontier entries (the one-launch pull's gather capacity)
 struct WsDst {                       // a cursor's working-set arrays
     int32_t* w_id;
@@ -330,6 +331,46 @@ struct BatchArgs {
 };
 cudaError_t launch_batch_intervals(const BatchArgs& a, const uint16_t* codes_bf16,
                                    const uint16_t* qcodes_bf16, int num_sms, cudaStream_t st);
+// ---- batched interval pass over the Int8 codes (batch_stream.cu) -------------
+constexpr int kStreamQueries = 128;   // most queries per pass
+int batch_stream_queries(int m_pad);  // queries per pass over rows of m_pad bytes
+// Widest row: 96 queries' f16 codes beside the code boxes; wider rows take the
+// bf16 pass (more, smaller passes would read the codes again).
+constexpr int kStreamMaxWidth = 1024;
+struct StreamArgs {
+    int64_t rows;                 // corpus rows [0, rows) are scanned
+    int m_pad;
+    int nq, nq_pad;               // queries; nq_pad multiple of 32, <= kStreamQueries
+    const float* scale;
+    const float* vnorm;
+    const float* enorm;
+    const uint32_t* tomb;         // tombstones of the snapshot, or null
+    const QueryScalars* qs;       // [nq]
+    int mode;                     // 0: sample, 1: filter
+    int tile_stride;              // process 128-row tiles 0, s, 2s, ...
+    int group_max;                // sample: 1: the largest of each 32 rows, 0: every row
+    float* dump_lo;               // sample: [nq][dump_ld]; entry 4 i + g: rows 32 g .. of
+    int64_t dump_ld;              //   tile i s, or entry 128 i + r: row r of tile i s
+    const float* tau;             // filter: [nq] thresholds
+    const float* theta;           // filter: [nq] from launch_stream_theta
+    int32_t* w_id;                // filter: as BatchArgs
+    float* w_lo;
+    float* w_hi;
+    int w_cap;
+    unsigned int* w_len;
+    unsigned int* h_eff;
+    int* status;
+};
+bool batch_stream_supported(int m_pad, int num_sms);
+cudaError_t launch_batch_stream(const StreamArgs& a, const int8_t* codes, const uint16_t* qcodes_f16,
+                                int num_sms, cudaStream_t st);
+cudaError_t launch_stream_theta(const QueryScalars* qs, int nq, const unsigned int* maxes,
+                                const float* tau, float* theta, cudaStream_t st);
+// dst[0 .. count) = the codes as f16, dst[count .. padded) = 0.
+cudaError_t launch_codes_to_f16(const int8_t* src, uint16_t* dst, int64_t count, int64_t padded,
+                                cudaStream_t st);
+// The driver's cuTensorMapEncodeTiled (null if unavailable).
+void* tensor_map_encoder();
 // status_out[i] = *refs[i].status; ctr_out[i] = *refs[i].ctr (ctr_out may be null).
 cudaError_t launch_gather_state(const CursorRef* refs, int n, int* status_out,
                                 DevCounters* ctr_out, cudaStream_t st);

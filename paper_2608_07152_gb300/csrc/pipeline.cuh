@@ -56,13 +56,18 @@ __device__ inline bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Wait for the phase with the given parity to complete; false after
+constexpr int kWaitTries = 64;   // attempts before the timer is read
+
+// Wait for the phase with the given parity to complete; false after about
 // limit_ns nanoseconds of device time.  limit_ns == 0 does not wait at all:
 // true only if the phase has already completed.
 __device__ inline bool mbar_wait(uint64_t* bar, uint32_t parity,
                                  unsigned long long limit_ns = kWaitLimitNs) {
     if (limit_ns == 0) return mbar_test_wait(bar, parity);
-    if (mbar_try_wait(bar, parity)) return true;
+    // ordinary waits end here: reading the global timer takes about a
+    // microsecond, which a wait that has just begun must not add to itself
+    for (int i = 0; i < kWaitTries; ++i)
+        if (mbar_try_wait(bar, parity)) return true;
     const unsigned long long t0 = globaltimer();
     while (true) {
         for (int i = 0; i < 32; ++i)

@@ -763,7 +763,7 @@ cudaError_t launch_pull_cluster(const PullArgs& a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-constexpr int kCopiesPerLaunch = 64;
+constexpr int kCopiesPerLaunch = 512;   // 20 KB of kernel parameters
 struct RankCopyPack {
     RankCopy e[kCopiesPerLaunch];
 };

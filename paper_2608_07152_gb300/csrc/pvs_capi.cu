@@ -198,15 +198,15 @@ std::shared_ptr<SnapData> make_snapdata(const pvs_index* x) {
 }
 
 void cursor_free_device(pvs_cursor* c) {
-    dev_free(c->zq), dev_free(c->qraw), dev_free(c->qs);
+    if (c->small) cudaFree(c->small);
+    c->small = nullptr;
+    c->zq = nullptr;
     dev_free(c->lo), dev_free(c->hi), dev_free(c->bmax);
-    dev_free(c->w_id), dev_free(c->w_lo), dev_free(c->w_hi);
     dev_free(c->compact_scratch), dev_free(c->slot_top);
     c->slot_cap = 0;
-    dev_free(c->cand), dev_free(c->keys), dev_free(c->keys_tmp), dev_free(c->front);
-    if (c->sort_scratch) cudaFree(c->sort_scratch);
-    c->sort_scratch = nullptr;
-    dev_free(c->sel), dev_free(c->ctr), dev_free(c->d_status);
+    if (c->ws_slab) cudaFree(c->ws_slab);
+    c->ws_slab = nullptr;
+    c->w_id = nullptr;
     dev_free(c->d_ids), dev_free(c->d_scores);
     if (c->h_ids) cudaFreeHost(c->h_ids);
     if (c->h_scores) cudaFreeHost(c->h_scores);
@@ -285,27 +285,76 @@ pvs_status cursor_alloc_full(pvs_cursor* c) {
     return PVS_OK;
 }
 
+// Hands out parts of one allocation, each on a 256-byte boundary; with a null
+// base it only adds up their sizes.
+struct Carve {
+    char* base;
+    size_t used = 0;
+    template <typename T>
+    void take(T** p, size_t count) {
+        if (base) *p = reinterpret_cast<T*>(base + used);
+        used += (std::max<size_t>(count, 1) * sizeof(T) + 255) / 256 * 256;
+    }
+};
+
 // Working-set arrays and pull scratch for up to `cap` entries (contents are
-// not preserved when they grow).
+// not preserved when they grow): one allocation.
 pvs_status cursor_alloc_ws(pvs_cursor* c, int64_t cap) {
     cap = std::max<int64_t>(cap, 1);
-    if (!c->front) PVS_CUDA(dev_alloc(&c->front, (size_t)kFrontCap));
     if (c->w_id && c->cap_w >= cap) return PVS_OK;
-    dev_free(c->w_id), dev_free(c->w_lo), dev_free(c->w_hi);
-    dev_free(c->cand), dev_free(c->keys), dev_free(c->keys_tmp);
-    if (c->sort_scratch) cudaFree(c->sort_scratch);
-    c->sort_scratch = nullptr;
+    if (c->ws_slab) cudaFree(c->ws_slab);
+    c->ws_slab = nullptr;
+    c->w_id = nullptr;
     c->cap_w = 0;
     const size_t n = (size_t)cap;
-    PVS_CUDA(dev_alloc(&c->w_id, n));
-    PVS_CUDA(dev_alloc(&c->w_lo, n));
-    PVS_CUDA(dev_alloc(&c->w_hi, n));
-    PVS_CUDA(dev_alloc(&c->cand, n));
-    PVS_CUDA(dev_alloc(&c->keys, n));
-    PVS_CUDA(dev_alloc(&c->keys_tmp, n));
-    PVS_CUDA(cudaMalloc(&c->sort_scratch, radix_sort_scratch_bytes((int64_t)n)));
+    auto carve = [&](char* base) {
+        Carve k{base};
+        char* scratch = nullptr;
+        k.take(&c->w_id, n);
+        k.take(&c->w_lo, n);
+        k.take(&c->w_hi, n);
+        k.take(&c->cand, n);
+        k.take(&c->keys, n);
+        k.take(&c->keys_tmp, n);
+        k.take(&c->front, (size_t)kFrontCap);
+        k.take(&scratch, radix_sort_scratch_bytes((int64_t)n));
+        if (base) c->sort_scratch = scratch;
+        return k.used;
+    };
+    PVS_CUDA(cudaMalloc(&c->ws_slab, carve(nullptr)));
+    carve(static_cast<char*>(c->ws_slab));
     c->cap_w = cap;
     return PVS_OK;
+}
+
+// The cursor's query buffers, selection state, counters and status word: one
+// allocation.
+cudaError_t cursor_alloc_small(pvs_cursor* c, const pvs_index* x) {
+    if (c->small) return cudaSuccess;
+    auto carve = [&](char* base) {
+        Carve k{base};
+        k.take(&c->zq, (size_t)x->m_pad);
+        k.take(&c->qraw, (size_t)x->m_raw);
+        k.take(&c->qs, 1);
+        k.take(&c->sel, 1);
+        k.take(&c->ctr, 1);
+        k.take(&c->d_status, 1);
+        return k.used;
+    };
+    const cudaError_t e = cudaMalloc(&c->small, carve(nullptr));
+    if (e != cudaSuccess) {
+        c->small = nullptr;
+        return e;
+    }
+    carve(static_cast<char*>(c->small));
+    return cudaSuccess;
+}
+
+// The pinned words that a cursor's own copies and status polls use; batched
+// cursors read theirs through gather_state and mostly need none.
+cudaError_t cursor_pinned(pvs_cursor* c) {
+    if (c->h_small) return cudaSuccess;
+    return cudaMallocHost(&c->h_small, 16 * sizeof(unsigned int));
 }
 
 pvs_status cursor_alloc_rows(pvs_cursor* c) {
@@ -375,6 +424,7 @@ bool wait_published(const int* word) {
 // Read the device status word; a failure makes the cursor Failed.
 pvs_status check_device_status(pvs_cursor* c) {
     cudaStream_t st = c->stream;
+    PVS_CUDA(cursor_pinned(c));
     PVS_CUDA(cudaMemcpyAsync(c->h_small, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
     PVS_CUDA(cudaStreamSynchronize(st));
     const int s = (int)c->h_small[0];
@@ -648,7 +698,8 @@ pvs_status pull(pvs_cursor* c, int64_t n_eff, int64_t* d_ids, float* d_scores,
     }
     const int grid_w = grid_for(c, std::min<int64_t>(c->rows, (int64_t)1 << 22));
     // rows leave without the one-launch pull's frontier count: drop the frontier
-    cudaError_t e = cudaMemsetAsync(&c->ctr->front_k, 0, sizeof(unsigned int), st);
+    cudaError_t e = cursor_pinned(c);
+    if (e == cudaSuccess) e = cudaMemsetAsync(&c->ctr->front_k, 0, sizeof(unsigned int), st);
     if (e == cudaSuccess)
         e = launch_select_f32(c->w_lo, &c->ctr->w_len, (uint64_t)n_eff, c->sel, grid_w, st);
     if (e == cudaSuccess)
@@ -771,7 +822,9 @@ struct BatchQueries {
     int8_t* zq = nullptr;          // [nq][m_pad]
     float* qraw = nullptr;         // [nq][m_raw]
     QueryScalars* qs = nullptr;    // [nq]
-    uint16_t* qcodes = nullptr;    // [nq_pad][m_pad] bf16, zero rows past nq
+    // [nq_pad][m_pad], zero rows past nq: f16 for the pass over the Int8 codes
+    // (batch_stream.cu), bf16 for the bf16 one (batch_gemm.cu)
+    uint16_t* qcodes = nullptr;
 };
 
 // bf16 copy of every code row (the tensor-core pass reads it), extended on
@@ -800,7 +853,7 @@ pvs_status ensure_bf16(pvs_index* x, cudaStream_t st) {
 // reports a non-finite query; otherwise the caller reads bq->qs[i].status
 // later, at its own synchronisation point.
 pvs_status encode_batch(pvs_index* x, const float* queries, int nq, bool on_device, DevBuf& buf,
-                        BatchQueries* bq, cudaStream_t st, bool check_now = true) {
+                        BatchQueries* bq, cudaStream_t st, bool check_now, bool f16) {
     bq->nq = nq;
     bq->nq_pad = (int)round_up(nq, 32);
     bq->zq = buf.get<int8_t>((size_t)nq * x->m_pad);
@@ -817,9 +870,12 @@ pvs_status encode_batch(pvs_index* x, const float* queries, int nq, bool on_devi
     }
     if (!bq->zq || !bq->qraw || !bq->qs || !bq->qcodes) return PVS_ERR_OOM;
     PVS_CUDA(launch_encode_queries(qd, nq, x->m, x->m_pad, x->m_raw, bq->zq, bq->qraw, bq->qs, st));
-    PVS_CUDA(cudaMemsetAsync(bq->qcodes, 0, (size_t)bq->nq_pad * x->m_pad * sizeof(uint16_t), st));
-    PVS_CUDA(launch_codes_to_bf16(bq->zq, bq->qcodes, (int64_t)nq * x->m_pad, st));
-    {
+    if (f16) {
+        PVS_CUDA(launch_codes_to_f16(bq->zq, bq->qcodes, (int64_t)nq * x->m_pad,
+                                     (int64_t)bq->nq_pad * x->m_pad, st));
+    } else {
+        PVS_CUDA(cudaMemsetAsync(bq->qcodes, 0, (size_t)bq->nq_pad * x->m_pad * sizeof(uint16_t), st));
+        PVS_CUDA(launch_codes_to_bf16(bq->zq, bq->qcodes, (int64_t)nq * x->m_pad, st));
         std::lock_guard<std::mutex> lock(x->pass_mutex);
         pvs_status s = ensure_bf16(x, st);
         if (s != PVS_OK) return s;
@@ -859,13 +915,7 @@ pvs_status acquire_cursor(pvs_index* x, const std::shared_ptr<SnapData>& sd, pvs
     c->rows = sd->rows;
     c->visible = sd->visible;
     *out = c;
-    if (!c->zq &&
-        (dev_alloc(&c->zq, (size_t)x->m_pad) != cudaSuccess ||
-         dev_alloc(&c->qraw, (size_t)x->m_raw) != cudaSuccess ||
-         dev_alloc(&c->qs, 1) != cudaSuccess || dev_alloc(&c->sel, 1) != cudaSuccess ||
-         dev_alloc(&c->ctr, 1) != cudaSuccess || dev_alloc(&c->d_status, 1) != cudaSuccess ||
-         cudaMallocHost(&c->h_small, 16 * sizeof(unsigned int)) != cudaSuccess))
-        return PVS_ERR_OOM;
+    if (cursor_alloc_small(c, x) != cudaSuccess) return PVS_ERR_OOM;
     if (zero_state) {
         PVS_CUDA(cudaMemsetAsync(c->ctr, 0, sizeof(DevCounters), c->stream));
         PVS_CUDA(cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream));
@@ -875,11 +925,11 @@ pvs_status acquire_cursor(pvs_index* x, const std::shared_ptr<SnapData>& sd, pvs
 }
 
 // Up to kBatchMax cursors from one batched pass:
-//   1. encode the queries; bf16 query codes for the MMA;
-//   2. thresholds: on every 16th 128-row tile (every tile for small corpora)
-//      the pass dumps all intervals; tau_q = the k-th largest lower bound of
-//      query q there, k sized so that about 3x the horizon rows of the whole
-//      corpus reach it;
+//   1. encode the queries; f16 (or bf16) query codes for the MMA;
+//   2. thresholds: on every stride-th 128-row tile (every tile for small
+//      corpora) the pass leaves the lower bounds; tau_q = the k-th largest of
+//      query q there, k sized so that about twice the horizon's rows of the
+//      whole corpus reach it;
 //   3. the filter pass appends every row with hi >= tau_q to query q's
 //      working set and counts the rows with lo >= tau_q: those rows precede
 //      every row outside the working set, so the cursor can deliver that many
@@ -887,32 +937,41 @@ pvs_status acquire_cursor(pvs_index* x, const std::shared_ptr<SnapData>& sd, pvs
 //   4. each working set is sorted by id into its cursor.
 // A query whose working set overflows, or whose count is 0, falls back to a
 // single-query interval pass at its first pull.
+// Steps 2 and 3 read the Int8 codes up to kStreamQueries queries at a time
+// (batch_stream.cu) for rows of 128 .. kStreamMaxWidth bytes, else a bf16 copy
+// of them (batch_gemm.cu).
 pvs_status open_batch_group(pvs_index* x, const std::shared_ptr<SnapData>& sd,
                             const float* queries, int nq, bool on_device, int horizon,
                             cudaStream_t st, pvs_cursor** out) {
     DevBuf buf(st, x->scratch_pool);
     BatchQueries bq;
+    const bool stream = batch_stream_supported(x->m_pad, x->num_sms);
     // one synchronisation at the end: query statuses are read with the pass's
-    pvs_status s = encode_batch(x, queries, nq, on_device, buf, &bq, st, /*check_now=*/false);
+    pvs_status s = encode_batch(x, queries, nq, on_device, buf, &bq, st, /*check_now=*/false, stream);
     if (s != PVS_OK) return s;
-    for (int i = 0; i < nq; ++i) {
-        s = acquire_cursor(x, sd, &out[i], /*zero_state=*/false);
-        if (s != PVS_OK) return s;
-        out[i]->stream = st;
-    }
-    QueryDst* d_qd = buf.get<QueryDst>((size_t)nq);
-    if (!d_qd) return PVS_ERR_OOM;
-    {
+    // cursors with the queries' encodings and fresh counters (queued behind the
+    // passes, which do not need them: the host works while the passes run)
+    auto open_cursors = [&]() -> pvs_status {
+        for (int i = 0; i < nq; ++i) {
+            pvs_status cs = acquire_cursor(x, sd, &out[i], /*zero_state=*/false);
+            if (cs != PVS_OK) return cs;
+            out[i]->stream = st;
+        }
+        QueryDst* d_qd = buf.get<QueryDst>((size_t)nq);
+        if (!d_qd) return PVS_ERR_OOM;
         // a pageable source is staged before cudaMemcpyAsync returns
         std::vector<QueryDst> qd(nq);
         for (int i = 0; i < nq; ++i)
             qd[i] = QueryDst{out[i]->zq, out[i]->qraw, out[i]->qs, out[i]->ctr, out[i]->d_status};
         PVS_CUDA(cudaMemcpyAsync(d_qd, qd.data(), nq * sizeof(QueryDst), cudaMemcpyHostToDevice, st));
         PVS_CUDA(launch_copy_queries(bq.zq, bq.qraw, bq.qs, d_qd, nq, x->m_pad, x->m_raw, st));
-    }
-    std::vector<QueryScalars> h_qs(nq);
+        return PVS_OK;
+    };
     const int64_t rows = sd->rows;
     if (rows == 0) {
+        s = open_cursors();
+        if (s != PVS_OK) return s;
+        std::vector<QueryScalars> h_qs(nq);
         PVS_CUDA(cudaMemcpyAsync(h_qs.data(), bq.qs, nq * sizeof(QueryScalars),
                                  cudaMemcpyDeviceToHost, st));
         PVS_CUDA(cudaStreamSynchronize(st));
@@ -922,70 +981,114 @@ pvs_status open_batch_group(pvs_index* x, const std::shared_ptr<SnapData>& sd,
     }
 
     // Sample every stride-th tile and take tau_q = the k_s-th largest sampled
-    // lower bound, k_s = 2 H / stride + 4: about 2 H rows of the corpus reach
-    // it.  It misses the horizon (fewer than H rows reach it) only when at
-    // least k_s of the top-H rows were sampled; that count is about
-    // Poisson(H / stride), so this happens for about 1e-5 of the queries
-    // (H = 200: stride 12, k_s = 38, mean 16.7), which then rescan.
+    // lower bound.  The number of the horizon's rows in the sample is about
+    // Poisson with mean H / stride, and tau_q misses the horizon (fewer than H
+    // rows reach it) only when at least k_s of them were sampled: five
+    // standard deviations and 4 above the mean, about 1e-6 of the queries,
+    // which then rescan.  About stride k_s rows reach tau_q: 2 H at the means
+    // of 16 and more taken here.
     const int64_t ntiles = (rows + 127) / 128;
-    int stride = (int)std::min<int64_t>(16, std::max<int64_t>(1, (3 * (int64_t)horizon) / 48));
+    int stride = (int)std::min<int64_t>(32, std::max<int64_t>(1, (int64_t)horizon / 16));
     if (ntiles < 8 * (int64_t)stride) stride = 1;
-    const int64_t ld = ((ntiles + stride - 1) / stride) * 128;
+    const double mean = (double)horizon / stride;
     const unsigned int k_s =
         stride == 1 ? (unsigned int)horizon
-                    : (unsigned int)((2 * (int64_t)horizon + stride - 1) / stride + 4);
-    const int w_cap = (int)std::min<int64_t>((int64_t)kWsSortMax, std::max<int64_t>(rows, 1));
+                    : (unsigned int)std::ceil(mean + 5.0 * std::sqrt(mean) + 4.0);
+    const int64_t sampled = (ntiles + stride - 1) / stride;
+    // one value per 32 rows where that leaves 16 times more values than the
+    // rank taken (few of the k_s largest then share a group)
+    const bool group_max = stream && stride > 1 && sampled * 4 >= 16 * (int64_t)k_s;
+    const int64_t ld = sampled * (group_max ? 4 : 128);
+    // working sets: half the sort's capacity holds 16 times the horizon up to
+    // 512 ranks; wide intervals over deep horizons take the rest
+    const int64_t cap = horizon <= 512 ? kWsSortMax / 2 : kWsSortMax;
+    const int w_cap = (int)std::min<int64_t>(cap, std::max<int64_t>(rows, 1));
     float* dlo = buf.get<float>((size_t)nq * ld);
-    float* dhi = dlo;   // the sampling pass needs the lower bounds only
     float* tau = buf.get<float>((size_t)nq);
-    float* rmax = buf.get<float>((size_t)nq);
-    int* status = buf.get<int>(1);
+    float* rmax = buf.get<float>((size_t)nq);   // theta of the streaming pass
     int32_t* wid = buf.get<int32_t>((size_t)nq * w_cap);
     float* wlo = buf.get<float>((size_t)nq * w_cap);
     float* whi = buf.get<float>((size_t)nq * w_cap);
-    unsigned int* wlen = buf.get<unsigned int>((size_t)nq);
-    unsigned int* heff = buf.get<unsigned int>((size_t)nq);
+    // the pass's status word, then per query its working-set length and count
+    unsigned int* verdict = buf.get<unsigned int>(1 + 2 * (size_t)nq);
     WsDst* d_ws = buf.get<WsDst>((size_t)nq);
-    if (!dlo || !dhi || !tau || !rmax || !status || !wid || !wlo || !whi || !wlen ||
-        !heff || !d_ws)
-        return PVS_ERR_OOM;
-    PVS_CUDA(cudaMemsetAsync(status, 0, sizeof(int), st));
-    PVS_CUDA(cudaMemsetAsync(wlen, 0, nq * sizeof(unsigned int), st));
-    PVS_CUDA(cudaMemsetAsync(heff, 0, nq * sizeof(unsigned int), st));
-
-    BatchArgs a{};
-    a.rows = rows;
-    a.m_pad = x->m_pad;
-    a.nq = nq;
-    a.nq_pad = bq.nq_pad;
-    a.scale = x->scale;
-    a.vnorm = x->vnorm;
-    a.enorm = x->enorm;
-    a.tomb = sd->d_tomb;
-    a.qs = bq.qs;
-    a.status = status;
-    // 2. thresholds from the sampled tiles
-    a.mode = 0;
-    a.tile_stride = stride;
-    a.dump_lo = dlo;
-    a.dump_hi = nullptr;
-    a.dump_ld = ld;
-    PVS_CUDA(launch_batch_intervals(a, x->codes_bf16, bq.qcodes, x->num_sms, st));
+    if (!dlo || !tau || !rmax || !wid || !wlo || !whi || !verdict || !d_ws) return PVS_ERR_OOM;
+    int* status = reinterpret_cast<int*>(verdict);
+    unsigned int* wlen = verdict + 1;
+    unsigned int* heff = wlen + nq;
+    PVS_CUDA(cudaMemsetAsync(verdict, 0, (1 + 2 * (size_t)nq) * sizeof(unsigned int), st));
+    // one launch per batch_stream_queries queries, or one bf16 launch for all
+    auto pass = [&](bool filter) -> cudaError_t {
+        if (!stream) {
+            BatchArgs a{};
+            a.rows = rows;
+            a.m_pad = x->m_pad;
+            a.nq = nq;
+            a.nq_pad = bq.nq_pad;
+            a.scale = x->scale;
+            a.vnorm = x->vnorm;
+            a.enorm = x->enorm;
+            a.tomb = sd->d_tomb;
+            a.qs = bq.qs;
+            a.status = status;
+            a.mode = filter ? 1 : 0;
+            a.tile_stride = filter ? 1 : stride;
+            if (filter) {
+                a.tau = tau;
+                a.rmax = rmax;
+                a.w_id = wid;
+                a.w_lo = wlo;
+                a.w_hi = whi;
+                a.w_cap = w_cap;
+                a.w_len = wlen;
+                a.h_eff = heff;
+            } else {
+                a.dump_lo = dlo;
+                a.dump_ld = ld;
+            }
+            return launch_batch_intervals(a, x->codes_bf16, bq.qcodes, x->num_sms, st);
+        }
+        const int per_pass = batch_stream_queries(x->m_pad);
+        for (int q0 = 0; q0 < nq; q0 += per_pass) {
+            StreamArgs a{};
+            a.rows = rows;
+            a.m_pad = x->m_pad;
+            a.nq = std::min(per_pass, nq - q0);
+            a.nq_pad = (int)round_up(a.nq, 32);
+            a.scale = x->scale;
+            a.vnorm = x->vnorm;
+            a.enorm = x->enorm;
+            a.tomb = sd->d_tomb;
+            a.qs = bq.qs + q0;
+            a.status = status;
+            a.mode = filter ? 1 : 0;
+            a.tile_stride = filter ? 1 : stride;
+            a.group_max = group_max ? 1 : 0;
+            if (filter) {
+                a.tau = tau + q0;
+                a.theta = rmax + q0;
+                a.w_id = wid + (size_t)q0 * w_cap;
+                a.w_lo = wlo + (size_t)q0 * w_cap;
+                a.w_hi = whi + (size_t)q0 * w_cap;
+                a.w_cap = w_cap;
+                a.w_len = wlen + q0;
+                a.h_eff = heff + q0;
+            } else {
+                a.dump_lo = dlo + (size_t)q0 * ld;
+                a.dump_ld = ld;
+            }
+            const cudaError_t e = launch_batch_stream(a, x->codes, bq.qcodes + (size_t)q0 * x->m_pad,
+                                                      x->num_sms, st);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    };
+    // 2. thresholds from the sampled tiles (norm maxima over all rows: a valid bound)
+    PVS_CUDA(pass(false));
     PVS_CUDA(launch_batch_tau(dlo, ld, (unsigned int)ld, nq, k_s, tau, st));
-    PVS_CUDA(launch_rmax(bq.qs, nq, x->norm_maxes, rmax, st));   // maxima over all rows: a valid bound
+    PVS_CUDA(stream ? launch_stream_theta(bq.qs, nq, x->norm_maxes, tau, rmax, st)
+                    : launch_rmax(bq.qs, nq, x->norm_maxes, rmax, st));
     // 3. the filter pass over every row
-    a.mode = 1;
-    a.tile_stride = 1;
-    a.dump_lo = a.dump_hi = nullptr;
-    a.dump_ld = 0;
-    a.tau = tau;
-    a.rmax = rmax;
-    a.w_id = wid;
-    a.w_lo = wlo;
-    a.w_hi = whi;
-    a.w_cap = w_cap;
-    a.w_len = wlen;
-    a.h_eff = heff;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     PVS_CUDA(cudaEventCreate(&ev0));
     PVS_CUDA(cudaEventCreate(&ev1));
@@ -993,26 +1096,29 @@ pvs_status open_batch_group(pvs_index* x, const std::shared_ptr<SnapData>& sd,
         std::lock_guard<std::mutex> lock(x->pass_mutex);   // one HBM pass at a time
         if (x->pass_done) PVS_CUDA(cudaStreamWaitEvent(st, x->pass_done, 0));
         PVS_CUDA(cudaEventRecord(ev0, st));
-        PVS_CUDA(launch_batch_intervals(a, x->codes_bf16, bq.qcodes, x->num_sms, st));
+        PVS_CUDA(pass(true));
         PVS_CUDA(cudaEventRecord(ev1, st));
         if (!x->pass_done)
             PVS_CUDA(cudaEventCreateWithFlags(&x->pass_done, cudaEventDisableTiming));
         PVS_CUDA(cudaEventRecord(x->pass_done, st));
     }
     // 4. ordered working sets into the cursors
-    std::vector<WsDst> ws(nq);
-    for (int i = 0; i < nq; ++i) {
-        s = cursor_alloc_ws(out[i], w_cap);
-        if (s != PVS_OK) return s;
-        ws[i] = WsDst{out[i]->w_id, out[i]->w_lo, out[i]->w_hi, &out[i]->ctr->w_len};
+    s = open_cursors();
+    if (s != PVS_OK) return s;
+    {
+        std::vector<WsDst> ws(nq);
+        for (int i = 0; i < nq; ++i) {
+            s = cursor_alloc_ws(out[i], w_cap);
+            if (s != PVS_OK) return s;
+            ws[i] = WsDst{out[i]->w_id, out[i]->w_lo, out[i]->w_hi, &out[i]->ctr->w_len};
+        }
+        PVS_CUDA(cudaMemcpyAsync(d_ws, ws.data(), nq * sizeof(WsDst), cudaMemcpyHostToDevice, st));
     }
-    PVS_CUDA(cudaMemcpyAsync(d_ws, ws.data(), nq * sizeof(WsDst), cudaMemcpyHostToDevice, st));
     PVS_CUDA(launch_ws_sort(wid, wlo, whi, w_cap, wlen, d_ws, nq, st));
-    std::vector<unsigned int> h_wlen(nq), h_heff(nq);
-    int h_status = 0;
-    PVS_CUDA(cudaMemcpyAsync(h_wlen.data(), wlen, nq * sizeof(unsigned int), cudaMemcpyDeviceToHost, st));
-    PVS_CUDA(cudaMemcpyAsync(h_heff.data(), heff, nq * sizeof(unsigned int), cudaMemcpyDeviceToHost, st));
-    PVS_CUDA(cudaMemcpyAsync(&h_status, status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    std::vector<unsigned int> h_verdict(1 + 2 * (size_t)nq);
+    std::vector<QueryScalars> h_qs(nq);
+    PVS_CUDA(cudaMemcpyAsync(h_verdict.data(), verdict, h_verdict.size() * sizeof(unsigned int),
+                             cudaMemcpyDeviceToHost, st));
     PVS_CUDA(cudaMemcpyAsync(h_qs.data(), bq.qs, nq * sizeof(QueryScalars), cudaMemcpyDeviceToHost,
                              st));
     PVS_CUDA(cudaStreamSynchronize(st));
@@ -1022,13 +1128,14 @@ pvs_status open_batch_group(pvs_index* x, const std::shared_ptr<SnapData>& sd,
     cudaEventDestroy(ev1);
     for (int i = 0; i < nq; ++i)   // a non-finite query fails the batch
         if (h_qs[i].status != 0) return (pvs_status)h_qs[i].status;
-    if (h_status != 0) return (pvs_status)h_status;
+    if ((int)h_verdict[0] != 0) return (pvs_status)(int)h_verdict[0];
     for (int i = 0; i < nq; ++i) {
         pvs_cursor* c = out[i];
-        if (h_wlen[i] <= (unsigned int)w_cap && h_heff[i] > 0) {
+        const unsigned int len = h_verdict[1 + (size_t)i], reach = h_verdict[1 + (size_t)(nq + i)];
+        if (len <= (unsigned int)w_cap && reach > 0) {
             c->batch_ws = true;
             c->fresh_ws = true;
-            c->horizon = h_heff[i];
+            c->horizon = reach;
             c->horizon_base = 0;
         }
         c->batch_passes = 1;
@@ -1407,12 +1514,7 @@ pvs_status pvs::cursor_open_on(pvs_index* x, const pvs_snapshot* snap, const flo
     c->rows = c->snap->rows;
     c->visible = c->snap->visible;
     cudaStream_t st = c->stream;
-    if (!c->zq &&
-        (dev_alloc(&c->zq, (size_t)x->m_pad) != cudaSuccess ||
-         dev_alloc(&c->qraw, (size_t)x->m_raw) != cudaSuccess ||
-         dev_alloc(&c->qs, 1) != cudaSuccess || dev_alloc(&c->sel, 1) != cudaSuccess ||
-         dev_alloc(&c->ctr, 1) != cudaSuccess || dev_alloc(&c->d_status, 1) != cudaSuccess ||
-         cudaMallocHost(&c->h_small, 16 * sizeof(unsigned int)) != cudaSuccess))
+    if (cursor_alloc_small(c, x) != cudaSuccess || cursor_pinned(c) != cudaSuccess)
         return bail(PVS_ERR_OOM);
     cudaError_t e = cudaSuccess;
     if (st != x->stream) {   // after the index's queued builds and appends
@@ -1588,6 +1690,39 @@ pvs_status pvs::cursor_open_group(pvs_index* x, const pvs_snapshot* snap, const 
     return PVS_OK;
 }
 
+pvs_status pvs::cursor_open_serving(pvs_index* x, const pvs_snapshot* snap, const float* queries,
+                                    int32_t nq, int32_t queries_on_device, int32_t horizon,
+                                    cudaStream_t stream, pvs_cursor** out, int64_t* passes,
+                                    double* pass_ms) {
+    DeviceGuard device_guard(index_device(x));
+    *passes = 0;
+    *pass_ms = 0.0;
+    for (int32_t i = 0; i < nq; ++i) out[i] = nullptr;
+    std::shared_ptr<SnapData> sd = snap ? snap->data : make_snapdata(x);
+    if (!sd) return PVS_ERR_OOM;
+    pvs_status s = open_batch_group(x, sd, queries, nq, queries_on_device != 0, horizon, stream, out);
+    std::vector<pvs_cursor*> wide;   // working sets past the batched pass's capacity
+    if (s == PVS_OK) {
+        *passes = 1;
+        *pass_ms = out[0]->batch_ms;
+        for (int32_t i = 0; i < nq; ++i)
+            if (!out[i]->batch_ws && out[i]->visible > 0) wide.push_back(out[i]);
+    }
+    const int32_t group = kGroupMax / 2;
+    for (size_t i = 0; s == PVS_OK && i + 1 < wide.size(); i += group) {
+        const int32_t n = (int32_t)std::min<size_t>(group, wide.size() - i);
+        if (n < 2 || !interval_group_supported(x->m_pad, n)) break;   // each at its first pull
+        s = group_pass(x, wide.data() + i, n, stream);
+        ++*passes;
+    }
+    if (s != PVS_OK)
+        for (int32_t i = 0; i < nq; ++i) {
+            if (out[i]) pvs_cursor_close(out[i]);
+            out[i] = nullptr;
+        }
+    return s;
+}
+
 extern "C" {
 
 pvs_status pvs_cursor_open(pvs_index* x, const pvs_snapshot* snap, const float* query,
@@ -1642,7 +1777,8 @@ pvs_status pvs_batch_bounds(pvs_index* x, const pvs_snapshot* snap, const float*
     cudaStream_t st = x->stream;
     DevBuf buf(st, x->scratch_pool);
     BatchQueries bq;
-    pvs_status s = encode_batch(x, queries, nq, queries_on_device, buf, &bq, st);
+    pvs_status s = encode_batch(x, queries, nq, queries_on_device, buf, &bq, st,
+                                /*check_now=*/true, /*f16=*/false);
     if (s != PVS_OK) return s;
     const int64_t ntiles = (rows + 127) / 128;
     const int64_t ld = ntiles * 128;
@@ -1694,7 +1830,10 @@ static pvs_status delivery_state(pvs_cursor* c) {
 // never past the list's end); large requests exactly.
 static int64_t pull_size(const pvs_cursor* c, int64_t need, int32_t readahead) {
     if (need > kPullFusedMax) return need;
-    const int64_t want = std::min<int64_t>(kPullFusedMax, need * std::max<int32_t>(1, readahead));
+    int64_t want = std::min<int64_t>(kPullFusedMax, need * std::max<int32_t>(1, readahead));
+    // not past what a batched working set certifies: a rescan for ranks that
+    // nobody has asked for costs a pass over the codes
+    if (c->batch_ws) want = std::min(want, c->horizon_base + c->horizon - c->emitted);
     return std::min<int64_t>(std::max(want, need), c->visible - c->emitted);
 }
 
@@ -1716,7 +1855,7 @@ pvs_status pvs::next_batch_rows(pvs_cursor* const* cursors, int32_t nc, int32_t 
     }
     for (int32_t i = 0; i < nc; ++i)
         if (cursors[i]->state < 0) return PVS_ERR_FAILED;
-    if (n > kPullFusedMax) {   // large pulls: one cursor at a time
+    if (n > kPullBatchMax || (n > kPullFusedMax && nc == 1)) {   // one cursor at a time
         for (int32_t i = 0; i < nc; ++i) {
             pvs_status s = outputs_on_device
                                ? pvs_next_device(cursors[i], n, ids[i], scores[i], &n_out[i])
@@ -1769,7 +1908,9 @@ pvs_status pvs::next_batch_rows(pvs_cursor* const* cursors, int32_t nc, int32_t 
     for (int32_t i = 0; i < nc; ++i) {
         if (pulls[i] <= 0) continue;
         pvs_cursor* c = cursors[i];
-        pvs_status s = cursor_out_reserve(c, pulls[i]);   // nothing is ahead now
+        // a pull of exactly what is asked goes straight to the caller's device row
+        const bool direct = outputs_on_device && pulls[i] == rest[i];
+        pvs_status s = direct ? PVS_OK : cursor_out_reserve(c, pulls[i]);   // nothing is ahead now
         if (s != PVS_OK) return fail(c, s);
         s = prepare_pull(c, pulls[i]);
         if (s != PVS_OK) return fail(c, s);
@@ -1788,8 +1929,8 @@ pvs_status pvs::next_batch_rows(pvs_cursor* const* cursors, int32_t nc, int32_t 
         a.keys = reinterpret_cast<unsigned long long*>(c->keys);
         // device outputs: the cursor's device buffers; host outputs: its
         // pinned buffers, which the kernels write directly
-        a.out_ids = outputs_on_device ? c->d_ids : c->h_ids;
-        a.out_scores = outputs_on_device ? c->d_scores : c->h_scores;
+        a.out_ids = direct ? ids[i] + take[i] : outputs_on_device ? c->d_ids : c->h_ids;
+        a.out_scores = direct ? scores[i] + take[i] : outputs_on_device ? c->d_scores : c->h_scores;
         a.status = c->d_status;
         a.ctr = c->ctr;
         a.front = nullptr;   // a few pulls per batch: a frontier would not pay for itself
@@ -1798,9 +1939,10 @@ pvs_status pvs::next_batch_rows(pvs_cursor* const* cursors, int32_t nc, int32_t 
         who.push_back(i);
     }
     if (!args.empty()) {
+        // first pulls of new working sets, and deep ones: refinement on every SM
         bool fresh = false;
-        for (int32_t i : who) fresh = fresh || cursors[i]->fresh_ws;
-        if (fresh) {   // first pull of new working sets: refinement on every SM
+        for (int32_t i : who) fresh = fresh || cursors[i]->fresh_ws || pulls[i] > kPullFusedMax;
+        if (fresh) {
             const int per = std::min(64, std::max(4, 2 * x->num_sms / (int)args.size()));
             PVS_CUDA(launch_pull_batch(args.data(), (int)args.size(), per, x->m_raw, st));
         } else {
@@ -1819,6 +1961,7 @@ pvs_status pvs::next_batch_rows(pvs_cursor* const* cursors, int32_t nc, int32_t 
     if (outputs_on_device) {
         for (int32_t i : who) {
             pvs_cursor* c = cursors[i];
+            if (pulls[i] == rest[i]) continue;   // written in place
             copies.push_back(RankCopy{c->d_ids, c->d_scores, ids[i] + take[i],
                                       scores[i] + take[i], (int)rest[i]});
         }
@@ -1892,6 +2035,7 @@ static pvs_status pull_to_pinned(pvs_cursor* c, int64_t r, int64_t at = 0) {
     if (r <= kPullFusedMax) {
         // the kernels write ids, scores and the status word straight into the
         // cursor's pinned host buffers: one launch, one wait
+        if (cursor_pinned(c) != cudaSuccess) return fail(c, PVS_ERR_OOM);
         int* mirror = reinterpret_cast<int*>(c->h_small) + 2;
         *reinterpret_cast<volatile int*>(mirror) = kStatusPending;
         s = pull(c, r, c->h_ids + at, c->h_scores + at, mirror);

@@ -93,7 +93,8 @@ struct pvs_cursor {
     int64_t rows = 0, visible = 0, emitted = 0;
     int state = PVS_OK;
     bool scanned = false;
-    // query
+    // query (zq .. qs, sel, ctr and d_status are parts of `small`)
+    void* small = nullptr;
     int8_t* zq = nullptr;
     float* qraw = nullptr;
     pvs::QueryScalars* qs = nullptr;
@@ -105,8 +106,10 @@ struct pvs_cursor {
     // bounds of hi from then on: refinement and delivery only lower hi)
     float* bmax = nullptr;
     bool bmax_valid = false;
-    // working set (ordered by id): rows that can hold the next `horizon` ranks
+    // working set (ordered by id): rows that can hold the next `horizon` ranks;
+    // its arrays and the pull scratch are parts of ws_slab
     int64_t cap_w = 0;                // capacity of the working-set arrays
+    void* ws_slab = nullptr;
     bool batch_ws = false;            // working set came from a batched pass (no full bounds)
     bool fresh_ws = false;            // no pull since the working set was built (many candidates)
     int32_t* w_id = nullptr;
@@ -259,6 +262,15 @@ pvs_status next_batch_rows(pvs_cursor* const* cursors, int32_t nc, int32_t n,
 pvs_status cursor_open_group(pvs_index* x, const pvs_snapshot* snap, const float* queries,
                              int32_t nq, int32_t queries_on_device, cudaStream_t pass_stream,
                              const cudaStream_t* cursor_streams, pvs_cursor** out);
+// Open nq cursors for requests of about `horizon` ranks, all on `stream`: one
+// batched pass (open_batch_group); the queries whose working sets it cannot hold
+// share grouped passes instead.  On an error every cursor is closed.
+// *passes, *pass_ms: passes over the codes that were queued, and the
+// device time of the batched one.
+pvs_status cursor_open_serving(pvs_index* x, const pvs_snapshot* snap, const float* queries,
+                               int32_t nq, int32_t queries_on_device, int32_t horizon,
+                               cudaStream_t stream, pvs_cursor** out, int64_t* passes,
+                               double* pass_ms);
 // Open a cursor whose device work runs on `stream` (null: the index's stream).
 pvs_status cursor_open_on(pvs_index* x, const pvs_snapshot* snap, const float* query,
                           int32_t query_on_device, cudaStream_t stream, pvs_cursor** out);
