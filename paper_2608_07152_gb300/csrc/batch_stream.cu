@@ -403,26 +403,34 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
                 tc::wait_ld();
                 if (a.mode == 0) {
                     const int64_t srow = i * kRows + r_in_tile;
-                    float best = -INFINITY;   // lane k: the 32 rows' largest lower bound, query k
                     bool bad = false;
 #pragma unroll
                     for (int k = 0; k < 32; ++k) {   // (branch-free: the 32 chains overlap)
-                        const int q = cc * 32 + k;
                         float lo, hi;
-                        interval_epilogue(__float2int_rn(__uint_as_float(d[k])), sh.qs[q], sv, vn, en,
-                                          lo, hi);
+                        interval_epilogue(__float2int_rn(__uint_as_float(d[k])), sh.qs[cc * 32 + k],
+                                          sv, vn, en, lo, hi);
                         bad |= live && !(isfinite(lo) && isfinite(hi));   // (padding queries: 0)
-                        lo = live ? lo : -INFINITY;
-                        if (a.group_max) {
-                            const uint32_t m = __reduce_max_sync(0xffffffffu, fkey(lo));
-                            best = lane == k ? fkey_inv(m) : best;
-                        } else if (q < a.nq) {
-                            a.dump_lo[(int64_t)q * a.dump_ld + srow] = lo;
+                        d[k] = __float_as_uint(live ? lo : -INFINITY);
+                    }
+                    if (a.group_max) {
+                        uint32_t best = 0;   // lane k: the 32 rows' largest key, query k
+#pragma unroll
+                        for (int k = 0; k < 32; ++k) {
+                            const uint32_t m =
+                                __reduce_max_sync(0xffffffffu, fkey(__uint_as_float(d[k])));
+                            best = lane == k ? m : best;
                         }
+                        if (cc * 32 + lane < a.nq)
+                            a.dump_lo[(int64_t)(cc * 32 + lane) * a.dump_ld + i * 4 + quarter] =
+                                fkey_inv(best);
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 32; ++k)
+                            if (cc * 32 + k < a.nq)
+                                a.dump_lo[(int64_t)(cc * 32 + k) * a.dump_ld + srow] =
+                                    __uint_as_float(d[k]);
                     }
                     if (bad) set_status(a.status, PVS_ERR_OVERFLOW);
-                    if (a.group_max && cc * 32 + lane < a.nq)
-                        a.dump_lo[(int64_t)(cc * 32 + lane) * a.dump_ld + i * 4 + quarter] = best;
                     continue;
                 }
                 // any pair of the chunk that may reach its threshold?  One

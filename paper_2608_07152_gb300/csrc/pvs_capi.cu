@@ -928,7 +928,7 @@ pvs_status acquire_cursor(pvs_index* x, const std::shared_ptr<SnapData>& sd, pvs
 //   1. encode the queries; f16 (or bf16) query codes for the MMA;
 //   2. thresholds: on every stride-th 128-row tile (every tile for small
 //      corpora) the pass leaves the lower bounds; tau_q = the k-th largest of
-//      query q there, k sized so that about twice the horizon's rows of the
+//      query q there, k sized so that 1.5 to 2.5 times the horizon's rows of the
 //      whole corpus reach it;
 //   3. the filter pass appends every row with hi >= tau_q to query q's
 //      working set and counts the rows with lo >= tau_q: those rows precede
@@ -983,17 +983,19 @@ pvs_status open_batch_group(pvs_index* x, const std::shared_ptr<SnapData>& sd,
     // Sample every stride-th tile and take tau_q = the k_s-th largest sampled
     // lower bound.  The number of the horizon's rows in the sample is about
     // Poisson with mean H / stride, and tau_q misses the horizon (fewer than H
-    // rows reach it) only when at least k_s of them were sampled: five
-    // standard deviations and 4 above the mean, about 1e-6 of the queries,
-    // which then rescan.  About stride k_s rows reach tau_q: 2 H at the means
-    // of 16 and more taken here.
+    // rows reach it) only when at least k_s of them were sampled: 4.5 standard
+    // deviations and 3 above the mean, less than 1e-5 of the queries, which
+    // then rescan.  About stride k_s rows reach tau_q: 1.6 H at means of 62.  (At a mean of
+    // 31, 2 H rows: past the end of more clusters of near neighbours, where the
+    // threshold falls into the bulk of the corpus and no working set holds
+    // what reaches it.)
     const int64_t ntiles = (rows + 127) / 128;
-    int stride = (int)std::min<int64_t>(32, std::max<int64_t>(1, (int64_t)horizon / 16));
+    int stride = (int)std::min<int64_t>(16, std::max<int64_t>(1, (int64_t)horizon / 16));
     if (ntiles < 8 * (int64_t)stride) stride = 1;
     const double mean = (double)horizon / stride;
     const unsigned int k_s =
         stride == 1 ? (unsigned int)horizon
-                    : (unsigned int)std::ceil(mean + 5.0 * std::sqrt(mean) + 4.0);
+                    : (unsigned int)std::ceil(mean + 4.5 * std::sqrt(mean) + 3.0);
     const int64_t sampled = (ntiles + stride - 1) / stride;
     // one value per 32 rows where that leaves 16 times more values than the
     // rank taken (few of the k_s largest then share a group)
