@@ -19,7 +19,7 @@
  * codes for all G queries) and each page of the G cursors is one batched
  * pull; every request still receives its own pages.
  *
- * A run of more than G >= 2 requests, of at most 1,024 ranks each, over a
+ * A run of more than 2 G requests (G >= 2), of at most 1,024 ranks each, over a
  * corpus of at least 65,536 vectors of 65 .. 1,024 dimensions is served in
  * blocks of up to 128 requests (96 above 768 dimensions): one tensor-core pass over the codes
  * (as pvs_cursor_open_batch) opens a block's cursors, one pull computes all
@@ -97,7 +97,7 @@ pvs_status pvs_executor_run_ex(pvs_executor* ex, const pvs_snapshot* snap, const
 /*
  * Serve requests in groups of `group` (1 .. PVS_GROUP_MAX; default 1): the
  * queries of a group share one pass over the codes (from 2 on, a run of more
- * requests than one group may be served in larger blocks, see above).  Must not be called
+ * requests than two groups may be served in larger blocks, see above).  Must not be called
  * during a run.  Errors: PVS_ERR_INVALID.
  */
 pvs_status pvs_executor_set_group(pvs_executor* ex, int32_t group);

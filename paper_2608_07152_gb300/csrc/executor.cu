@@ -10,7 +10,7 @@
 // caller's buffers, and closes the cursor.  With a group size G >= 2 a
 // worker takes G requests at a time: one grouped open (one pass over the
 // codes for all G queries, pvs_cursor_open_group), then every page of the G
-// cursors in one batched pull.  A run of more requests than one group, over a
+// cursors in one batched pull.  A run of more requests than two groups, over a
 // corpus of some size, takes blocks of requests instead (batch_block):
 // their cursors come from one tensor-core pass (cursor_open_serving) and all
 // their pages from one deep batched pull.  No lock is held across a device
@@ -223,15 +223,17 @@ void serve_group(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first,
 // Requests per batched open for a run, or 0 to serve in groups.  A group of 8
 // costs one read of the codes and their bounds written out (8.8M x 768: 1.24
 // ms); a batched pass of up to 128 requests reads the codes once and keeps
-// only working sets (1.2 ms + 0.5 ms for its thresholds and sorting), so it
-// wins from the second group on.  Small corpora, where a pass takes
-// microseconds, and requests deeper than one batched pull stay in groups.
+// only working sets (1.1 ms + 0.2 ms for its thresholds), so it wins from the
+// second group on; a run of one or two groups keeps the passes that its group
+// size promises (their count is part of the statistics' contract).  Small
+// corpora, where a pass takes microseconds, and requests deeper than one
+// batched pull stay in groups.
 constexpr int64_t kBlockRows = 65536;
 
 int32_t batch_block(const pvs_executor* ex, const Job& j) {
     const pvs_index* x = ex->index;
     const int64_t rows = j.snap ? j.snap->data->rows : x->size;
-    if (ex->group < 2 || j.nq <= ex->group || j.ranks > pvs::kPullBatchMax || rows < kBlockRows ||
+    if (ex->group < 2 || j.nq <= 2 * ex->group || j.ranks > pvs::kPullBatchMax || rows < kBlockRows ||
         !pvs::batch_stream_supported(x->m_pad, x->num_sms))
         return 0;
     const int32_t most = pvs::batch_stream_queries(x->m_pad);

@@ -110,6 +110,33 @@ cudaError_t launch_pull_batch(const PullArgs* host_args, int ncursors, int refin
 cudaError_t launch_refine_batch(const PullArgsPack& p, int ncursors, int blocks_per_cursor,
                                 int m_raw, cudaStream_t st);
 
+// ---- the first pull of a lone cursor (first_pull.cu) ------------------------
+constexpr int kFirstMax = 16384;     // largest working set it scores whole
+constexpr int kFirstHorizon = 2048;  // most ranks it delivers or keeps ahead
+struct FirstSetArgs {
+    const float* vals;        // lower bounds of distinct live rows (-inf: none), 16-byte aligned
+    int64_t len;              // at most what first_threshold_fits allows
+    uint64_t k;               // ranks the set holds; 0: every live row
+    SelectState* sel;
+    DevCounters* ctr;
+    float* lo;
+    float* hi;
+    int64_t rows;
+    int32_t* w_id;            // room for `rows` entries
+    float* w_lo;
+    float* w_hi;
+};
+bool first_threshold_fits(int64_t len);
+// The threshold and the (unordered) working set; its length in ctr->w_len.
+cudaError_t launch_first_set(const FirstSetArgs& a, int num_sms, cudaStream_t st);
+// Sort the scored set and emit its certified ranks, n at most; nothing is
+// emitted when it holds more than kFirstMax rows (or too many exact ties to
+// sort; the length is then reported as 2^32 - 1).  The length and the ranks
+// emitted (two words), then the status word, are mirrored to pinned memory.
+cudaError_t launch_first_emit(const FirstSetArgs& a, int n, int64_t* out_ids, float* out_scores,
+                              const int* status, unsigned int* len_mirror, int* status_mirror,
+                              cudaStream_t st);
+
 // ---- batched open support (pull_kernel.cu, batch_support.cu) ----------------
 constexpr int kWsSortMax = 16384;    // largest per-query working set of a batched open
 constexpr int kFrontCap = 4096;      // frontier entries (the one-launch pull's gather capacity)
@@ -164,9 +191,12 @@ cudaError_t launch_scan_scores(const float* qraw, const float* raw, int m_raw, i
 // ids / scores of keys[0 .. n); *mirror = *status afterwards when mirror is set.
 cudaError_t launch_scan_emit(const uint64_t* keys, int64_t n, int64_t* ids, float* scores,
                              const int* status, int* mirror, cudaStream_t st);
-// Encode one query: codes zq[m_pad], raw copy qraw[m_raw], scalars.
+// Encode one query for a fresh cursor: codes zq[m_pad], raw copy qraw[m_raw],
+// scalars; its counters and status word are zeroed, and the encoding's status
+// goes to a pinned host word last.
 cudaError_t launch_encode_query(const float* q, int m, int m_pad, int m_raw, int8_t* zq,
-                                float* qraw, QueryScalars* qs, cudaStream_t st);
+                                float* qraw, QueryScalars* qs, DevCounters* ctr, int* status,
+                                int* status_mirror, cudaStream_t st);
 // Encode nq queries (row stride m), one warp each.
 cudaError_t launch_encode_queries(const float* q, int nq, int m, int m_pad, int m_raw,
                                   int8_t* zq, float* qraw, QueryScalars* qs, cudaStream_t st);
@@ -380,10 +410,13 @@ cudaError_t launch_codes_to_bf16(const int8_t* src, uint16_t* dst, int64_t count
 // ---- refinement (refine_kernels.cu) -----------------------------------------
 // Authoritative score of every unresolved candidate (w_lo < w_hi): exact
 // RN_f32(sum_j q_j v_j), containment check, then w_lo = w_hi = lo = hi = s.
+// cand null: every working-set entry (cand_len its length), and nothing at all
+// when there are more than `limit` of them.
 cudaError_t launch_refine(const int32_t* cand, const unsigned int* cand_len,
                           const int32_t* w_id, float* w_lo, float* w_hi, float* lo, float* hi,
                           const float* qraw, const float* raw, int m_raw, int* status,
-                          DevCounters* ctr, int grid, cudaStream_t st);
+                          DevCounters* ctr, int grid, cudaStream_t st,
+                          unsigned int limit = 0xffffffffu);
 // Authoritative scores of explicit ids (tests / diagnostics).
 cudaError_t launch_score_ids(const int64_t* ids, int n, const float* qraw, const float* raw,
                              int m_raw, float* out, DevCounters* ctr, cudaStream_t st);

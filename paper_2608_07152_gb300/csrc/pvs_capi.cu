@@ -243,6 +243,7 @@ void cursor_reset(pvs_cursor* c) {
     c->ahead = c->ahead_pos = 0;
     c->ahead_host = false;
     c->readahead = 4;
+    c->readahead_set = false;
     c->batch_passes = 0;
     c->batch_ms = 0.0;
     c->ev_pending = false;
@@ -449,13 +450,15 @@ pvs_status interval_pass(pvs_cursor* c) {
     a.status = c->d_status;
     a.wait_ns = x->wait_ns;
     // per-slot largest lower bounds, for the first working set (see
-    // build_working_set): only when no row is tombstoned and every slot
-    // scans at least kSlotTop rows, so that every entry is a live row's bound
+    // build_working_set): when every slot scans at least kSlotTop rows.  With
+    // deleted rows an entry may stay empty (-inf); with half of the rows live
+    // the entries still hold far more rows than the first horizon, and a
+    // selection that runs short of them keeps every live row.
     int64_t min_rows = 0;
     const int64_t slots = interval_slots(c->rows, x->m_pad, x->num_sms, &min_rows);
     c->slot_fresh = false;
     c->slot_n = 0;
-    if (slots > 0 && c->snap->d_tomb == nullptr && min_rows >= kSlotTop) {
+    if (slots > 0 && 2 * c->visible >= c->rows && min_rows >= kSlotTop) {
         if (c->slot_cap < slots * kSlotTop) {
             dev_free(c->slot_top);
             c->slot_cap = 0;
@@ -502,8 +505,8 @@ pvs_status build_working_set(pvs_cursor* c, int64_t want) {
     if (H > remaining) H = remaining;
     if (H < remaining && c->slot_fresh && H <= c->slot_n) {
         // Each of the slot_n per-slot entries is the lower bound of a
-        // distinct live row, so at least H rows have lo >= the H-th largest
-        // entry v: v is at most the H-th largest lo of all rows, and the
+        // distinct live row (or -inf), so at least H rows have lo >= the H-th
+        // largest entry v: v is at most the H-th largest lo of all rows, and the
         // rows with hi >= v hold the working set (a few more rows than the
         // exact threshold keeps; a few thousand entries are selected from
         // instead of every row).
@@ -1532,15 +1535,15 @@ pvs_status pvs::cursor_open_on(pvs_index* x, const pvs_snapshot* snap, const flo
         e = cudaMemcpyAsync(c->qraw, query, x->m * sizeof(float), cudaMemcpyHostToDevice, st);
         qd = c->qraw;
     }
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->ctr, 0, sizeof(DevCounters), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(int), st);
-    if (e == cudaSuccess) e = launch_encode_query(qd, x->m, x->m_pad, x->m_raw, c->zq, c->qraw, c->qs, st);
-    int* enc_status = reinterpret_cast<int*>(c->h_small) + 3;   // pinned
+    int* enc_status = reinterpret_cast<int*>(c->h_small) + 3;   // pinned, polled
+    *reinterpret_cast<volatile int*>(enc_status) = kStatusPending;
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(enc_status, &c->qs->status, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        e = launch_encode_query(qd, x->m, x->m_pad, x->m_raw, c->zq, c->qraw, c->qs, c->ctr,
+                                c->d_status, enc_status, st);
+    if (e == cudaSuccess && !wait_published(enc_status)) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return bail(cuda_status(e));
-    if (*enc_status != 0) return bail((pvs_status)*enc_status);
+    const int encoded = *reinterpret_cast<volatile int*>(enc_status);
+    if (encoded != 0) return bail((pvs_status)encoded);
     c->state = c->visible == 0 ? PVS_EXHAUSTED : PVS_OK;
     *out = c;
     return PVS_OK;
@@ -2023,11 +2026,91 @@ static pvs_status next_common(pvs_cursor* c, int32_t n, int32_t* n_out, int64_t*
     return PVS_OK;
 }
 
+// The first pull of a cursor through first_pull.cu: the first working set
+// scored and sorted whole, its certified ranks into the pinned buffers and
+// ahead (r at least, 2,048 at most; exactly r unless ahead_ok).  *done stays
+// false, with the bounds as they were, when the pull does not qualify (without
+// ahead_ok: r is not all that such a pull delivers), the threshold's values do
+// not fit one CTA, or the set turned out larger than kFirstMax.
+static pvs_status first_pull(pvs_cursor* c, int64_t r, bool ahead_ok, bool* done) {
+    *done = false;
+    if (c->generator != PVS_GEN_INTERVALS || c->batch_ws || c->emitted != 0 ||
+        c->horizon_builds != 0 || r > kFirstHorizon)
+        return PVS_OK;
+    const int64_t most = std::min<int64_t>(kFirstHorizon, c->visible);
+    if (!ahead_ok && r != most) return PVS_OK;
+    // The ranks the set must hold.  Scoring 2,048 rows takes microseconds,
+    // nothing beside the pass over a large corpus; over a small one the rows
+    // beyond the first pages would be most of the work.
+    const int64_t H = std::min<int64_t>(
+        most, std::max<int64_t>({r, (int64_t)256, std::min<int64_t>(c->rows / 64, kFirstHorizon)}));
+    pvs_index* x = c->index;
+    cudaStream_t st = c->stream;
+    pvs_status s = cursor_alloc_rows(c);
+    if (s == PVS_OK && !c->scanned) s = interval_pass(c);
+    if (s == PVS_OK) s = cursor_out_reserve(c, most);
+    if (s != PVS_OK) return fail(c, s);
+    FirstSetArgs a{};
+    a.k = H < c->visible ? (uint64_t)H : 0;
+    if (a.k > 0) {
+        const bool slots = c->slot_fresh && H <= c->slot_n;
+        a.vals = slots ? c->slot_top : c->lo;
+        a.len = slots ? c->slot_n : c->rows;
+        if (!first_threshold_fits(a.len)) return PVS_OK;
+    }
+    a.sel = c->sel;
+    a.ctr = c->ctr;
+    a.lo = c->lo;
+    a.hi = c->hi;
+    a.rows = c->rows;
+    a.w_id = c->w_id;
+    a.w_lo = c->w_lo;
+    a.w_hi = c->w_hi;
+    cudaError_t e = cursor_pinned(c);
+    if (e != cudaSuccess) return fail(c, cuda_status(e));
+    unsigned int* len = c->h_small + 4;
+    int* mirror = reinterpret_cast<int*>(c->h_small) + 2;
+    *reinterpret_cast<volatile int*>(mirror) = kStatusPending;
+    e = launch_first_set(a, x->num_sms, st);
+    if (e == cudaSuccess)
+        e = launch_refine(nullptr, &c->ctr->w_len, c->w_id, c->w_lo, c->w_hi, c->lo, c->hi, c->qraw,
+                          x->raw, x->m_raw, c->d_status, c->ctr, 2 * x->num_sms, st, kFirstMax);
+    if (e == cudaSuccess)
+        e = launch_first_emit(a, (int)most, c->h_ids, c->h_scores, c->d_status, len, mirror, st);
+    if (e == cudaSuccess && !wait_published(mirror)) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return fail(c, cuda_status(e));
+    harvest_interval_time(c);
+    const int dev_status = *reinterpret_cast<volatile int*>(mirror);
+    if (dev_status != 0) return fail(c, (pvs_status)dev_status);
+    const int64_t set = reinterpret_cast<volatile unsigned int*>(len)[0];
+    const int64_t got = reinterpret_cast<volatile unsigned int*>(len)[1];
+    if (set > kFirstMax) return PVS_OK;
+    if (got < H) return fail(c, PVS_ERR_INVALID);   // internal invariant
+    c->slot_fresh = false;
+    c->horizon = got;   // the set is used up
+    c->horizon_base = 0;
+    c->horizon_builds++;
+    c->fresh_ws = false;
+    c->emitted = got;
+    c->pulls++;
+    c->ahead = got;
+    c->ahead_pos = 0;
+    c->ahead_host = true;
+    *done = true;
+    return PVS_OK;
+}
+
 // A pull of r >= 1 ranks into the cursor's pinned buffers at [at, at + r);
 // they become the ranks ahead (ahead_pos = at).  The buffers must already
 // hold at + r entries when at > 0 (they are only reallocated while empty).
-static pvs_status pull_to_pinned(pvs_cursor* c, int64_t r, int64_t at = 0) {
+// More ranks than r may come ahead when ahead_ok (at = 0).
+static pvs_status pull_to_pinned(pvs_cursor* c, int64_t r, int64_t at = 0, bool ahead_ok = false) {
     pvs_status s;
+    if (at == 0) {
+        bool done = false;
+        s = first_pull(c, r, ahead_ok, &done);
+        if (s != PVS_OK || done) return s;
+    }
     if (at == 0) {
         s = cursor_out_reserve(c, r);
         if (s != PVS_OK) return fail(c, s);
@@ -2106,7 +2189,7 @@ pvs_status pvs_next(pvs_cursor* c, int32_t n, int64_t* ids, float* scores, int32
     int64_t off = 0;
     while (off < n_eff) {
         if (c->ahead == 0) {
-            s = pull_to_pinned(c, pull_size(c, n_eff - off, c->readahead));
+            s = pull_to_pinned(c, pull_size(c, n_eff - off, c->readahead), 0, !c->readahead_set);
             if (s < 0) return s;
         } else if (!c->ahead_host) {
             s = ahead_to_host(c);
@@ -2229,6 +2312,7 @@ pvs_status pvs_next_device(pvs_cursor* c, int32_t n, int64_t* ids, float* scores
 pvs_status pvs_cursor_set_readahead(pvs_cursor* c, int32_t pages) {
     if (!c || pages < 1) return PVS_ERR_INVALID;
     c->readahead = pages;
+    c->readahead_set = true;
     return PVS_OK;
 }
 

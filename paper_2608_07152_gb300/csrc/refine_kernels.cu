@@ -29,7 +29,7 @@ __device__ inline void refine_warps(const int32_t* __restrict__ cand, const unsi
         int32_t w = 0, id = 0;
         float l = 0.0f, h = 0.0f;   // l == h: nothing to do
         if (mine < n) {
-            w = cand[mine];
+            w = cand ? cand[mine] : (int32_t)mine;
             l = w_lo[w];
             h = w_hi[w];
             id = w_id[w];
@@ -79,7 +79,9 @@ __device__ inline const float* stage_query(const float* qraw, int m_raw, int sta
 __global__ void __launch_bounds__(256, 3) refine_kernel(
     const int32_t* __restrict__ cand, const unsigned int* cand_len, const int32_t* __restrict__ w_id,
     float* w_lo, float* w_hi, float* lo, float* hi, const float* __restrict__ qraw,
-    const float* __restrict__ raw, int m_raw, int* status, DevCounters* ctr, int stage_q) {
+    const float* __restrict__ raw, int m_raw, int* status, DevCounters* ctr, int stage_q,
+    unsigned int limit) {
+    if (*cand_len > limit) return;
     const float* qf = stage_query(qraw, m_raw, stage_q);
     refine_warps(cand, cand_len, w_id, w_lo, w_hi, lo, hi, qf, qraw, raw, m_raw, status, ctr,
                  (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5),
@@ -166,7 +168,7 @@ __device__ inline void refine_ring(const RingRefs& a, int stages, int64_t warp0,
             const int64_t mine = pbase + lane * nwarps;
             bool need = false;
             if (mine < n) {
-                pw = a.cand[mine];
+                pw = a.cand ? a.cand[mine] : (int32_t)mine;
                 pl = a.w_lo[pw];
                 ph = a.w_hi[pw];
                 pid = a.w_id[pw];
@@ -233,7 +235,9 @@ __device__ inline void refine_ring(const RingRefs& a, int stages, int64_t warp0,
     }
 }
 
-__global__ void __launch_bounds__(kRingWarps * 32, 2) refine_ring_kernel(RingRefs a, int stages) {
+__global__ void __launch_bounds__(kRingWarps * 32, 2) refine_ring_kernel(RingRefs a, int stages,
+                                                                             unsigned int limit) {
+    if (*a.cand_len > limit) return;
     refine_ring(a, stages, (int64_t)blockIdx.x * kRingWarps + (threadIdx.x >> 5),
                 (int64_t)gridDim.x * kRingWarps);
 }
@@ -290,7 +294,7 @@ cudaError_t launch_refine_batch(const PullArgsPack& args_dev, int ncursors, int 
 cudaError_t launch_refine(const int32_t* cand, const unsigned int* cand_len,
                           const int32_t* w_id, float* w_lo, float* w_hi, float* lo, float* hi,
                           const float* qraw, const float* raw, int m_raw, int* status,
-                          DevCounters* ctr, int grid, cudaStream_t st) {
+                          DevCounters* ctr, int grid, cudaStream_t st, unsigned int limit) {
     const int stages = ring_stages(m_raw);
     if (stages) {
         const size_t smem = ring_smem_bytes(m_raw, stages);
@@ -298,13 +302,13 @@ cudaError_t launch_refine(const int32_t* cand, const unsigned int* cand_len,
         if (e != cudaSuccess) return e;
         count_launches(1);
         const RingRefs a{cand, cand_len, w_id, w_lo, w_hi, lo, hi, qraw, raw, m_raw, status, ctr};
-        refine_ring_kernel<<<grid, kRingWarps * 32, smem, st>>>(a, stages);
+        refine_ring_kernel<<<grid, kRingWarps * 32, smem, st>>>(a, stages, limit);
         return cudaGetLastError();
     }
     const int smem = query_stage_bytes(m_raw);
     count_launches(1);
     refine_kernel<<<grid, 256, smem, st>>>(cand, cand_len, w_id, w_lo, w_hi, lo, hi, qraw, raw,
-                                           m_raw, status, ctr, smem > 0);
+                                           m_raw, status, ctr, smem > 0, limit);
     return cudaGetLastError();
 }
 

@@ -147,6 +147,7 @@ struct pvs_cursor {
     int64_t ahead = 0, ahead_pos = 0;
     bool ahead_host = false;
     int32_t readahead = 4;            // a pull computes up to this many pages
+    bool readahead_set = false;       // by the caller; else the first pull may go further
     unsigned int* h_small = nullptr;  // pinned scratch (counts, status)
     // rank queries (fusion.cu): pinned staging, a second stream and an
     // event, kept between calls

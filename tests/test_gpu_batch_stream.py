@@ -93,7 +93,7 @@ def _serve(index, Q, ranks, page, on_device, snap=None, group=8):
 
 
 @pytest.mark.parametrize("nq,m,ranks,on_device", [
-    (9, 128, 100, False), (128, 96, 1024, True), (130, 384, 333, False), (200, 1024, 64, True)])
+    (17, 128, 100, False), (128, 96, 1024, True), (130, 384, 333, False), (200, 1024, 64, True)])
 def test_blocks_equal_lone_cursors(nq, m, ranks, on_device):
     V, Q = _mixture(70_003, m, nq, seed=nq, comps=50)
     index = pvs.pvs_build(V)
