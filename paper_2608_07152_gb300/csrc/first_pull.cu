@@ -20,11 +20,12 @@
 // working set and the first page, then a pull for every further 80 ranks.
 #include "kernels.h"
 #include "pvs_common.cuh"
+#include "sort_regs.cuh"
 
 namespace pvs {
 namespace {
 
-constexpr int kThreads = 1024;
+constexpr int kThreads = kSortThreads;
 constexpr int kWarps = kThreads / 32;
 constexpr int kBins = 2048;
 constexpr int kStageMax = 50 * 1024;   // values staged in shared memory (200 KB)
@@ -224,53 +225,6 @@ __global__ void __launch_bounds__(256) first_set_kernel(const float* __restrict_
             w_lo[at] = lo[r0 + j];
             w_hi[at] = hi[r0 + j];
             ++at;
-        }
-    }
-}
-
-// ---- descending sort of at most 1024 E keys, E per thread in registers -------
-// (the network of bitonic_desc_reg_kernel: strides under E within a thread,
-// under 32 E by shuffles, the rest through shared memory)
-template <int E>
-__device__ __forceinline__ void sort_desc(uint64_t (&v)[E], uint64_t* sk) {
-    const int t = threadIdx.x;
-    auto keep = [](uint64_t& a, uint64_t b, int i, int s, int size) {
-        const bool keep_max = ((i & s) == 0) == ((i & size) == 0);
-        a = keep_max ? (a > b ? a : b) : (a < b ? a : b);
-    };
-#pragma unroll 1
-    for (int size = 2; size <= 1024 * E; size <<= 1) {
-#pragma unroll 1
-        for (int s = size >> 1; s >= 32 * E; s >>= 1) {   // another warp's element
-            // element e of thread t at e 1024 + t: no bank conflicts
-#pragma unroll
-            for (int e = 0; e < E; ++e) sk[e * kThreads + t] = v[e];
-            __syncthreads();
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-                keep(v[e], sk[e * kThreads + (t ^ (s / E))], t * E + e, s, size);
-            __syncthreads();
-        }
-#pragma unroll 1
-        for (int s = min(size >> 1, 16 * E); s >= E; s >>= 1) {   // another lane's
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const uint64_t w = __shfl_xor_sync(0xffffffffu, v[e], s / E);
-                keep(v[e], w, t * E + e, s, size);
-            }
-        }
-#pragma unroll
-        for (int s = E / 2; s > 0; s >>= 1) {   // this thread's
-            if (s >= size) continue;
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                if (e & s) continue;
-                const bool desc = ((t * E + e) & size) == 0;
-                const uint64_t a = v[e], b = v[e | s];
-                const bool swap = (a < b) == desc;
-                v[e] = swap ? b : a;
-                v[e | s] = swap ? a : b;
-            }
         }
     }
 }

@@ -103,6 +103,27 @@ int grid_of(int64_t n) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, 152 * 8));
 }
 
+// Bitonic sort of pow2 keys in shared memory, ascending (after a barrier; ends
+// with one).
+__device__ __forceinline__ void sort_ascending(uint64_t* sk, int pow2) {
+    for (int size = 2; size <= pow2; size <<= 1) {
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            for (int i = threadIdx.x; i < pow2; i += blockDim.x) {
+                const int j = i ^ stride;
+                if (j > i) {
+                    const bool up = (i & size) == 0;
+                    const uint64_t a = sk[i], b = sk[j];
+                    if ((a > b) == up) {
+                        sk[i] = b;
+                        sk[j] = a;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+
 // The queried items' keys (score, id) in ascending order, in one CTA:
 // keys[i] = rank_key(score of ids[i], ids[i]), bitonic sort in shared memory.
 __global__ void __launch_bounds__(kRankQueryMax) query_keys_kernel(const int64_t* __restrict__ ids,
@@ -122,22 +143,7 @@ __global__ void __launch_bounds__(kRankQueryMax) query_keys_kernel(const int64_t
         sk[i] = k;
     }
     __syncthreads();
-    for (int size = 2; size <= pow2; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = threadIdx.x; i < pow2; i += blockDim.x) {
-                const int j = i ^ stride;
-                if (j > i) {
-                    const bool up = (i & size) == 0;
-                    const uint64_t a = sk[i], b = sk[j];
-                    if ((a > b) == up) {
-                        sk[i] = b;
-                        sk[j] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    }
+    sort_ascending(sk, pow2);
     for (int i = threadIdx.x; i < n; i += blockDim.x) keys[i] = sk[i];
 }
 
@@ -776,10 +782,46 @@ __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
     }
 }
 
-__global__ void gather_ranks_kernel(const int32_t* __restrict__ rank_of,
-                                    const int32_t* __restrict__ ids, int n, int32_t* out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = rank_of[ids[i]];
+// Ranks of a few items in a complete sparse ranking held as scores (S of every
+// item): the items' keys, sorted; rank_count_kernel counts every visible row's
+// key against them (lo = hi = S, so every row is placed); then an item's rank
+// is 1 + the rows above its key.  An item outside the support (S = 0, or
+// deleted) has key 0 and rank 0.
+__device__ __forceinline__ uint64_t sparse_key(const float* scores, const uint32_t* tomb,
+                                               int32_t id) {
+    const float s = scores[id];
+    return s > 0.0f && !tombstoned(tomb, id) ? rank_key(s, (uint32_t)id) : 0ull;
+}
+
+__global__ void __launch_bounds__(kRankQueryMax) sparse_keys_kernel(
+    const int32_t* __restrict__ ids, int n, const float* __restrict__ scores,
+    const uint32_t* __restrict__ tomb, uint64_t* keys) {
+    __shared__ uint64_t sk[kRankQueryMax];
+    int pow2 = 1;
+    while (pow2 < n) pow2 <<= 1;
+    for (int i = threadIdx.x; i < pow2; i += blockDim.x)
+        sk[i] = i < n ? sparse_key(scores, tomb, ids[i]) : ~0ull;   // padding sorts last
+    __syncthreads();
+    sort_ascending(sk, pow2);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) keys[i] = sk[i];
+}
+
+__global__ void __launch_bounds__(kRankQueryMax) sparse_ranks_kernel(
+    const int32_t* __restrict__ ids, int n, const float* __restrict__ scores,
+    const uint32_t* __restrict__ tomb, const uint64_t* __restrict__ keys,
+    const unsigned long long* __restrict__ hist, int32_t* out) {
+    __shared__ uint64_t sk[kRankQueryMax];
+    __shared__ unsigned long long h[kRankQueryMax + 1];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) sk[i] = keys[i];
+    for (int i = threadIdx.x; i <= n; i += blockDim.x) h[i] = hist[i];
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const uint64_t k = sparse_key(scores, tomb, ids[i]);
+        unsigned long long above = 0;
+        if (k)
+            for (int t = keys_at_most(sk, n, k); t <= n; ++t) above += h[t];
+        out[i] = k ? (int32_t)(above + 1) : 0;
+    }
 }
 
 // Every id of a sparse list: inside the snapshot, not deleted, not repeated
@@ -966,7 +1008,7 @@ void free_staged_list(StagedList* s) {
     cudaGetDevice(&prev);
     if (s->index) cudaSetDevice(s->index->device);
     if (s->stream) {
-        if (s->rank_of) cudaFreeAsync(s->rank_of, s->stream);
+        if (s->scores) cudaFreeAsync(s->scores, s->stream);
         if (s->list) cudaFreeAsync(s->list, s->stream);
         if (s->seen) cudaFreeAsync(s->seen, s->stream);
         if (s->status) cudaFreeAsync(s->status, s->stream);
@@ -1208,7 +1250,7 @@ pvs_status rank_queries(pvs_cursor* c, const int32_t* dense_ids, int32_t nd, boo
     }
     // sparse (second stream; a copy from pageable memory may hold this thread
     // until it is done, so the dense work is queued first): a PBM ranking's
-    // table read at the queried ids, or one pass over a host list (staged
+    // scores counted against the queried ids', or one pass over a host list (staged
     // ahead, or copied and checked here) that finds the queried ids, sorted
     // and without repeats
     int32_t* d_srank = nullptr;
@@ -1218,7 +1260,7 @@ pvs_status rank_queries(pvs_cursor* c, const int32_t* dense_ids, int32_t nd, boo
         return PVS_ERR_INVALID;
     }
     if (nsq > 0) {
-        const bool table = staged && staged->rank_of;
+        const bool table = staged && staged->scores;
         int nfind = nsq;
         if (!table) {
             uniq.assign(sparse_ids, sparse_ids + nsq);
@@ -1264,9 +1306,25 @@ pvs_status rank_queries(pvs_cursor* c, const int32_t* dense_ids, int32_t nd, boo
                                     cudaMemcpyDeviceToDevice, st2));
         }
         if (table) {
-            count_launches(1);
-            gather_ranks_kernel<<<(nsq + 255) / 256, 256, 0, st2>>>(staged->rank_of, d_sids, nsq,
-                                                                    d_srank);
+            uint64_t* d_keys = static_cast<uint64_t*>(alloc((size_t)nsq * 8, st2));
+            unsigned long long* d_hist =
+                static_cast<unsigned long long*>(alloc((size_t)(nsq + 1) * 16, st2));
+            if (!d_keys || !d_hist) {
+                cleanup();
+                return PVS_ERR_OOM;
+            }
+            RQ_CUDA(cudaMemsetAsync(d_hist, 0, (size_t)(nsq + 1) * 16, st2));
+            count_launches(3);
+            sparse_keys_kernel<<<1, kRankQueryMax, 0, st2>>>(d_sids, nsq, staged->scores,
+                                                             staged->tomb, d_keys);
+            const int64_t blocks = std::min<int64_t>(4 * (int64_t)std::max(x->num_sms, 1),
+                                                     (rows + kCountTile - 1) / kCountTile);
+            rank_count_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), kCountWarps * 32, 0, st2>>>(
+                staged->scores, staged->scores, rows, staged->tomb, c->qraw, x->raw, x->m_raw,
+                d_keys, nsq, 0, nullptr, nullptr, nullptr, x->m_pad, 1, c->qs, d_hist,
+                d_hist + nsq + 1, status + 1, c->ctr);
+            sparse_ranks_kernel<<<1, kRankQueryMax, 0, st2>>>(d_sids, nsq, staged->scores,
+                                                              staged->tomb, d_keys, d_hist, d_srank);
         } else {
             const int64_t n_list = staged ? std::max<int64_t>(ns, 0) : ns;
             RQ_CUDA(cudaMemsetAsync(d_srank, 0, (size_t)nfind * 4, st2));

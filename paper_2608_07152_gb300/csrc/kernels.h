@@ -327,8 +327,10 @@ constexpr int kBitonicMax = 8192;
 cudaError_t launch_bitonic_desc(uint64_t* keys, int count, cudaStream_t st);
 // LSD radix sort of `count` 64-bit keys descending; result in keys.
 size_t radix_sort_scratch_bytes(int64_t count);
+// high_word: by the upper 32 bits only, stably (keys already in descending
+// order of their lower word come out fully sorted, in half the passes).
 cudaError_t launch_radix_sort_desc(uint64_t* keys, uint64_t* tmp, int64_t count, void* scratch,
-                                   cudaStream_t st);
+                                   cudaStream_t st, bool high_word = false);
 // Emit the first n sorted keys: ids/scores out (device), mark emitted.
 cudaError_t launch_emit(const uint64_t* keys, int n, const int32_t* w_id, float* w_lo,
                         float* w_hi, float* lo, float* hi, int64_t* out_ids, float* out_scores,

@@ -115,7 +115,7 @@ struct pbm_cursor {
     int64_t* starts = nullptr;        // [nq][nchunk + 1]
     float* H = nullptr;               // [n_ranges], as computed at open
     uint64_t* rkeys = nullptr;        // [n_ranges] range keys, sorted descending at open
-    uint64_t* pool = nullptr;         // [n_items] rank keys of scored items
+    uint64_t* pool = nullptr;         // [n_ranges * block] rank keys of scored items
     pvs::PbmCounters* ctr = nullptr;  // device
     pvs::PbmCounters* h_ctr = nullptr;   // pinned mirror
     unsigned long long* sel64 = nullptr;   // [258]
@@ -393,7 +393,9 @@ pvs_status open_cursor(pbm_index* x, const std::shared_ptr<pvs::SnapData>& snap,
     c->last_key = ~0ull;
     c->n_pos = 0;
     c->next = 0;
-    c->E = 64;
+    // the first expansion: a 128th of a large id space costs a launch the same
+    // as 64 ranges and saves rounds, each with a host round trip
+    c->E = (uint64_t)std::max<int64_t>(64, x->n_ranges / 128);
     c->emitted = c->pulls = c->rounds = c->served_ahead = 0;
     c->state = PVS_OK;
     auto bail = [&](pvs_status s) {
@@ -414,7 +416,7 @@ pvs_status open_cursor(pbm_index* x, const std::shared_ptr<pvs::SnapData>& snap,
     }
     if ((!c->H && dalloc(&c->H, (size_t)x->n_ranges) != cudaSuccess) ||
         (!c->rkeys && dalloc(&c->rkeys, (size_t)x->n_ranges) != cudaSuccess) ||
-        (!c->pool && dalloc(&c->pool, (size_t)x->n_items) != cudaSuccess) ||
+        (!c->pool && dalloc(&c->pool, (size_t)x->n_ranges * (size_t)x->block) != cudaSuccess) ||
         (!c->ctr && dalloc(&c->ctr, 1) != cudaSuccess) ||
         (!c->sel64 && dalloc(&c->sel64, 258) != cudaSuccess) ||
         (!c->h_ctr && cudaMallocHost(reinterpret_cast<void**>(&c->h_ctr),
@@ -440,12 +442,14 @@ pvs_status open_cursor(pbm_index* x, const std::shared_ptr<pvs::SnapData>& snap,
         pvs::launch_pbm_range_keys(c->H, x->n_ranges, x->block, c->rkeys, st) != cudaSuccess)
         return bail(PVS_ERR_CUDA);
     // the expansion order: range keys sorted descending (the sort's scratch is
-    // the gather buffers, sized for at least n_ranges keys)
+    // the gather buffers, sized for at least n_ranges keys); they start in id
+    // order, so equal bounds keep it and only the bounds need sorting
     if (ensure_buffers(c, (uint64_t)x->n_ranges) != PVS_OK) return bail(PVS_ERR_OOM);
     if (x->n_ranges > 1 &&
         ((uint64_t)x->n_ranges <= (uint64_t)pvs::kBitonicMax
              ? pvs::launch_bitonic_desc(c->rkeys, (int)x->n_ranges, st)
-             : pvs::launch_radix_sort_desc(c->rkeys, c->tmp, x->n_ranges, c->sort_scratch, st)) !=
+             : pvs::launch_radix_sort_desc(c->rkeys, c->tmp, x->n_ranges, c->sort_scratch, st,
+                                           /*high_word=*/true)) !=
             cudaSuccess)
         return bail(PVS_ERR_CUDA);
     if (cudaMemcpyAsync(c->h_ctr, c->ctr, sizeof(pvs::PbmCounters), cudaMemcpyDeviceToHost,
@@ -463,10 +467,10 @@ namespace pvs {
 const SnapData* pbm_cursor_snapshot(const pbm_cursor* c) { return c->snap.get(); }
 
 // The complete sparse ranking of the cursor's query as a staged list: every
-// item's S in the query's term order (the expand kernel's evaluation), the
-// visible items with S > 0 sorted by key, their positions scattered into
-// rank_of.  Runs on a stream of its own and waits for it once (for the
-// member count), so the caller may be a helper thread.
+// item's S in the query's term order (the expand kernel's evaluation).  An
+// item's rank is a count over them (rank_queries); sorting the ranking for a
+// few items' positions took 30 launches and a host round trip.  Queued on a
+// stream of its own.
 pvs_status pbm_stage_ranks(pbm_cursor* c, pvs_index* owner, StagedList** out) {
     *out = nullptr;
     if (!c || !c->index || !owner || c->state < 0) return PVS_ERR_INVALID;
@@ -479,52 +483,22 @@ pvs_status pbm_stage_ranks(pbm_cursor* c, pvs_index* owner, StagedList** out) {
     if (!s) return PVS_ERR_OOM;
     s->index = owner;
     s->rows = x->n_items;
+    s->tomb = c->snap ? c->snap->d_tomb : nullptr;
     const size_t n = (size_t)std::max<int64_t>(x->n_items, 1);
-    const uint32_t* tomb = c->snap ? c->snap->d_tomb : nullptr;
-    float* acc = nullptr;
-    uint64_t* keys = nullptr;
-    uint64_t* tmp = nullptr;
-    void* scratch = nullptr;
-    unsigned long long* count = nullptr;
-    unsigned long long* h_count = nullptr;
     cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
-    auto pool_alloc = [&](void** p, size_t bytes) {
-        if (e == cudaSuccess)
-            e = cudaMallocFromPoolAsync(p, std::max<size_t>(bytes, 16), owner->scratch_pool,
-                                        s->stream);
-    };
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ready, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMallocHost(&h_count, sizeof(unsigned long long));
-    pool_alloc(reinterpret_cast<void**>(&s->rank_of), n * 4);
-    pool_alloc(reinterpret_cast<void**>(&s->status), sizeof(int));
-    pool_alloc(reinterpret_cast<void**>(&acc), n * 4);
-    pool_alloc(reinterpret_cast<void**>(&keys), n * 8);
-    pool_alloc(reinterpret_cast<void**>(&count), sizeof(unsigned long long));
-    const int grid = std::max(1, x->num_sms) * 8;
-    if (e == cudaSuccess) e = cudaMemsetAsync(s->rank_of, 0, n * 4, s->stream);
+    if (e == cudaSuccess)
+        e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&s->scores), n * 4,
+                                    owner->scratch_pool, s->stream);
+    if (e == cudaSuccess)
+        e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&s->status), 16, owner->scratch_pool,
+                                    s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->status, 0, sizeof(int), s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, n * 4, s->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(count, 0, sizeof(unsigned long long), s->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->scores, 0, n * 4, s->stream);
     if (e == cudaSuccess)
         e = launch_pbm_score_all(PbmQuery{c->terms, c->weights, c->nq}, x->term_off, x->docs,
-                                 x->imps, acc, grid, s->stream);
-    if (e == cudaSuccess)
-        e = launch_pbm_member_keys(acc, x->n_items, tomb, keys, count, grid, s->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(h_count, count, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
-                            s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    const int64_t m = e == cudaSuccess ? (int64_t)*h_count : 0;
-    if (m > 1) {
-        pool_alloc(reinterpret_cast<void**>(&tmp), (size_t)m * 8);
-        pool_alloc(&scratch, radix_sort_scratch_bytes(m));
-        if (e == cudaSuccess) e = launch_radix_sort_desc(keys, tmp, m, scratch, s->stream);
-    }
-    if (e == cudaSuccess) e = launch_pbm_rank_of(keys, m, s->rank_of, grid, s->stream);
+                                 x->imps, s->scores, std::max(1, x->num_sms) * 8, s->stream);
     if (e == cudaSuccess) e = cudaEventRecord(s->ready, s->stream);
-    for (void* p : {(void*)acc, (void*)keys, (void*)tmp, scratch, (void*)count})
-        if (p) cudaFreeAsync(p, s->stream);
-    if (h_count) cudaFreeHost(h_count);
     if (e != cudaSuccess) {
         cudaGetLastError();
         free_staged_list(s);
@@ -621,6 +595,7 @@ pvs_status pbm_next(pbm_cursor* c, int32_t n, int64_t* ids, float* scores, int32
         pvs::PbmExpandArgs a{};
         a.ranges = c->rkeys + c->next;
         a.count = (int64_t)k;
+        a.pos = c->next;
         a.q = pvs::PbmQuery{c->terms, c->weights, c->nq};
         a.starts = c->starts;
         a.nchunk = x->nchunk;
@@ -633,7 +608,7 @@ pvs_status pbm_next(pbm_cursor* c, int32_t n, int64_t* ids, float* scores, int32
         a.tomb = c->snap ? c->snap->d_tomb : nullptr;
         a.pool = c->pool;
         a.ctr = c->ctr;
-        e = pvs::launch_pbm_expand(a, (int)std::min<uint64_t>(k, (uint64_t)x->num_sms * 4), st);
+        e = pvs::launch_pbm_expand(a, x->num_sms, st);
         if (e != cudaSuccess) return fail(c, cuda_status(e));
         c->next += (int64_t)k;
         last = k;
@@ -642,15 +617,35 @@ pvs_status pbm_next(pbm_cursor* c, int32_t n, int64_t* ids, float* scores, int32
     // the next pull starts from the size of the expansion that last sufficed
     if (last) c->E = std::max<uint64_t>(16, last);
     const uint64_t m = std::min<uint64_t>(need, window);
-    if (served) {
+    if (!served && m > 0 && m <= (uint64_t)pvs::kPbmFastWindow) {
+        // a window past kPbmFastWindow: its first kPbmFastWindow keys serve
+        // this pull and the next ones (selecting each pull's own few keys
+        // anew took 17 launches a page)
+        const uint64_t keep = pvs::kPbmFastWindow;
+        cudaError_t e = pvs::launch_pbm_select64(c->pool, c->ctr, c->last_key, keep, c->sel64, st);
+        if (e == cudaSuccess)
+            e = pvs::launch_pbm_collect(c->pool, c->sel64, c->last_key, c->buf, c->buf_cap, c->ctr,
+                                        st);
+        if (e == cudaSuccess)
+            e = pvs::launch_pbm_finish(c->buf, c->ctr, need, false, c->h_ids, c->h_scores, c->h_ctr,
+                                       st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return fail(c, cuda_status(e));
+        if (c->h_ctr->status != 0) return fail(c, (pvs_status)c->h_ctr->status);
+        if (c->h_ctr->collected != keep) return fail(c, PVS_ERR_INVALID);   // internal invariant
+        std::memcpy(ids, c->h_ids, m * sizeof(int64_t));
+        std::memcpy(scores, c->h_scores, m * sizeof(float));
+        c->ahead_pos = (int64_t)m;
+        c->ahead_len = (int64_t)keep;
+        c->ahead_complete = false;
+    } else if (served) {
         std::memcpy(ids, c->h_ids, m * sizeof(int64_t));
         std::memcpy(scores, c->h_scores, m * sizeof(float));
         c->ahead_pos = (int64_t)m;
         c->ahead_len = (int64_t)window;
         c->ahead_complete = complete;
     } else if (m > 0) {
-        // large window: the m-th largest key first (or the whole window when
-        // it fits the gather buffer), then a device sort of the m keys
+        // a large pull: the m-th largest key first, then a device sort of the m keys
         pvs_status s = ensure_buffers(c, m);
         if (s != PVS_OK) return fail(c, s);
         cudaError_t e = pvs::launch_pbm_select64(c->pool, c->ctr, c->last_key, m, c->sel64, st);

@@ -22,6 +22,7 @@
 
 #include "pbm_kernels.h"
 #include "pvs_common.cuh"
+#include "sort_regs.cuh"
 
 namespace pvs {
 
@@ -389,7 +390,28 @@ cudaError_t launch_pbm_window(const uint64_t* sorted, int64_t next, int64_t n_ra
     return cudaGetLastError();
 }
 
-constexpr int kFinishThreads = 1024;
+constexpr int kFinishThreads = kSortThreads;
+
+// The whole window, sorted, to pinned memory: every key in it is certified,
+// so the host can serve later pulls from what lies beyond `need`.
+template <int E>
+__device__ __forceinline__ void finish_sorted(const uint64_t* keys_in, int count, uint64_t* sk,
+                                              int64_t* h_ids, float* h_scores) {
+    uint64_t v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = threadIdx.x + e * kFinishThreads;
+        v[e] = i < count ? keys_in[i] : 0ull;   // 0 sorts last
+    }
+    sort_desc<E>(v, sk);
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int r = threadIdx.x * E + e;
+        if (r >= count) continue;
+        h_ids[r] = (int64_t)rank_key_id(v[e]);
+        h_scores[r] = rank_key_score(v[e]);
+    }
+}
 
 __global__ void __launch_bounds__(kFinishThreads) pbm_finish_kernel(const uint64_t* keys_in,
                                                                     const PbmCounters* ctr,
@@ -401,34 +423,11 @@ __global__ void __launch_bounds__(kFinishThreads) pbm_finish_kernel(const uint64
     const unsigned long long count = ctr->collected;
     if (need > 0 && count >= 1 && (count >= need || complete) &&
         count <= (unsigned long long)kPbmFastWindow) {
-        int pow2 = 1;
-        while ((unsigned long long)pow2 < count) pow2 <<= 1;
-        for (int i = threadIdx.x; i < pow2; i += blockDim.x)
-            keys[i] = (unsigned long long)i < count ? keys_in[i] : 0ull;   // 0 sorts last
-        __syncthreads();
-        // bitonic sort, descending
-        for (int k = 2; k <= pow2; k <<= 1) {
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = threadIdx.x; i < pow2; i += blockDim.x) {
-                    const int ixj = i ^ j;
-                    if (ixj > i) {
-                        const uint64_t a = keys[i], b = keys[ixj];
-                        const bool swap = (i & k) == 0 ? a < b : a > b;
-                        if (swap) {
-                            keys[i] = b;
-                            keys[ixj] = a;
-                        }
-                    }
-                }
-                __syncthreads();
-            }
-        }
-        // the whole window, sorted: every key in it is certified, so the
-        // host can serve later pulls from what lies beyond `need`
-        for (int i = threadIdx.x; (unsigned long long)i < count; i += blockDim.x) {
-            h_ids[i] = (int64_t)rank_key_id(keys[i]);
-            h_scores[i] = rank_key_score(keys[i]);
-        }
+        const int n = (int)count;
+        if (n <= 1024) finish_sorted<1>(keys_in, n, keys, h_ids, h_scores);
+        else if (n <= 2048) finish_sorted<2>(keys_in, n, keys, h_ids, h_scores);
+        else if (n <= 4096) finish_sorted<4>(keys_in, n, keys, h_ids, h_scores);
+        else finish_sorted<8>(keys_in, n, keys, h_ids, h_scores);
     }
     __syncthreads();
     if (threadIdx.x == 0) *h_mirror = *ctr;
@@ -455,14 +454,88 @@ cudaError_t launch_pbm_finish(const uint64_t* keys, const PbmCounters* ctr, uint
 // them.
 constexpr int kExpandThreads = 256;
 
+__device__ __forceinline__ uint64_t item_key(const PbmExpandArgs& a, float v, int64_t id) {
+    if (!isfinite(v)) set_status(&a.ctr->status, PVS_ERR_OVERFLOW);
+    const bool dead = a.tomb != nullptr && ((__ldg(a.tomb + (id >> 5)) >> (id & 31)) & 1u);
+    return (v > 0.0f && !dead) ? rank_key(v, (uint32_t)id) : 0ull;
+}
+
+// The same, one warp per range: up to 32 query terms (a lane finds each
+// term's block) and ranges of up to kWarpBlock items.  A range holds a few
+// postings of each term, so a range's time is its chain of dependent loads;
+// eight times the ranges in flight per CTA (4M items, 128-item ranges: 22 to
+// 37 us per launch of one CTA per range).
+constexpr int kWarpBlock = 512;
+
+__global__ void __launch_bounds__(kExpandThreads) pbm_expand_warp_kernel(PbmExpandArgs a) {
+    extern __shared__ float warp_scores[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nwarps = blockDim.x >> 5;
+    float* s = warp_scores + (size_t)warp * a.block;
+    const int nq = a.q.nq;
+    const float w_mine = lane < nq ? a.q.weights[lane] : 0.0f;
+    const int64_t per = a.nchunk + 1;
+    unsigned long long visited = 0, items = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctr->pool_len = (unsigned long long)((a.pos + a.count) * a.block);
+        a.ctr->ranges_expanded += (unsigned long long)a.count;
+    }
+    for (int64_t e = (int64_t)blockIdx.x * nwarps + warp; e < a.count;
+         e += (int64_t)gridDim.x * nwarps) {
+        const int64_t r = (int64_t)rank_key_id(a.ranges[e]) / a.block;
+        const int64_t k = r / kPbmChunk;
+        const int64_t first = r * a.block;
+        const int64_t rest = a.n_items - first;
+        const int cnt = (int)(rest < a.block ? rest : a.block);
+        int64_t pb = 0, pe = 0;
+        if (lane < nq) {
+            const int64_t s1 = a.starts[lane * per + k + 1];
+            const int64_t j = lower_bound_i32(a.blk_range, a.starts[lane * per + k], s1, r);
+            if (j < s1 && a.blk_range[j] == r) {
+                pb = a.blk_pbeg[j];
+                pe = a.blk_pbeg[j + 1];
+            }
+        }
+        visited += (unsigned long long)(pe - pb);
+        items += lane == 0 ? (unsigned long long)cnt : 0ull;
+        for (int x = lane; x < a.block; x += 32) s[x] = 0.0f;
+        __syncwarp();
+        unsigned int has = __ballot_sync(0xffffffffu, pe > pb);
+        while (has) {   // terms in query order
+            const int i = __ffs(has) - 1;
+            has &= has - 1;
+            const int64_t b0 = __shfl_sync(0xffffffffu, pb, i), b1 = __shfl_sync(0xffffffffu, pe, i);
+            const float wi = __shfl_sync(0xffffffffu, w_mine, i);
+            for (int64_t p = b0 + lane; p < b1; p += 32) {
+                const int64_t x = (int64_t)a.docs[p] - first;
+                if (x >= 0 && x < cnt)
+                    s[x] = __fadd_rn(s[x], __fmul_rn(wi, a.imps[p]));
+                else
+                    set_status(&a.ctr->status, PVS_ERR_INVALID);   // metadata out of order
+            }
+            __syncwarp();
+        }
+        uint64_t* pool = a.pool + (a.pos + e) * a.block;
+        for (int x = lane; x < a.block; x += 32)
+            pool[x] = x < cnt ? item_key(a, s[x], first + x) : 0ull;
+        __syncwarp();   // s is reused by the next range
+    }
+    visited = warp_sum(visited);
+    if (lane == 0) {
+        if (visited) atomicAdd(&a.ctr->postings, visited);
+        if (items) atomicAdd(&a.ctr->items, items);
+    }
+}
+
 __global__ void __launch_bounds__(kExpandThreads) pbm_expand_kernel(PbmExpandArgs a) {
     __shared__ float s[kPbmMaxBlock];
     __shared__ float w[kPbmMaxTerms];
     __shared__ int64_t pb[kPbmMaxTerms];
     __shared__ int64_t pe[kPbmMaxTerms];
-    __shared__ unsigned long long base_sh;
     const int nq = a.q.nq;
     for (int i = threadIdx.x; i < nq; i += blockDim.x) w[i] = a.q.weights[i];
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        a.ctr->pool_len = (unsigned long long)((a.pos + a.count) * a.block);
     const int64_t per = a.nchunk + 1;
     for (int64_t e = blockIdx.x; e < a.count; e += gridDim.x) {
         const int64_t r = (int64_t)rank_key_id(a.ranges[e]) / a.block;
@@ -498,29 +571,30 @@ __global__ void __launch_bounds__(kExpandThreads) pbm_expand_kernel(PbmExpandArg
             __syncthreads();
         }
         if (threadIdx.x == 0) {
-            base_sh = atomicAdd(&a.ctr->pool_len, (unsigned long long)cnt);
             atomicAdd(&a.ctr->ranges_expanded, 1ull);
             atomicAdd(&a.ctr->postings, visited);
             atomicAdd(&a.ctr->items, (unsigned long long)cnt);
         }
-        __syncthreads();
-        const unsigned long long base = base_sh;
-        for (int x = threadIdx.x; x < cnt; x += blockDim.x) {
-            const float v = s[x];
-            if (!isfinite(v)) set_status(&a.ctr->status, PVS_ERR_OVERFLOW);
-            const int64_t id = first + x;
-            const bool dead =
-                a.tomb != nullptr && ((__ldg(a.tomb + (id >> 5)) >> (id & 31)) & 1u);
-            a.pool[base + x] = (v > 0.0f && !dead) ? rank_key(v, (uint32_t)id) : 0ull;
-        }
+        uint64_t* pool = a.pool + (a.pos + e) * a.block;
+        for (int x = threadIdx.x; x < a.block; x += blockDim.x)
+            pool[x] = x < cnt ? item_key(a, s[x], first + x) : 0ull;
         __syncthreads();   // s, pb, pe are reused by the next range
     }
 }
 
-cudaError_t launch_pbm_expand(const PbmExpandArgs& a, int grid, cudaStream_t st) {
-    if (grid < 1) grid = 1;
+cudaError_t launch_pbm_expand(const PbmExpandArgs& a, int num_sms, cudaStream_t st) {
+    if (a.count <= 0) return cudaSuccess;
     count_launches(1);
-    pbm_expand_kernel<<<grid, kExpandThreads, 0, st>>>(a);
+    if (a.q.nq <= 32 && a.block <= kWarpBlock) {
+        constexpr int kWarps = kExpandThreads / 32;
+        const int64_t want = (a.count + kWarps - 1) / kWarps;
+        const unsigned grid = (unsigned)(want < 8 * (int64_t)num_sms ? want : 8 * (int64_t)num_sms);
+        pbm_expand_warp_kernel<<<grid, kExpandThreads, (size_t)kWarps * a.block * sizeof(float),
+                                 st>>>(a);
+        return cudaGetLastError();
+    }
+    const int64_t most = 4 * (int64_t)num_sms;
+    pbm_expand_kernel<<<(unsigned)(a.count < most ? a.count : most), kExpandThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -592,19 +666,27 @@ __global__ void pbm_sel_hist_kernel(const uint64_t* __restrict__ pool, const Pbm
         if (h[i]) atomicAdd(&sel[2 + i], (unsigned long long)h[i]);
 }
 
-__global__ void pbm_sel_pick_kernel(int shift, unsigned long long* sel) {
-    if (threadIdx.x != 0) return;
-    unsigned long long k = sel[1], cum = 0;
-    for (int d = 255; d >= 0; --d) {
-        const unsigned long long c = sel[2 + d];
-        if (cum + c >= k) {
-            sel[0] |= (unsigned long long)d << shift;
-            sel[1] = k - cum;
-            break;
-        }
-        cum += c;
+// One block of 256 threads, thread t the digit 255 - t: the digit whose keys
+// hold the wanted rank (suffix counts by a scan).
+__global__ void __launch_bounds__(256) pbm_sel_pick_kernel(int shift, unsigned long long* sel) {
+    __shared__ unsigned long long tot[8];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const unsigned long long c = sel[2 + 255 - t];
+    const unsigned long long k = sel[1];
+    unsigned long long incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long up = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += up;
     }
-    for (int i = 0; i < 256; ++i) sel[2 + i] = 0;
+    if (lane == 31) tot[warp] = incl;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) incl += tot[w];
+    if (incl - c < k && k <= incl) {   // one thread
+        sel[0] |= (unsigned long long)(255 - t) << shift;
+        sel[1] = k - (incl - c);
+    }
+    sel[2 + 255 - t] = 0;
 }
 
 cudaError_t launch_pbm_select64(const uint64_t* pool, const PbmCounters* ctr, uint64_t hi,
@@ -614,7 +696,7 @@ cudaError_t launch_pbm_select64(const uint64_t* pool, const PbmCounters* ctr, ui
     for (int shift = 56; shift >= 0; shift -= 8) {
         count_launches(2);
         pbm_sel_hist_kernel<<<152 * 4, 256, 0, st>>>(pool, ctr, hi, shift, sel64);
-        pbm_sel_pick_kernel<<<1, 32, 0, st>>>(shift, sel64);
+        pbm_sel_pick_kernel<<<1, 256, 0, st>>>(shift, sel64);
     }
     return cudaGetLastError();
 }
@@ -663,40 +745,6 @@ cudaError_t launch_pbm_score_all(const PbmQuery& q, const int64_t* term_off, con
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
-}
-
-__global__ void pbm_member_keys_kernel(const float* __restrict__ acc, int64_t n,
-                                       const uint32_t* __restrict__ tomb, uint64_t* keys,
-                                       unsigned long long* count) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += stride) {
-        const float s = acc[x];
-        if (s > 0.0f && !tombstoned(tomb, x))
-            keys[atomicAdd(count, 1ull)] = rank_key(s, (uint32_t)x);
-    }
-}
-
-cudaError_t launch_pbm_member_keys(const float* acc, int64_t n, const uint32_t* tomb,
-                                   uint64_t* keys, unsigned long long* count, int grid,
-                                   cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    count_launches(1);
-    pbm_member_keys_kernel<<<grid, 256, 0, st>>>(acc, n, tomb, keys, count);
-    return cudaGetLastError();
-}
-
-__global__ void pbm_rank_of_kernel(const uint64_t* __restrict__ keys, int64_t m, int32_t* rank_of) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride)
-        rank_of[rank_key_id(keys[i])] = (int32_t)(i + 1);
-}
-
-cudaError_t launch_pbm_rank_of(const uint64_t* keys, int64_t m, int32_t* rank_of, int grid,
-                               cudaStream_t st) {
-    if (m <= 0) return cudaSuccess;
-    count_launches(1);
-    pbm_rank_of_kernel<<<grid, 256, 0, st>>>(keys, m, rank_of);
-    return cudaGetLastError();
 }
 
 }  // namespace pvs

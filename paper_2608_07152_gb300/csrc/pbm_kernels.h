@@ -85,9 +85,12 @@ constexpr int kPbmFastWindow = 8192;
 cudaError_t launch_pbm_finish(const uint64_t* keys, const PbmCounters* ctr, uint64_t need,
                               bool complete, int64_t* h_ids, float* h_scores,
                               PbmCounters* h_mirror, cudaStream_t st);
+// The range at position pos + e of the sorted order puts its items' keys at
+// pool[(pos + e) * block ..] (key 0 past the last item of the id space).
 struct PbmExpandArgs {
     const uint64_t* ranges;       // sorted range keys of the ranges to expand
     int64_t count;                // how many
+    int64_t pos;                  // ranges expanded before these
     PbmQuery q;
     const int64_t* starts;
     int64_t nchunk;
@@ -101,7 +104,7 @@ struct PbmExpandArgs {
     uint64_t* pool;
     PbmCounters* ctr;
 };
-cudaError_t launch_pbm_expand(const PbmExpandArgs& a, int grid, cudaStream_t st);
+cudaError_t launch_pbm_expand(const PbmExpandArgs& a, int num_sms, cudaStream_t st);
 // Pool keys k with ctr->kmax < k < hi and k >= *from (from may be null)
 // appended to out in any order (ctr->collected counts them; at most cap written).
 cudaError_t launch_pbm_collect(const uint64_t* pool, const unsigned long long* from, uint64_t hi,
@@ -118,13 +121,5 @@ cudaError_t launch_pbm_emit(const uint64_t* keys, int m, int64_t* ids, float* sc
 // by the caller), the evaluation of the expand kernel for every item.
 cudaError_t launch_pbm_score_all(const PbmQuery& q, const int64_t* term_off, const int32_t* docs,
                                  const float* imps, float* acc, int grid, cudaStream_t st);
-// keys[0 .. *count) = rank keys of the visible items with acc > 0, in any
-// order (*count zeroed by the caller).
-cudaError_t launch_pbm_member_keys(const float* acc, int64_t n, const uint32_t* tomb,
-                                   uint64_t* keys, unsigned long long* count, int grid,
-                                   cudaStream_t st);
-// rank_of[id of keys[i]] = i + 1 for i < m (keys sorted descending).
-cudaError_t launch_pbm_rank_of(const uint64_t* keys, int64_t m, int32_t* rank_of, int grid,
-                               cudaStream_t st);
 
 }  // namespace pvs

@@ -219,18 +219,18 @@ constexpr int32_t kRankQueryMax = 1024;
 // A sparse list on the device ahead of need.  From a host list
 // (stage_sparse_list): the ids copied, and checked as in fuse_complete (the
 // verdict is read when the ranks are used); rank_queries finds its ids in the
-// list.  From a PBM query (pbm_stage_ranks): rank_of[x] = position + 1 of id
-// x (0: not in the list).  Built on its own stream (stage_sparse_list may hold
+// list.  From a PBM query (pbm_stage_ranks): scores[x] = S(x) of every item;
+// rank_queries counts the items above the queried ones.  Built on its own stream (stage_sparse_list may hold
 // the calling thread while the pageable list is copied); rank_queries orders
 // its reads after it.
 struct StagedList {
     pvs_index* index = nullptr;       // device and scratch pool
     cudaStream_t stream = nullptr;
     cudaEvent_t ready = nullptr;      // recorded after the scatter
-    int32_t* rank_of = nullptr;       // [rows], or null: look the ids up in `list`
+    float* scores = nullptr;          // [rows], or null: look the ids up in `list`
     int64_t* list = nullptr;          // the list's ids on the device (or null)
     uint32_t* seen = nullptr;         // a bit per id, set by the check of `list`
-    const uint32_t* tomb = nullptr;   // the snapshot's deletions, for the check
+    const uint32_t* tomb = nullptr;   // the snapshot's deletions
     int64_t n = 0;                    // ids in `list`
     bool checked = true;              // the check of `list` is queued
     int* status = nullptr;            // the scatter's verdict on the ids
@@ -244,7 +244,7 @@ pvs_status stage_sparse_list(pvs_cursor* dense, const int64_t* sparse, int64_t n
 pvs_status check_staged_list(StagedList* s);
 // The complete ranking of a PBM cursor's query (U_s = the visible items with
 // S > 0, by (S desc, id asc), S evaluated as the PBM kernels do, App. A.2)
-// staged the same way (pbm_capi.cu); scratch from pool_owner's pool.
+// staged as scores (pbm_capi.cu); memory from pool_owner's pool.
 pvs_status pbm_stage_ranks(pbm_cursor* sparse, pvs_index* pool_owner, StagedList** out);
 void free_staged_list(StagedList* s);
 // `staged` (or null): the same list, already scattered.
