@@ -292,26 +292,127 @@ __device__ inline float exact_dot_warp_eft(const float* q_fast, const float* __r
     return exact_dot_warp_slow(q, v, m_raw, used_fallback);
 }
 
-// The same score with the row already in shared memory (v_sh, generic loads);
-// v (global) is the same row for the exact path.
-__device__ inline float exact_dot_warp_eft_smem(const float* q_fast, const float* __restrict__ q,
+// ---- two chains per instruction (f32x2), for rows staged in shared memory -----
+__device__ __forceinline__ uint64_t f2_pack(float x, float y) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float& x, float& y) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_fma_ru(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rp.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// Two chains of the error-free transformations above (components x, z and
+// y, w of the float4s), one f32x2 instruction a step.  There is no packed
+// subtraction: a - b is fma(b, -1, a), exact in the product, and the
+// product's error comes negated from the negated query.  vv: sum of squares of
+// the row, rounded up.
+struct EftAcc2 {
+    uint64_t s = 0, c = 0, vv = 0;
+    __device__ __forceinline__ void add_products(uint64_t x, uint64_t xneg, uint64_t y,
+                                                 uint64_t m1) {
+        const uint64_t p = f2_mul(x, y);
+        const uint64_t nep = f2_fma(xneg, y, p);       // -(x y - p)
+        const uint64_t s1 = f2_add(s, p);              // TwoSum(s, p)
+        const uint64_t bb = f2_fma(s, m1, s1);
+        const uint64_t es = f2_add(f2_fma(f2_fma(bb, m1, s1), m1, s), f2_fma(bb, m1, p));
+        s = s1;
+        c = f2_add(c, f2_fma(nep, m1, es));
+        vv = f2_fma_ru(y, y, vv);
+    }
+};
+
+// RU(||x||) over m_raw floats of shared memory, by one warp.
+__device__ __forceinline__ float norm_up_warp(const float* x, int m_raw) {
+    float s = 0.0f;
+    for (int j = threadIdx.x & 31; j < m_raw; j += kWarp) s = __fmaf_ru(x[j], x[j], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s = __fadd_ru(s, __shfl_xor_sync(0xffffffffu, s, o));
+    return __fsqrt_ru(s);
+}
+
+// The same score with the row already in shared memory (v_sh), and the query
+// and its negative (q_sh, qneg_sh; q_norm >= ||q||); v (global) is the same
+// row for the exact path.  In place of running sums of |error terms| the
+// error of the error sum is bounded in advance.  With u = 2^-24, K products
+// per chain and S = sum |q_j v_j| <= ||q|| ||v||: every partial sum is at most
+// (1 + K u) S_chain, so the error terms of a chain sum to at most
+// u (K + 1) S_chain in magnitude, and the roundings of each of them and of each
+// partial sum of theirs to u^2 (K + 1)^2 S_chain.  Merging the 64 chains takes
+// six levels; at each, the partial error sums are at most u (K + 7) S together
+// and are rounded twice: 12 u^2 (K + 7) S.  (1.01 covers the factors 1 + O(K u).)
+// What bounds it is the instructions a product costs (17 with two running
+// sums of magnitudes, 11 half ones here) and their issue, not memory: 256
+// working sets of 977 rows of 768 took 227 us as one chain an instruction and
+// take 199 us (3.8 TB/s of rows), 256 of about 1,100 rows 254 us and 204 us.
+__device__ inline float exact_dot_warp_eft_smem(const float* q_sh, const float* qneg_sh,
+                                                float q_norm, const float* __restrict__ q,
                                                 const float* v_sh, const float* __restrict__ v,
                                                 int m_raw, bool* used_fallback) {
     const int lane = threadIdx.x & 31;
-    const float4* q4 = reinterpret_cast<const float4*>(q_fast);
-    const float4* v4 = reinterpret_cast<const float4*>(v_sh);
-    EftAcc acc, acc2;   // two dependency chains, merged as in the butterfly
+    const ulonglong2* q2 = reinterpret_cast<const ulonglong2*>(q_sh);
+    const ulonglong2* n2 = reinterpret_cast<const ulonglong2*>(qneg_sh);
+    const ulonglong2* v2 = reinterpret_cast<const ulonglong2*>(v_sh);
+    const uint64_t m1 = f2_pack(-1.0f, -1.0f);
+    EftAcc2 acc;
     const int n4 = m_raw >> 2;
+#pragma unroll 3
     for (int j = lane; j < n4; j += kWarp) {
-        const float4 x = q4[j], y = v4[j];
-        acc.add_product(x.x, y.x);
-        acc2.add_product(x.y, y.y);
-        acc.add_product(x.z, y.z);
-        acc2.add_product(x.w, y.w);
+        const ulonglong2 x = q2[j], xn = n2[j], y = v2[j];
+        acc.add_products(x.x, xn.x, y.x, m1);
+        acc.add_products(x.y, xn.y, y.y, m1);
     }
-    acc.merge(acc2.s, acc2.c, acc2.a1, acc2.a2);
-    float r;
-    if (eft_finish(acc, m_raw, &r)) {
+    float s, s2, c, c2, vv, vv2;
+    f2_unpack(acc.s, s, s2);
+    f2_unpack(acc.c, c, c2);
+    f2_unpack(acc.vv, vv, vv2);
+    vv = __fadd_ru(vv, vv2);
+    auto merge = [&](float so, float co) {   // commutative: all lanes end alike
+        float es;
+        two_sum_f(s, so, s, es);
+        c = __fadd_rn(__fadd_rn(c, co), es);
+    };
+    merge(s2, c2);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const float so = __shfl_xor_sync(0xffffffffu, s, off);
+        const float co = __shfl_xor_sync(0xffffffffu, c, off);
+        vv = __fadd_ru(vv, __shfl_xor_sync(0xffffffffu, vv, off));
+        merge(so, co);
+    }
+    float r, e2;
+    two_sum_f(s, c, r, e2);
+    const float ar = fabsf(r);
+    const float K = (float)(2 * ((n4 + 31) / 32));
+    const float coef = (1.01f * 0x1p-48f) * ((K + 1.0f) * (K + 1.0f) + 12.0f * (K + 7.0f));
+    const float S = __fmul_ru(q_norm, __fsqrt_ru(vv));
+    const float bound =
+        __fadd_ru(fabsf(e2), __fadd_ru(__fmul_ru(coef, S), __fmul_ru((float)m_raw, 0x1p-149f)));
+    const unsigned int bits = __float_as_uint(ar);
+    const float ulp = __uint_as_float(bits & 0x7f800000u) * 0x1p-23f;
+    const float half_gap = (bits & 0x007fffffu) ? ulp * 0.5f : ulp * 0.25f;
+    // (a value that is not finite, or outside the range, fails the comparison)
+    if (ar >= 0x1p-100f && ar <= 0x1p+126f && isfinite(c) && bound < half_gap) {
         *used_fallback = false;
         return r;
     }

@@ -128,11 +128,11 @@ struct RingRefs {
     DevCounters* ctr;
 };
 
-// Dynamic shared memory: q [m_raw] | rows [kRingWarps][stages][m_raw] |
+// Dynamic shared memory: q [m_raw] | -q [m_raw] | rows [kRingWarps][stages][m_raw] |
 // bars [kRingWarps][stages] | meta [kRingWarps][stages] (int4: w, lo, hi, id).
 __host__ __device__ inline size_t ring_smem_bytes(int m_raw, int stages) {
     const size_t row = (size_t)m_raw * sizeof(float);
-    return row + (size_t)kRingWarps * stages * (row + sizeof(uint64_t) + sizeof(int4));
+    return 2 * row + (size_t)kRingWarps * stages * (row + sizeof(uint64_t) + sizeof(int4));
 }
 
 __device__ inline void refine_ring(const RingRefs& a, int stages, int64_t warp0, int64_t nwarps) {
@@ -140,14 +140,20 @@ __device__ inline void refine_ring(const RingRefs& a, int stages, int64_t warp0,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int n4 = a.m_raw >> 2;
     float4* q_sh = ring_sh;
-    float4* rows = ring_sh + n4 + (size_t)warp * stages * n4;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(ring_sh + n4 + (size_t)kRingWarps * stages * n4) +
-                     warp * stages;
+    float4* qneg_sh = ring_sh + n4;
+    float4* rows = ring_sh + 2 * n4 + (size_t)warp * stages * n4;
+    uint64_t* bars =
+        reinterpret_cast<uint64_t*>(ring_sh + 2 * n4 + (size_t)kRingWarps * stages * n4) +
+        warp * stages;
     int4* meta = reinterpret_cast<int4*>(reinterpret_cast<uint64_t*>(
-                     ring_sh + n4 + (size_t)kRingWarps * stages * n4) + kRingWarps * stages) +
+                     ring_sh + 2 * n4 + (size_t)kRingWarps * stages * n4) + kRingWarps * stages) +
                  warp * stages;
     const float4* q4 = reinterpret_cast<const float4*>(a.qraw);
-    for (int i = threadIdx.x; i < n4; i += blockDim.x) q_sh[i] = q4[i];
+    for (int i = threadIdx.x; i < n4; i += blockDim.x) {
+        const float4 x = q4[i];
+        q_sh[i] = x;
+        qneg_sh[i] = make_float4(-x.x, -x.y, -x.z, -x.w);
+    }
     if (lane == 0) {
         for (int st = 0; st < stages; ++st) mbar_init(&bars[st], 1);
         mbar_fence_init();
@@ -196,6 +202,7 @@ __device__ inline void refine_ring(const RingRefs& a, int stages, int64_t warp0,
     int issued = 0;
     while (issued < stages && issue(issued)) ++issued;
     __syncwarp();
+    const float q_norm = norm_up_warp(reinterpret_cast<const float*>(q_sh), a.m_raw);
     unsigned long long refined = 0, fallbacks = 0;
     int k = 0;
     for (; k < issued; ++k) {
@@ -206,7 +213,9 @@ __device__ inline void refine_ring(const RingRefs& a, int stages, int64_t warp0,
         const float lj = __int_as_float(md.y), hj = __int_as_float(md.z);
         const float* vg = a.raw + (int64_t)md.w * a.m_raw;
         bool fb;
-        const float s = exact_dot_warp_eft_smem(reinterpret_cast<const float*>(q_sh), a.qraw,
+        const float s = exact_dot_warp_eft_smem(reinterpret_cast<const float*>(q_sh),
+                                                reinterpret_cast<const float*>(qneg_sh), q_norm,
+                                                a.qraw,
                                                 reinterpret_cast<const float*>(rows + (size_t)st * n4),
                                                 vg, a.m_raw, &fb);
         if (lane == 0) {
