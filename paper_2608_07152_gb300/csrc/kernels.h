@@ -58,11 +58,11 @@ struct CursorRef {
 // ---- fused single-CTA pull (pull_kernel.cu) ----------------------------------
 constexpr int kPullFusedMax = 256;   // largest pull served by one fused launch
 constexpr int kPullBatchMax = 1024;  // largest pull of the three-launch batch form
-struct PullArgs {
+// What a pull of one of many cursors needs.
+struct PullCore {
     int32_t* w_id;
     float* w_lo;
     float* w_hi;
-    const unsigned int* w_len;
     float* lo;                // bounds of every row (kept in step with the working set)
     float* hi;
     const float* qraw;
@@ -74,8 +74,10 @@ struct PullArgs {
     int64_t* out_ids;         // device
     float* out_scores;        // device
     int* status;
-    DevCounters* ctr;
-    int32_t* front;           // frontier of working-set indices, kFrontCap entries
+    DevCounters* ctr;         // w_len: rows of the working set
+};
+struct PullArgs : PullCore {
+    int32_t* front;           // frontier of working-set indices, kFrontCap entries (null: none)
     int* status_mirror;       // pinned host word: the status after the pull (null: none)
 };
 cudaError_t launch_pull_fused(const PullArgs& a, int refine_grid, cudaStream_t st);
@@ -83,16 +85,20 @@ cudaError_t launch_pull_fused(const PullArgs& a, int refine_grid, cudaStream_t s
 // parameters, up to kPullPack cursors per launch (the parameter space holds
 // 32,764 bytes), so no copy of them is staged; every CTA reads only its own
 // cursor's entry, one address for all its threads.  The host array is read
-// at launch.
-constexpr int kPullPack = 224;
+// at launch.  A pull of many keeps no frontier (a few pulls per batch would
+// not pay for it) and mirrors no status word, so the entries leave them out
+// and a pack holds 264.  At 224 the last 32 of 256 cursors made second
+// launches that left most SMs idle (refinement of 256 x 977 rows of 768:
+// 157 + 41 us, against 171 us in one launch; the batch 1,028 and 965 us).
+constexpr int kPullPack = 264;
 struct PullArgsPack {
-    PullArgs a[kPullPack];
+    PullCore a[kPullPack];
 };
 static_assert(sizeof(PullArgsPack) <= 31 * 1024, "kernel parameter space");
 // One launch per pull (n <= kPullFusedMax): a cluster of CTAs selects,
 // refines and emits (one cluster per cursor in the batch form).
 cudaError_t launch_pull_cluster(const PullArgs& a, cudaStream_t st);
-cudaError_t launch_pull_cluster_batch(const PullArgs* host_args, int ncursors, cudaStream_t st);
+cudaError_t launch_pull_cluster_batch(const PullCore* host_args, int ncursors, cudaStream_t st);
 // Ranks computed ahead, handed to the callers' buffers: for every entry,
 // count ids and scores from src to dst (device or pinned host memory), in
 // stream order, one launch per 512 entries (the entries are read at launch).
@@ -104,7 +110,7 @@ struct RankCopy {
     int count;
 };
 cudaError_t launch_copy_ranks(const RankCopy* host, int n, cudaStream_t st);
-cudaError_t launch_pull_batch(const PullArgs* host_args, int ncursors, int refine_blocks_per_cursor,
+cudaError_t launch_pull_batch(const PullCore* host_args, int ncursors, int refine_blocks_per_cursor,
                               int m_raw, cudaStream_t st);
 // ncursors <= kPullPack entries of p.
 cudaError_t launch_refine_batch(const PullArgsPack& p, int ncursors, int blocks_per_cursor,

@@ -151,7 +151,7 @@ __device__ inline void bitonic_desc_smem(unsigned long long* sk, int pow2) {
 // ctr->cand for the refinement and emission launches.
 __device__ inline void pull_select_body(const PullArgs& a, PullShared& sh) {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const unsigned int len = *a.w_len;
+    const unsigned int len = a.ctr->w_len;
     const int n = a.n;
     if (t == 0) {
         sh.prefix = 0;
@@ -197,11 +197,20 @@ __global__ void __launch_bounds__(kPullThreads, 2) pull_select_kernel(PullArgs a
     pull_select_body(a, sh);
 }
 
+// One of many cursors: no frontier, no mirrored status.
+__device__ inline PullArgs of_many(const PullCore& c) {
+    PullArgs a;
+    static_cast<PullCore&>(a) = c;
+    a.front = nullptr;
+    a.status_mirror = nullptr;
+    return a;
+}
+
 // One CTA per cursor.
 __global__ void __launch_bounds__(kPullThreads, 2)
     pull_select_batch_kernel(const __grid_constant__ PullArgsPack p) {
     __shared__ PullShared sh;
-    pull_select_body(p.a[blockIdx.x], sh);
+    pull_select_body(of_many(p.a[blockIdx.x]), sh);
 }
 
 // Sort the m keys in sh.sk (descending) and emit the first n: ids, scores,
@@ -345,7 +354,7 @@ __global__ void __launch_bounds__(kPullThreads, 2) pull_emit_kernel(PullArgs a) 
 __global__ void __launch_bounds__(kPullThreads, 2)
     pull_emit_batch_kernel(const __grid_constant__ PullArgsPack p) {
     __shared__ PullShared sh;
-    pull_emit_body(p.a[blockIdx.x], sh);
+    pull_emit_body(of_many(p.a[blockIdx.x]), sh);
 }
 
 // ---- one launch per pull: a cluster of CTAs per cursor -------------------------
@@ -452,7 +461,7 @@ __device__ inline FastSelect pull_select_fast(const PullArgs& a, PullShared& sh)
         }
         __syncthreads();
     } else {
-        len = *a.w_len;
+        len = a.ctr->w_len;
         uint32_t mx = 0;   // 0: no live row (every live key is larger)
         auto live_key = [](float l) -> uint32_t { return l == -INFINITY ? 0u : fkey(l); };
         const unsigned int len4 = len >> 2;   // working-set arrays are 16-byte aligned
@@ -752,7 +761,7 @@ __global__ void __cluster_dims__(kPullCluster, 1, 1) __launch_bounds__(kPullThre
 __global__ void __cluster_dims__(kPullClusterBatch, 1, 1) __launch_bounds__(kPullThreads, 2)
     pull_cluster_batch_kernel(const __grid_constant__ PullArgsPack p) {
     __shared__ PullShared sh;
-    pull_cluster_body<kPullClusterBatch>(p.a[blockIdx.x / kPullClusterBatch], sh);
+    pull_cluster_body<kPullClusterBatch>(of_many(p.a[blockIdx.x / kPullClusterBatch]), sh);
 }
 
 cudaError_t launch_pull_cluster(const PullArgs& a, cudaStream_t st) {
@@ -790,7 +799,7 @@ cudaError_t launch_copy_ranks(const RankCopy* host, int n, cudaStream_t st) {
 }
 
 // Packs of up to kPullPack cursors' arguments (the last one partial).
-static std::vector<PullArgsPack> pull_packs(const PullArgs* host, int n) {
+static std::vector<PullArgsPack> pull_packs(const PullCore* host, int n) {
     std::vector<PullArgsPack> packs((size_t)((n + kPullPack - 1) / kPullPack));
     for (int i = 0; i < n; ++i) packs[(size_t)(i / kPullPack)].a[i % kPullPack] = host[i];
     return packs;
@@ -800,7 +809,7 @@ static int pack_count(int n, size_t k) {
     return rest < kPullPack ? rest : kPullPack;
 }
 
-cudaError_t launch_pull_cluster_batch(const PullArgs* host_args, int ncursors, cudaStream_t st) {
+cudaError_t launch_pull_cluster_batch(const PullCore* host_args, int ncursors, cudaStream_t st) {
     if (ncursors <= 0) return cudaSuccess;
     const std::vector<PullArgsPack> packs = pull_packs(host_args, ncursors);
     for (size_t k = 0; k < packs.size(); ++k) {
@@ -989,7 +998,7 @@ cudaError_t launch_ws_sort(const int32_t* w_id_b, const float* w_lo_b, const flo
 }
 
 // Selection for every pack, then refinement for every pack, then emission.
-cudaError_t launch_pull_batch(const PullArgs* host_args, int ncursors, int refine_blocks_per_cursor,
+cudaError_t launch_pull_batch(const PullCore* host_args, int ncursors, int refine_blocks_per_cursor,
                               int m_raw, cudaStream_t st) {
     if (ncursors <= 0) return cudaSuccess;
     const std::vector<PullArgsPack> packs = pull_packs(host_args, ncursors);

@@ -674,7 +674,6 @@ pvs_status pull(pvs_cursor* c, int64_t n_eff, int64_t* d_ids, float* d_scores,
         a.w_id = c->w_id;
         a.w_lo = c->w_lo;
         a.w_hi = c->w_hi;
-        a.w_len = &c->ctr->w_len;
         a.lo = c->lo;
         a.hi = c->hi;
         a.qraw = c->qraw;
@@ -1907,7 +1906,7 @@ pvs_status pvs::next_batch_rows(pvs_cursor* const* cursors, int32_t nc, int32_t 
         pvs_status s = build_first_working_sets(cursors, nc, pulls.data());
         if (s != PVS_OK) return s;
     }
-    std::vector<PullArgs> args;
+    std::vector<PullCore> args;
     std::vector<int32_t> who;
     args.reserve(nc);
     for (int32_t i = 0; i < nc; ++i) {
@@ -1919,11 +1918,10 @@ pvs_status pvs::next_batch_rows(pvs_cursor* const* cursors, int32_t nc, int32_t 
         if (s != PVS_OK) return fail(c, s);
         s = prepare_pull(c, pulls[i]);
         if (s != PVS_OK) return fail(c, s);
-        PullArgs a;
+        PullCore a;
         a.w_id = c->w_id;
         a.w_lo = c->w_lo;
         a.w_hi = c->w_hi;
-        a.w_len = &c->ctr->w_len;
         a.lo = c->scanned ? c->lo : nullptr;
         a.hi = c->scanned ? c->hi : nullptr;
         a.qraw = c->qraw;
@@ -1938,8 +1936,6 @@ pvs_status pvs::next_batch_rows(pvs_cursor* const* cursors, int32_t nc, int32_t 
         a.out_scores = direct ? scores[i] + take[i] : outputs_on_device ? c->d_scores : c->h_scores;
         a.status = c->d_status;
         a.ctr = c->ctr;
-        a.front = nullptr;   // a few pulls per batch: a frontier would not pay for itself
-        a.status_mirror = nullptr;
         args.push_back(a);
         who.push_back(i);
     }
