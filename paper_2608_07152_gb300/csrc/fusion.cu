@@ -173,7 +173,19 @@ constexpr int kCountWarps = 8;
 // before a tile could overflow the queue.
 constexpr int kCountTile = kCountWarps * 32 * 4;
 constexpr int kPlaceQueue = 2048;
-static_assert(kPlaceQueue >= 2 * kCountTile, "queue");
+// The rows of a block's step of the residual level: a multiple is placed
+// per flush, so that its warps end together.
+constexpr int kPlaceStripe = kCountWarps * 32;
+static_assert(kPlaceQueue >= 2 * kCountTile && kPlaceStripe <= kPlaceQueue - kCountTile, "queue");
+
+// One shared-memory add per distinct bin (>= 0) among the lanes of a warp.
+__device__ __forceinline__ void count_bins(unsigned int* sh, int bin, int lane) {
+    const unsigned int live = __ballot_sync(0xffffffffu, bin >= 0);
+    if (bin >= 0) {
+        const unsigned int same = __match_any_sync(live, bin);
+        if (lane == __ffs(same) - 1) atomicAdd(&sh[bin], (unsigned int)__popc(same));
+    }
+}
 
 // Pinned staging of one rank query: ids in (8 B dense, 4 B sparse), per dense
 // item two 8-byte counts (plus one) and its key, per sparse item its rank,
@@ -363,6 +375,15 @@ pvs_status ensure_resid(pvs_index* x, cudaStream_t st, int* status) {
     return PVS_OK;
 }
 
+// What a count reads beside the bounds when the cursor's pass kept `mid`
+// (null: it did not).
+struct MidRefs {
+    const float* mid;
+    const float* vnorm;
+    const float* enorm;
+    const int8_t* zq;
+};
+
 // The query in integers for the residual level, computed by every block of
 // a rank count into shared memory: q = s_q zq + e_q with |zq_j| <= Q (Q
 // keeps every integer dot product below 2^31), zq as 16-bit pairs twice,
@@ -374,6 +395,13 @@ pvs_status ensure_resid(pvs_index* x, cudaStream_t st, int* status) {
 struct ResidQuery {
     float sq, eq;
     int bias;
+};
+// The query in two digits (fine_digit), for counts with IntervalArgs::mid.
+struct FineQuery {
+    float rest;        // >= ||q - s_q zq - s_e ze||
+    float digit;       // >= ||s_e ze||
+    float norm;        // >= ||s_q zq + s_e ze||
+    float code_norm;   // >= 8 sqrt(m_pad)
 };
 
 // D1 = zq.z and D2 = zq.z2 over one row, exact integers, by the eight
@@ -464,13 +492,104 @@ __device__ __forceinline__ bool resid_bounds(int D1, int D2, const float4 rp,
     return isfinite(*fl) && isfinite(*fh);
 }
 
+// D2 alone, from the residual codes alone (0.5 B per dimension): the cursor's
+// pass has kept a finer centre of every row (IntervalArgs::mid), so the codes
+// need not be read again.  Up to six 8-byte loads a lane in flight.
+__device__ __forceinline__ int resid_dot_group8(const uint8_t* __restrict__ z2,
+                                                const int32_t* __restrict__ zqp, int bias,
+                                                int m_pad, bool valid) {
+    const int sl = threadIdx.x & 7;
+    const int n16 = m_pad >> 4;
+    const uint2* rc = reinterpret_cast<const uint2*>(z2);
+    const int4* qp = reinterpret_cast<const int4*>(zqp);
+    int acc = 0, acc_b = 0;
+    if (valid) {
+#pragma unroll 1
+        for (int c0 = sl; c0 < n16; c0 += 48) {
+            uint2 b[6];
+#pragma unroll
+            for (int u = 0; u < 6; ++u) {
+                const int c = c0 + 8 * u;
+                b[u] = c < n16 ? __ldg(rc + c) : make_uint2(0x88888888u, 0x88888888u);
+            }
+#pragma unroll
+            for (int u = 0; u < 6; ++u) {
+                const int c = c0 + 8 * u;
+                if (c >= n16) break;
+                const int4 p0 = qp[c], p1 = qp[n16 + c];
+                const int l0 = (int)(b[u].x & 0x0F0F0F0Fu), h0 = (int)((b[u].x >> 4) & 0x0F0F0F0Fu);
+                const int l1 = (int)(b[u].y & 0x0F0F0F0Fu), h1 = (int)((b[u].y >> 4) & 0x0F0F0F0Fu);
+                acc = __dp2a_lo(p0.x, l0, acc);
+                acc = __dp2a_hi(p0.y, l0, acc);
+                acc = __dp2a_lo(p0.z, h0, acc);
+                acc = __dp2a_hi(p0.w, h0, acc);
+                acc_b = __dp2a_lo(p1.x, l1, acc_b);
+                acc_b = __dp2a_hi(p1.y, l1, acc_b);
+                acc_b = __dp2a_lo(p1.z, h1, acc_b);
+                acc_b = __dp2a_hi(p1.w, h1, acc_b);
+            }
+        }
+    }
+    acc += acc_b;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return acc - 8 * bias;   // nibbles hold z2 + 8
+}
+
+// Bounds of q.v from c = IntervalArgs::mid.  With w1 = s z, v = w1 + r1 and
+// q = q2 + f, q2 = s_q zq + s_e ze the query in two digits:
+//   q.v = q2.w1 + q2.r1 + f.v,
+// |q2.r1| <= (||q|| + ||f||) ||r1|| and |f.v| <= ||f|| ||v||.  c has at most six
+// roundings of relative error u = 2^-24 on its way from the integer dots D, D':
+// |c - q2.w1| <= 4.1 u (|s s_q D| + |s s_e D'|) (plus the subnormal range), and
+// |s s_q D| <= |q2.w1| + |s s_e D'|, |s s_e D'| <= ||s_e ze|| ||w1||; 2^-21 and
+// 2^-20 leave a factor of two.  (s <= ||w1|| unless both dots are 0.)
+__device__ __forceinline__ float mid_error(float c, float w1, const FineQuery& fq) {
+    float E = __fmul_ru(fabsf(c), 0x1p-21f);
+    E = __fadd_ru(E, __fmul_ru(__fmul_ru(fq.digit, w1), 0x1p-20f));
+    return __fadd_ru(E, __fadd_ru(__fmul_ru(w1, 0x1p-147f), 0x1p-147f));
+}
+__device__ __forceinline__ bool mid_bounds(float c, float vn, float en, const FineQuery& fq,
+                                           float* fl, float* fh) {
+    float E = mid_error(c, __fadd_ru(vn, en), fq);
+    E = __fadd_ru(E, __fmul_ru(fq.rest, vn));
+    E = __fadd_ru(E, __fmul_ru(fq.norm, en));
+    *fl = __fsub_rd(c, E);
+    *fh = __fadd_ru(c, E);
+    return isfinite(*fl) && isfinite(*fh);
+}
+// Bounds of q.v from c and the residual codes: with w2 = s2 z2 and r2 = r1 - w2,
+//   q.v = q2.w1 + f.w1 + (s_q' zq' + e').w2 + q.r2,
+// zq' the 16-bit codes and ||e'|| <= eq.  ||w2|| <= 8 sqrt(m_pad) s2, and
+// ||w1|| <= ||w1 + w2|| + ||w2||.  t = RN(s_q' RN(s2 RN(D2))) has at most three
+// roundings, RN(c + t) one more: within the factor of two again.
+__device__ __forceinline__ bool fine_bounds(float c, int D2, const float4 rp,
+                                            const ResidQuery& rq, const FineQuery& fq,
+                                            float qnorm, float* fl, float* fh) {
+    const float t = __fmul_rn(rq.sq, __fmul_rn(rp.y, __int2float_rn(D2)));
+    const float w2 = __fmul_ru(rp.y, fq.code_norm);
+    const float w1 = __fadd_ru(rp.w, w2);
+    float E = mid_error(c, w1, fq);
+    E = __fadd_ru(E, __fmul_ru(fabsf(t), 0x1p-21f));
+    E = __fadd_ru(E, __fadd_ru(__fmul_ru(rq.sq, 0x1p-147f), 0x1p-147f));
+    E = __fadd_ru(E, __fmul_ru(fq.rest, w1));
+    E = __fadd_ru(E, __fmul_ru(rq.eq, w2));
+    E = __fadd_ru(E, __fmul_ru(qnorm, rp.z));
+    const float f = __fadd_rn(c, t);
+    *fl = __fsub_rd(f, E);
+    *fh = __fadd_ru(f, E);
+    return isfinite(*fl) && isfinite(*fh);
+}
+
 // hist[j] = number of visible rows whose key lies above exactly j of the
 // queried keys (sorted ascending); the rank of the item with the j-th
 // smallest key is then 1 + sum of hist[t] for t > j.  A row's key lies in
 // [key(lo, y), key(hi, y)]; when no queried key falls in that range the
 // count is fixed by the bounds.  Otherwise, with `exact`, the row's
-// authoritative score is placed: first by the bounds of its residual codes
-// (resid_dots_group8 and resid_bounds, 1.5 B per dimension; the block queues
+// authoritative score is placed: where the pass kept `mid`, by its tighter
+// bounds (mid_bounds, 12 B a row); then by the bounds of its residual codes
+// (fine_bounds, 0.5 B per dimension; without `mid` resid_dots_group8 and
+// resid_bounds, 1.5 B; the block queues
 // such rows and places them eight lanes per row), else by the fp32 dot with
 // its error bound, else exactly (and it must lie in its interval, App. A.1);
 // without, the row counts in hist[a] (a = the queried keys below key(lo, y):
@@ -478,6 +597,12 @@ __device__ __forceinline__ bool resid_bounds(int D1, int D2, const float4 rp,
 // keys at most key(hi, y)): maybe[a] += 1, maybe[b] -= 1, so that the prefix
 // sum of `maybe` at j counts the rows that may lie above the j-th key.  A
 // row with hi = -inf has been delivered and lies above every queried key.
+// Bound by the rows it reads where most intervals straddle: 12 keys from the
+// middle of 8.8M x 768, of which 7.5M rows straddle, read 11.9 GB in 1,840 us
+// through the codes; with `mid` 6.5M straddle and read 5.7 GB.  A search by one
+// lane in eight, and by one lane of the warp for the fp32 rows, then made the
+// instructions the bound (1,440 us); with a row in every lane it takes 933 us
+// (2M x 1,024: 346 us, 157 now).  More registers for fewer blocks: 985 us.
 __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
     const float* __restrict__ lo, const float* __restrict__ hi, int64_t rows,
     const uint32_t* __restrict__ tomb, const float* __restrict__ qraw,
@@ -485,7 +610,7 @@ __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
     const int8_t* __restrict__ codes, const uint8_t* __restrict__ resid,
     const float4* __restrict__ rparam, int m_pad, int qrange,
     const QueryScalars* __restrict__ qs, unsigned long long* hist, unsigned long long* maybe,
-    int* status, DevCounters* ctr) {
+    int* status, DevCounters* ctr, const MidRefs mref) {
     __shared__ uint64_t sk[kRankQueryMax];
     __shared__ unsigned int sh[kRankQueryMax + 1];
     __shared__ int sm[kRankQueryMax + 1];
@@ -506,9 +631,11 @@ __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
     int32_t* zqn = reinterpret_cast<int32_t*>(rq_smem);   // m_pad / 2 pairs
     int32_t* zqp = zqn + (m_pad >> 1);
     __shared__ ResidQuery srq;
-    __shared__ float red_f[kCountWarps];
+    __shared__ FineQuery sfq;
+    __shared__ float red_f[kCountWarps], red_e[kCountWarps];
     __shared__ int red_i[kCountWarps];
     const bool use_resid = exact && resid != nullptr;
+    const bool use_mid = use_resid && mref.mid != nullptr;
     float qnorm = 0.0f;
     if (use_resid) {
         const int w = threadIdx.x >> 5;
@@ -528,9 +655,17 @@ __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
         }
         int16_t* zn16 = reinterpret_cast<int16_t*>(zqn);
         int16_t* zp16 = reinterpret_cast<int16_t*>(zqp);
-        float ss = 0.0f;
+        float ss = 0.0f, sf = 0.0f;
         int bias = 0;
+        const float s_q = qs->s;
+        const FineScale fine = fine_scale(s_q);
         for (int j = threadIdx.x; j < m_pad; j += blockDim.x) {
+            if (use_mid && j < m_raw) {   // |q_j - s_q zq_j - s_e ze_j|, rounded up
+                const float e = fine_rest(qraw[j], s_q, mref.zq[j]);
+                const float f = fmaf(-fine.s, (float)fine_digit(e, fine.inv), e);
+                const float b = __fadd_ru(abs_before_rn(f), __fsub_ru(abs_before_rn(e), fabsf(e)));
+                sf = __fadd_ru(sf, __fmul_ru(b, b));
+            }
             int c = 0;
             if (j < m_raw && mq > 0.0f) {
                 c = (int)fminf(fmaxf(rintf(__fdiv_rn(qraw[j], sq)), -Qf), Qf);
@@ -548,20 +683,29 @@ __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
             bias += c;
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ss = __fadd_ru(ss, __shfl_xor_sync(0xffffffffu, ss, o));
+        for (int o = 16; o > 0; o >>= 1) {
+            ss = __fadd_ru(ss, __shfl_xor_sync(0xffffffffu, ss, o));
+            sf = __fadd_ru(sf, __shfl_xor_sync(0xffffffffu, sf, o));
+        }
         bias = __reduce_add_sync(0xffffffffu, bias);
         if (lane == 0) {
             red_f[w] = ss;
+            red_e[w] = sf;
             red_i[w] = bias;
         }
         __syncthreads();
         if (threadIdx.x == 0) {
-            float st = 0.0f;
+            float st = 0.0f, ft = 0.0f;
             int bt = 0;
             for (int i = 0; i < kCountWarps; ++i) {
                 st = __fadd_ru(st, red_f[i]);
+                ft = __fadd_ru(ft, red_e[i]);
                 bt += red_i[i];
             }
+            sfq.rest = __fsqrt_ru(ft);
+            sfq.digit = __fadd_ru(qs->enorm, sfq.rest);
+            sfq.norm = __fadd_ru(qs->qnorm, sfq.rest);
+            sfq.code_norm = __fmul_ru(8.0f, __fsqrt_ru((float)m_pad));
             srq.sq = sq;
             srq.eq = __fsqrt_ru(st);
             srq.bias = bt;
@@ -571,28 +715,8 @@ __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
     }
     const int64_t rbytes = m_pad >> 1;
     const int warp = threadIdx.x >> 5;
-    // row r's bin from its fp32 row, by the whole warp: first a plain fp32
-    // dot with its error bound, which places the authoritative score RN(q.v)
-    // in [fl, fh] and fixes the bin unless a queried key falls in that range;
-    // then the exact dot
-    auto place_fp32 = [&](int64_t r, float lr, float hr) {
-        float err;
-        const float f = fast_dot_warp(qraw, raw + r * (int64_t)m_raw, m_raw, &err);
-        int fast_bin = -1;
-        if (lane == 0 && isfinite(f) && isfinite(err)) {
-            // a score of zero is reported as +0, whose key is above -0's
-            const float fl = __fsub_rd(f, err);
-            const float fh = __fadd_ru(f, err) == 0.0f ? 0.0f : __fadd_ru(f, err);
-            const int a = keys_below(sk, nq, rank_key(fl, (uint32_t)r));
-            const int b = keys_at_most(sk, nq, rank_key(fh, (uint32_t)r));
-            if (a == b) {
-                fast_bin = a;
-                if (fh < lr || fl > hr) set_status(status, PVS_ERR_INTERVAL);
-                atomicAdd(&sh[a], 1u);
-                ++scored;
-            }
-        }
-        if (__shfl_sync(0xffffffffu, fast_bin, 0) >= 0) return;
+    // the exact dot of a row by the whole warp, for the bins its bounds leave open
+    auto place_exact = [&](int64_t r, float lr, float hr) {
         bool fb = false;
         const float s = exact_dot_warp_eft(qraw, qraw, raw + r * (int64_t)m_raw, m_raw, &fb);
         if (lane == 0) {
@@ -603,8 +727,53 @@ __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
             fallbacks += fb ? 1 : 0;
         }
     };
-    // with the residual codes, the block queues its straddling rows and
-    // places them eight lanes per row; the rows they leave open are queued
+    // the bins of a list of rows from their fp32 rows: a plain fp32 dot a warp
+    // with its error bound places the authoritative score RN(q.v) in [fl, fh]
+    // and fixes the bin unless a queried key falls in that range; then the
+    // exact dot.  A warp's dots of 32 rows come first, then a row in every lane.
+    auto place_fp32 = [&](const int32_t* list, int count) {
+        for (int i0 = warp; i0 < count; i0 += 32 * kCountWarps) {
+            const int mine = i0 + lane * kCountWarps;
+            const bool valid = mine < count;
+            const int32_t r = valid ? list[mine] : 0;
+            const float lr = valid ? lo[r] : 0.0f, hr = valid ? hi[r] : 0.0f;
+            float f = 0.0f, err = 0.0f;
+            const int steps = min(32, (count - i0 + kCountWarps - 1) / kCountWarps);
+#pragma unroll 1
+            for (int t = 0; t < steps; ++t) {
+                const int64_t rt = __shfl_sync(0xffffffffu, r, t);
+                float et;
+                const float ft = fast_dot_warp(qraw, raw + rt * (int64_t)m_raw, m_raw, &et);
+                if (lane == t) {
+                    f = ft;
+                    err = et;
+                }
+            }
+            int bin = -1;
+            if (valid && isfinite(f) && isfinite(err)) {
+                // a score of zero is reported as +0, whose key is above -0's
+                const float fl = __fsub_rd(f, err);
+                const float fh = __fadd_ru(f, err) == 0.0f ? 0.0f : __fadd_ru(f, err);
+                const int a = keys_below(sk, nq, rank_key(fl, (uint32_t)r));
+                const int b = keys_at_most(sk, nq, rank_key(fh, (uint32_t)r));
+                if (a == b) {
+                    bin = a;
+                    if (fh < lr || fl > hr) set_status(status, PVS_ERR_INTERVAL);
+                }
+            }
+            count_bins(sh, bin, lane);
+            unsigned int open = __ballot_sync(0xffffffffu, valid && bin < 0);
+            if (lane == 0) scored += steps - __popc(open);
+            while (open) {
+                const int src = __ffs(open) - 1;
+                open &= open - 1;
+                place_exact(__shfl_sync(0xffffffffu, r, src), __shfl_sync(0xffffffffu, lr, src),
+                            __shfl_sync(0xffffffffu, hr, src));
+            }
+        }
+    };
+    // the block queues its straddling rows; with the residual codes it places
+    // them eight lanes per row, and the rows these leave open are queued
     // again and scored one warp per row
     __shared__ int32_t q_rows[kPlaceQueue];
     __shared__ int32_t f_rows[kPlaceQueue];
@@ -634,9 +803,28 @@ __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
                         hv[u] = hi[y0 + u];
                     }
             }
+            float mv[4] = {0.f, 0.f, 0.f, 0.f}, vn[4] = {0.f, 0.f, 0.f, 0.f};
+            float en[4] = {0.f, 0.f, 0.f, 0.f};
+            if (use_mid) {   // (allocations: 16-byte aligned)
+                if (y0 + 3 < rows) {
+                    const float4 M = *reinterpret_cast<const float4*>(mref.mid + y0);
+                    const float4 V = *reinterpret_cast<const float4*>(mref.vnorm + y0);
+                    const float4 N = *reinterpret_cast<const float4*>(mref.enorm + y0);
+                    mv[0] = M.x, mv[1] = M.y, mv[2] = M.z, mv[3] = M.w;
+                    vn[0] = V.x, vn[1] = V.y, vn[2] = V.z, vn[3] = V.w;
+                    en[0] = N.x, en[1] = N.y, en[2] = N.z, en[3] = N.w;
+                } else {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (y0 + u < rows) {
+                            mv[u] = mref.mid[y0 + u];
+                            vn[u] = mref.vnorm[y0 + u];
+                            en[u] = mref.enorm[y0 + u];
+                        }
+                }
+            }
             // the four rows share one tombstone word
             const uint32_t tw = (tomb && y0 < rows) ? tomb[y0 >> 5] >> (y0 & 31) : 0u;
-            unsigned int strad[4] = {0u, 0u, 0u, 0u};   // straddling lanes per row slot
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int64_t y = y0 + u;
@@ -654,18 +842,27 @@ __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
                             bin = a;
                         } else if (exact) {
                             straddle = true;
+                            float rl, rh;
+                            if (use_mid && mid_bounds(mv[u], vn[u], en[u], sfq, &rl, &rh)) {
+                                // RN(q.v) lies in [rl, rh] as q.v does, and in [l, h]
+                                if (rh < l || rl > h) set_status(status, PVS_ERR_INTERVAL);
+                                rl = fmaxf(rl, l);
+                                rh = fminf(rh, h);
+                                if (rh == 0.0f) rh = 0.0f;   // -0 is reported as +0
+                                const int a2 = keys_below(sk, nq, rank_key(rl, (uint32_t)y));
+                                const int b2 = keys_at_most(sk, nq, rank_key(rh, (uint32_t)y));
+                                if (a2 == b2) {
+                                    bin = a2;
+                                    straddle = false;
+                                }
+                            }
                         } else {
                             bin = a;
                             mb = b;
                         }
                     }
                 }
-                // one shared-memory add per distinct bin of the warp
-                const unsigned int live = __ballot_sync(0xffffffffu, bin >= 0);
-                if (bin >= 0) {
-                    const unsigned int same = __match_any_sync(live, bin);
-                    if (lane == __ffs(same) - 1) atomicAdd(&sh[bin], (unsigned int)__popc(same));
-                }
+                count_bins(sh, bin, lane);
                 // bounds mode: maybe[a] += 1, maybe[b] -= 1, per distinct key of the warp
                 const unsigned int mlive = __ballot_sync(0xffffffffu, mb >= 0);
                 if (mb >= 0) {
@@ -675,98 +872,101 @@ __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
                     if (lane == __ffs(sb) - 1) atomicAdd(&sm[mb], -__popc(sb));
                 }
                 const unsigned int todo = __ballot_sync(0xffffffffu, straddle);
-                if (use_resid) {   // one queue reservation per warp
-                    if (todo) {
-                        int qb = 0;
-                        if (lane == __ffs(todo) - 1) qb = atomicAdd(&q_n, __popc(todo));
-                        qb = __shfl_sync(0xffffffffu, qb, __ffs(todo) - 1);
-                        if (straddle) q_rows[qb + __popc(todo & lanemask_lt)] = (int32_t)y;
-                    }
-                } else {
-                    strad[u] = todo;
-                }
-            }
-            // without the residual codes, each straddling row from its fp32 row
-#pragma unroll 1
-            for (int u = 0; u < 4 && !use_resid; ++u) {
-                unsigned int rest = strad[u];
-                while (rest) {
-                    const int src = __ffs(rest) - 1;
-                    rest &= rest - 1;
-                    if (rest) {   // the next row to score, into L2 while this one is scored
-                        const char* nrow = reinterpret_cast<const char*>(
-                            raw + (base + 4 * (__ffs(rest) - 1) + u) * (int64_t)m_raw);
-                        for (int off = lane * 128; off < m_raw * 4; off += 32 * 128)
-                            asm volatile("prefetch.global.L2 [%0];" ::"l"(nrow + off));
-                    }
-                    const int64_t r = base + 4 * src + u;
-                    place_fp32(r, lo[r], hi[r]);
+                if (todo) {   // one queue reservation per warp
+                    int qb = 0;
+                    if (lane == __ffs(todo) - 1) qb = atomicAdd(&q_n, __popc(todo));
+                    qb = __shfl_sync(0xffffffffu, qb, __ffs(todo) - 1);
+                    if (straddle) q_rows[qb + __popc(todo & lanemask_lt)] = (int32_t)y;
                 }
             }
         }
         const bool last = tb + step >= rows;   // the same in every thread of the block
-        if (!use_resid) {
+        if (!exact) {
             if (last) break;
             continue;
         }
         __syncthreads();
         const int n = q_n;
-        if (n > kPlaceQueue - kCountTile || last) {
-            // four rows per warp, eight lanes per row
+        if (!use_resid) {   // each straddling row from its fp32 row
+            place_fp32(q_rows, n);
+            __syncthreads();
+            if (threadIdx.x == 0) q_n = 0;
+            __syncthreads();
+        } else if (n > kPlaceQueue - kCountTile || last) {
+            // kPlaceStripe rows a step: a warp's dots take four rows at a time,
+            // eight lanes a row, and lane (g, t) keeps those of the step's row
+            // 32 t + 4 warp + g, so that the bounds and the searches then run
+            // with a row in every lane.  A remainder stays for the next flush.
             const int sl = lane & 7;
-            for (int i0 = warp * 4; i0 < n; i0 += kCountWarps * 4) {
-                const int i = i0 + (lane >> 3);
-                const bool valid = i < n;
-                const int64_t r = valid ? q_rows[i] : 0;
-                const int inext = i + kCountWarps * 4;   // the group's next row, into L2
-                if (inext < n) {
-                    const int64_t pr = q_rows[inext];
-                    const char* zc = reinterpret_cast<const char*>(codes + pr * (int64_t)m_pad);
-                    const char* rc = reinterpret_cast<const char*>(resid + pr * rbytes);
-                    for (int off = sl * 128; off < m_pad; off += 8 * 128)
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(zc + off));
-                    for (int off = sl * 128; off < rbytes; off += 8 * 128)
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(rc + off));
-                    if (sl == 7) asm volatile("prefetch.global.L2 [%0];" ::"l"(rparam + pr));
+            const int first = last ? 0 : n % kPlaceStripe;
+            for (int s0 = first; s0 < n; s0 += kPlaceStripe) {
+                const int mine = s0 + 32 * sl + 4 * warp + (lane >> 3);
+                const bool valid = mine < n;
+                const int64_t r = valid ? q_rows[mine] : 0;
+                float4 rp = make_float4(0.f, 0.f, 0.f, 0.f);
+                float mr = 0.0f, lr = 0.0f, hr = 0.0f;
+                if (valid) {
+                    rp = __ldg(rparam + r);
+                    if (use_mid) mr = mref.mid[r];
+                    lr = lo[r];
+                    hr = hi[r];
                 }
-                int D1, D2;
-                resid_dots_group8(zqn, zqp, srq.bias, codes + r * (int64_t)m_pad,
-                                  resid + r * rbytes, m_pad, valid, &D1, &D2);
-                int open = 0;   // the row needs its fp32 row
-                if (valid && sl == 0) {
+                int D1 = 0, D2 = 0;
+#pragma unroll 1
+                for (int t = 0; t < 8 && s0 + 32 * t + 4 * warp < n; ++t) {
+                    const int i = s0 + 32 * t + 4 * warp + (lane >> 3);
+                    const bool vt = i < n;
+                    const int64_t rt = vt ? q_rows[i] : 0;
+                    int d1 = 0, d2;
+                    if (use_mid)
+                        d2 = resid_dot_group8(resid + rt * rbytes, zqp, srq.bias, m_pad, vt);
+                    else
+                        resid_dots_group8(zqn, zqp, srq.bias, codes + rt * (int64_t)m_pad,
+                                          resid + rt * rbytes, m_pad, vt, &d1, &d2);
+                    if (sl == t) {
+                        D1 = d1;
+                        D2 = d2;
+                    }
+                }
+                int bin = -1;
+                if (valid) {
                     float rl, rh;
-                    bool placed = false;
-                    if (resid_bounds(D1, D2, rparam[r], srq, qnorm, &rl, &rh)) {
+                    if (use_mid ? fine_bounds(mr, D2, rp, srq, sfq, qnorm, &rl, &rh)
+                                : resid_bounds(D1, D2, rp, srq, qnorm, &rl, &rh)) {
                         // RN(q.v) lies in [rl, rh] as q.v does; a score of
                         // zero is reported as +0, whose key is above -0's
                         const float rh0 = rh == 0.0f ? 0.0f : rh;
-                        const int a = keys_below(sk, nq, rank_key(rl, (uint32_t)r));
-                        const int b = keys_at_most(sk, nq, rank_key(rh0, (uint32_t)r));
-                        if (a == b) {
-                            placed = true;
-                            if (rh < lo[r] || rl > hi[r]) set_status(status, PVS_ERR_INTERVAL);
-                            atomicAdd(&sh[a], 1u);
+                        const int ka = keys_below(sk, nq, rank_key(rl, (uint32_t)r));
+                        const int kb = keys_at_most(sk, nq, rank_key(rh0, (uint32_t)r));
+                        if (ka == kb) {
+                            bin = ka;
+                            if (rh < lr || rl > hr) set_status(status, PVS_ERR_INTERVAL);
                         }
                     }
-                    if (!placed) {
-                        f_rows[atomicAdd(&f_n, 1)] = (int32_t)r;
-                        open = 1;
+                }
+                count_bins(sh, bin, lane);
+                unsigned int open = __ballot_sync(0xffffffffu, valid && bin < 0);
+                if (open) {   // rows that need their fp32 row: queued, and on their way to L2
+                    int fb = 0;
+                    if (lane == 0) fb = atomicAdd(&f_n, __popc(open));
+                    fb = __shfl_sync(0xffffffffu, fb, 0);
+                    if ((open >> lane) & 1u) f_rows[fb + __popc(open & lanemask_lt)] = (int32_t)r;
+                    while (open) {
+                        const int64_t ro = __shfl_sync(0xffffffffu, (int)r, __ffs(open) - 1);
+                        open &= open - 1;
+                        const char* vr = reinterpret_cast<const char*>(raw + ro * (int64_t)m_raw);
+                        for (int off = lane * 128; off < m_raw * 4; off += 32 * 128)
+                            asm volatile("prefetch.global.L2 [%0];" ::"l"(vr + off));
                     }
                 }
-                if (__shfl_sync(0xffffffffu, open, lane & ~7)) {   // its fp32 row, into L2
-                    const char* vr = reinterpret_cast<const char*>(raw + r * (int64_t)m_raw);
-                    for (int off = sl * 128; off < m_raw * 4; off += 8 * 128)
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(vr + off));
-                }
             }
             __syncthreads();
-            const int nf = f_n;
-            for (int i = warp; i < nf; i += kCountWarps) {
-                const int64_t r = f_rows[i];
-                place_fp32(r, lo[r], hi[r]);
-            }
+            place_fp32(f_rows, f_n);
             __syncthreads();
-            if (threadIdx.x == 0) q_n = f_n = 0;
+            if (threadIdx.x == 0) {
+                q_n = first;
+                f_n = 0;
+            }
             __syncthreads();
         }
         if (last) break;
@@ -1242,7 +1442,8 @@ pvs_status rank_queries(pvs_cursor* c, const int32_t* dense_ids, int32_t nd, boo
                             resid ? (size_t)x->m_pad * 4 : 0, st>>>(
             c->lo, c->hi, rows, tomb, c->qraw, x->raw, x->m_raw, d_keys, nd, exact ? 1 : 0,
             resid ? x->codes : nullptr, resid ? x->resid : nullptr, x->rparam, x->m_pad, qrange,
-            c->qs, d_hist, d_maybe, status, c->ctr);
+            c->qs, d_hist, d_maybe, status, c->ctr,
+            MidRefs{c->mid_valid ? c->mid : nullptr, x->vnorm, x->enorm, c->zq});
         RQ_CUDA(cudaGetLastError());
         RQ_CUDA(cudaMemcpyAsync(h_hist, d_hist, (size_t)(nd + 1) * 16, cudaMemcpyDeviceToHost,
                                 st));
@@ -1322,7 +1523,7 @@ pvs_status rank_queries(pvs_cursor* c, const int32_t* dense_ids, int32_t nd, boo
             rank_count_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), kCountWarps * 32, 0, st2>>>(
                 staged->scores, staged->scores, rows, staged->tomb, c->qraw, x->raw, x->m_raw,
                 d_keys, nsq, 0, nullptr, nullptr, nullptr, x->m_pad, 1, c->qs, d_hist,
-                d_hist + nsq + 1, status + 1, c->ctr);
+                d_hist + nsq + 1, status + 1, c->ctr, MidRefs{});
             sparse_ranks_kernel<<<1, kRankQueryMax, 0, st2>>>(d_sids, nsq, staged->scores,
                                                               staged->tomb, d_keys, d_hist, d_srank);
         } else {

@@ -27,7 +27,12 @@ constexpr int kIntervalThreads = (kConsumerWarps + 1) * 32;
 
 // CPL = 16-byte chunks per lane per row = m_pad / 64 (compile-time), or 0 for
 // a runtime count with the query chunks read from global memory.
-template <int CPL>
+// MID: the row's dot product with the query's second digit as well, and the
+// sum of both into a.mid.  The pass stays bound by its one reading of the
+// codes: a second dp4a per word and 4 bytes written per row (8.8M x 768: 987 us, 1,022
+// with MID; 2M x 1,024: 296 and 294).  The digits are made by the consumers while
+// the first tiles are on their way (before the ring starts: 2M x 1,024 328 us).
+template <int CPL, bool MID>
 __global__ void __launch_bounds__(kIntervalThreads, 1)
     interval_pass_kernel(IntervalArgs a, int stages, int rotate, int cpl_rt) {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -101,6 +106,27 @@ __global__ void __launch_bounds__(kIntervalThreads, 1)
             qreg[j] = zq4[4 * jj + p];
         }
     }
+    // the second digits, by the consumers while the first tiles are on their way
+    int8_t* z2 = reinterpret_cast<int8_t*>(empty + stages);
+    FineScale fine{0.0f, 0.0f};
+    if constexpr (MID) {
+        fine = fine_scale(q.s);
+        for (int j = threadIdx.x; j < m_pad; j += kConsumerWarps * 32) {
+            const float v = j < a.m_raw ? a.qraw[j] : 0.0f;
+            z2[j] = (int8_t)fine_digit(fine_rest(v, q.s, a.zq[j]), fine.inv);
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kConsumerWarps * 32) : "memory");
+    }
+    const int4* z24 = reinterpret_cast<const int4*>(z2);
+    int4 ereg[CPL > 0 && MID ? CPL : 1];
+    if constexpr (CPL > 0 && MID) {
+#pragma unroll
+        for (int j = 0; j < CPL; ++j) {
+            int jj = j + par;
+            if (jj >= CPL) jj -= CPL;
+            ereg[j] = z24[4 * jj + p];
+        }
+    }
 
     // the slot's kSlotTop largest live lower bounds, descending
     float top[kSlotTop];
@@ -118,7 +144,7 @@ __global__ void __launch_bounds__(kIntervalThreads, 1)
         const uint8_t* stage = smem + (size_t)s * stage_bytes;
         const int64_t row = t * TR + r_in_tile;
         const int4* rowp = reinterpret_cast<const int4*>(stage + r_in_tile * m_pad);
-        int acc0 = 0, acc1 = 0;
+        int acc0 = 0, acc1 = 0, fine0 = 0, fine1 = 0;
         if (row < a.rows) {
             if constexpr (CPL > 0) {
 #pragma unroll
@@ -130,6 +156,12 @@ __global__ void __launch_bounds__(kIntervalThreads, 1)
                     acc1 = __dp4a(cv.y, qreg[j].y, acc1);
                     acc0 = __dp4a(cv.z, qreg[j].z, acc0);
                     acc1 = __dp4a(cv.w, qreg[j].w, acc1);
+                    if constexpr (MID) {
+                        fine0 = __dp4a(cv.x, ereg[j].x, fine0);
+                        fine1 = __dp4a(cv.y, ereg[j].y, fine1);
+                        fine0 = __dp4a(cv.z, ereg[j].z, fine0);
+                        fine1 = __dp4a(cv.w, ereg[j].w, fine1);
+                    }
                 }
             } else {
                 for (int j = 0; j < cpl; ++j) {
@@ -141,12 +173,24 @@ __global__ void __launch_bounds__(kIntervalThreads, 1)
                     acc1 = __dp4a(cv.y, qv.y, acc1);
                     acc0 = __dp4a(cv.z, qv.z, acc0);
                     acc1 = __dp4a(cv.w, qv.w, acc1);
+                    if constexpr (MID) {
+                        const int4 ev = z24[4 * jj + p];
+                        fine0 = __dp4a(cv.x, ev.x, fine0);
+                        fine1 = __dp4a(cv.y, ev.y, fine1);
+                        fine0 = __dp4a(cv.z, ev.z, fine0);
+                        fine1 = __dp4a(cv.w, ev.w, fine1);
+                    }
                 }
             }
         }
         int dot = acc0 + acc1;
         dot += __shfl_xor_sync(0xffffffffu, dot, 1);
         dot += __shfl_xor_sync(0xffffffffu, dot, 2);
+        int dot2 = fine0 + fine1;
+        if constexpr (MID) {
+            dot2 += __shfl_xor_sync(0xffffffffu, dot2, 1);
+            dot2 += __shfl_xor_sync(0xffffffffu, dot2, 2);
+        }
         if (p == 0 && row < a.rows) {
             const float* ps = reinterpret_cast<const float*>(stage + TR * m_pad);
             float lo, hi;
@@ -156,6 +200,10 @@ __global__ void __launch_bounds__(kIntervalThreads, 1)
             if (tombstoned(a.tomb, row)) lo = hi = -INFINITY;
             a.lo[row] = lo;
             a.hi[row] = hi;
+            if constexpr (MID)
+                a.mid[row] = __fmul_rn(
+                    ps[r_in_tile], __fadd_rn(__fmul_rn(q.s, __int2float_rn(dot)),
+                                             __fmul_rn(fine.s, __int2float_rn(dot2))));
             if (lo > top[kSlotTop - 1]) {   // insertion into the descending list
                 top[kSlotTop - 1] = lo;
 #pragma unroll
@@ -177,23 +225,28 @@ __global__ void __launch_bounds__(kIntervalThreads, 1)
     }
 }
 
-template <int CPL>
-static cudaError_t launch_tpl(const IntervalArgs& a, int num_sms, cudaStream_t st) {
+template <int CPL, bool MID>
+static cudaError_t launch_pass(const IntervalArgs& a, int num_sms, cudaStream_t st) {
     const int stage_bytes = kTileRows * a.m_pad + 3 * kTileRows * 4;
     int stages = (200 * 1024) / stage_bytes;
     if (stages > 8) stages = 8;
     if (stages < 2) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)stages * stage_bytes + 2 * stages * sizeof(uint64_t);
-    cudaError_t e = raise_smem_limit((const void*)interval_pass_kernel<CPL>, smem);
+    const size_t smem = (size_t)stages * stage_bytes + 2 * stages * sizeof(uint64_t) +
+                        (MID ? (size_t)a.m_pad : 0);
+    cudaError_t e = raise_smem_limit((const void*)interval_pass_kernel<CPL, MID>, smem);
     if (e != cudaSuccess) return e;
     const int64_t ntiles = (a.rows + kTileRows - 1) / kTileRows;
     const int grid = (int)(ntiles < num_sms ? ntiles : num_sms);
     const int chunks = a.m_pad / 16;
     const int rotate = (chunks % 8) == 0 ? 1 : 0;
     count_launches(1);
-    interval_pass_kernel<CPL><<<grid, kIntervalThreads, smem, st>>>(a, stages, rotate,
-                                                                     a.m_pad / 64);
+    interval_pass_kernel<CPL, MID><<<grid, kIntervalThreads, smem, st>>>(a, stages, rotate,
+                                                                          a.m_pad / 64);
     return cudaGetLastError();
+}
+template <int CPL>
+static cudaError_t launch_tpl(const IntervalArgs& a, int num_sms, cudaStream_t st) {
+    return a.mid ? launch_pass<CPL, true>(a, num_sms, st) : launch_pass<CPL, false>(a, num_sms, st);
 }
 
 // The staged kernel serves these row widths (the others take the unstaged one).
@@ -204,6 +257,8 @@ static bool staged_width(int m_pad) {
     }
     return kTileRows * m_pad + 3 * kTileRows * 4 <= 100 * 1024;
 }
+
+bool interval_writes_mid(int m_pad) { return staged_width(m_pad); }
 
 int64_t interval_slots(int64_t rows, int m_pad, int num_sms, int64_t* min_rows_per_slot) {
     *min_rows_per_slot = 0;

@@ -225,6 +225,12 @@ struct IntervalArgs {
     // the staged pass (slot = CTA x row position in a tile; each row belongs
     // to one slot), kSlotTop per slot, -inf where a slot had fewer live rows
     float* slot_top = nullptr;
+    // optional (staged passes): for every row, s (s_q zq + s_e ze).z in
+    // binary32, ze the query's second digit (fine_digit): what an exact rank
+    // count needs of the codes, for 4 bytes a row.  It wants the query itself.
+    float* mid = nullptr;
+    const float* qraw = nullptr;
+    int m_raw = 0;
     // limit of each wait for a tile or a free stage (device ns; 0: never
     // wait).  Waits for the pass's own copies in flight before it exits keep
     // the full 2 s limit whatever this is, so no copy outlives the kernel.
@@ -232,6 +238,8 @@ struct IntervalArgs {
 };
 constexpr int kSlotTop = 4;
 cudaError_t launch_interval_pass(const IntervalArgs& a, int num_sms, cudaStream_t st);
+// A pass over rows of m_pad bytes can write `mid`.
+bool interval_writes_mid(int m_pad);
 // Slots whose kSlotTop lower bounds a pass over `rows` rows of m_pad bytes
 // writes to slot_top (0: that pass writes none), and the fewest rows any
 // of them scans.

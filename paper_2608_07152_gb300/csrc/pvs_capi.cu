@@ -201,7 +201,8 @@ void cursor_free_device(pvs_cursor* c) {
     if (c->small) cudaFree(c->small);
     c->small = nullptr;
     c->zq = nullptr;
-    dev_free(c->lo), dev_free(c->hi), dev_free(c->bmax);
+    dev_free(c->lo), dev_free(c->hi), dev_free(c->bmax), dev_free(c->mid);
+    c->mid_cap = 0;
     dev_free(c->compact_scratch), dev_free(c->slot_top);
     c->slot_cap = 0;
     if (c->ws_slab) cudaFree(c->ws_slab);
@@ -234,6 +235,7 @@ void cursor_reset(pvs_cursor* c) {
     c->state = PVS_OK;
     c->scanned = false;
     c->bmax_valid = false;
+    c->want_mid = c->mid_valid = false;
     c->batch_ws = false;
     c->fresh_ws = false;
     c->horizon = c->horizon_base = 0;
@@ -266,7 +268,7 @@ constexpr size_t kCursorPoolBytes = size_t(4) << 30;
 size_t cursor_device_bytes(const pvs_cursor* c) {
     return (size_t)c->cap_rows * 12 + (size_t)c->cap_rows / 4 + (size_t)c->cap_w * 40 + 4096 +
            kFrontCap * 4 +
-           (size_t)c->scan_cap * 20;
+           (size_t)c->mid_cap * 4 + (size_t)c->scan_cap * 20;
 }
 
 // Allocate the per-row state of a cursor (first pull); a pooled cursor keeps
@@ -468,6 +470,20 @@ pvs_status interval_pass(pvs_cursor* c) {
         a.slot_top = c->slot_top;
         c->slot_n = slots * kSlotTop;
     }
+    c->mid_valid = false;
+    if (c->want_mid && interval_writes_mid(x->m_pad)) {
+        if (c->mid_cap < c->rows) {
+            dev_free(c->mid);
+            c->mid_cap = 0;
+            if (dev_alloc(&c->mid, (size_t)c->rows) == cudaSuccess) c->mid_cap = c->rows;
+            else cudaGetLastError();   // the rank count then reads the codes
+        }
+        if (c->mid_cap >= c->rows) {
+            a.mid = c->mid;
+            a.qraw = c->qraw;
+            a.m_raw = x->m_raw;
+        }
+    }
     if (!c->ev_begin) {
         PVS_CUDA(cudaEventCreate(&c->ev_begin));
         PVS_CUDA(cudaEventCreate(&c->ev_end));
@@ -481,6 +497,7 @@ pvs_status interval_pass(pvs_cursor* c) {
     PVS_CUDA(cudaEventRecord(c->ev_begin, c->stream));
     PVS_CUDA(launch_interval_pass(a, x->num_sms, c->stream));
     c->slot_fresh = a.slot_top != nullptr;
+    c->mid_valid = a.mid != nullptr;
     PVS_CUDA(cudaEventRecord(c->ev_end, c->stream));
     PVS_CUDA(cudaEventRecord(x->pass_done, c->stream));
     c->ev_pending = true;

@@ -71,6 +71,26 @@ __device__ __forceinline__ void interval_epilogue(int dot, const QueryScalars& q
     hi = __fadd_ru(c, r);
 }
 
+// What the query's codes leave of it, in a second digit: e_j = RN(q_j - s_q
+// zq_j) (one FMA; at most about s_q / 2), ze_j = rint(e_j / s_e) in [-127, 127]
+// with s_e = RN(s_q / 254).  Every kernel that uses the digits derives the same
+// ones.  No digits (all 0) where s_e or its inverse leaves the normal range.
+struct FineScale {
+    float s, inv;
+};
+__device__ __forceinline__ FineScale fine_scale(float s_q) {
+    FineScale f{__fdiv_rn(s_q, 254.0f), 0.0f};
+    f.inv = __fdiv_rn(1.0f, f.s);
+    if (!(f.s >= 0x1p-120f && f.s <= 0x1p+120f)) f.s = f.inv = 0.0f;
+    return f;
+}
+__device__ __forceinline__ float fine_rest(float q, float s_q, int z) {
+    return __fmaf_rn(-s_q, (float)z, q);
+}
+__device__ __forceinline__ int fine_digit(float e, float inv) {
+    return (int)fminf(fmaxf(rintf(__fmul_rn(e, inv)), -127.0f), 127.0f);
+}
+
 __device__ __forceinline__ bool tombstoned(const uint32_t* tomb, int64_t row) {
     return tomb != nullptr && ((__ldg(tomb + (row >> 5)) >> (row & 31)) & 1u);
 }

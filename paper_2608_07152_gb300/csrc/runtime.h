@@ -102,6 +102,11 @@ struct pvs_cursor {
     int64_t cap_rows = 0;
     float* lo = nullptr;
     float* hi = nullptr;
+    // a finer centre of every row's score (IntervalArgs::mid), written by the
+    // pass when a fusion asked for it before the pass; exact rank counts use it
+    float* mid = nullptr;
+    int64_t mid_cap = 0;
+    bool want_mid = false, mid_valid = false;
     // the largest hi of each 16-row block, written by a grouped pass (upper
     // bounds of hi from then on: refinement and delivery only lower hi)
     float* bmax = nullptr;
