@@ -6,7 +6,9 @@
 // The raw float32 row is copied next to the codes for authoritative scoring.
 #include <algorithm>
 
+#include "f32x2.cuh"
 #include "kernels.h"
+#include "pipeline.cuh"
 #include "pvs_common.cuh"
 
 namespace pvs {
@@ -19,25 +21,105 @@ static __device__ __noinline__ RowQuant quantize_row_slow(const float* v, int m,
     return quantize_row_warp(v, m, m_pad, z, fixed_s);
 }
 
+// A sum of squares x^2 2^(-2e), |x| < 2^e, to about 2^-37 of its value, two
+// chains of float32 at a time: s from 1 on, so that it is at least each
+// product and s' = RN(s + p) has the exact error p - (s' - s) (Dekker's
+// FastTwoSum); the products' errors are exact too (one FMA), and both sum to c.
+// n squares a chain: |c| <= 2 n u s with u = 2^-24, and the 2 n additions to it
+// and that of two chains' c round by u |c| at most, so 64 chains err by at most
+// 4 n (n + 1) u^2 (64 + S) in all.
+struct SquareSum {
+    uint64_t s, c = 0;
+    const uint64_t scale, neg_scale, m1;   // 2^-e, -2^-e, -1 in both halves
+    __device__ __forceinline__ explicit SquareSum(float f)
+        : s(f2_pack(1.0f, 1.0f)), scale(f2_pack(f, f)), neg_scale(f2_pack(-f, -f)),
+          m1(f2_pack(-1.0f, -1.0f)) {}
+    __device__ __forceinline__ void add(float a, float b) {
+        const uint64_t v = f2_pack(a, b);
+        const uint64_t x = f2_mul(v, scale);
+        const uint64_t np = f2_mul(x, f2_mul(v, neg_scale));   // -RN(x^2)
+        const uint64_t ep = f2_fma(x, x, np);
+        const uint64_t s1 = f2_fma(np, m1, s);                 // s + p
+        const uint64_t es = f2_fma(np, m1, f2_fma(s1, m1, s));
+        c = f2_add(c, f2_add(ep, es));
+        s = s1;
+    }
+    // The sum over the warp's 64 chains in units of 2^-38 (the same in every
+    // lane): s - 1 is a multiple of 2^-23, below 2^5 for up to 32 squares a lane;
+    // c rounds by half a unit a lane.
+    __device__ __forceinline__ long long warp_total() const {
+        float s0, s1, c0, c1;
+        f2_unpack(s, s0, s1);
+        f2_unpack(c, c0, c1);
+        const int a = (int)__fmul_rn(__fsub_rn(s0, 1.0f), 0x1p23f) +
+                      (int)__fmul_rn(__fsub_rn(s1, 1.0f), 0x1p23f);
+        const int b = __float2int_rn(__fmul_rn(__fadd_rn(c0, c1), 0x1p38f));
+        const int ahi = __reduce_add_sync(0xffffffffu, a >> 16);
+        const int alo = __reduce_add_sync(0xffffffffu, a & 0xffff);
+        const int bt = __reduce_add_sync(0xffffffffu, b);
+        return ((((long long)ahi << 16) + alo) << 15) + bt;
+    }
+};
+// 2^-e for the biased exponent field E of the largest |x| (e = E - 126)
+__device__ __forceinline__ float norm_scale(int E) {
+    return E <= 252 ? __uint_as_float((uint32_t)(253 - E) << 23) : __uint_as_float(0x00400000u >> (E - 253));
+}
+// norm_finish of the integer sum T of norm_term_bits, from the total of a
+// SquareSum of n squares a chain, of m in all: T 2^-48 lies in [S, S + m 2^-48).
+// Both ends of the interval round to the same bound, or *settled is false.
+__device__ inline float norm_from_squares(long long total, int e, int n, int m, bool* settled) {
+    const double S = (double)total * 0x1p-38;
+    const double u2 = 4.04 * 0x1p-48 * (double)(n * (n + 1));
+    const double E = u2 * (64.0 + S) + 0x1p-33 + (double)m * 0x1p-48;
+    const double r = __dsqrt_rn(S) * pow2d(e);
+    // |sqrt(S + d) / sqrt(S) - 1| <= |d| / S for |d| <= S / 2
+    const double d = r * (E / S + 0x1p-50);
+    const float lo = __double2float_ru(r - d), hi = __double2float_ru(r + d);
+    *settled = lo == hi;
+    return hi;
+}
+// Both integer sums of a row again, exactly, by the warp: the rows whose
+// intervals hold a rounding boundary (one norm in about 2^12).
+static __device__ __noinline__ void exact_norm_sums(const float* v, int m, float s, int Ev, int Ee,
+                                                    unsigned long long* T) {
+    const float rs = __frcp_rn(s);
+    unsigned long long a = 0, b = 0;
+    for (int j = threadIdx.x & 31; j < m; j += kWarp) {
+        uint32_t y;
+        const float x = v[j];
+        const float e = __fmaf_rn(-s, code_of(x, s, rs, y), x);
+        a += norm_term_bits(__float_as_uint(fabsf(x)), Ev);
+        b += norm_term_bits(__float_as_uint(fabsf(e)), Ee);
+    }
+    T[0] = warp_sum(a);
+    T[1] = warp_sum(b);
+}
+
 // One warp per row, `per_warp` (<= 32) rows of a warp in turn.  Everything per
 // element is float32 and integer work:
 //   - the code comes from the product with 1 / s (code_of);
 //   - the residual v - s c is exact in one FMA: v and s c are multiples of
 //     u = max(ulp(s) / 2, 2^-149) (v >= s / 2 where c != 0) and
 //     |v - s c| < 2^floor(log2 s) <= 2^24 u, checked per row;
-//   - the norm bounds sum norm_term_bits.
+//   - the norm bounds are those of sums of norm_term_bits, found from a sum of
+//     squares with an error bound (SquareSum); wider rows sum the terms.
 // Lane r keeps the sums of the batch's r-th row, and the binary64 square
 // roots run once for the batch, one row per lane.
 //
 // Bound by: HBM (4m bytes read, 5m + 12 written per row); the element work is
-// about 30 instructions.  With binary64 norm terms and four passes over the row the
-// kernel was bound by the FP64 pipe: 213 ms at 8.8M x 768 (0.29 TB/s); now 21.6 ms
-// (2.8 TB/s), bound by issue.
+// about 25 instructions.  With binary64 norm terms and four passes over the row
+// the FP64 pipe was the bound (500k x 768: 12.1 ms), then the latency of
+// one row after the other (1,290 us with integer terms, 1,166 with sums of
+// squares): a warp's loads waited for its last row's reductions.  Rows now come
+// ahead through a ring of bulk copies, two or three per warp: 628 us
+// (5.5 TB/s), 1M x 1,024 3,670 -> 1,606 us, 1M x 384 1,048 -> 693 us, 2M x 128
+// 867 -> 797 us.  Three
+// blocks of fewer registers from 513 dimensions on: 670 and 1,920 us.
 // NV4: float4 of the row per lane, in registers (m_pad <= 128 NV4); 0: wider
 // rows are read again (from L1 / L2) in each of the three steps.
 
 template <int NV4>
-__global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 3) build_kernel(const float* __restrict__ vecs, int64_t n,
+__global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 4) build_kernel(const float* __restrict__ vecs, int64_t n,
                                                     int m, int m_pad, int m_raw,
                                                     int8_t* __restrict__ codes,
                                                     float* __restrict__ scale,
@@ -45,15 +127,51 @@ __global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 3) build_kernel(const float
                                                     float* __restrict__ enorm,
                                                     float* __restrict__ raw, int* status,
                                                     const float* fixed_scale, int aligned,
-                                                    int per_warp) {
+                                                    int per_warp, int stages) {
     constexpr int kKeep = NV4 > 0 ? NV4 : 1;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t stride = (int64_t)gridDim.x * (blockDim.x >> 5) * per_warp;
     const float fs = fixed_scale ? *fixed_scale : 0.0f;
     const int steps = NV4 > 0 ? NV4 : (m_pad + 127) / 128;
-    for (int64_t row0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) *
-                        per_warp;
-         row0 < n; row0 += stride) {
+    const int64_t first = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * per_warp;
+    // the ring: rows [warps][stages][m] | barriers [warps][stages]; lane 0
+    // issues the rows in the order they are read
+    extern __shared__ float4 build_ring[];
+    const int n4 = m >> 2;
+    float4* ring = build_ring + (size_t)warp * stages * n4;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(build_ring + (size_t)(blockDim.x >> 5) * stages * n4) +
+                     warp * stages;
+    const uint32_t row_bytes = (uint32_t)m * sizeof(float);
+    uint64_t pol = 0;
+    int64_t next0 = first;   // the next row to issue: next0 + nextb
+    int nextb = 0;
+    int in_flight = 0;       // rows issued and not read; the oldest in buffer st
+    int st = 0;
+    uint32_t parity = 0;     // of buffer st
+    auto issue = [&](int buf) {
+        if (next0 >= n) return;
+        if (lane == 0) {
+            fence_proxy_async_smem();   // the warp's reads of this buffer come first
+            mbar_arrive_expect_tx(&bars[buf], row_bytes);
+            bulk_g2s(ring + (size_t)buf * n4, vecs + (next0 + nextb) * (int64_t)m, row_bytes,
+                     &bars[buf], pol);
+        }
+        ++in_flight;
+        if (++nextb == per_warp || next0 + nextb >= n) {
+            nextb = 0;
+            next0 += stride;
+        }
+    };
+    if (NV4 > 0 && stages) {
+        if (lane == 0) {
+            pol = l2_evict_first_policy();
+            for (int b = 0; b < stages; ++b) mbar_init(&bars[b], 1);
+            mbar_fence_init();
+        }
+        __syncwarp();
+        for (int b = 0; b < stages; ++b) issue(b);
+    }
+    for (int64_t row0 = first; row0 < n; row0 += stride) {
         const int batch = (int)(n - row0 < per_warp ? n - row0 : per_warp);
         // this lane's row of the batch
         unsigned long long tv = 0, te = 0;
@@ -66,7 +184,9 @@ __global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 3) build_kernel(const float
             auto load = [&](int i) {
                 const int j = 4 * (lane + 32 * i);
                 float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (aligned) {
+                if (NV4 > 0 && stages) {
+                    if (j < m) x = ring[(size_t)st * n4 + (j >> 2)];
+                } else if (aligned) {
                     if (j < m) x = __ldcs(reinterpret_cast<const float4*>(v + j));
                 } else {
                     if (j < m) x.x = v[j];
@@ -78,6 +198,16 @@ __global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 3) build_kernel(const float
             };
             float4 keep[kKeep];
             uint32_t mx = 0;
+            // warp-uniform: every lane must agree before the warp-wide steps below
+            if (NV4 > 0 && stages && !__all_sync(0xffffffffu, mbar_wait(&bars[st], parity))) {
+                // a copy did not arrive in time: record it, drain every copy in flight
+                if (lane == 0) set_status(status, PVS_ERR_TIMEOUT);
+                for (int k = 0; k < in_flight; ++k) {
+                    mbar_wait(&bars[st], parity);
+                    if (++st == stages) st = 0, parity ^= 1u;
+                }
+                return;
+            }
 #pragma unroll
             for (int i = 0; i < steps; ++i) {
                 const float4 x = load(i);
@@ -88,6 +218,11 @@ __global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 3) build_kernel(const float
                 mx = max(max(mx, __float_as_uint(fabsf(x.z))), __float_as_uint(fabsf(x.w)));
             }
             mx = __reduce_max_sync(0xffffffffu, mx);
+            if (NV4 > 0 && stages) {   // every lane has its values: the buffer is free
+                --in_flight;
+                issue(st);
+                if (++st == stages) st = 0, parity ^= 1u;
+            }
             if (mx >= 0x7f800000u) {   // an infinity or a NaN
                 if (lane == 0) set_status(status, PVS_ERR_NONFINITE);
                 done |= lane == b;
@@ -102,6 +237,7 @@ __global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 3) build_kernel(const float
             bool slow = mx != 0 && (mx < 0x00800000u || s < kFastScaleMin);
             const int Ev = max((int)(mx >> 23), 1);   // (0: sums of 0)
             unsigned long long a = 0, c2 = 0;
+            SquareSum sq(NV4 > 0 ? norm_scale(Ev) : 0.0f);
             if (!slow) {
 #pragma unroll
                 for (int i = 0; i < steps; ++i) {
@@ -115,7 +251,11 @@ __global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 3) build_kernel(const float
                         if (fs > 0.0f && fabsf(c) > 127.0f) out_of_range = true;
                         e[k] = __fmaf_rn(-s, c, xs[k]);
                         emx = max(emx, __float_as_uint(fabsf(e[k])));
-                        a += norm_term_bits(__float_as_uint(fabsf(xs[k])), Ev);
+                        if constexpr (NV4 == 0) a += norm_term_bits(__float_as_uint(fabsf(xs[k])), Ev);
+                    }
+                    if constexpr (NV4 > 0) {
+                        sq.add(x.x, x.y);
+                        sq.add(x.z, x.w);
                     }
                     const int j4 = lane + 32 * i;
                     if (4 * j4 < m_pad)
@@ -142,13 +282,12 @@ __global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 3) build_kernel(const float
                 continue;
             }
             const int Ee = max((int)(emx >> 23), 1);
+            SquareSum eq(NV4 > 0 ? norm_scale(Ee) : 0.0f);
 #pragma unroll
             for (int i = 0; i < steps; ++i) {
                 if constexpr (NV4 > 0) {
-                    c2 += norm_term_bits(__float_as_uint(fabsf(keep[i].x)), Ee);
-                    c2 += norm_term_bits(__float_as_uint(fabsf(keep[i].y)), Ee);
-                    c2 += norm_term_bits(__float_as_uint(fabsf(keep[i].z)), Ee);
-                    c2 += norm_term_bits(__float_as_uint(fabsf(keep[i].w)), Ee);
+                    eq.add(keep[i].x, keep[i].y);
+                    eq.add(keep[i].z, keep[i].w);
                 } else {
                     const float4 x = load(i);
                     const float xs[4] = {x.x, x.y, x.z, x.w};
@@ -160,8 +299,13 @@ __global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 3) build_kernel(const float
                     }
                 }
             }
-            a = warp_sum(a);
-            c2 = warp_sum(c2);
+            if constexpr (NV4 > 0) {
+                a = mx ? (unsigned long long)sq.warp_total() : 0ull;
+                c2 = emx ? (unsigned long long)eq.warp_total() : 0ull;
+            } else {
+                a = warp_sum(a);
+                c2 = warp_sum(c2);
+            }
             if (lane == b) {
                 s_of = s;
                 tv = a;
@@ -170,10 +314,36 @@ __global__ void __launch_bounds__(256, NV4 > 4 ? 2 : 3) build_kernel(const float
                 ee = Ee - 126;
             }
         }
+        if constexpr (NV4 > 0) {
+            bool open = false;
+            if (lane < batch && !done) {
+                bool ok = true;
+                vn = tv ? norm_from_squares((long long)tv, ev, 2 * NV4, m, &ok) : 0.0f;
+                open = !ok;
+                en = te ? norm_from_squares((long long)te, ee, 2 * NV4, m, &ok) : 0.0f;
+                open |= !ok;
+            }
+            unsigned int todo = __ballot_sync(0xffffffffu, open);
+            while (todo) {
+                const int b = __ffs(todo) - 1;
+                todo &= todo - 1;
+                unsigned long long T[2];
+                const int Ev = __shfl_sync(0xffffffffu, ev, b) + 126;
+                const int Ee = __shfl_sync(0xffffffffu, ee, b) + 126;
+                exact_norm_sums(vecs + (row0 + b) * (int64_t)m, m,
+                                __shfl_sync(0xffffffffu, s_of, b), Ev, Ee, T);
+                if (lane == b) {
+                    vn = norm_finish((long long)T[0], ev);
+                    en = norm_finish((long long)T[1], ee);
+                }
+            }
+        }
         if (lane < batch) {
             if (!done) {
-                vn = norm_finish((long long)tv, ev);
-                en = norm_finish((long long)te, ee);
+                if constexpr (NV4 == 0) {
+                    vn = norm_finish((long long)tv, ev);
+                    en = norm_finish((long long)te, ee);
+                }
                 if (isinf(vn) || isinf(en)) set_status(status, PVS_ERR_OVERFLOW);
             }
             scale[row0 + lane] = s_of;
@@ -194,10 +364,18 @@ cudaError_t launch_build(const float* vecs, int64_t n, int m, int m_pad, int m_r
     if (blocks > 152 * 64) blocks = 152 * 64;
     const int aligned =
         m % 4 == 0 && (reinterpret_cast<uintptr_t>(vecs) & 15u) == 0 ? 1 : 0;
+    // rows of up to 1,024 dimensions on 16-byte boundaries come through the
+    // ring, three a warp where three blocks of them fit on an SM
+    const size_t row = (size_t)m * sizeof(float) + sizeof(uint64_t);
+    const int stages = !aligned || m_pad > 1024 ? 0 : 3 * 8 * 3 * row <= 216 * 1024 ? 3 : 2;
+    const size_t smem = 8 * (size_t)stages * row;
     auto run = [&](auto kernel) {
+        const cudaError_t e = raise_smem_limit((const void*)kernel, smem);
+        if (e != cudaSuccess) return e;
         count_launches(1);
-        kernel<<<(unsigned)blocks, 256, 0, st>>>(vecs, n, m, m_pad, m_raw, codes, scale, vnorm,
-                                                 enorm, raw, status, fixed_scale, aligned, per_warp);
+        kernel<<<(unsigned)blocks, 256, smem, st>>>(vecs, n, m, m_pad, m_raw, codes, scale, vnorm,
+                                                    enorm, raw, status, fixed_scale, aligned,
+                                                    per_warp, stages);
         return cudaGetLastError();
     };
     switch ((m_pad + 127) / 128) {

@@ -17,6 +17,7 @@
 // A result that rounds to zero is +0.
 #pragma once
 
+#include "f32x2.cuh"
 #include "pvs_common.cuh"
 
 namespace pvs {
@@ -293,35 +294,6 @@ __device__ inline float exact_dot_warp_eft(const float* q_fast, const float* __r
 }
 
 // ---- two chains per instruction (f32x2), for rows staged in shared memory -----
-__device__ __forceinline__ uint64_t f2_pack(float x, float y) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ void f2_unpack(uint64_t v, float& x, float& y) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-}
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t f2_fma_ru(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rp.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 // Two chains of the error-free transformations above (components x, z and
 // y, w of the float4s), one f32x2 instruction a step.  There is no packed
 // subtraction: a - b is fma(b, -1, a), exact in the product, and the
