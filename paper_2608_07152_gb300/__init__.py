@@ -361,11 +361,11 @@ def pvs_cursor_open_group(index, queries, snap=None, pass_stream=None, cursor_st
 
 class CursorBatch(tuple):
     """The cursors of a batched open (immutable), with the C array of their
-    handles built once for the batch calls."""
+    handles for the batch calls."""
 
-    def __new__(cls, handles):
-        self = super().__new__(cls, [ctypes.c_void_p(h) for h in handles])
-        self._arr = (ctypes.c_void_p * max(len(handles), 1))(*handles)
+    def __new__(cls, arr, nq):
+        self = super().__new__(cls, map(ctypes.c_void_p, arr[:nq]))
+        self._arr = arr
         return self
 
 
@@ -381,7 +381,7 @@ def pvs_cursor_open_batch(index, queries, horizon: int, snap=None, stream=None):
                                       ctypes.c_void_p(handle) if handle else None,
                                       ctypes.cast(arr, ctypes.POINTER(ctypes.c_void_p))),
            "pvs_cursor_open_batch")
-    return CursorBatch([arr[i] for i in range(nq)])
+    return CursorBatch(arr, nq)
 
 
 def pvs_next(cursor, n: int):

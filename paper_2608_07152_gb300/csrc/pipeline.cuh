@@ -64,8 +64,7 @@ constexpr int kWaitTries = 64;   // attempts before the timer is read
 __device__ inline bool mbar_wait(uint64_t* bar, uint32_t parity,
                                  unsigned long long limit_ns = kWaitLimitNs) {
     if (limit_ns == 0) return mbar_test_wait(bar, parity);
-    // ordinary waits end here: reading the global timer takes about a
-    // microsecond, which a wait that has just begun must not add to itself
+    // ordinary waits end here, without reading the global timer
     for (int i = 0; i < kWaitTries; ++i)
         if (mbar_try_wait(bar, parity)) return true;
     const unsigned long long t0 = globaltimer();

@@ -763,20 +763,34 @@ struct DevBuf {
     cudaStream_t st = nullptr;
     cudaMemPool_t pool = nullptr;
     std::vector<void*> ptrs;
+    char* at = nullptr;      // the rest of the last allocation
+    size_t left = 0;
     DevBuf(cudaStream_t s, cudaMemPool_t p) : st(s), pool(p) {}
-    template <typename T>
-    T* get(size_t count) {
+    static size_t padded(size_t bytes) { return (std::max<size_t>(bytes, 1) + 255) / 256 * 256; }
+    // One allocation for the next gets of `bytes` (their padded sizes) in all.
+    bool reserve(size_t bytes) {
         void* p = nullptr;
-        const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
         const cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, st)
                                    : cudaMallocAsync(&p, bytes, st);
         if (e != cudaSuccess) {
             cudaGetLastError();
-            return nullptr;
+            return false;
         }
         ptrs.push_back(p);
-        return static_cast<T*>(p);
+        at = static_cast<char*>(p);
+        left = bytes;
+        return true;
     }
+    template <typename T>
+    T* get(size_t count) {
+        const size_t bytes = padded(count * sizeof(T));
+        if (bytes > left && !reserve(std::max(bytes, kSmall))) return nullptr;
+        T* p = reinterpret_cast<T*>(at);
+        at += bytes;
+        left -= bytes;
+        return p;
+    }
+    static constexpr size_t kSmall = size_t(64) << 10;   // several small arrays share one
     ~DevBuf() {
         for (void* p : ptrs) cudaFreeAsync(p, st);
     }
@@ -964,41 +978,8 @@ pvs_status open_batch_group(pvs_index* x, const std::shared_ptr<SnapData>& sd,
                             cudaStream_t st, pvs_cursor** out) {
     DevBuf buf(st, x->scratch_pool);
     BatchQueries bq;
-    const bool stream = batch_stream_supported(x->m_pad, x->num_sms);
-    // one synchronisation at the end: query statuses are read with the pass's
-    pvs_status s = encode_batch(x, queries, nq, on_device, buf, &bq, st, /*check_now=*/false, stream);
-    if (s != PVS_OK) return s;
-    // cursors with the queries' encodings and fresh counters (queued behind the
-    // passes, which do not need them: the host works while the passes run)
-    auto open_cursors = [&]() -> pvs_status {
-        for (int i = 0; i < nq; ++i) {
-            pvs_status cs = acquire_cursor(x, sd, &out[i], /*zero_state=*/false);
-            if (cs != PVS_OK) return cs;
-            out[i]->stream = st;
-        }
-        QueryDst* d_qd = buf.get<QueryDst>((size_t)nq);
-        if (!d_qd) return PVS_ERR_OOM;
-        // a pageable source is staged before cudaMemcpyAsync returns
-        std::vector<QueryDst> qd(nq);
-        for (int i = 0; i < nq; ++i)
-            qd[i] = QueryDst{out[i]->zq, out[i]->qraw, out[i]->qs, out[i]->ctr, out[i]->d_status};
-        PVS_CUDA(cudaMemcpyAsync(d_qd, qd.data(), nq * sizeof(QueryDst), cudaMemcpyHostToDevice, st));
-        PVS_CUDA(launch_copy_queries(bq.zq, bq.qraw, bq.qs, d_qd, nq, x->m_pad, x->m_raw, st));
-        return PVS_OK;
-    };
     const int64_t rows = sd->rows;
-    if (rows == 0) {
-        s = open_cursors();
-        if (s != PVS_OK) return s;
-        std::vector<QueryScalars> h_qs(nq);
-        PVS_CUDA(cudaMemcpyAsync(h_qs.data(), bq.qs, nq * sizeof(QueryScalars),
-                                 cudaMemcpyDeviceToHost, st));
-        PVS_CUDA(cudaStreamSynchronize(st));
-        for (int i = 0; i < nq; ++i)
-            if (h_qs[i].status != 0) return (pvs_status)h_qs[i].status;
-        return PVS_OK;
-    }
-
+    const bool stream = batch_stream_supported(x->m_pad, x->num_sms);
     // Sample every stride-th tile and take tau_q = the k_s-th largest sampled
     // lower bound.  The number of the horizon's rows in the sample is about
     // Poisson with mean H / stride, and tau_q misses the horizon (fewer than H
@@ -1024,6 +1005,52 @@ pvs_status open_batch_group(pvs_index* x, const std::shared_ptr<SnapData>& sd,
     // 512 ranks; wide intervals over deep horizons take the rest
     const int64_t cap = horizon <= 512 ? kWsSortMax / 2 : kWsSortMax;
     const int w_cap = (int)std::min<int64_t>(cap, std::max<int64_t>(rows, 1));
+    // one allocation for all of the open's scratch (a dozen, and their frees,
+    // were 30 us of a 256-query open while the device waited)
+    const size_t nqp = (size_t)round_up(nq, 32);
+    if (!buf.reserve(DevBuf::padded((size_t)nq * x->m_pad) + DevBuf::padded((size_t)nq * x->m_raw * 4) +
+                     DevBuf::padded((size_t)nq * sizeof(QueryScalars)) +
+                     DevBuf::padded(nqp * x->m_pad * 2) +
+                     (on_device ? 0 : DevBuf::padded((size_t)nq * x->m * 4)) +
+                     DevBuf::padded((size_t)nq * ld * 4) + 2 * DevBuf::padded((size_t)nq * 4) +
+                     3 * DevBuf::padded((size_t)nq * w_cap * 4) +
+                     DevBuf::padded((1 + 2 * (size_t)nq) * 4) +
+                     DevBuf::padded((size_t)nq * sizeof(WsDst)) +
+                     DevBuf::padded((size_t)nq * sizeof(QueryDst))))
+        return PVS_ERR_OOM;
+    // one synchronisation at the end: query statuses are read with the pass's
+    pvs_status s = encode_batch(x, queries, nq, on_device, buf, &bq, st, /*check_now=*/false, stream);
+    if (s != PVS_OK) return s;
+    // cursors with the queries' encodings and fresh counters (queued behind the
+    // passes, which do not need them: the host works while the passes run)
+    auto open_cursors = [&]() -> pvs_status {
+        for (int i = 0; i < nq; ++i) {
+            pvs_status cs = acquire_cursor(x, sd, &out[i], /*zero_state=*/false);
+            if (cs != PVS_OK) return cs;
+            out[i]->stream = st;
+        }
+        QueryDst* d_qd = buf.get<QueryDst>((size_t)nq);
+        if (!d_qd) return PVS_ERR_OOM;
+        // a pageable source is staged before cudaMemcpyAsync returns
+        std::vector<QueryDst> qd(nq);
+        for (int i = 0; i < nq; ++i)
+            qd[i] = QueryDst{out[i]->zq, out[i]->qraw, out[i]->qs, out[i]->ctr, out[i]->d_status};
+        PVS_CUDA(cudaMemcpyAsync(d_qd, qd.data(), nq * sizeof(QueryDst), cudaMemcpyHostToDevice, st));
+        PVS_CUDA(launch_copy_queries(bq.zq, bq.qraw, bq.qs, d_qd, nq, x->m_pad, x->m_raw, st));
+        return PVS_OK;
+    };
+    if (rows == 0) {
+        s = open_cursors();
+        if (s != PVS_OK) return s;
+        std::vector<QueryScalars> h_qs(nq);
+        PVS_CUDA(cudaMemcpyAsync(h_qs.data(), bq.qs, nq * sizeof(QueryScalars),
+                                 cudaMemcpyDeviceToHost, st));
+        PVS_CUDA(cudaStreamSynchronize(st));
+        for (int i = 0; i < nq; ++i)
+            if (h_qs[i].status != 0) return (pvs_status)h_qs[i].status;
+        return PVS_OK;
+    }
+
     float* dlo = buf.get<float>((size_t)nq * ld);
     float* tau = buf.get<float>((size_t)nq);
     float* rmax = buf.get<float>((size_t)nq);   // theta of the streaming pass
