@@ -249,13 +249,15 @@ static cudaError_t launch_tpl(const IntervalArgs& a, int num_sms, cudaStream_t s
     return a.mid ? launch_pass<CPL, true>(a, num_sms, st) : launch_pass<CPL, false>(a, num_sms, st);
 }
 
-// The staged kernel serves these row widths (the others take the unstaged one).
+// Widths with the query in registers: every multiple of 64 bytes up to 1,024.
+// Read again for each row, from L1, the query costs as many loads as the row:
+// 1M x 448 took 118 us (3.9 TB/s) that way, 102 us in registers.
+constexpr int kMaxCpl = 16;
+
+// The staged kernel serves rows of which two stages fit (the others take the
+// unstaged one).
 static bool staged_width(int m_pad) {
-    switch (m_pad / 64) {
-        case 1: case 2: case 4: case 6: case 8: case 12: case 16: return true;
-        default: break;
-    }
-    return kTileRows * m_pad + 3 * kTileRows * 4 <= 100 * 1024;
+    return m_pad <= 64 * kMaxCpl || kTileRows * m_pad + 3 * kTileRows * 4 <= 100 * 1024;
 }
 
 bool interval_writes_mid(int m_pad) { return staged_width(m_pad); }
@@ -276,14 +278,23 @@ cudaError_t launch_interval_pass(const IntervalArgs& a, int num_sms, cudaStream_
     switch (a.m_pad / 64) {
         case 1: return launch_tpl<1>(a, num_sms, st);
         case 2: return launch_tpl<2>(a, num_sms, st);
+        case 3: return launch_tpl<3>(a, num_sms, st);
         case 4: return launch_tpl<4>(a, num_sms, st);
+        case 5: return launch_tpl<5>(a, num_sms, st);
         case 6: return launch_tpl<6>(a, num_sms, st);
+        case 7: return launch_tpl<7>(a, num_sms, st);
         case 8: return launch_tpl<8>(a, num_sms, st);
+        case 9: return launch_tpl<9>(a, num_sms, st);
+        case 10: return launch_tpl<10>(a, num_sms, st);
+        case 11: return launch_tpl<11>(a, num_sms, st);
         case 12: return launch_tpl<12>(a, num_sms, st);
-        case 16: return launch_tpl<16>(a, num_sms, st);
+        case 13: return launch_tpl<13>(a, num_sms, st);
+        case 14: return launch_tpl<14>(a, num_sms, st);
+        case 15: return launch_tpl<15>(a, num_sms, st);
+        case kMaxCpl: return launch_tpl<kMaxCpl>(a, num_sms, st);
         default: break;
     }
-    if (kTileRows * a.m_pad + 3 * kTileRows * 4 <= 100 * 1024) return launch_tpl<0>(a, num_sms, st);
+    if (staged_width(a.m_pad)) return launch_tpl<0>(a, num_sms, st);
     return launch_interval_simple(a, st);
 }
 
