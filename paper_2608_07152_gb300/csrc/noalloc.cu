@@ -27,6 +27,7 @@
 #include "exact_dot.cuh"
 #include "kernels.h"
 #include "pvs_common.cuh"
+#include "rank_by_count.cuh"
 
 namespace pvs {
 
@@ -124,41 +125,15 @@ __global__ void __launch_bounds__(kScoreWarps * 32) noalloc_score_kernel(
     }
 }
 
-// The position of a key in the descending order is the number of larger
-// keys (they are distinct): a block takes 32 keys, one a lane, its warps a
-// share of all keys each, staged in shared memory and read by every lane
-// at once.  n^2 comparisons on every SM and no order of steps: 1,000 keys
-// in 5 us, against 11 us for the network of one block that sorted them.
-constexpr int kRankWarps = 8;
-constexpr int kRankStage = 2048;   // keys staged at a time (16 KB)
 __global__ void __launch_bounds__(kRankWarps * 32) noalloc_rank_emit_kernel(
     const unsigned long long* __restrict__ scratch, int n, int top, int64_t* out_ids,
     float* out_scores) {
-    __shared__ __align__(16) unsigned long long sk[kRankStage];
-    __shared__ int larger[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i = blockIdx.x * 32 + lane;
-    const unsigned long long key = i < n ? scratch[i] : 0ull;
-    if (threadIdx.x < 32) larger[threadIdx.x] = 0;
-    int count = 0;
-    for (int base = 0; base < n; base += kRankStage) {
-        const int m = min(kRankStage, n - base);
-        for (int j = threadIdx.x; j < kRankStage; j += blockDim.x)
-            sk[j] = j < m ? scratch[base + j] : 0ull;   // 0: larger than no key
-        __syncthreads();
-        const ulonglong2* s2 = reinterpret_cast<const ulonglong2*>(sk);
-#pragma unroll 4
-        for (int j = warp; 2 * j < m; j += kRankWarps) {
-            const ulonglong2 x = s2[j];
-            count += (x.x > key) + (x.y > key);
-        }
-        __syncthreads();
-    }
-    atomicAdd(&larger[lane], count);
-    __syncthreads();
-    if (warp == 0 && i < n && larger[lane] < top) {
-        out_ids[larger[lane]] = rank_key_id(key);
-        out_scores[larger[lane]] = rank_key_score(key);
+    __shared__ RankShared sh;
+    uint64_t key;
+    const int r = position_by_count(reinterpret_cast<const uint64_t*>(scratch), n, sh, key);
+    if (threadIdx.x < kRankKeys && blockIdx.x * kRankKeys + threadIdx.x < n && r < top) {
+        out_ids[r] = rank_key_id(key);
+        out_scores[r] = rank_key_score(key);
     }
 }
 
@@ -230,7 +205,7 @@ extern "C" pvs_status pvs_rank_exact_noalloc(const float* query, const float* ve
     }
     if (e == cudaSuccess && top > 0) {
         count_launches(1);
-        noalloc_rank_emit_kernel<<<(n + 31) / 32, kRankWarps * 32, 0, st>>>(scratch, n, top,
+        noalloc_rank_emit_kernel<<<(n + kRankKeys - 1) / kRankKeys, kRankWarps * 32, 0, st>>>(scratch, n, top,
                                                                             out_ids, out_scores);
         e = cudaGetLastError();
     }

@@ -22,7 +22,7 @@
 
 #include "pbm_kernels.h"
 #include "pvs_common.cuh"
-#include "sort_regs.cuh"
+#include "rank_by_count.cuh"
 
 namespace pvs {
 
@@ -390,57 +390,33 @@ cudaError_t launch_pbm_window(const uint64_t* sorted, int64_t next, int64_t n_ra
     return cudaGetLastError();
 }
 
-constexpr int kFinishThreads = kSortThreads;
-
-// The whole window, sorted, to pinned memory: every key in it is certified,
+// The whole window, ordered, to pinned memory: every key in it is certified,
 // so the host can serve later pulls from what lies beyond `need`.
-template <int E>
-__device__ __forceinline__ void finish_sorted(const uint64_t* keys_in, int count, uint64_t* sk,
-                                              int64_t* h_ids, float* h_scores) {
-    uint64_t v[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int i = threadIdx.x + e * kFinishThreads;
-        v[e] = i < count ? keys_in[i] : 0ull;   // 0 sorts last
-    }
-    sort_desc<E>(v, sk);
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int r = threadIdx.x * E + e;
-        if (r >= count) continue;
-        h_ids[r] = (int64_t)rank_key_id(v[e]);
-        h_scores[r] = rank_key_score(v[e]);
-    }
-}
-
-__global__ void __launch_bounds__(kFinishThreads) pbm_finish_kernel(const uint64_t* keys_in,
-                                                                    const PbmCounters* ctr,
-                                                                    uint64_t need, int complete,
-                                                                    int64_t* h_ids,
-                                                                    float* h_scores,
-                                                                    PbmCounters* h_mirror) {
-    extern __shared__ uint64_t keys[];
+__global__ void __launch_bounds__(kRankWarps * 32) pbm_finish_kernel(const uint64_t* keys,
+                                                                     const PbmCounters* ctr,
+                                                                     uint64_t need, int complete,
+                                                                     int64_t* h_ids,
+                                                                     float* h_scores,
+                                                                     PbmCounters* h_mirror) {
+    __shared__ RankShared sh;
     const unsigned long long count = ctr->collected;
-    if (need > 0 && count >= 1 && (count >= need || complete) &&
-        count <= (unsigned long long)kPbmFastWindow) {
-        const int n = (int)count;
-        if (n <= 1024) finish_sorted<1>(keys_in, n, keys, h_ids, h_scores);
-        else if (n <= 2048) finish_sorted<2>(keys_in, n, keys, h_ids, h_scores);
-        else if (n <= 4096) finish_sorted<4>(keys_in, n, keys, h_ids, h_scores);
-        else finish_sorted<8>(keys_in, n, keys, h_ids, h_scores);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *h_mirror = *ctr;
+    if (need == 0 || count < 1 || (count < need && !complete) ||
+        count > (unsigned long long)kPbmFastWindow || blockIdx.x * kRankKeys >= count)
+        return;
+    uint64_t key;
+    const int r = position_by_count(keys, (int)count, sh, key);
+    if (threadIdx.x < kRankKeys && blockIdx.x * kRankKeys + threadIdx.x < count) {
+        h_ids[r] = (int64_t)rank_key_id(key);
+        h_scores[r] = rank_key_score(key);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) *h_mirror = *ctr;
 }
 
 cudaError_t launch_pbm_finish(const uint64_t* keys, const PbmCounters* ctr, uint64_t need,
                               bool complete, int64_t* h_ids, float* h_scores,
                               PbmCounters* h_mirror, cudaStream_t st) {
-    cudaError_t e = raise_smem_limit((const void*)pbm_finish_kernel,
-                                     kPbmFastWindow * sizeof(uint64_t));
-    if (e != cudaSuccess) return e;
     count_launches(1);
-    pbm_finish_kernel<<<1, kFinishThreads, kPbmFastWindow * sizeof(uint64_t), st>>>(
+    pbm_finish_kernel<<<kPbmFastWindow / kRankKeys, kRankWarps * 32, 0, st>>>(
         keys, ctr, need, complete ? 1 : 0, h_ids, h_scores, h_mirror);
     return cudaGetLastError();
 }

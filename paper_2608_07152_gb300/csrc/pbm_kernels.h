@@ -76,11 +76,11 @@ cudaError_t launch_pbm_range_keys(const float* H, int64_t n_ranges, int block, u
 cudaError_t launch_pbm_window(const uint64_t* sorted, int64_t next, int64_t n_ranges,
                               const uint64_t* pool, uint64_t hi, uint64_t* out, uint64_t cap,
                               PbmCounters* ctr, cudaStream_t st);
-// One CTA: when 1 <= ctr->collected <= kPbmFastWindow and either need <=
+// When 1 <= ctr->collected <= kPbmFastWindow and either need <=
 // ctr->collected or `complete` (the window holds every remaining rank),
-// sorts the collected keys and writes all of them as ids / scores to h_ids /
-// h_scores; always copies *ctr to *h_mirror last.  h_* may be pinned host
-// memory.
+// orders the collected keys and writes all of them as ids / scores to h_ids /
+// h_scores; always copies *ctr to *h_mirror.  h_* may be pinned host memory
+// (complete once the stream is).
 constexpr int kPbmFastWindow = 8192;
 cudaError_t launch_pbm_finish(const uint64_t* keys, const PbmCounters* ctr, uint64_t need,
                               bool complete, int64_t* h_ids, float* h_scores,
