@@ -644,7 +644,8 @@ __global__ void pbm_sel_hist_kernel(const uint64_t* __restrict__ pool, const Pbm
 
 // One block of 256 threads, thread t the digit 255 - t: the digit whose keys
 // hold the wanted rank (suffix counts by a scan).
-__global__ void __launch_bounds__(256) pbm_sel_pick_kernel(int shift, unsigned long long* sel) {
+__global__ void __launch_bounds__(256) pbm_sel_pick_kernel(int shift, unsigned long long* sel,
+                                                           unsigned long long past) {
     __shared__ unsigned long long tot[8];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const unsigned long long c = sel[2 + 255 - t];
@@ -659,20 +660,23 @@ __global__ void __launch_bounds__(256) pbm_sel_pick_kernel(int shift, unsigned l
     __syncthreads();
     for (int w = 0; w < warp; ++w) incl += tot[w];
     if (incl - c < k && k <= incl) {   // one thread
-        sel[0] |= (unsigned long long)(255 - t) << shift;
+        sel[0] = (sel[0] | ((unsigned long long)(255 - t) << shift)) + past;
         sel[1] = k - (incl - c);
     }
     sel[2 + 255 - t] = 0;
 }
 
 cudaError_t launch_pbm_select64(const uint64_t* pool, const PbmCounters* ctr, uint64_t hi,
-                                uint64_t k, unsigned long long* sel64, cudaStream_t st) {
+                                uint64_t k, bool scores_only, unsigned long long* sel64,
+                                cudaStream_t st) {
     count_launches(1);
     pbm_sel_init_kernel<<<1, 256, 0, st>>>(sel64, (unsigned long long)k);
-    for (int shift = 56; shift >= 0; shift -= 8) {
+    const int last = scores_only ? 32 : 0;
+    for (int shift = 56; shift >= last; shift -= 8) {
         count_launches(2);
         pbm_sel_hist_kernel<<<152 * 4, 256, 0, st>>>(pool, ctr, hi, shift, sel64);
-        pbm_sel_pick_kernel<<<1, 256, 0, st>>>(shift, sel64);
+        pbm_sel_pick_kernel<<<1, 256, 0, st>>>(shift, sel64,
+                                               scores_only && shift == last ? 1ull << 32 : 0ull);
     }
     return cudaGetLastError();
 }

@@ -110,9 +110,12 @@ cudaError_t launch_pbm_expand(const PbmExpandArgs& a, int num_sms, cudaStream_t 
 cudaError_t launch_pbm_collect(const uint64_t* pool, const unsigned long long* from, uint64_t hi,
                                uint64_t* out, uint64_t cap, PbmCounters* ctr, cudaStream_t st);
 // 64-bit radix selection: sel64[0] = the k-th largest (1-based) pool key k'
-// with ctr->kmax < k' < hi; sel64 holds 2 + 256 words of state.
+// with ctr->kmax < k' < hi; sel64 holds 2 + 256 words of state.  scores_only:
+// sel64[0] = the least key of any score above that of k' (half the passes;
+// fewer than k keys reach it).
 cudaError_t launch_pbm_select64(const uint64_t* pool, const PbmCounters* ctr, uint64_t hi,
-                                uint64_t k, unsigned long long* sel64, cudaStream_t st);
+                                uint64_t k, bool scores_only, unsigned long long* sel64,
+                                cudaStream_t st);
 // ids[i], scores[i] of the first m keys of a descending key array.
 cudaError_t launch_pbm_emit(const uint64_t* keys, int m, int64_t* ids, float* scores,
                             cudaStream_t st);
