@@ -31,8 +31,8 @@
 // for every tile; it serves row widths this kernel has no room for.
 //
 // Modes:
-//   sample  lower bounds of every tile_stride-th tile: one float per row, or the
-//           largest of each 32 rows (a distinct row's bound either way, so the
+//   sample  lower bounds of every tile_stride-th tile: one float per row, or that of the
+//           row of the largest centre among 32 (a distinct row's bound either way, so the
 //           k-th largest stored never exceeds the k-th largest lower bound);
 //   filter  rows whose upper bound reaches the query's threshold tau_q are
 //           appended to its working set, rows whose lower bound does are
@@ -401,6 +401,44 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
                 uint32_t d[32];
                 tc::ld_32x32b_x32(tcol + (uint32_t)(cc * 32), d);
                 tc::wait_ld();
+                if (a.mode == 0 && a.group_max) {
+                    // per query the row of the largest centre (of equal ones to
+                    // 18 bits, the last lane's), whose own lower bound the 32
+                    // rows leave; then a query in every lane.  (Every row's
+                    // bound made the epilogue's instructions the sample's
+                    // time: 553k x 768 x 64 queries 190 us, 113 so.)
+                    int m[32];
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) {   // (branch-free: the 32 chains overlap)
+                        const float c = live ? __fmul_rn(__uint_as_float(d[k]), sv) : -INFINITY;
+                        int b = __float_as_int(c);
+                        b ^= (b >> 31) & 0x7fffffff;   // ordered as the floats are
+                        m[k] = __reduce_max_sync(0xffffffffu, (b & ~31) | lane);
+                    }
+                    int best = 0;
+                    uint32_t dot = 0;
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) {
+                        const uint32_t dk = __shfl_sync(0xffffffffu, d[k], m[k] & 31);
+                        best = lane == k ? m[k] & 31 : best;
+                        dot = lane == k ? dk : dot;
+                    }
+                    const float bs = __shfl_sync(0xffffffffu, sv, best);
+                    const float bv = __shfl_sync(0xffffffffu, vn, best);
+                    const float be = __shfl_sync(0xffffffffu, en, best);
+                    const unsigned int alive = __ballot_sync(0xffffffffu, live);
+                    if (cc * 32 + lane < a.nq) {
+                        float lo, hi;
+                        interval_epilogue(__float2int_rn(__uint_as_float(dot)),
+                                          sh.qs[cc * 32 + lane], bs, bv, be, lo, hi);
+                        const bool any = (alive >> best) & 1u;
+                        if (any && !(isfinite(lo) && isfinite(hi)))
+                            set_status(a.status, PVS_ERR_OVERFLOW);
+                        a.dump_lo[(int64_t)(cc * 32 + lane) * a.dump_ld + i * 4 + quarter] =
+                            any ? lo : -INFINITY;
+                    }
+                    continue;
+                }
                 if (a.mode == 0) {
                     const int64_t srow = i * kRows + r_in_tile;
                     bool bad = false;
@@ -412,24 +450,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
                         bad |= live && !(isfinite(lo) && isfinite(hi));   // (padding queries: 0)
                         d[k] = __float_as_uint(live ? lo : -INFINITY);
                     }
-                    if (a.group_max) {
-                        uint32_t best = 0;   // lane k: the 32 rows' largest key, query k
 #pragma unroll
-                        for (int k = 0; k < 32; ++k) {
-                            const uint32_t m =
-                                __reduce_max_sync(0xffffffffu, fkey(__uint_as_float(d[k])));
-                            best = lane == k ? m : best;
-                        }
-                        if (cc * 32 + lane < a.nq)
-                            a.dump_lo[(int64_t)(cc * 32 + lane) * a.dump_ld + i * 4 + quarter] =
-                                fkey_inv(best);
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 32; ++k)
-                            if (cc * 32 + k < a.nq)
-                                a.dump_lo[(int64_t)(cc * 32 + k) * a.dump_ld + srow] =
-                                    __uint_as_float(d[k]);
-                    }
+                    for (int k = 0; k < 32; ++k)
+                        if (cc * 32 + k < a.nq)
+                            a.dump_lo[(int64_t)(cc * 32 + k) * a.dump_ld + srow] =
+                                __uint_as_float(d[k]);
                     if (bad) set_status(a.status, PVS_ERR_OVERFLOW);
                     continue;
                 }
