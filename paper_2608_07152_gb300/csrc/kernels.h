@@ -333,9 +333,10 @@ cudaError_t launch_compact_ordered(const float* lo, const float* hi, int64_t row
 cudaError_t launch_candidates(const float* w_lo, const float* w_hi, const unsigned int* w_len,
                               const SelectState* sel, int32_t* cand, unsigned int* cand_len,
                               int grid, cudaStream_t st);
-// keys[i] = rank_key(w_lo[cand[i]], cand[i]) for i < *cand_len.
-cudaError_t launch_make_keys(const int32_t* cand, const unsigned int* cand_len,
-                             const float* w_lo, uint64_t* keys, int grid, cudaStream_t st);
+// rank_key(w_lo[w], w) of the live rows w with fkey(w_lo[w]) >= sel->prefix, in
+// any order; *count of them.
+cudaError_t launch_top_keys(const float* w_lo, const unsigned int* w_len, const SelectState* sel,
+                            uint64_t* keys, unsigned int* count, int grid, cudaStream_t st);
 // Sort `count` 64-bit keys descending, in place (count <= kBitonicMax).
 constexpr int kBitonicMax = 8192;
 cudaError_t launch_bitonic_desc(uint64_t* keys, int count, cudaStream_t st);
@@ -349,6 +350,12 @@ cudaError_t launch_radix_sort_desc(uint64_t* keys, uint64_t* tmp, int64_t count,
 cudaError_t launch_emit(const uint64_t* keys, int n, const int32_t* w_id, float* w_lo,
                         float* w_hi, float* lo, float* hi, int64_t* out_ids, float* out_scores,
                         cudaStream_t st);
+// The same from `count` distinct keys in any order: each key's position is
+// counted, count^2 comparisons on every SM (8,192 keys 25 us).
+constexpr int kCountEmitMax = 8192;
+cudaError_t launch_count_emit(const uint64_t* keys, int count, int n, const int32_t* w_id,
+                              float* w_lo, float* w_hi, float* lo, float* hi, int64_t* out_ids,
+                              float* out_scores, cudaStream_t st);
 
 // ---- batched interval pass on the tensor cores (batch_gemm.cu) --------------
 struct BatchArgs {

@@ -14,6 +14,7 @@
 
 #include "kernels.h"
 #include "pvs_common.cuh"
+#include "rank_by_count.cuh"
 
 namespace pvs {
 
@@ -498,20 +499,32 @@ cudaError_t launch_candidates(const float* w_lo, const float* w_hi, const unsign
     return cudaGetLastError();
 }
 
-__global__ void make_keys_kernel(const int32_t* __restrict__ cand, const unsigned int* cand_len,
-                                 const float* __restrict__ w_lo, uint64_t* keys) {
-    const int64_t n = *cand_len;
+// The keys of the rows whose lower bound (their score, once refined) reaches
+// the selected threshold, in any order.
+__global__ void top_keys_kernel(const float* __restrict__ w_lo, const unsigned int* w_len,
+                                const SelectState* sel, uint64_t* keys, unsigned int* count) {
+    const uint32_t t = (uint32_t)sel->prefix;
+    const int64_t len = *w_len;
+    const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int32_t w = cand[i];
-        keys[i] = rank_key(w_lo[w], (uint32_t)w);
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < len; i0 += stride) {
+        const int64_t i = i0 + threadIdx.x;
+        const float s = i < len ? w_lo[i] : -INFINITY;
+        const bool f = s != -INFINITY && fkey(s) >= t;
+        const unsigned int bal = __ballot_sync(0xffffffffu, f);
+        unsigned int base = 0;
+        if (lane == 0 && bal) base = atomicAdd(count, (unsigned int)__popc(bal));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (f) keys[base + __popc(bal & ((1u << lane) - 1u))] = rank_key(s, (uint32_t)i);
     }
 }
 
-cudaError_t launch_make_keys(const int32_t* cand, const unsigned int* cand_len,
-                             const float* w_lo, uint64_t* keys, int grid, cudaStream_t st) {
+cudaError_t launch_top_keys(const float* w_lo, const unsigned int* w_len, const SelectState* sel,
+                            uint64_t* keys, unsigned int* count, int grid, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned int), st);
+    if (e != cudaSuccess) return e;
     count_launches(1);
-    make_keys_kernel<<<grid, 256, 0, st>>>(cand, cand_len, w_lo, keys);
+    top_keys_kernel<<<grid, 256, 0, st>>>(w_lo, w_len, sel, keys, count);
     return cudaGetLastError();
 }
 
@@ -807,12 +820,9 @@ cudaError_t launch_radix_sort_desc(uint64_t* keys, uint64_t* tmp, int64_t count,
 // ---------------------------------------------------------------------------
 // emit the first n sorted keys and mark them emitted
 // ---------------------------------------------------------------------------
-__global__ void emit_kernel(const uint64_t* __restrict__ keys, int n, const int32_t* w_id,
-                            float* w_lo, float* w_hi, float* lo, float* hi, int64_t* out_ids,
-                            float* out_scores) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint64_t k = keys[i];
+__device__ __forceinline__ void emit_key(uint64_t k, int i, const int32_t* w_id, float* w_lo,
+                                         float* w_hi, float* lo, float* hi, int64_t* out_ids,
+                                         float* out_scores) {
     const uint32_t w = rank_key_id(k);
     const int32_t id = w_id[w];
     out_ids[i] = id;
@@ -823,6 +833,35 @@ __global__ void emit_kernel(const uint64_t* __restrict__ keys, int n, const int3
         lo[id] = -INFINITY;
         hi[id] = -INFINITY;
     }
+}
+
+__global__ void emit_kernel(const uint64_t* __restrict__ keys, int n, const int32_t* w_id,
+                            float* w_lo, float* w_hi, float* lo, float* hi, int64_t* out_ids,
+                            float* out_scores) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) emit_key(keys[i], i, w_id, w_lo, w_hi, lo, hi, out_ids, out_scores);
+}
+
+// The same from `count` keys in any order (a few thousand: every key meets
+// every other).
+__global__ void __launch_bounds__(kRankWarps * 32) count_emit_kernel(
+    const uint64_t* __restrict__ keys, int count, int n, const int32_t* w_id, float* w_lo,
+    float* w_hi, float* lo, float* hi, int64_t* out_ids, float* out_scores) {
+    __shared__ RankShared sh;
+    uint64_t key;
+    const int r = position_by_count(keys, count, sh, key);
+    if (threadIdx.x < kRankKeys && blockIdx.x * kRankKeys + threadIdx.x < count && r < n)
+        emit_key(key, r, w_id, w_lo, w_hi, lo, hi, out_ids, out_scores);
+}
+
+cudaError_t launch_count_emit(const uint64_t* keys, int count, int n, const int32_t* w_id,
+                              float* w_lo, float* w_hi, float* lo, float* hi, int64_t* out_ids,
+                              float* out_scores, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    count_launches(1);
+    count_emit_kernel<<<(count + kRankKeys - 1) / kRankKeys, kRankWarps * 32, 0, st>>>(
+        keys, count, n, w_id, w_lo, w_hi, lo, hi, out_ids, out_scores);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_emit(const uint64_t* keys, int n, const int32_t* w_id, float* w_lo,
