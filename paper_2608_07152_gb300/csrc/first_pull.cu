@@ -1,13 +1,13 @@
 // The first pull of a lone cursor in four launches (Sec. 2.3.1 incremental
 // ranking, Sec. 2.1 exact prefix): the first working set is the rows that can
-// hold the next H ranks; all of them are scored exactly and sorted, and the
-// first ranks come out in order.
+// hold the next H ranks; all of them are scored exactly, and the first ranks
+// come out in order.
 //
 //   1. first_threshold_kernel  a value v that at least H rows' lower bounds reach;
 //   2. first_set_kernel        W = the live rows with hi >= v (unordered);
 //   3. refine_ring_kernel      the exact score of every row of W, on every SM;
-//   4. first_emit_kernel       W sorted by rank key (score desc, id asc), the
-//                              first n ranks written and marked.
+//   4. first_emit_kernel       W's certified rows ordered by rank key (score desc, id
+//                              asc), the first n ranks written and marked.
 // Every row outside W has hi < v, so the rows of W that score v or more, H at
 // least, are the first ranks: all of them are certified, usually many more
 // than H (intervals are wider than the spread of the best scores).  More than
@@ -20,16 +20,14 @@
 // working set and the first page, then a pull for every further 80 ranks.
 #include "kernels.h"
 #include "pvs_common.cuh"
-#include "sort_regs.cuh"
 
 namespace pvs {
 namespace {
 
-constexpr int kThreads = kSortThreads;
+constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
 constexpr int kBins = 2048;
 constexpr int kStageMax = 50 * 1024;   // values staged in shared memory (200 KB)
-constexpr int kSortMax = 4096;         // keys sorted at once
 
 struct ThresholdShared {
     unsigned int hist[kBins];
@@ -147,6 +145,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (t == 0) {
         sel->prefix = 0;
         ctr->w_len = 0;
+        ctr->cand = 0;   // the emission's blocks that are done
         ctr->front_k = 0;
         ctr->front_hint = 0;
     }
@@ -252,161 +251,75 @@ __device__ __forceinline__ void emit_rank(const FirstEmitArgs& a, int r, uint64_
     a.hi[id] = -INFINITY;
 }
 
-// Order the keys (E per thread; 0: none) and emit; returns the ranks emitted.
-// A key's rank is the number of larger keys: those of the bins above (2,048
-// bins, linear in score) and the larger ones of its own bin, two or three for
-// scores spread like real ones.  Where a bin holds more than kBinMax (ties,
-// an outlier that stretches the range) the keys are sorted instead.  (Sorting
-// always: 34 us at 2,200 rows under the profiler, against 15 us.)
-constexpr unsigned int kBinMax = 48;
+// Order the certified rows of the scored set and emit the first n.  A key's
+// rank is the number of larger keys, and every key larger than a certified
+// one is certified too: each block gathers the certified keys in shared memory
+// and counts for its share of the set, 32 rows at a time, one a lane, its warps
+// a part of the keys each.  The last block to finish publishes.  Bound by
+// latency: one block that ranked by bins of the scores, or sorted where a
+// bin was crowded, took 14 us at 2,200 rows and 24 to 45 us in clusters of near
+// neighbours; now 11, and 12 to 15 us.
+constexpr int kEmitWarps = 32;
 
-template <int E>
-__device__ __forceinline__ int emit_first(const FirstEmitArgs& a, uint64_t (&v)[E], uint64_t* sk,
-                                          ThresholdShared& sh) {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const uint32_t tau = (uint32_t)a.sel->prefix;
-    float mn = INFINITY, mx = -INFINITY;
-    int certified = 0;   // certified ranks come first
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        certified += __syncthreads_count(v[e] != 0 && (uint32_t)(v[e] >> 32) >= tau);
-        if (v[e] == 0) continue;
-        const float s = rank_key_score(v[e]);
-        mn = fminf(mn, s);
-        mx = fmaxf(mx, s);
-    }
-    mx = warp_max(mx);
-    mn = -warp_max(-mn);
-    if (lane == 0) {
-        sh.red[warp][0] = mn;
-        sh.red[warp][1] = mx;
-    }
-    for (int i = t; i < kBins; i += kThreads) sh.hist[i] = 0;
-    __syncthreads();
-    mx = warp_max(sh.red[lane][1]);
-    mn = -warp_max(-sh.red[lane][0]);
-    const float scale = mx > mn ? (kBins - 0.5f) / (mx - mn) : 0.0f;
-    int bin[E];
-    unsigned int at[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {   // larger scores in earlier bins
-        bin[e] = -1;
-        if (v[e] == 0) continue;
-        bin[e] = min(kBins - 1, max(0, (int)((mx - rank_key_score(v[e])) * scale)));
-        at[e] = atomicAdd(&sh.hist[bin[e]], 1u);
-    }
-    __syncthreads();
-    // exclusive prefix sums over the bins: thread t holds bins 2 t and 2 t + 1
-    const unsigned int h0 = sh.hist[2 * t], h1 = sh.hist[2 * t + 1];
-    if (__syncthreads_or(h0 > kBinMax || h1 > kBinMax)) {
-        sort_desc<E>(v, sk);
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int r = t * E + e;
-            if (r < a.n && r < certified) emit_rank(a, r, v[e]);
-        }
-        return min(certified, a.n);
-    }
-    unsigned int incl = h0 + h1;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned int up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += up;
-    }
-    if (lane == 31) sh.warp_tot[warp] = incl;
-    __syncthreads();
-    unsigned int first = incl - h0 - h1;
-    for (int w = 0; w < warp; ++w) first += sh.warp_tot[w];
-    sh.hist[2 * t] = first;
-    sh.hist[2 * t + 1] = first + h0;
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < E; ++e)
-        if (bin[e] >= 0) sk[sh.hist[bin[e]] + at[e]] = v[e];
-    // the end of the last bin: every key
-    int total = 0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) total += __syncthreads_count(v[e] != 0);
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        if (bin[e] < 0) continue;
-        const unsigned int b0 = sh.hist[bin[e]];
-        const unsigned int b1 = bin[e] + 1 < kBins ? sh.hist[bin[e] + 1] : (unsigned int)total;
-        unsigned int r = b0;
-        for (unsigned int i = b0; i < b1; ++i) r += sk[i] > v[e];
-        if ((int)r < a.n && (int)r < certified) emit_rank(a, (int)r, v[e]);
-    }
-    return min(certified, a.n);
-}
-
-template <int E>
-__device__ __forceinline__ int emit_set(const FirstEmitArgs& a, unsigned int len, uint64_t* sk,
-                                        ThresholdShared& sh) {
-    uint64_t v[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const unsigned int i = threadIdx.x + (unsigned int)(e * kThreads);
-        v[e] = i < len ? rank_key(a.w_lo[i], (uint32_t)a.w_id[i]) : 0ull;
-    }
-    return emit_first<E>(a, v, sk, sh);
-}
-
-// A set of more than kSortMax rows: only those that can be among the n emitted
-// are sorted (a floor that n of the scores reach; exact ties below a full
-// bin can leave more than kSortMax of them: -1, nothing emitted).
-__device__ __forceinline__ int emit_pruned(const FirstEmitArgs& a, unsigned int len, uint64_t* sk,
-                                           float* scores, ThresholdShared& sh,
-                                           unsigned int* count) {
-    const int t = threadIdx.x;
-    float vmin = INFINITY, vmax = -INFINITY;
-    for (unsigned int i = t; i < len; i += kThreads) {
-        const float v = a.w_lo[i];
-        scores[i] = v;
-        vmin = fminf(vmin, v);
-        vmax = fmaxf(vmax, v);
-    }
-    if (t == 0) *count = 0;
-    __syncthreads();
-    const uint32_t floor_key = fkey(block_floor(scores, (int)len, (unsigned int)a.n, vmin, vmax, sh));
-    for (unsigned int i = t; i < len; i += kThreads) {
-        if (fkey(scores[i]) < floor_key) continue;
-        const unsigned int pos = atomicAdd(count, 1u);
-        if (pos < (unsigned int)kSortMax) sk[pos] = rank_key(scores[i], (uint32_t)a.w_id[i]);
-    }
-    __syncthreads();
-    const unsigned int m = *count;
-    if (m > (unsigned int)kSortMax) return -1;
-    constexpr int E = kSortMax / kThreads;
-    uint64_t v[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const unsigned int i = (unsigned int)(t + e * kThreads);
-        v[e] = i < m ? sk[i] : 0ull;
-    }
-    __syncthreads();
-    return emit_first<E>(a, v, sk, sh);
-}
-
-__global__ void __launch_bounds__(kThreads, 1) first_emit_kernel(const FirstEmitArgs a) {
-    extern __shared__ uint64_t sk[];   // kSortMax keys, then kFirstMax scores
-    __shared__ ThresholdShared sh;
+__global__ void __launch_bounds__(kEmitWarps * 32, 1) first_emit_kernel(const FirstEmitArgs a) {
+    extern __shared__ ulonglong2 emit_sh[];   // kFirstMax keys
+    uint64_t* sk = reinterpret_cast<uint64_t*>(emit_sh);
     __shared__ unsigned int count;
+    __shared__ unsigned int larger[32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const unsigned int len = a.ctr->w_len;
-    int emitted = -1;
-    if (len <= (unsigned int)kFirstMax) {
-        if (len <= 1024) emitted = emit_set<1>(a, len, sk, sh);
-        else if (len <= 2048) emitted = emit_set<2>(a, len, sk, sh);
-        else if (len <= (unsigned int)kSortMax) emitted = emit_set<4>(a, len, sk, sh);
-        else emitted = emit_pruned(a, len, sk, reinterpret_cast<float*>(sk + kSortMax), sh, &count);
-        __threadfence_system();   // this thread's ranks, before the words below
+    const bool fits = len <= (unsigned int)kFirstMax;
+    const uint32_t tau = (uint32_t)a.sel->prefix;
+    unsigned int m = 0;
+    if (fits) {
+        auto key_of = [&](unsigned int i) {
+            return i < len ? rank_key(a.w_lo[i], (uint32_t)a.w_id[i]) : 0ull;
+        };
+        uint64_t next = key_of(blockIdx.x * 32u + lane);   // of this block's first rows
+        if (t == 0) count = 0;
+        __syncthreads();
+        for (unsigned int i0 = warp * 32; i0 < len; i0 += kEmitWarps * 32) {
+            const uint64_t key = key_of(i0 + lane);
+            const bool take = key != 0 && (uint32_t)(key >> 32) >= tau;
+            const unsigned int bal = __ballot_sync(0xffffffffu, take);
+            unsigned int base = 0;
+            if (lane == 0 && bal) base = atomicAdd(&count, (unsigned int)__popc(bal));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (take) sk[base + __popc(bal & ((1u << lane) - 1u))] = key;
+        }
+        __syncthreads();
+        m = count;
+        if (t == 0 && (m & 1u)) sk[m] = 0ull;   // larger than no key (m < kFirstMax: it is odd)
+        for (unsigned int i0 = blockIdx.x * 32u; i0 < len; i0 += gridDim.x * 32u) {
+            const uint64_t key = next;
+            next = key_of(i0 + gridDim.x * 32u + lane);
+            const bool mine = key != 0 && (uint32_t)(key >> 32) >= tau;
+            if (t < 32) larger[t] = 0;
+            __syncthreads();
+            if (__any_sync(0xffffffffu, mine)) {   // the same in every warp
+                unsigned int above = 0;
+#pragma unroll 4
+                for (unsigned int j = warp; 2 * j < m; j += kEmitWarps) {
+                    const ulonglong2 x = emit_sh[j];
+                    above += (x.x > key) + (x.y > key);
+                }
+                atomicAdd(&larger[lane], above);
+            }
+            __syncthreads();
+            if (warp == 0 && mine && larger[lane] < (unsigned int)a.n)
+                emit_rank(a, (int)larger[lane], key);
+            __syncthreads();
+        }
     }
+    __threadfence_system();   // this thread's ranks, before the words below
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (t == 0 && atomicAdd(&a.ctr->cand, 1u) == gridDim.x - 1) {
+        __threadfence_system();   // the other blocks' ranks
         a.ctr->cand = len;
-        if (emitted >= 0) a.ctr->cand_total += len;
-        volatile unsigned int* m = a.len_mirror;
-        m[0] = emitted >= 0 ? len : 0xffffffffu;   // (nothing emitted)
-        m[1] = emitted >= 0 ? (unsigned int)emitted : 0u;
+        if (fits) a.ctr->cand_total += len;
+        volatile unsigned int* words = a.len_mirror;
+        words[0] = fits ? len : 0xffffffffu;   // (nothing emitted)
+        words[1] = fits ? min(m, (unsigned int)a.n) : 0u;
         __threadfence_system();
         *reinterpret_cast<volatile int*>(a.status_mirror) =
             *reinterpret_cast<const volatile int*>(a.status);
@@ -436,14 +349,14 @@ cudaError_t launch_first_set(const FirstSetArgs& a, int num_sms, cudaStream_t st
 
 cudaError_t launch_first_emit(const FirstSetArgs& a, int n, int64_t* out_ids, float* out_scores,
                               const int* status, unsigned int* len_mirror, int* status_mirror,
-                              cudaStream_t st) {
-    constexpr size_t smem = (size_t)kSortMax * sizeof(uint64_t) + (size_t)kFirstMax * sizeof(float);
+                              int num_sms, cudaStream_t st) {
+    constexpr size_t smem = (size_t)kFirstMax * sizeof(uint64_t);
     cudaError_t e = raise_smem_limit((const void*)first_emit_kernel, smem);
     if (e != cudaSuccess) return e;
     const FirstEmitArgs f{a.w_id, a.w_lo, a.lo, a.hi, n, a.sel, out_ids, out_scores, a.ctr, status,
                           len_mirror, status_mirror};
     count_launches(1);
-    first_emit_kernel<<<1, kThreads, smem, st>>>(f);
+    first_emit_kernel<<<num_sms, kEmitWarps * 32, smem, st>>>(f);
     return cudaGetLastError();
 }
 

@@ -135,13 +135,13 @@ struct FirstSetArgs {
 bool first_threshold_fits(int64_t len);
 // The threshold and the (unordered) working set; its length in ctr->w_len.
 cudaError_t launch_first_set(const FirstSetArgs& a, int num_sms, cudaStream_t st);
-// Sort the scored set and emit its certified ranks, n at most; nothing is
-// emitted when it holds more than kFirstMax rows (or too many exact ties to
-// sort; the length is then reported as 2^32 - 1).  The length and the ranks
+// Order the scored set and emit its certified ranks, n at most; nothing is
+// emitted when it holds more than kFirstMax rows (the length is then reported as
+// 2^32 - 1).  The length and the ranks
 // emitted (two words), then the status word, are mirrored to pinned memory.
 cudaError_t launch_first_emit(const FirstSetArgs& a, int n, int64_t* out_ids, float* out_scores,
                               const int* status, unsigned int* len_mirror, int* status_mirror,
-                              cudaStream_t st);
+                              int num_sms, cudaStream_t st);
 
 // ---- batched open support (pull_kernel.cu, batch_support.cu) ----------------
 constexpr int kWsSortMax = 16384;    // largest per-query working set of a batched open

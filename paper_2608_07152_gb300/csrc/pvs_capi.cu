@@ -2132,7 +2132,8 @@ static pvs_status first_pull(pvs_cursor* c, int64_t r, bool ahead_ok, bool* done
         e = launch_refine(nullptr, &c->ctr->w_len, c->w_id, c->w_lo, c->w_hi, c->lo, c->hi, c->qraw,
                           x->raw, x->m_raw, c->d_status, c->ctr, 2 * x->num_sms, st, kFirstMax);
     if (e == cudaSuccess)
-        e = launch_first_emit(a, (int)most, c->h_ids, c->h_scores, c->d_status, len, mirror, st);
+        e = launch_first_emit(a, (int)most, c->h_ids, c->h_scores, c->d_status, len, mirror,
+                              x->num_sms, st);
     if (e == cudaSuccess && !wait_published(mirror)) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return fail(c, cuda_status(e));
     harvest_interval_time(c);
