@@ -501,20 +501,20 @@ def main_batched(args, pvs, synth, torch, np, rank, world, local, dev, pg):
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": warm, "ms_per_step": elapsed / args.steps * 1e3,
-        "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bf16",
+        "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f16",
         "data": "synthetic",
         "config": {"workload": BATCH_WORKLOAD, "N": n, "d": DIM, "queries_per_batch": BATCH_Q,
                    "ranks_per_query": BATCH_RANKS, "chunk": BATCH_CHUNK,
                    "batches_in_flight": BATCH_PIPELINE,
-                   "l2": "no flush: each batch pass streams 1.5 GB of bf16 codes (> 129 MB L2)",
+                   "l2": "no flush: each batch streams 0.77 GB of Int8 codes twice (> 129 MB L2)",
                    "parallelism": f"replicas x{world}"},
         "e2e": {"value": e2e_value, "unit": UNIT,
                 "h2d_bytes_per_step": BATCH_Q * DIM * 4,
                 "d2h_bytes_per_step": BATCH_Q * BATCH_RANKS * (8 + 4)},
         "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": achieved / peak,
-                     "traffic": interval_traffic(n, "batch_interval_kernel_traffic.json"),
-                     "peak_kind": peak_kind, "kernel": "batch_interval_kernel (filter pass)"},
+                     "traffic": None,
+                     "peak_kind": peak_kind, "kernel": "batch_stream_kernel (a batch's filter passes)"},
         "gpu_launches": launches,
         "batch_pass_ms": batch_ms,
         "per_query": {"refined_mean": statistics.mean(s["refined"] for s in stats),
