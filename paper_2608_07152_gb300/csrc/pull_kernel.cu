@@ -278,6 +278,115 @@ static __device__ __noinline__ void emit_many(const PullArgs& a, PullShared& sh,
     emit_sorted(a, sh, n);
 }
 
+// kPullThreads to kPullSortCap candidates (the list may sit in sh.hist): a key's
+// rank is the number of keys in the bins above its own (kHistBins, linear in
+// score) and of the larger ones in its bin, two or three for scores spread
+// like real ones.  Where a bin holds more than kBinMax (ties, an outlier that
+// stretches the range) the keys are sorted.  (Sorting always: 28 us for 256 CTAs
+// of about 1,000 keys, 11 us so; 48 CTAs 24 and 10.)  Out of line, as emit_many.
+constexpr unsigned int kBinMax = 256;
+static __device__ __noinline__ void emit_binned(const PullArgs& a, PullShared& sh,
+                                                const int32_t* cand, unsigned int c) {
+    constexpr int E = kPullSortCap / kPullThreads;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    unsigned long long v[E];
+    float mn = INFINITY, mx = -INFINITY;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const unsigned int i = (unsigned int)(t + e * kPullThreads);
+        v[e] = 0ull;
+        if (i >= c) continue;
+        const int32_t w = cand[i];
+        const float s = a.w_lo[w];
+        v[e] = rank_key(s, (uint32_t)w);
+        mn = fminf(mn, s);
+        mx = fmaxf(mx, s);
+    }
+    mx = warp_max(mx);
+    mn = -warp_max(-mn);
+    float* red = reinterpret_cast<float*>(sh.sk);   // [2][kPullWarps]
+    if (lane == 0) {
+        red[warp] = mn;
+        red[kPullWarps + warp] = mx;
+    }
+    __syncthreads();   // the list is read
+    for (int i = t; i < kHistBins; i += kPullThreads) sh.hist[i] = 0;
+    mn = red[0];
+    mx = red[kPullWarps];
+    for (int w = 1; w < kPullWarps; ++w) {
+        mn = fminf(mn, red[w]);
+        mx = fmaxf(mx, red[kPullWarps + w]);
+    }
+    __syncthreads();
+    const float scale = mx > mn ? (kHistBins - 0.5f) / (mx - mn) : 0.0f;
+    int bin[E];
+    unsigned int at[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {   // larger scores in earlier bins
+        bin[e] = -1;
+        if (v[e] == 0ull) continue;
+        bin[e] = min(kHistBins - 1, max(0, (int)((mx - rank_key_score(v[e])) * scale)));
+        at[e] = atomicAdd(&sh.hist[bin[e]], 1u);
+    }
+    __syncthreads();
+    unsigned int h[kBinsPerThread], own = 0;
+    bool crowded = false;
+#pragma unroll
+    for (int b = 0; b < kBinsPerThread; ++b) {
+        h[b] = sh.hist[kBinsPerThread * t + b];
+        own += h[b];
+        crowded |= h[b] > kBinMax;
+    }
+    if (__syncthreads_or(crowded)) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const unsigned int i = (unsigned int)(t + e * kPullThreads);
+            if (i < c) sh.sk[i] = v[e];
+        }
+        emit_sorted(a, sh, (int)c);
+        return;
+    }
+    unsigned int incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned int up = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += up;
+    }
+    if (lane == 31) sh.warp_tot[warp] = incl;
+    __syncthreads();
+    unsigned int first = incl - own;
+    for (int w = 0; w < warp; ++w) first += sh.warp_tot[w];
+#pragma unroll
+    for (int b = 0; b < kBinsPerThread; ++b) {
+        sh.hist[kBinsPerThread * t + b] = first;
+        first += h[b];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (bin[e] >= 0) sh.sk[sh.hist[bin[e]] + at[e]] = v[e];
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        if (bin[e] < 0) continue;
+        const unsigned int b0 = sh.hist[bin[e]];
+        const unsigned int b1 = bin[e] + 1 < kHistBins ? sh.hist[bin[e] + 1] : c;
+        unsigned int r = b0;
+        for (unsigned int i = b0; i < b1; ++i) r += sh.sk[i] > v[e];
+        if (r >= (unsigned int)a.n) continue;
+        const uint32_t w = rank_key_id(v[e]);
+        const int32_t id = a.w_id[w];
+        a.out_ids[r] = id;
+        a.out_scores[r] = rank_key_score(v[e]);
+        a.w_lo[w] = -INFINITY;
+        a.w_hi[w] = -INFINITY;
+        if (a.lo) {
+            a.lo[id] = -INFINITY;
+            a.hi[id] = -INFINITY;
+        }
+    }
+}
+
 // Steps 4-5 (one CTA): order the candidates (all scored by now) and emit the
 // first n.
 __device__ inline void pull_emit_list(const PullArgs& a, PullShared& sh, const int32_t* cand,
@@ -320,11 +429,7 @@ __device__ inline void pull_emit_list(const PullArgs& a, PullShared& sh, const i
         }
         return;
     }
-    for (unsigned int j = t; j < c; j += kPullThreads) {
-        const int32_t w = cand[j];
-        sh.sk[j] = rank_key(a.w_lo[w], (uint32_t)w);
-    }
-    emit_sorted(a, sh, (int)c);
+    emit_binned(a, sh, cand, c);
 }
 
 // The status word as it stands after a pull, into the caller's pinned host
