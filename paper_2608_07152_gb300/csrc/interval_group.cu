@@ -26,6 +26,9 @@
 // 9 .. 16 (split) both take every tile, group 0 for queries 0 .. 7 and
 // group 1 for queries 8 .. 15, so a tile is released once all eight warps
 // have read it (query fragments in registers: m_pad up to 768).
+// A ring of an odd number of stages (three, at m_pad = 1024) is one whose
+// buffers the alternating groups share: its full barriers are those of
+// ring_turns.h, so that each group waits for every phase of the barriers it uses.
 // (Rows staged one bulk copy each, into a padded pitch free of bank
 // conflicts, made the TMA issue rate the limit: 2.4 ms per pass.  With
 // unpadded rows the fragment loads below are 2-way bank conflicted, which
@@ -52,6 +55,7 @@
 #include "kernels.h"
 #include "pipeline.cuh"
 #include "pvs_common.cuh"
+#include "ring_turns.h"
 
 namespace pvs {
 namespace {
@@ -141,14 +145,15 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
     const int pitch = m_pad;
     const int stage_bytes = group_stage_bytes(m_pad);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)stages * stage_bytes);
-    uint64_t* empty = full + stages;
+    const int bars = turn_bars(stages);                // full barriers (ring_turns.h)
+    uint64_t* empty = full + bars;
     uint2* bsm = reinterpret_cast<uint2*>(empty + stages);   // [STEPS][32] when !kRegB
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntiles = (a.rows + TR - 1) / TR;
 
     if (threadIdx.x == 0) {
+        for (int b = 0; b < bars; ++b) mbar_init(&full[b], 1);
         for (int s = 0; s < stages; ++s) {
-            mbar_init(&full[s], 1);
             // the warps that read a tile: one group, or both when split
             mbar_init(&empty[s], a.nq > kGroupHalf ? kGroupWarps : kGroupWarps / 2);
         }
@@ -175,20 +180,21 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
             const uint32_t cb = (uint32_t)rows_t * (uint32_t)m_pad;
             const uint32_t pb = (uint32_t)((rows_t + 3) & ~3) * 4u;
             uint8_t* dst = smem + (size_t)s * stage_bytes;
-            mbar_arrive_expect_tx(&full[s], cb + 3u * pb);
-            bulk_g2s(dst, a.codes + r0 * m_pad, cb, &full[s], pol);
+            uint64_t* bar = &full[turn_bar(k, stages)];
+            mbar_arrive_expect_tx(bar, cb + 3u * pb);
+            bulk_g2s(dst, a.codes + r0 * m_pad, cb, bar, pol);
             uint8_t* pd = dst + (size_t)TR * pitch;
-            bulk_g2s(pd, a.scale + r0, pb, &full[s], pol);
-            bulk_g2s(pd + TR * 4, a.vnorm + r0, pb, &full[s], pol);
-            bulk_g2s(pd + 2 * TR * 4, a.enorm + r0, pb, &full[s], pol);
+            bulk_g2s(pd, a.scale + r0, pb, bar, pol);
+            bulk_g2s(pd + TR * 4, a.vnorm + r0, pb, bar, pol);
+            bulk_g2s(pd + 2 * TR * 4, a.enorm + r0, pb, bar, pol);
         }
-        // drain: the last copy into every used stage has landed before exit
+        // drain: the last copy counted on every used barrier has landed before exit
         // (with the full wait limit, whatever a.wait_ns is)
         {
             const int issued = k;
-            for (int s = 0; s < stages && s < issued; ++s) {
-                const int last = issued - 1 - ((issued - 1 - s) % stages);
-                if (!mbar_wait(&full[s], (uint32_t)(last / stages) & 1u) && ok)
+            for (int b = 0; b < bars && b < issued; ++b) {
+                const int last = issued - 1 - ((issued - 1 - b) % bars);
+                if (!mbar_wait(&full[b], turn_parity(last, stages)) && ok)
                     for (int g = 0; g < a.nq; ++g) set_status(a.status[g], PVS_ERR_TIMEOUT);
             }
         }
@@ -237,9 +243,9 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
     int k = split ? 0 : grp;
     for (int64_t t = blockIdx.x + (split ? 0 : (int64_t)grp * gridDim.x); t < ntiles;
          t += (int64_t)kstep * gridDim.x, k += kstep) {
-        const int s = k % stages;
-        const uint32_t ph = (uint32_t)(k / stages) & 1u;
-        if (!mbar_wait(&full[s], ph, a.wait_ns)) {
+        const int bar = turn_bar(k, stages);
+        const int s = turn_buffer(bar, stages);
+        if (!mbar_wait(&full[bar], turn_parity(k, stages), a.wait_ns)) {
             if (lane == 0)
                 for (int m = 0; m < a.nq; ++m) set_status(a.status[m], PVS_ERR_TIMEOUT);
             break;
@@ -328,7 +334,8 @@ cudaError_t launch_group_tpl(const IntervalGroupArgs& a, int num_sms, cudaStream
     int stages = (kGroupSmemMax - bbytes - 256) / stage_bytes;
     if (stages > 8) stages = 8;
     if (stages < 2) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)stages * stage_bytes + 2 * stages * sizeof(uint64_t) + bbytes;
+    const size_t smem = (size_t)stages * stage_bytes +
+                        (turn_bars(stages) + stages) * sizeof(uint64_t) + bbytes;
     cudaError_t e = raise_smem_limit((const void*)interval_group_kernel<CPJ>, smem);
     if (e != cudaSuccess) return e;
     const int64_t ntiles = (a.rows + kTileRows - 1) / kTileRows;
