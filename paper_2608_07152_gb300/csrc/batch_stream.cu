@@ -18,10 +18,12 @@
 //   warps 2-9   converters: a thread owns a row (= a TMEM lane), reads its 128
 //               bytes of a box, widens them to f16 in registers (exact) and
 //               stores them as the A operand in TMEM; two groups of four warps
-//               take alternate boxes.  A box is handed over in two halves (32
-//               columns each, eight buffers): the loop converter -> issuer ->
-//               MMA -> commit -> converter crosses the pair twice and takes
-//               thousands of cycles, so many small buffers keep the MMAs fed;
+//               take alternate boxes (full barriers of ring_turns.h: the ring
+//               has seven buffers at 768 bytes and 128 queries).  A box is
+//               handed over in two halves (32 columns each, eight buffers):
+//               the loop converter -> issuer -> MMA -> commit -> converter
+//               crosses the pair twice and takes thousands of cycles, so many
+//               small buffers keep the MMAs fed;
 //   warps 10-17 epilogue: one row per thread, 32 query columns per
 //               tcgen05.ld, two queries per f32x2 instruction; two
 //               accumulators let it run under the next tile's MMAs.
@@ -47,6 +49,7 @@
 
 #include "kernels.h"
 #include "pvs_common.cuh"
+#include "ring_turns.h"
 #include "tc.cuh"
 
 namespace pvs {
@@ -67,7 +70,7 @@ constexpr int kStreamThreads = (2 + kConvWarps + kEpiWarps) * 32;
 constexpr int kSmemMax = 226 * 1024;
 
 struct StreamShared {
-    uint64_t full[kMaxStages];    // TMA -> converters
+    uint64_t full[2 * kMaxStages];   // TMA -> converters (ring_turns.h)
     uint64_t empty[kMaxStages];   // converters -> TMA
     uint64_t afull[kABufs];       // both CTAs' converters -> MMA (even CTA)
     uint64_t aempty[kABufs];      // MMA -> converters (both CTAs)
@@ -149,6 +152,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
     const uint32_t crank = cluster_ctarank();
     const bool leader = crank == 0;
     const int64_t slot0 = blockIdx.x / 2, nslots = gridDim.x / 2;
+    const int bars = turn_bars(stages);             // full barriers of the ring
     // tile slots of this pair: slot0, slot0 + nslots, ... while 2 t < niter
     const int64_t pair_tiles = (niter + 1) / 2;
     const int nmine = slot0 < pair_tiles ? (int)((pair_tiles - slot0 + nslots - 1) / nslots) : 0;
@@ -161,10 +165,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
         sh.tau[i] = on && a.tau ? a.tau[i] : INFINITY;
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < stages; ++s) {
-            mbar_init(&sh.full[s], 1);
-            mbar_init(&sh.empty[s], 4);                  // one converter group
-        }
+        for (int f = 0; f < bars; ++f) mbar_init(&sh.full[f], 1);
+        for (int s = 0; s < stages; ++s) mbar_init(&sh.empty[s], 4);   // one converter group
         for (int b = 0; b < kABufs; ++b) {
             mbar_init(&sh.afull[b], 8);                  // one group of each CTA
             mbar_init(&sh.aempty[b], 1);
@@ -200,7 +202,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
             for (int kc = 0; kc < kchunks; ++kc)
                 tc::tma_load_2d_pair(bsm + (size_t)kc * bhalf * 128, &tmB, kc * 64,
                                      (int)crank * bhalf, bb);
-            int s = 0, issued = 0;
+            int s = 0, f = 0, issued = 0;
             uint32_t ph = 1;
             bool ok = true;
             for (int it = 0; it < nmine && ok; ++it) {
@@ -212,20 +214,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
                         ok = false;
                         break;
                     }
-                    mbar_arrive_expect_tx(&sh.full[s], kBoxBytes);
+                    mbar_arrive_expect_tx(&sh.full[f], kBoxBytes);
                     tc::tma_load_2d_hint(ring + (size_t)s * kBoxBytes, &tmA, k * kBox, (int)r0,
-                                         &sh.full[s], pol);
+                                         &sh.full[f], pol);
                     ++issued;
+                    if (++f == bars) f = 0;
                     if (++s == stages) {
                         s = 0;
                         ph ^= 1u;
                     }
                 }
             }
-            // drain: the last copy into every used stage has landed before exit
-            for (int st = 0; st < stages && st < issued; ++st) {
-                const int last = issued - 1 - ((issued - 1 - st) % stages);
-                if (!mbar_wait(&sh.full[st], (uint32_t)(last / stages) & 1u)) give_up(sh, a.status);
+            // drain: the last copy counted on every used barrier has landed before exit
+            for (int b = 0; b < bars && b < issued; ++b) {
+                const int last = issued - 1 - ((issued - 1 - b) % bars);
+                if (!mbar_wait(&sh.full[b], turn_parity(last, stages))) give_up(sh, a.status);
             }
         }
     } else if (warp == 1) {
@@ -286,12 +289,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
         const int r = quarter * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
         const int total = nmine * boxes;
-        int s = grp % stages;
+        int fb = grp;                               // the box's full barrier, and its phase
         uint32_t ph = 0;
         uint32_t b = 2 * (uint32_t)grp, aph = 1;    // the box's first half buffer, and its phase
         for (int g = grp; g < total; g += 2) {
+            const int s = turn_buffer(fb, stages);
             // warp-uniform: the TMEM stores below are warp-wide
-            if (!__all_sync(0xffffffffu, !aborted(sh) && mbar_wait(&sh.full[s], ph))) {
+            if (!__all_sync(0xffffffffu, !aborted(sh) && mbar_wait(&sh.full[fb], ph))) {
                 if (lane == 0) give_up(sh, a.status);
                 break;
             }
@@ -324,9 +328,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
             }
             b ^= 4u;                                // boxes g and g + 2: the other four buffers
             if (((g >> 1) & 1) != 0) aph ^= 1u;     // both visited once
-            s += 2;
-            if (s >= stages) {
-                s -= stages;
+            fb += 2;
+            if (fb >= bars) {
+                fb -= bars;
                 ph ^= 1u;
             }
         }

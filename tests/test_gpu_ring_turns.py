@@ -43,3 +43,30 @@ def test_grouped_pass_of_three_stages_equals_lone_passes(n, m, nq):
                         pvs.pvs_cursor_close(cur)
     finally:
         pvs.pvs_index_free(index)
+
+
+@pytest.mark.parametrize("n,m,nq", [(200_003, 768, 128), (128 * 305 + 1, 1000, 96), (70_003, 704, 97)])
+def test_batched_pass_of_seven_boxes_equals_lone_cursors(n, m, nq):
+    g = torch.Generator(device="cuda").manual_seed(n + m)
+    V = torch.randn((n, m), generator=g, device="cuda")
+    Q = torch.randn((nq, m), generator=g, device="cuda")
+    index = pvs.pvs_build(V)
+    try:
+        want = []
+        for q in Q:
+            cur = pvs.pvs_cursor_open(index, q)
+            try:
+                want.append(pvs.pvs_next(cur, 64)[:2])
+            finally:
+                pvs.pvs_cursor_close(cur)
+        for _ in range(5):
+            cursors = pvs.pvs_cursor_open_batch(index, Q, 64)
+            try:
+                ids, sc, _ = pvs.pvs_next_batch(cursors, 64)
+            finally:
+                pvs.pvs_cursor_close_batch(cursors)
+            for i, (wi, ws) in enumerate(want):
+                assert np.array_equal(ids[i], wi)
+                assert np.array_equal(sc[i].view(np.uint32), ws.view(np.uint32))
+    finally:
+        pvs.pvs_index_free(index)

@@ -115,7 +115,7 @@ def test_no_wait_passes_before_its_fill(model, stages):
     assert model(stages, True) == stages % 2
 
 
-KERNELS = ["interval_group.cu"]
+KERNELS = ["interval_group.cu", "batch_stream.cu"]
 
 
 @pytest.mark.parametrize("name", KERNELS)
