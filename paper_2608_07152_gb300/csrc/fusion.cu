@@ -940,14 +940,21 @@ __global__ void __launch_bounds__(kCountWarps * 32, 4) rank_count_kernel(
             if (last) break;
             continue;
         }
-        __syncthreads();
-        const int n = q_n;
+        // Whether the queue may not hold another tile, decided once for the
+        // block: every thread reads the count before the barrier (read after it,
+        // a late warp would meet the next tile's adds, decide otherwise and miss
+        // the flush's barriers).  The count only grows within a tile, and the
+        // thread that adds last reads the total, so one of them knows.
+        const bool full = __syncthreads_or(*reinterpret_cast<volatile int*>(&q_n) >
+                                           kPlaceQueue - kCountTile);
+        // (below, the count is read where a barrier comes before the next add)
         if (!use_resid) {   // each straddling row from its fp32 row
-            place_fp32(q_rows, n);
+            place_fp32(q_rows, q_n);
             __syncthreads();
             if (threadIdx.x == 0) q_n = 0;
             __syncthreads();
-        } else if (n > kPlaceQueue - kCountTile || last) {
+        } else if (full || last) {
+            const int n = q_n;
             // kPlaceStripe rows a step: a warp's dots take four rows at a time,
             // eight lanes a row, and lane (g, t) keeps those of the step's row
             // 32 t + 4 warp + g, so that the bounds and the searches then run
