@@ -158,9 +158,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
     const int nmine = slot0 < pair_tiles ? (int)((pair_tiles - slot0 + nslots - 1) / nslots) : 0;
 
     for (int i = threadIdx.x; i < kStreamQueries; i += blockDim.x) {
-        const bool on = i < a.nq;
+        const bool on = i < a.nq && a.qs[i].status == 0;
         sh.qs[i] = on ? a.qs[i] : QueryScalars{};
-        // padding columns are never candidates
+        // padding columns, and queries the encoder refused, are never candidates
         sh.ntheta[i] = on ? (a.theta ? -a.theta[i] : INFINITY) : -INFINITY;
         sh.tau[i] = on && a.tau ? a.tau[i] : INFINITY;
     }

@@ -13,7 +13,9 @@
 // cursors in one batched pull.  A run of more requests than two groups, over a
 // corpus of some size, takes blocks of requests instead (batch_block):
 // their cursors come from one tensor-core pass (cursor_open_serving) and all
-// their pages from one deep batched pull.  No lock is held across a device
+// their pages from one deep batched pull.  Requests that the block does not serve
+// (a working set past the pass's capacity, a cursor's error) follow in groups,
+// on every worker that has no block, one group's cursors open at a time.  No lock is held across a device
 // wait; the job lock is taken only at the start and end of a run.
 #include <algorithm>
 #include <atomic>
@@ -58,6 +60,13 @@ struct pvs_executor {
     std::atomic<int32_t> next{0};       // next request index to hand out
     std::mutex run_mutex;               // one run at a time
     int32_t group = 1;                  // requests per grouped open
+    // a run in blocks: the requests that finished blocks left, served in groups
+    // by whichever worker is free
+    std::mutex left_mutex;
+    std::condition_variable left_cv;
+    std::vector<int32_t> left;
+    int32_t blocks_done = 0;
+    int32_t left_groups = 0;            // groups of them being served
     std::atomic<int64_t> requests{0}, failed{0}, pages{0}, ranks{0};
     std::atomic<int64_t> passes{0}, refined{0};
     std::mutex ms_mutex;
@@ -148,19 +157,21 @@ pvs_status serve_one(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t i,
     return s == PVS_EXHAUSTED ? PVS_EXHAUSTED : (s < 0 ? s : PVS_OK);
 }
 
-// Requests first .. first+count-1 (2 <= count <= PVS_GROUP_MAX) from one
-// grouped open; each page of every cursor in one batched pull.  A failed
+// Requests req[0 .. count) (2 <= count <= PVS_GROUP_MAX) from one
+// grouped open; `step` ranks of every cursor in one batched pull.  A failed
 // open (a bad query) serves the group's requests one by one instead; a
 // failure of the batched pull leaves the failed cursors' requests with
 // their error and the others continuing one by one.
-void serve_group(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first, int32_t count) {
-    const int32_t dim = ex->index->m;
+void serve_group(pvs_executor* ex, const Job& j, cudaStream_t st, const int32_t* req, int32_t count,
+                 int32_t step) {
+    const float* queries[PVS_GROUP_MAX];
+    for (int32_t i = 0; i < count; ++i) queries[i] = j.queries + (size_t)req[i] * ex->index->m;
     pvs_cursor* cs[PVS_GROUP_MAX] = {nullptr};
-    pvs_status s = pvs::cursor_open_group(ex->index, j.snap, j.queries + (size_t)first * dim,
-                                          count, j.on_device, st, nullptr, cs);
+    pvs_status s = pvs::cursor_open_group(ex->index, j.snap, queries, count, j.on_device, st,
+                                          nullptr, cs);
     if (s != PVS_OK) {   // e.g. one non-finite query: the others go on alone
         for (int32_t i = 0; i < count; ++i)
-            j.status[first + i] = serve_one(ex, j, st, first + i, nullptr, 0);
+            j.status[req[i]] = serve_one(ex, j, st, req[i], nullptr, 0);
         return;
     }
     int32_t got[PVS_GROUP_MAX] = {0};
@@ -171,13 +182,13 @@ void serve_group(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first,
     int32_t total = 0;
     bool batch_ok = true;
     while (total < j.ranks) {
-        const int32_t n = std::min(j.page, j.ranks - total);
+        const int32_t n = std::min(step, j.ranks - total);
         for (int32_t i = 0; i < count; ++i) {
-            id_rows[i] = j.ids + (size_t)(first + i) * j.ranks + got[i];
-            sc_rows[i] = j.scores + (size_t)(first + i) * j.ranks + got[i];
+            id_rows[i] = j.ids + (size_t)req[i] * j.ranks + got[i];
+            sc_rows[i] = j.scores + (size_t)req[i] * j.ranks + got[i];
         }
         s = pvs::next_batch_rows(cs, count, n, j.on_device, id_rows, sc_rows, n_out);
-        ++pages;
+        pages += (n + j.page - 1) / j.page;
         if (s < 0) {
             batch_ok = false;
             break;
@@ -195,7 +206,7 @@ void serve_group(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first,
         for (int32_t i = 0; i < count; ++i) states[i] = PVS_ERR_CUDA;
     count_passes(ex, cs, count, true);
     for (int32_t i = 0; i < count; ++i) {
-        const int32_t r = first + i;
+        const int32_t r = req[i];
         if (!batch_ok) {
             pvs_stats st_i;
             const bool failed = pvs_cursor_stats(cs[i], &st_i) != PVS_OK || st_i.state < 0;
@@ -230,6 +241,16 @@ void serve_group(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first,
 // batched pull stay in groups.
 constexpr int64_t kBlockRows = 65536;
 
+// Groups of left-over requests served at once, over all workers: their cursors
+// hold some 45 bytes a row each.  All of a block's at once held 100 cursors'
+// row state (4.3 GB for 100 requests over 1M near-duplicates of 128 dimensions,
+// 46 GB at 8.8M rows).  1, 2, 4 and 8 groups: 223, 159, 124 and 112 ms a run there
+// (110 with all at once), first runs 227, 165, 139 and 167; 100 requests for 250
+// ranks over 2M x 640 unit normals, half of them left over: 20.7, 17.3, 16.0 and
+// 14.3 ms (16.0), first runs 22, 22, 25 and 32 (21: a group's cursors are
+// allocated while other groups run).
+constexpr int32_t kLeftGroups = 4;
+
 int32_t batch_block(const pvs_executor* ex, const Job& j) {
     const pvs_index* x = ex->index;
     const int64_t rows = j.snap ? j.snap->data->rows : x->size;
@@ -263,29 +284,47 @@ struct BlockOut {
 };
 
 // Requests first .. first+count-1 from one batched open and one pull of all
-// their ranks.  Returns false, with nothing delivered, when any of it failed
-// (a non-finite query, an error of one cursor): the caller serves them in
-// groups, which gives each request its own status.
-bool serve_block(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first, int32_t count) {
+// their ranks.  `left` receives the requests that are still to be served (a query
+// refused, a working set past the pass's capacity, a cursor's error; all of them
+// when the open or the pull failed), each of which then gets its own status.
+void serve_block(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first, int32_t count,
+                 std::vector<int32_t>& left) {
     const pvs_index* x = ex->index;
-    std::vector<pvs_cursor*> cs((size_t)count, nullptr);
-    int64_t passes = 0;
+    left.clear();
+    std::vector<pvs_cursor*> opened((size_t)count, nullptr), cs;
+    std::vector<pvs_status> each((size_t)count, PVS_OK);
     double pass_ms = 0.0;
     if (pvs::cursor_open_serving(ex->index, j.snap, j.queries + (size_t)first * x->m, count,
-                                 j.on_device, j.ranks, st, cs.data(), &passes, &pass_ms) != PVS_OK)
-        return false;
+                                 j.on_device, j.ranks, st, opened.data(), each.data(),
+                                 &pass_ms) != PVS_OK) {
+        for (int32_t i = 0; i < count; ++i) left.push_back(first + i);
+        return;
+    }
+    std::vector<int32_t> req, refused;   // the requests of cs, and of refused queries
+    for (int32_t i = 0; i < count; ++i) {
+        if (opened[(size_t)i]) {
+            cs.push_back(opened[(size_t)i]);
+            req.push_back(first + i);
+        } else if (each[(size_t)i] != PVS_OK) {   // (on its own: not to fail a group's open)
+            refused.push_back(first + i);
+        } else {
+            left.push_back(first + i);
+        }
+    }
+    const int32_t held = (int32_t)cs.size();
     const size_t at = (size_t)first * j.ranks, total = (size_t)count * j.ranks;
     BlockOut buf;
     bool ok = j.on_device || buf.get(x, total, st) == cudaSuccess;
-    std::vector<int32_t> n_out((size_t)count, 0), states((size_t)count, 0);
+    std::vector<int32_t> n_out((size_t)held, 0);
     if (ok) {
-        std::vector<int64_t*> id_rows((size_t)count);
-        std::vector<float*> sc_rows((size_t)count);
-        for (int32_t i = 0; i < count; ++i) {
-            id_rows[(size_t)i] = (j.on_device ? j.ids + at : buf.ids) + (size_t)i * j.ranks;
-            sc_rows[(size_t)i] = (j.on_device ? j.scores + at : buf.scores) + (size_t)i * j.ranks;
+        std::vector<int64_t*> id_rows((size_t)held);
+        std::vector<float*> sc_rows((size_t)held);
+        for (int32_t i = 0; i < held; ++i) {
+            const size_t row = (size_t)(req[(size_t)i] - first) * j.ranks;
+            id_rows[(size_t)i] = (j.on_device ? j.ids + at : buf.ids) + row;
+            sc_rows[(size_t)i] = (j.on_device ? j.scores + at : buf.scores) + row;
         }
-        ok = pvs::next_batch_rows(cs.data(), count, j.ranks, 1, id_rows.data(), sc_rows.data(),
+        ok = pvs::next_batch_rows(cs.data(), held, j.ranks, 1, id_rows.data(), sc_rows.data(),
                                   n_out.data()) >= 0;
     }
     if (ok && !j.on_device)   // the block's rows are consecutive on both sides
@@ -293,31 +332,33 @@ bool serve_block(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first,
                              st) == cudaSuccess &&
              cudaMemcpyAsync(j.scores + at, buf.scores, total * sizeof(float),
                              cudaMemcpyDeviceToHost, st) == cudaSuccess;
-    std::vector<pvs_stats> stats((size_t)count);
-    if (ok) ok = pvs_cursor_stats_batch(cs.data(), count, stats.data()) == PVS_OK;   // (waits)
-    for (int32_t i = 0; ok && i < count; ++i) ok = stats[(size_t)i].state >= 0;
-    if (ok) {
-        int64_t refined = 0;
-        for (int32_t i = 0; i < count; ++i) {
-            const pvs_stats& c = stats[(size_t)i];
-            refined += c.refined;
-            // passes of the queries that the batched one left: grouped (counted
-            // by the open) or their own
-            if (cs[(size_t)i]->group_size == 1) passes += c.interval_passes;
-            pass_ms += c.interval_ms / cs[(size_t)i]->group_size;
-            const int32_t r = first + i, got = n_out[(size_t)i];
-            fill_rest(j, st, r, got);
-            j.n_out[r] = got;
-            j.status[r] = got < j.ranks ? PVS_EXHAUSTED : PVS_OK;
-            count_request(ex, PVS_OK, std::max(1, (got + j.page - 1) / j.page), got);
+    std::vector<pvs_stats> stats((size_t)held);
+    if (ok) ok = pvs_cursor_stats_batch(cs.data(), held, stats.data()) == PVS_OK;   // (waits)
+    int64_t passes = 1, refined = 0;
+    for (int32_t i = 0; i < held; ++i) {
+        const int32_t r = req[(size_t)i], got = n_out[(size_t)i];
+        if (!ok || stats[(size_t)i].state < 0) {
+            left.push_back(r);
+            continue;
         }
-        ex->passes.fetch_add(passes, std::memory_order_relaxed);
-        ex->refined.fetch_add(refined, std::memory_order_relaxed);
+        const pvs_stats& c = stats[(size_t)i];
+        refined += c.refined;
+        passes += c.interval_passes;   // (none: the working sets hold every rank)
+        pass_ms += c.interval_ms;
+        fill_rest(j, st, r, got);
+        j.n_out[r] = got;
+        j.status[r] = got < j.ranks ? PVS_EXHAUSTED : PVS_OK;
+        count_request(ex, PVS_OK, std::max(1, (got + j.page - 1) / j.page), got);
+    }
+    ex->passes.fetch_add(passes, std::memory_order_relaxed);
+    ex->refined.fetch_add(refined, std::memory_order_relaxed);
+    {
         std::lock_guard<std::mutex> lk(ex->ms_mutex);
         ex->interval_ms += pass_ms;
     }
-    pvs_cursor_close_batch(cs.data(), count);   // (waits for the stream)
-    return ok;
+    pvs_cursor_close_batch(cs.data(), held);   // (waits for the stream)
+    // after the block's copy of all its rows
+    for (int32_t r : refused) j.status[r] = serve_one(ex, j, st, r, nullptr, 0);
 }
 
 void worker_main(pvs_executor* ex, int w) {
@@ -334,19 +375,51 @@ void worker_main(pvs_executor* ex, int w) {
             j = ex->job;
         }
         const int32_t G = ex->group;
-        auto serve = [&](int32_t i, int32_t count) {
-            if (count == 1)
-                j.status[i] = serve_one(ex, j, st, i, nullptr, 0);
+        // one group's requests, `ranks` of each at a time
+        auto serve = [&](const std::vector<int32_t>& req, int32_t ranks) {
+            if (req.size() == 1)
+                j.status[req[0]] = serve_one(ex, j, st, req[0], nullptr, 0);
             else
-                serve_group(ex, j, st, i, count);
+                serve_group(ex, j, st, req.data(), (int32_t)req.size(), ranks);
         };
+        std::vector<int32_t> req;
         const int32_t step = j.block ? j.block : G;
+        const int32_t blocks = j.block ? (j.nq + j.block - 1) / j.block : 0;
         for (;;) {
             const int32_t i = ex->next.fetch_add(step, std::memory_order_relaxed);
             if (i >= j.nq) break;
             const int32_t count = std::min(step, j.nq - i);
-            if (j.block && count > G && serve_block(ex, j, st, i, count)) continue;
-            for (int32_t k = 0; k < count; k += G) serve(i + k, std::min(G, count - k));
+            if (j.block && count > G) {
+                serve_block(ex, j, st, i, count, req);
+            } else {
+                req.resize((size_t)count);
+                for (int32_t k = 0; k < count; ++k) req[(size_t)k] = i + k;
+            }
+            if (!j.block) {
+                serve(req, j.page);
+                continue;
+            }
+            std::lock_guard<std::mutex> lk(ex->left_mutex);
+            ex->left.insert(ex->left.end(), req.begin(), req.end());
+            ++ex->blocks_done;
+            ex->left_cv.notify_all();
+        }
+        while (j.block) {   // what the blocks left, a group at a time
+            std::unique_lock<std::mutex> lk(ex->left_mutex);
+            ex->left_cv.wait(lk, [&] {
+                return ex->left.empty() ? ex->blocks_done == blocks
+                                        : ex->left_groups < kLeftGroups;
+            });
+            if (ex->left.empty()) break;
+            const size_t n = std::min<size_t>((size_t)G, ex->left.size());
+            req.assign(ex->left.end() - (ptrdiff_t)n, ex->left.end());
+            ex->left.resize(ex->left.size() - n);
+            ++ex->left_groups;
+            lk.unlock();
+            serve(req, j.ranks);   // (a block's requests are at most one batched pull deep)
+            lk.lock();
+            --ex->left_groups;
+            ex->left_cv.notify_all();
         }
         std::lock_guard<std::mutex> lk(ex->m);
         if (--ex->busy == 0) ex->done_cv.notify_all();
@@ -437,6 +510,9 @@ pvs_status pvs_executor_run_ex(pvs_executor* ex, const pvs_snapshot* snap, const
                       n_out, status, 0};
         ex->job.block = batch_block(ex, ex->job);
         ex->next.store(0, std::memory_order_relaxed);
+        ex->left.clear();
+        ex->blocks_done = 0;
+        ex->left_groups = 0;
         ex->busy = (int)ex->threads.size();
         ++ex->generation;
     }

@@ -939,20 +939,25 @@ pvs_status encode_batch(pvs_index* x, const float* queries, int nq, bool on_devi
     return PVS_OK;
 }
 
+// A closed cursor to be opened again (null: none): one without row state, or,
+// with `rows`, one with it where there is one.
+pvs_cursor* pooled_cursor(pvs_index* x, bool rows) {
+    std::lock_guard<std::mutex> lock(x->pool_mutex);
+    std::vector<pvs_cursor*>& pool =
+        rows && !x->row_cursor_pool.empty() ? x->row_cursor_pool : x->cursor_pool;
+    if (pool.empty()) return nullptr;
+    pvs_cursor* c = pool.back();
+    pool.pop_back();
+    x->pool_bytes -= cursor_device_bytes(c);
+    return c;
+}
+
 // A cursor with its small buffers, fresh counters and the given snapshot.
 // With zero_state false the caller zeroes the counters and status word on the
 // device itself (the batched open does it in its query copy).
 pvs_status acquire_cursor(pvs_index* x, const std::shared_ptr<SnapData>& sd, pvs_cursor** out,
                           bool zero_state = true) {
-    pvs_cursor* c = nullptr;
-    {
-        std::lock_guard<std::mutex> lock(x->pool_mutex);
-        if (!x->cursor_pool.empty()) {
-            c = x->cursor_pool.back();
-            x->cursor_pool.pop_back();
-            x->pool_bytes -= cursor_device_bytes(c);
-        }
-    }
+    pvs_cursor* c = pooled_cursor(x, /*rows=*/false);
     if (!c) {
         c = new (std::nothrow) pvs_cursor();
         if (!c) return PVS_ERR_OOM;
@@ -989,9 +994,12 @@ pvs_status acquire_cursor(pvs_index* x, const std::shared_ptr<SnapData>& sd, pvs
 // Steps 2 and 3 read the Int8 codes up to kStreamQueries queries at a time
 // (batch_stream.cu) for rows of 128 .. kStreamMaxWidth bytes, else a bf16 copy
 // of them (batch_gemm.cu).
+// A query that the encoder refuses fails the batch; with `each` (the streaming
+// pass only, which passes over such queries) it gets its status there, and the
+// others their cursors.
 pvs_status open_batch_group(pvs_index* x, const std::shared_ptr<SnapData>& sd,
                             const float* queries, int nq, bool on_device, int horizon,
-                            cudaStream_t st, pvs_cursor** out) {
+                            cudaStream_t st, pvs_cursor** out, pvs_status* each = nullptr) {
     DevBuf buf(st, x->scratch_pool);
     BatchQueries bq;
     const int64_t rows = sd->rows;
@@ -1062,8 +1070,10 @@ pvs_status open_batch_group(pvs_index* x, const std::shared_ptr<SnapData>& sd,
         PVS_CUDA(cudaMemcpyAsync(h_qs.data(), bq.qs, nq * sizeof(QueryScalars),
                                  cudaMemcpyDeviceToHost, st));
         PVS_CUDA(cudaStreamSynchronize(st));
-        for (int i = 0; i < nq; ++i)
-            if (h_qs[i].status != 0) return (pvs_status)h_qs[i].status;
+        for (int i = 0; i < nq; ++i) {
+            if (each) each[i] = (pvs_status)h_qs[i].status;
+            else if (h_qs[i].status != 0) return (pvs_status)h_qs[i].status;
+        }
         return PVS_OK;
     }
 
@@ -1190,8 +1200,10 @@ pvs_status open_batch_group(pvs_index* x, const std::shared_ptr<SnapData>& sd,
     cudaEventElapsedTime(&pass_ms, ev0, ev1);
     cudaEventDestroy(ev0);
     cudaEventDestroy(ev1);
-    for (int i = 0; i < nq; ++i)   // a non-finite query fails the batch
-        if (h_qs[i].status != 0) return (pvs_status)h_qs[i].status;
+    for (int i = 0; i < nq; ++i) {   // a non-finite query fails the batch, or itself
+        if (each) each[i] = (pvs_status)h_qs[i].status;
+        else if (h_qs[i].status != 0) return (pvs_status)h_qs[i].status;
+    }
     if ((int)h_verdict[0] != 0) return (pvs_status)(int)h_verdict[0];
     for (int i = 0; i < nq; ++i) {
         pvs_cursor* c = out[i];
@@ -1501,11 +1513,13 @@ void pvs_index_free(pvs_index* x) {
     DeviceGuard device_guard(index_device(x));
     if (!x) return;
     if (x->stream) cudaStreamSynchronize(x->stream);
-    for (pvs_cursor* c : x->cursor_pool) {
-        cursor_free_device(c);
-        delete c;
+    for (auto* pool : {&x->cursor_pool, &x->row_cursor_pool}) {
+        for (pvs_cursor* c : *pool) {
+            cursor_free_device(c);
+            delete c;
+        }
+        pool->clear();
     }
-    x->cursor_pool.clear();
     x->pool_bytes = 0;
     dev_free(x->codes), dev_free(x->scale), dev_free(x->vnorm), dev_free(x->enorm);
     dev_free(x->raw), dev_free(x->d_status), dev_free(x->d_stage), dev_free(x->codes_bf16);
@@ -1552,15 +1566,7 @@ pvs_status pvs::cursor_open_on(pvs_index* x, const pvs_snapshot* snap, const flo
     *out = nullptr;
     if (!x || !query || (snap && snap->index != x)) return PVS_ERR_INVALID;
     if (query_on_device && !is_device_ptr(query)) return PVS_ERR_INVALID;
-    pvs_cursor* c = nullptr;
-    {
-        std::lock_guard<std::mutex> lock(x->pool_mutex);
-        if (!x->cursor_pool.empty()) {   // reuse a closed cursor's buffers
-            c = x->cursor_pool.back();
-            x->cursor_pool.pop_back();
-            x->pool_bytes -= cursor_device_bytes(c);
-        }
-    }
+    pvs_cursor* c = pooled_cursor(x, /*rows=*/true);   // reuse a closed cursor's buffers
     if (!c) {
         c = new (std::nothrow) pvs_cursor();
         if (!c) return PVS_ERR_OOM;
@@ -1703,14 +1709,14 @@ pvs_status group_pass(pvs_index* x, pvs_cursor* const* cs, int nq, cudaStream_t 
 
 }  // namespace
 
-pvs_status pvs::cursor_open_group(pvs_index* x, const pvs_snapshot* snap, const float* queries,
-                                  int32_t nq, int32_t queries_on_device, cudaStream_t pass_stream,
+pvs_status pvs::cursor_open_group(pvs_index* x, const pvs_snapshot* snap,
+                                  const float* const* queries, int32_t nq,
+                                  int32_t queries_on_device, cudaStream_t pass_stream,
                                   const cudaStream_t* cursor_streams, pvs_cursor** out) {
     DeviceGuard device_guard(index_device(x));
     if (!out || nq < 1 || nq > kGroupMax) return PVS_ERR_INVALID;
     for (int i = 0; i < nq; ++i) out[i] = nullptr;
     if (!x || !queries || (snap && snap->index != x)) return PVS_ERR_INVALID;
-    if (queries_on_device && !is_device_ptr(queries)) return PVS_ERR_INVALID;
     cudaStream_t ps = pass_stream ? pass_stream : x->stream;
     // one visible set for the whole group
     pvs_snapshot own;
@@ -1728,8 +1734,7 @@ pvs_status pvs::cursor_open_group(pvs_index* x, const pvs_snapshot* snap, const 
     };
     for (int i = 0; i < nq; ++i) {
         cudaStream_t st = cursor_streams && cursor_streams[i] ? cursor_streams[i] : ps;
-        pvs_status s = cursor_open_on(x, snap, queries + (int64_t)i * x->m, queries_on_device,
-                                      st, &cs[i]);
+        pvs_status s = cursor_open_on(x, snap, queries[i], queries_on_device, st, &cs[i]);
         if (s != PVS_OK) return bail(s);
     }
     // one query, nothing visible, or rows the grouped pass does not serve:
@@ -1756,34 +1761,26 @@ pvs_status pvs::cursor_open_group(pvs_index* x, const pvs_snapshot* snap, const 
 
 pvs_status pvs::cursor_open_serving(pvs_index* x, const pvs_snapshot* snap, const float* queries,
                                     int32_t nq, int32_t queries_on_device, int32_t horizon,
-                                    cudaStream_t stream, pvs_cursor** out, int64_t* passes,
+                                    cudaStream_t stream, pvs_cursor** out, pvs_status* each,
                                     double* pass_ms) {
     DeviceGuard device_guard(index_device(x));
-    *passes = 0;
     *pass_ms = 0.0;
     for (int32_t i = 0; i < nq; ++i) out[i] = nullptr;
     std::shared_ptr<SnapData> sd = snap ? snap->data : make_snapdata(x);
     if (!sd) return PVS_ERR_OOM;
-    pvs_status s = open_batch_group(x, sd, queries, nq, queries_on_device != 0, horizon, stream, out);
-    std::vector<pvs_cursor*> wide;   // working sets past the batched pass's capacity
-    if (s == PVS_OK) {
-        *passes = 1;
-        *pass_ms = out[0]->batch_ms;
-        for (int32_t i = 0; i < nq; ++i)
-            if (!out[i]->batch_ws && out[i]->visible > 0) wide.push_back(out[i]);
+    pvs_status s = open_batch_group(x, sd, queries, nq, queries_on_device != 0, horizon, stream, out,
+                                    each);
+    if (s == PVS_OK) *pass_ms = out[0]->batch_ms;
+    for (int32_t i = 0; i < nq; ++i) {
+        pvs_cursor* c = out[i];
+        // (a cursor with nothing visible is Exhausted and needs no working set)
+        const bool holds = c && s == PVS_OK && each[i] == PVS_OK &&
+                           (c->visible == 0 ||
+                            (c->batch_ws && c->horizon >= std::min<int64_t>(horizon, c->visible)));
+        if (holds) continue;
+        if (c) pvs_cursor_close(c);
+        out[i] = nullptr;
     }
-    const int32_t group = kGroupMax / 2;
-    for (size_t i = 0; s == PVS_OK && i + 1 < wide.size(); i += group) {
-        const int32_t n = (int32_t)std::min<size_t>(group, wide.size() - i);
-        if (n < 2 || !interval_group_supported(x->m_pad, n)) break;   // each at its first pull
-        s = group_pass(x, wide.data() + i, n, stream);
-        ++*passes;
-    }
-    if (s != PVS_OK)
-        for (int32_t i = 0; i < nq; ++i) {
-            if (out[i]) pvs_cursor_close(out[i]);
-            out[i] = nullptr;
-        }
     return s;
 }
 
@@ -1797,7 +1794,12 @@ pvs_status pvs_cursor_open(pvs_index* x, const pvs_snapshot* snap, const float* 
 pvs_status pvs_cursor_open_group(pvs_index* x, const pvs_snapshot* snap, const float* queries,
                                  int32_t nq, int32_t queries_on_device, void* pass_stream,
                                  void* const* cursor_streams, pvs_cursor** out) {
-    return pvs::cursor_open_group(x, snap, queries, nq, queries_on_device,
+    if (!out || nq < 1 || nq > PVS_GROUP_MAX) return PVS_ERR_INVALID;
+    for (int32_t i = 0; i < nq; ++i) out[i] = nullptr;
+    if (!x || !queries) return PVS_ERR_INVALID;
+    const float* rows[PVS_GROUP_MAX];
+    for (int32_t i = 0; i < nq; ++i) rows[i] = queries + (int64_t)i * x->m;
+    return pvs::cursor_open_group(x, snap, rows, nq, queries_on_device,
                                   static_cast<cudaStream_t>(pass_stream),
                                   reinterpret_cast<const cudaStream_t*>(cursor_streams), out);
 }
@@ -2507,11 +2509,11 @@ static void release_cursor(pvs_cursor* c) {
     if (x) {
         std::lock_guard<std::mutex> lock(x->pool_mutex);
         const size_t bytes = cursor_device_bytes(c);
-        if (x->cursor_pool.size() < kCursorPool &&
+        if (x->cursor_pool.size() + x->row_cursor_pool.size() < kCursorPool &&
             x->pool_bytes + bytes <= x->pool_limit) {   // keep the buffers for the next cursor
             x->pool_bytes += bytes;
             cursor_reset(c);
-            x->cursor_pool.push_back(c);
+            (c->cap_rows > 0 ? x->row_cursor_pool : x->cursor_pool).push_back(c);
             return;
         }
     }

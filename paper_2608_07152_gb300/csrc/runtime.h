@@ -45,7 +45,10 @@ struct pvs_index {
     int* d_status = nullptr;
     float* d_stage = nullptr;         // host-input staging
     size_t stage_floats = 0;
-    std::vector<pvs_cursor*> cursor_pool;   // closed cursors whose buffers are reused
+    // closed cursors whose buffers are reused: those without row state, which
+    // batched opens take, and those with it, which the others take first (mixed, a
+    // batch's hundreds of cursors would all come to hold row state in time)
+    std::vector<pvs_cursor*> cursor_pool, row_cursor_pool;
     size_t pool_bytes = 0;                  // device bytes held by pooled cursors
     size_t pool_limit = 0;                  // at most this many (a quarter of the device)
     std::mutex pool_mutex;                  // cursors may open / close on several threads
@@ -263,19 +266,22 @@ pvs_status next_batch_rows(pvs_cursor* const* cursors, int32_t nc, int32_t n,
                            int32_t outputs_on_device, int64_t* const* ids, float* const* scores,
                            int32_t* n_out);
 // Open nq <= kGroupMax cursors whose bounds come from one grouped interval
-// pass on pass_stream (null: the index's stream); cursor i's later work runs
-// on cursor_streams[i] (null array or entry: pass_stream).
-pvs_status cursor_open_group(pvs_index* x, const pvs_snapshot* snap, const float* queries,
+// pass on pass_stream (null: the index's stream); cursor i's query is
+// queries[i], its later work runs on cursor_streams[i] (null array or entry:
+// pass_stream).
+pvs_status cursor_open_group(pvs_index* x, const pvs_snapshot* snap, const float* const* queries,
                              int32_t nq, int32_t queries_on_device, cudaStream_t pass_stream,
                              const cudaStream_t* cursor_streams, pvs_cursor** out);
-// Open nq cursors for requests of about `horizon` ranks, all on `stream`: one
-// batched pass (open_batch_group); the queries whose working sets it cannot hold
-// share grouped passes instead.  On an error every cursor is closed.
-// *passes, *pass_ms: passes over the codes that were queued, and the
-// device time of the batched one.
+// Cursors for nq requests of `horizon` ranks, all on `stream`, from one batched
+// pass (open_batch_group, over the Int8 codes).  out[i] is null for a query that
+// the encoder refused (each[i] is its status) and, with each[i] PVS_OK, for one whose
+// next `horizon` ranks no working set of the pass holds: bounds of every row
+// (some 45 bytes each) would be its cursor's, so the caller serves such requests
+// apart, a few at a time.  No cursor is left open on an error of the pass.
+// *pass_ms: the pass's device time.
 pvs_status cursor_open_serving(pvs_index* x, const pvs_snapshot* snap, const float* queries,
                                int32_t nq, int32_t queries_on_device, int32_t horizon,
-                               cudaStream_t stream, pvs_cursor** out, int64_t* passes,
+                               cudaStream_t stream, pvs_cursor** out, pvs_status* each,
                                double* pass_ms);
 // Open a cursor whose device work runs on `stream` (null: the index's stream).
 pvs_status cursor_open_on(pvs_index* x, const pvs_snapshot* snap, const float* query,
