@@ -13,9 +13,9 @@
 // cursors in one batched pull.  A run of more requests than two groups, over a
 // corpus of some size, takes blocks of requests instead (batch_block):
 // their cursors come from one tensor-core pass (cursor_open_serving) and all
-// their pages from one deep batched pull.  Requests that the block does not serve
-// (a working set past the pass's capacity, a cursor's error) follow in groups,
-// on every worker that has no block, one group's cursors open at a time.  No lock is held across a device
+// their pages from one deep batched pull.  Requests that the block does not
+// serve (a working set past the pass's capacity, a cursor's error) follow in
+// groups, on whichever workers have no block.  No lock is held across a device
 // wait; the job lock is taken only at the start and end of a run.
 #include <algorithm>
 #include <atomic>
@@ -269,13 +269,8 @@ struct BlockOut {
     float* scores = nullptr;
     cudaError_t get(const pvs_index* x, size_t ranks, cudaStream_t stream) {
         st = stream;
-        void* p = nullptr;
-        cudaError_t e = cudaMallocFromPoolAsync(&p, ranks * sizeof(int64_t), x->scratch_pool, st);
-        if (e != cudaSuccess) return e;
-        ids = static_cast<int64_t*>(p);
-        e = cudaMallocFromPoolAsync(&p, ranks * sizeof(float), x->scratch_pool, st);
-        if (e == cudaSuccess) scores = static_cast<float*>(p);
-        return e;
+        const cudaError_t e = pvs::pool_alloc(&ids, ranks, x->scratch_pool, st);
+        return e == cudaSuccess ? pvs::pool_alloc(&scores, ranks, x->scratch_pool, st) : e;
     }
     ~BlockOut() {
         if (ids) cudaFreeAsync(ids, st);
@@ -328,10 +323,10 @@ void serve_block(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first,
                                   n_out.data()) >= 0;
     }
     if (ok && !j.on_device)   // the block's rows are consecutive on both sides
-        ok = cudaMemcpyAsync(j.ids + at, buf.ids, total * sizeof(int64_t), cudaMemcpyDeviceToHost,
-                             st) == cudaSuccess &&
-             cudaMemcpyAsync(j.scores + at, buf.scores, total * sizeof(float),
-                             cudaMemcpyDeviceToHost, st) == cudaSuccess;
+        ok = pvs::taken(cudaMemcpyAsync(j.ids + at, buf.ids, total * sizeof(int64_t),
+                                        cudaMemcpyDeviceToHost, st)) == cudaSuccess &&
+             pvs::taken(cudaMemcpyAsync(j.scores + at, buf.scores, total * sizeof(float),
+                                        cudaMemcpyDeviceToHost, st)) == cudaSuccess;
     std::vector<pvs_stats> stats((size_t)held);
     if (ok) ok = pvs_cursor_stats_batch(cs.data(), held, stats.data()) == PVS_OK;   // (waits)
     int64_t passes = 1, refined = 0;

@@ -398,11 +398,9 @@ pvs_status ensure_resid(pvs_index* x, cudaStream_t st, int* status) {
     std::lock_guard<std::mutex> lock(x->resid_mutex);
     if (!x->resid) {
         const size_t cap = (size_t)std::max<int64_t>(x->cap, 1);
-        if (cudaMalloc(reinterpret_cast<void**>(&x->resid), cap * (size_t)(x->m_pad >> 1)) !=
-                cudaSuccess ||
-            cudaMalloc(reinterpret_cast<void**>(&x->rparam), cap * sizeof(float4)) !=
-                cudaSuccess) {
-            const cudaError_t e = cudaGetLastError();
+        cudaError_t e = device_alloc(&x->resid, cap * (size_t)(x->m_pad >> 1));
+        if (e == cudaSuccess) e = device_alloc(&x->rparam, cap);
+        if (e != cudaSuccess) {
             cudaFree(x->resid), cudaFree(x->rparam);
             x->resid = nullptr, x->rparam = nullptr;
             return e == cudaErrorMemoryAllocation ? PVS_ERR_OOM : PVS_ERR_CUDA;
@@ -1152,12 +1150,9 @@ pvs_status fuse_complete(pvs_cursor* c, const int64_t* sparse, int64_t ns, const
     std::vector<void*> held;
     pvs_status result = PVS_OK;
     auto alloc = [&](size_t bytes, cudaStream_t s) -> void* {
-        void* p = nullptr;
-        if (cudaMallocFromPoolAsync(&p, std::max<size_t>(bytes, 16), x->scratch_pool, s) !=
-            cudaSuccess) {
-            cudaGetLastError();
+        char* p = nullptr;
+        if (pool_alloc(&p, std::max<size_t>(bytes, 16), x->scratch_pool, s) != cudaSuccess)
             return nullptr;
-        }
         held.push_back(p);
         return p;
     };
@@ -1311,15 +1306,11 @@ pvs_status stage_sparse_list(pvs_cursor* c, const int64_t* sparse, int64_t ns,
     // interval pass
     const size_t words = rows / 32 + 1;
     if (e == cudaSuccess)
-        e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&s->list),
-                                    (size_t)std::max<int64_t>(ns, 1) * 8, x->scratch_pool,
-                                    s->stream);
+        e = pool_alloc(&s->list, (size_t)std::max<int64_t>(ns, 1), x->scratch_pool, s->stream);
     if (e == cudaSuccess)
-        e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&s->seen), words * 4,
-                                    x->scratch_pool, s->stream);
+        e = pool_alloc(&s->seen, words, x->scratch_pool, s->stream);
     if (e == cudaSuccess)
-        e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&s->status), sizeof(int),
-                                    x->scratch_pool, s->stream);
+        e = pool_alloc(&s->status, 1, x->scratch_pool, s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->seen, 0, words * 4, s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->status, 0, sizeof(int), s->stream);
     if (e == cudaSuccess && ns > 0)
@@ -1395,7 +1386,8 @@ pvs_status rank_queries(pvs_cursor* c, const int32_t* dense_ids, int32_t nd, boo
              cudaStreamCreateWithFlags(&c->rq_stream, cudaStreamNonBlocking) != cudaSuccess) ||
             (!c->rq_event &&
              cudaEventCreateWithFlags(&c->rq_event, cudaEventDisableTiming) != cudaSuccess) ||
-            (!c->rq_pinned && cudaMallocHost(&c->rq_pinned, kRankQueryPinned) != cudaSuccess)) {
+            (!c->rq_pinned && pinned_alloc(reinterpret_cast<char**>(&c->rq_pinned),
+                                           kRankQueryPinned) != cudaSuccess)) {
             cudaGetLastError();
             return PVS_ERR_CUDA;
         }
@@ -1404,12 +1396,9 @@ pvs_status rank_queries(pvs_cursor* c, const int32_t* dense_ids, int32_t nd, boo
     cudaEvent_t ev = c->rq_event;
     std::vector<void*> held;
     auto alloc = [&](size_t bytes, cudaStream_t s) -> void* {
-        void* p = nullptr;
-        if (cudaMallocFromPoolAsync(&p, std::max<size_t>(bytes, 16), x->scratch_pool, s) !=
-            cudaSuccess) {
-            cudaGetLastError();
+        char* p = nullptr;
+        if (pool_alloc(&p, std::max<size_t>(bytes, 16), x->scratch_pool, s) != cudaSuccess)
             return nullptr;
-        }
         held.push_back(p);
         return p;
     };

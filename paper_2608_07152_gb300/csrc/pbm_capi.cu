@@ -41,13 +41,9 @@ namespace {
 constexpr int kDefaultBlock = 128;
 constexpr uint64_t kCollectCap = 65536;   // smallest gather buffer (keys)
 
-pvs_status cuda_status(cudaError_t e) {
-    if (e == cudaSuccess) return PVS_OK;
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        return PVS_ERR_OOM;
-    }
-    return PVS_ERR_CUDA;
+pvs_status cuda_status(cudaError_t e) {   // (the error is reported here, once)
+    if (pvs::taken(e) == cudaSuccess) return PVS_OK;
+    return e == cudaErrorMemoryAllocation ? PVS_ERR_OOM : PVS_ERR_CUDA;
 }
 
 #define PBM_CUDA(x)                                      \
@@ -55,12 +51,6 @@ pvs_status cuda_status(cudaError_t e) {
         cudaError_t _e = (x);                            \
         if (_e != cudaSuccess) return cuda_status(_e);   \
     } while (0)
-
-template <typename T>
-cudaError_t dalloc(T** p, size_t count) {
-    *p = nullptr;
-    return cudaMalloc(reinterpret_cast<void**>(p), (count ? count : 1) * sizeof(T));
-}
 
 template <typename T>
 void dfree(T*& p) {
@@ -184,11 +174,12 @@ pvs_status ensure_buffers(pbm_cursor* c, uint64_t count) {
     dfree(c->out_ids);
     dfree(c->out_scores);
     c->buf_cap = 0;
-    PBM_CUDA(dalloc(&c->buf, need));
-    PBM_CUDA(dalloc(&c->tmp, need));
-    PBM_CUDA(cudaMalloc(&c->sort_scratch, pvs::radix_sort_scratch_bytes((int64_t)need)));
-    PBM_CUDA(dalloc(&c->out_ids, need));
-    PBM_CUDA(dalloc(&c->out_scores, need));
+    PBM_CUDA(pvs::device_alloc(&c->buf, need));
+    PBM_CUDA(pvs::device_alloc(&c->tmp, need));
+    PBM_CUDA(pvs::device_alloc(reinterpret_cast<char**>(&c->sort_scratch),
+                               pvs::radix_sort_scratch_bytes((int64_t)need)));
+    PBM_CUDA(pvs::device_alloc(&c->out_ids, need));
+    PBM_CUDA(pvs::device_alloc(&c->out_scores, need));
     c->buf_cap = need;
     return PVS_OK;
 }
@@ -263,10 +254,10 @@ pvs_status pbm_build(const int64_t* term_off, int32_t n_terms, const int32_t* do
     x->nchunk = (x->n_ranges + pvs::kPbmChunk - 1) / pvs::kPbmChunk;
     cudaStream_t st = x->stream;
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    if (dalloc(&x->term_off, off.size()) != cudaSuccess ||
-        dalloc(&x->docs, (size_t)n_postings) != cudaSuccess ||
-        dalloc(&x->imps, (size_t)n_postings) != cudaSuccess ||
-        dalloc(&x->blk_off, (size_t)n_terms + 1) != cudaSuccess)
+    if (pvs::device_alloc(&x->term_off, off.size()) != cudaSuccess ||
+        pvs::device_alloc(&x->docs, (size_t)n_postings) != cudaSuccess ||
+        pvs::device_alloc(&x->imps, (size_t)n_postings) != cudaSuccess ||
+        pvs::device_alloc(&x->blk_off, (size_t)n_terms + 1) != cudaSuccess)
         return bail(PVS_ERR_OOM);
     if (cudaMemcpyAsync(x->term_off, off.data(), off.size() * sizeof(int64_t),
                         cudaMemcpyHostToDevice, st) != cudaSuccess ||
@@ -292,9 +283,9 @@ pvs_status pbm_build(const int64_t* term_off, int32_t n_terms, const int32_t* do
         free_tmp();
         return bail(s);
     };
-    if (dalloc(&flags, (size_t)n_postings) != cudaSuccess ||
-        dalloc(&scratch, pvs::pbm_scan_scratch_elems(n_postings)) != cudaSuccess ||
-        dalloc(&status, 1) != cudaSuccess || dalloc(&nb_dev, 1) != cudaSuccess)
+    if (pvs::device_alloc(&flags, (size_t)n_postings) != cudaSuccess ||
+        pvs::device_alloc(&scratch, pvs::pbm_scan_scratch_elems(n_postings)) != cudaSuccess ||
+        pvs::device_alloc(&status, 1) != cudaSuccess || pvs::device_alloc(&nb_dev, 1) != cudaSuccess)
         return bail2(PVS_ERR_OOM);
     if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess ||
         pvs::launch_pbm_mark(x->term_off, n_terms, x->docs, x->imps, n_postings, n_items, block,
@@ -310,9 +301,9 @@ pvs_status pbm_build(const int64_t* term_off, int32_t n_terms, const int32_t* do
         return bail2(PVS_ERR_CUDA);
     if (h_status != 0) return bail2((pvs_status)h_status);
     x->nb = (int64_t)h_nb;
-    if (dalloc(&x->blk_range, (size_t)x->nb) != cudaSuccess ||
-        dalloc(&x->blk_pbeg, (size_t)x->nb + 1) != cudaSuccess ||
-        dalloc(&x->blk_max, (size_t)x->nb) != cudaSuccess)
+    if (pvs::device_alloc(&x->blk_range, (size_t)x->nb) != cudaSuccess ||
+        pvs::device_alloc(&x->blk_pbeg, (size_t)x->nb + 1) != cudaSuccess ||
+        pvs::device_alloc(&x->blk_max, (size_t)x->nb) != cudaSuccess)
         return bail2(PVS_ERR_OOM);
     const int64_t p_end = n_postings;
     if (pvs::launch_pbm_write_blocks(flags, x->docs, n_postings, block, scratch, x->blk_range,
@@ -408,23 +399,21 @@ pvs_status open_cursor(pbm_index* x, const std::shared_ptr<pvs::SnapData>& snap,
         dfree(c->starts);
         c->nq_cap = 0;
         const int cap = std::max(nq, 16);
-        if (dalloc(&c->terms, (size_t)cap) != cudaSuccess ||
-            dalloc(&c->weights, (size_t)cap) != cudaSuccess ||
-            dalloc(&c->starts, (size_t)cap * (size_t)(x->nchunk + 1)) != cudaSuccess)
+        if (pvs::device_alloc(&c->terms, (size_t)cap) != cudaSuccess ||
+            pvs::device_alloc(&c->weights, (size_t)cap) != cudaSuccess ||
+            pvs::device_alloc(&c->starts, (size_t)cap * (size_t)(x->nchunk + 1)) != cudaSuccess)
             return bail(PVS_ERR_OOM);
         c->nq_cap = cap;
     }
-    if ((!c->H && dalloc(&c->H, (size_t)x->n_ranges) != cudaSuccess) ||
-        (!c->rkeys && dalloc(&c->rkeys, (size_t)x->n_ranges) != cudaSuccess) ||
-        (!c->pool && dalloc(&c->pool, (size_t)x->n_ranges * (size_t)x->block) != cudaSuccess) ||
-        (!c->ctr && dalloc(&c->ctr, 1) != cudaSuccess) ||
-        (!c->sel64 && dalloc(&c->sel64, 258) != cudaSuccess) ||
-        (!c->h_ctr && cudaMallocHost(reinterpret_cast<void**>(&c->h_ctr),
-                                     sizeof(pvs::PbmCounters)) != cudaSuccess) ||
-        (!c->h_ids && cudaMallocHost(reinterpret_cast<void**>(&c->h_ids),
-                                     pvs::kPbmFastWindow * sizeof(int64_t)) != cudaSuccess) ||
-        (!c->h_scores && cudaMallocHost(reinterpret_cast<void**>(&c->h_scores),
-                                        pvs::kPbmFastWindow * sizeof(float)) != cudaSuccess))
+    if ((!c->H && pvs::device_alloc(&c->H, (size_t)x->n_ranges) != cudaSuccess) ||
+        (!c->rkeys && pvs::device_alloc(&c->rkeys, (size_t)x->n_ranges) != cudaSuccess) ||
+        (!c->pool && pvs::device_alloc(&c->pool, (size_t)x->n_ranges * (size_t)x->block) !=
+                         cudaSuccess) ||
+        (!c->ctr && pvs::device_alloc(&c->ctr, 1) != cudaSuccess) ||
+        (!c->sel64 && pvs::device_alloc(&c->sel64, 258) != cudaSuccess) ||
+        (!c->h_ctr && pvs::pinned_alloc(&c->h_ctr, 1) != cudaSuccess) ||
+        (!c->h_ids && pvs::pinned_alloc(&c->h_ids, pvs::kPbmFastWindow) != cudaSuccess) ||
+        (!c->h_scores && pvs::pinned_alloc(&c->h_scores, pvs::kPbmFastWindow) != cudaSuccess))
         return bail(PVS_ERR_OOM);
     std::memset(c->h_ctr, 0, sizeof(pvs::PbmCounters));
     cudaStream_t st = c->stream;
@@ -488,11 +477,8 @@ pvs_status pbm_stage_ranks(pbm_cursor* c, pvs_index* owner, StagedList** out) {
     cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ready, cudaEventDisableTiming);
     if (e == cudaSuccess)
-        e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&s->scores), n * 4,
-                                    owner->scratch_pool, s->stream);
-    if (e == cudaSuccess)
-        e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&s->status), 16, owner->scratch_pool,
-                                    s->stream);
+        e = pool_alloc(&s->scores, n, owner->scratch_pool, s->stream);
+    if (e == cudaSuccess) e = pool_alloc(&s->status, 1, owner->scratch_pool, s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->status, 0, sizeof(int), s->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s->scores, 0, n * 4, s->stream);
     if (e == cudaSuccess)

@@ -48,13 +48,9 @@ constexpr size_t kStageBytes = size_t(1) << 30;   // host-input staging chunk
 
 inline int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
-pvs_status cuda_status(cudaError_t e) {
-    if (e == cudaSuccess) return PVS_OK;
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        return PVS_ERR_OOM;
-    }
-    return PVS_ERR_CUDA;
+pvs_status cuda_status(cudaError_t e) {   // (the error is reported here, once)
+    if (taken(e) == cudaSuccess) return PVS_OK;
+    return e == cudaErrorMemoryAllocation ? PVS_ERR_OOM : PVS_ERR_CUDA;
 }
 
 #define PVS_CUDA(x)                                      \
@@ -62,13 +58,6 @@ pvs_status cuda_status(cudaError_t e) {
         cudaError_t _e = (x);                            \
         if (_e != cudaSuccess) return cuda_status(_e);   \
     } while (0)
-
-template <typename T>
-cudaError_t dev_alloc(T** p, size_t count) {
-    *p = nullptr;
-    if (count == 0) count = 1;
-    return cudaMalloc(reinterpret_cast<void**>(p), count * sizeof(T));
-}
 
 template <typename T>
 void dev_free(T*& p) {
@@ -92,11 +81,11 @@ pvs_status index_reserve(pvs_index* x, int64_t need) {
     cap = round_up(std::max<int64_t>(cap, 64), 64);
     int8_t* codes = nullptr;
     float *scale = nullptr, *vnorm = nullptr, *enorm = nullptr, *raw = nullptr;
-    cudaError_t e = dev_alloc(&codes, (size_t)cap * x->m_pad);
-    if (e == cudaSuccess) e = dev_alloc(&scale, (size_t)cap);
-    if (e == cudaSuccess) e = dev_alloc(&vnorm, (size_t)cap);
-    if (e == cudaSuccess) e = dev_alloc(&enorm, (size_t)cap);
-    if (e == cudaSuccess) e = dev_alloc(&raw, (size_t)cap * x->m_raw);
+    cudaError_t e = device_alloc(&codes, (size_t)cap * x->m_pad);
+    if (e == cudaSuccess) e = device_alloc(&scale, (size_t)cap);
+    if (e == cudaSuccess) e = device_alloc(&vnorm, (size_t)cap);
+    if (e == cudaSuccess) e = device_alloc(&enorm, (size_t)cap);
+    if (e == cudaSuccess) e = device_alloc(&raw, (size_t)cap * x->m_raw);
     if (e == cudaSuccess) {
         // zero the tail so that tile copies past the last row read zeros
         e = cudaMemsetAsync(scale, 0, cap * sizeof(float), x->stream);
@@ -151,7 +140,7 @@ pvs_status index_fill(pvs_index* x, const float* vecs, int64_t n, bool on_device
         const int64_t chunk = std::min<int64_t>(rows_per_chunk, n);
         if (x->stage_floats < (size_t)(chunk * x->m)) {
             dev_free(x->d_stage);
-            PVS_CUDA(dev_alloc(&x->d_stage, (size_t)(chunk * x->m)));
+            PVS_CUDA(device_alloc(&x->d_stage, (size_t)(chunk * x->m)));
             x->stage_floats = (size_t)(chunk * x->m);
         }
         for (int64_t r = 0; r < n; r += chunk) {
@@ -173,7 +162,7 @@ pvs_status index_fill(pvs_index* x, const float* vecs, int64_t n, bool on_device
 
 // Corpus maxima of the norm bounds over rows [0, size); waits for them.
 pvs_status refresh_norm_maxes(pvs_index* x) {
-    if (!x->norm_maxes) PVS_CUDA(dev_alloc(&x->norm_maxes, 2));
+    if (!x->norm_maxes) PVS_CUDA(device_alloc(&x->norm_maxes, 2));
     PVS_CUDA(launch_norm_max(x->vnorm, x->enorm, x->size, x->norm_maxes, x->stream));
     PVS_CUDA(cudaStreamSynchronize(x->stream));
     return PVS_OK;
@@ -186,12 +175,9 @@ std::shared_ptr<SnapData> make_snapdata(const pvs_index* x) {
     if (x->tombstoned > 0) {
         const size_t words = (size_t)((x->size + 31) / 32);
         s->h_tomb.assign(x->h_tomb.begin(), x->h_tomb.begin() + words);
-        if (cudaMalloc(&s->d_tomb, words * sizeof(uint32_t)) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        if (cudaMemcpy(s->d_tomb, s->h_tomb.data(), words * sizeof(uint32_t),
-                       cudaMemcpyHostToDevice) != cudaSuccess)
+        if (device_alloc(&s->d_tomb, words) != cudaSuccess) return nullptr;
+        if (taken(cudaMemcpy(s->d_tomb, s->h_tomb.data(), words * sizeof(uint32_t),
+                             cudaMemcpyHostToDevice)) != cudaSuccess)
             return nullptr;
     }
     return s;
@@ -280,10 +266,10 @@ pvs_status cursor_alloc_full(pvs_cursor* c) {
     c->cap_rows = 0;
     c->bmax_valid = false;
     const size_t n = (size_t)std::max<int64_t>(c->rows, 1);
-    PVS_CUDA(dev_alloc(&c->lo, n));
-    PVS_CUDA(dev_alloc(&c->hi, n));
-    PVS_CUDA(dev_alloc(&c->bmax, (n + kBmaxRows - 1) / kBmaxRows));
-    PVS_CUDA(dev_alloc(&c->compact_scratch, compact_scratch_elems((int64_t)n)));
+    PVS_CUDA(device_alloc(&c->lo, n));
+    PVS_CUDA(device_alloc(&c->hi, n));
+    PVS_CUDA(device_alloc(&c->bmax, (n + kBmaxRows - 1) / kBmaxRows));
+    PVS_CUDA(device_alloc(&c->compact_scratch, compact_scratch_elems((int64_t)n)));
     c->cap_rows = (int64_t)n;
     return PVS_OK;
 }
@@ -324,8 +310,10 @@ pvs_status cursor_alloc_ws(pvs_cursor* c, int64_t cap) {
         if (base) c->sort_scratch = scratch;
         return k.used;
     };
-    PVS_CUDA(cudaMalloc(&c->ws_slab, carve(nullptr)));
-    carve(static_cast<char*>(c->ws_slab));
+    char* slab = nullptr;
+    PVS_CUDA(device_alloc(&slab, carve(nullptr)));
+    c->ws_slab = slab;
+    carve(slab);
     c->cap_w = cap;
     return PVS_OK;
 }
@@ -344,12 +332,11 @@ cudaError_t cursor_alloc_small(pvs_cursor* c, const pvs_index* x) {
         k.take(&c->d_status, 1);
         return k.used;
     };
-    const cudaError_t e = cudaMalloc(&c->small, carve(nullptr));
-    if (e != cudaSuccess) {
-        c->small = nullptr;
-        return e;
-    }
-    carve(static_cast<char*>(c->small));
+    char* slab = nullptr;
+    const cudaError_t e = device_alloc(&slab, carve(nullptr));
+    if (e != cudaSuccess) return e;
+    c->small = slab;
+    carve(slab);
     return cudaSuccess;
 }
 
@@ -357,7 +344,7 @@ cudaError_t cursor_alloc_small(pvs_cursor* c, const pvs_index* x) {
 // cursors read theirs through gather_state and mostly need none.
 cudaError_t cursor_pinned(pvs_cursor* c) {
     if (c->h_small) return cudaSuccess;
-    return cudaMallocHost(&c->h_small, 16 * sizeof(unsigned int));
+    return pinned_alloc(&c->h_small, 16);
 }
 
 pvs_status cursor_alloc_rows(pvs_cursor* c) {
@@ -373,10 +360,10 @@ pvs_status cursor_out_reserve(pvs_cursor* c, int64_t n) {
     if (c->h_scores) cudaFreeHost(c->h_scores);
     c->h_ids = nullptr, c->h_scores = nullptr, c->out_cap = 0;
     const int64_t cap = std::max<int64_t>(n, 256);
-    PVS_CUDA(dev_alloc(&c->d_ids, (size_t)cap));
-    PVS_CUDA(dev_alloc(&c->d_scores, (size_t)cap));
-    PVS_CUDA(cudaMallocHost(&c->h_ids, cap * sizeof(int64_t)));
-    PVS_CUDA(cudaMallocHost(&c->h_scores, cap * sizeof(float)));
+    PVS_CUDA(device_alloc(&c->d_ids, (size_t)cap));
+    PVS_CUDA(device_alloc(&c->d_scores, (size_t)cap));
+    PVS_CUDA(pinned_alloc(&c->h_ids, (size_t)cap));
+    PVS_CUDA(pinned_alloc(&c->h_scores, (size_t)cap));
     c->out_cap = cap;
     return PVS_OK;
 }
@@ -464,7 +451,7 @@ pvs_status interval_pass(pvs_cursor* c) {
         if (c->slot_cap < slots * kSlotTop) {
             dev_free(c->slot_top);
             c->slot_cap = 0;
-            PVS_CUDA(dev_alloc(&c->slot_top, (size_t)(slots * kSlotTop)));
+            PVS_CUDA(device_alloc(&c->slot_top, (size_t)(slots * kSlotTop)));
             c->slot_cap = slots * kSlotTop;
         }
         a.slot_top = c->slot_top;
@@ -475,8 +462,8 @@ pvs_status interval_pass(pvs_cursor* c) {
         if (c->mid_cap < c->rows) {
             dev_free(c->mid);
             c->mid_cap = 0;
-            if (dev_alloc(&c->mid, (size_t)c->rows) == cudaSuccess) c->mid_cap = c->rows;
-            else cudaGetLastError();   // the rank count then reads the codes
+            if (device_alloc(&c->mid, (size_t)c->rows) == cudaSuccess) c->mid_cap = c->rows;
+            // (refused: the rank count then reads the codes)
         }
         if (c->mid_cap >= c->rows) {
             a.mid = c->mid;
@@ -657,9 +644,10 @@ pvs_status scan_pull(pvs_cursor* c, int64_t n_eff, int64_t* d_ids, float* d_scor
             if (c->scan_scratch) cudaFree(c->scan_scratch);
             c->scan_scratch = nullptr;
             c->scan_cap = 0;
-            if (dev_alloc(&c->scan_keys, (size_t)rows) != cudaSuccess ||
-                dev_alloc(&c->scan_tmp, (size_t)rows) != cudaSuccess ||
-                cudaMalloc(&c->scan_scratch, radix_sort_scratch_bytes(rows)) != cudaSuccess)
+            if (device_alloc(&c->scan_keys, (size_t)rows) != cudaSuccess ||
+                device_alloc(&c->scan_tmp, (size_t)rows) != cudaSuccess ||
+                device_alloc(reinterpret_cast<char**>(&c->scan_scratch),
+                             radix_sort_scratch_bytes(rows)) != cudaSuccess)
                 return fail(c, PVS_ERR_OOM);
             c->scan_cap = rows;
         }
@@ -785,15 +773,10 @@ struct DevBuf {
     static size_t padded(size_t bytes) { return (std::max<size_t>(bytes, 1) + 255) / 256 * 256; }
     // One allocation for the next gets of `bytes` (their padded sizes) in all.
     bool reserve(size_t bytes) {
-        void* p = nullptr;
-        const cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, st)
-                                   : cudaMallocAsync(&p, bytes, st);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
+        char* p = nullptr;
+        if (pool_alloc(&p, bytes, pool, st) != cudaSuccess) return false;
         ptrs.push_back(p);
-        at = static_cast<char*>(p);
+        at = p;
         left = bytes;
         return true;
     }
@@ -881,7 +864,7 @@ struct BatchQueries {
 // Caller holds x->pass_mutex.
 pvs_status ensure_bf16(pvs_index* x, cudaStream_t st) {
     if (!x->codes_bf16) {
-        PVS_CUDA(dev_alloc(&x->codes_bf16, (size_t)std::max<int64_t>(x->cap, 1) * x->m_pad));
+        PVS_CUDA(device_alloc(&x->codes_bf16, (size_t)std::max<int64_t>(x->cap, 1) * x->m_pad));
         x->bf16_rows = 0;
     }
     if (!x->bf16_ready) PVS_CUDA(cudaEventCreateWithFlags(&x->bf16_ready, cudaEventDisableTiming));
@@ -1319,7 +1302,7 @@ pvs_status index_create(int32_t dim, void* cuda_stream, pvs_index** out) {
             return bail(PVS_ERR_CUDA);
         x->own_stream = true;
     }
-    if (cudaMalloc(&x->d_status, sizeof(int)) != cudaSuccess) return bail(PVS_ERR_OOM);
+    if (device_alloc(&x->d_status, 1) != cudaSuccess) return bail(PVS_ERR_OOM);
     {
         cudaMemPoolProps props{};
         props.allocType = cudaMemAllocationTypePinned;
@@ -1359,7 +1342,7 @@ pvs_status pvs_build_ex(const float* vecs, int64_t n, int32_t dim, int32_t vecs_
         // one scale for the corpus: RN(max |v_j| / 127), from the largest entry
         x->quant = PVS_QUANT_GLOBAL;
         unsigned int* mx = nullptr;
-        if (dev_alloc(&x->gscale, 1) != cudaSuccess || dev_alloc(&mx, 1) != cudaSuccess) {
+        if (device_alloc(&x->gscale, 1) != cudaSuccess || device_alloc(&mx, 1) != cudaSuccess) {
             dev_free(mx);
             return bail(PVS_ERR_OOM);
         }
@@ -1657,7 +1640,7 @@ pvs_status group_pass(pvs_index* x, pvs_cursor* const* cs, int nq, cudaStream_t 
             if (c->slot_cap < slots * kSlotTop) {
                 dev_free(c->slot_top);
                 c->slot_cap = 0;
-                PVS_CUDA(dev_alloc(&c->slot_top, (size_t)(slots * kSlotTop)));
+                PVS_CUDA(device_alloc(&c->slot_top, (size_t)(slots * kSlotTop)));
                 c->slot_cap = slots * kSlotTop;
             }
             a.slot_top[i] = c->slot_top;
@@ -2487,8 +2470,8 @@ pvs_status pvs_cursor_score_ids(pvs_cursor* c, const int64_t* ids, int32_t n, fl
     cudaStream_t st = c->stream;
     int64_t* d_ids = nullptr;
     float* d_out = nullptr;
-    cudaError_t e = dev_alloc(&d_ids, (size_t)n);
-    if (e == cudaSuccess) e = dev_alloc(&d_out, (size_t)n);
+    cudaError_t e = device_alloc(&d_ids, (size_t)n);
+    if (e == cudaSuccess) e = device_alloc(&d_out, (size_t)n);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d_ids, ids, n * sizeof(int64_t), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/pvs.h"
+#include "alloc.h"
 #include "kernels.h"
 
 namespace pvs {
