@@ -188,12 +188,13 @@ void pvs_snapshot_free(pvs_snapshot* snap);
 pvs_status pvs_cursor_open(pvs_index* index, const pvs_snapshot* snap, const float* query,
                            int32_t query_on_device, pvs_cursor** out);
 
-/* Open nq cursors (queries: nq*dim floats) whose intervals come from one
- * tensor-core pass per group of up to 256 queries (the Int8 dot products of
- * all queries as one exact bf16 GEMM, Sec. 2.3.1 intervals in its
- * epilogue).  Each cursor keeps only the rows that can hold its first
- * ranks: `horizon` (>= 1) is the number of ranks it is prepared for; it can
- * usually deliver about three times that many before it needs a
+/* Open nq cursors (queries: nq*dim floats) whose intervals come from
+ * tensor-core passes over the codes (the Int8 dot products of many queries as
+ * one exact f16 or bf16 GEMM, Sec. 2.3.1 intervals in its epilogue): one for
+ * up to 128 queries where the rows have 65 .. 1,024 dimensions (96 above 768),
+ * else one for up to 256.  Each cursor keeps only the rows that can hold its
+ * first ranks: `horizon` (>= 1) is the number of ranks it is prepared for; it
+ * can usually deliver 1.5 to 3 times that many before it needs a
  * single-query interval pass, and later ranks still come out exactly, at the
  * cost of that pass.  The work runs on `cuda_stream` (a cudaStream_t; NULL:
  * the index's stream), and so do the cursors afterwards: batched opens on

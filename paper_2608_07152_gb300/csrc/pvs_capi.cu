@@ -965,8 +965,8 @@ pvs_status acquire_cursor(pvs_index* x, const std::shared_ptr<SnapData>& sd, pvs
 //   1. encode the queries; f16 (or bf16) query codes for the MMA;
 //   2. thresholds: on every stride-th 128-row tile (every tile for small
 //      corpora) the pass leaves the lower bounds; tau_q = the k-th largest of
-//      query q there, k sized so that 1.5 to 2.5 times the horizon's rows of the
-//      whole corpus reach it;
+//      query q there, k sized so that 1.5 to 3 times the horizon's rows of the
+//      whole corpus reach it (more for a horizon of a page);
 //   3. the filter pass appends every row with hi >= tau_q to query q's
 //      working set and counts the rows with lo >= tau_q: those rows precede
 //      every row outside the working set, so the cursor can deliver that many
@@ -995,9 +995,12 @@ pvs_status open_batch_group(pvs_index* x, const std::shared_ptr<SnapData>& sd,
     // then rescan.  About stride k_s rows reach tau_q: 1.6 H at means of 62.  (At a mean of
     // 31, 2 H rows: past the end of more clusters of near neighbours, where the
     // threshold falls into the bulk of the corpus and no working set holds
-    // what reaches it.)
+    // what reaches it.)  Short horizons still sample every fourth tile: reading
+    // every row in place of a sample took nq floats a row of scratch, 4.5 GB for
+    // 128 first pages over 8.8M rows, where now 52 to 96 rows reach the threshold
+    // and the scratch is 35 MB.
     const int64_t ntiles = (rows + 127) / 128;
-    int stride = (int)std::min<int64_t>(16, std::max<int64_t>(1, (int64_t)horizon / 16));
+    int stride = (int)std::min<int64_t>(16, std::max<int64_t>(4, (int64_t)horizon / 16));
     if (ntiles < 8 * (int64_t)stride) stride = 1;
     const double mean = (double)horizon / stride;
     const unsigned int k_s =
