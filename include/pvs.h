@@ -248,7 +248,10 @@ pvs_status pvs_next_batch(pvs_cursor** cursors, int32_t nc, int32_t n, int32_t o
  * copy (device outputs).  Exact either way (Sec. 2.1: the list is a stable
  * prefix, so a rank computed early is the rank delivered later).  pages = 1
  * computes exactly what is asked.  Until this is called, the first pvs_next of
- * a cursor may compute its whole first working set: up to 2,048 ranks ahead.
+ * a cursor may compute its whole first working set: up to 2,048 ranks ahead,
+ * from up to 16,384 scored rows.  Where one of those misses its interval
+ * (App. A.1), the ranks above it are delivered and the call that would reach it
+ * fails with PVS_ERR_INTERVAL.
  * Errors: PVS_ERR_INVALID (pages < 1). */
 pvs_status pvs_cursor_set_readahead(pvs_cursor* cursor, int32_t pages);
 

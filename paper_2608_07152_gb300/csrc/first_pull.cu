@@ -7,7 +7,8 @@
 //   2. first_set_kernel        W = the live rows with hi >= v (unordered);
 //   3. refine_ring_kernel      the exact score of every row of W, on every SM;
 //   4. first_emit_kernel       W's certified rows ordered by rank key (score desc, id
-//                              asc), the first n ranks written and marked.
+//                              asc), the first n ranks written and marked (those
+//                              above the first row that missed its interval).
 // Every row outside W has hi < v, so the rows of W that score v or more, H at
 // least, are the first ranks: all of them are certified, usually many more
 // than H (intervals are wider than the spread of the best scores).  More than
@@ -270,6 +271,7 @@ __global__ void __launch_bounds__(kEmitWarps * 32, 1) first_emit_kernel(const Fi
     const unsigned int len = a.ctr->w_len;
     const bool fits = len <= (unsigned int)kFirstMax;
     const uint32_t tau = (uint32_t)a.sel->prefix;
+    const uint64_t bad = a.ctr->bad_key;   // ranks from this key on are void (0: none)
     unsigned int m = 0;
     if (fits) {
         auto key_of = [&](unsigned int i) {
@@ -280,7 +282,7 @@ __global__ void __launch_bounds__(kEmitWarps * 32, 1) first_emit_kernel(const Fi
         __syncthreads();
         for (unsigned int i0 = warp * 32; i0 < len; i0 += kEmitWarps * 32) {
             const uint64_t key = key_of(i0 + lane);
-            const bool take = key != 0 && (uint32_t)(key >> 32) >= tau;
+            const bool take = key > bad && (uint32_t)(key >> 32) >= tau;
             const unsigned int bal = __ballot_sync(0xffffffffu, take);
             unsigned int base = 0;
             if (lane == 0 && bal) base = atomicAdd(&count, (unsigned int)__popc(bal));
@@ -293,7 +295,7 @@ __global__ void __launch_bounds__(kEmitWarps * 32, 1) first_emit_kernel(const Fi
         for (unsigned int i0 = blockIdx.x * 32u; i0 < len; i0 += gridDim.x * 32u) {
             const uint64_t key = next;
             next = key_of(i0 + gridDim.x * 32u + lane);
-            const bool mine = key != 0 && (uint32_t)(key >> 32) >= tau;
+            const bool mine = key > bad && (uint32_t)(key >> 32) >= tau;
             if (t < 32) larger[t] = 0;
             __syncthreads();
             if (__any_sync(0xffffffffu, mine)) {   // the same in every warp

@@ -47,6 +47,9 @@ struct DevCounters {
     unsigned int front_bound;
     unsigned int front_k;
     unsigned int front_hint;
+    // the largest rank key (by row id) of the scored rows that missed their
+    // interval (0: none); kept by launch_refine's and launch_refine_batch's kernels
+    unsigned long long bad_key;
 };
 
 // Where one cursor keeps its device status word and counters.
@@ -135,7 +138,8 @@ struct FirstSetArgs {
 bool first_threshold_fits(int64_t len);
 // The threshold and the (unordered) working set; its length in ctr->w_len.
 cudaError_t launch_first_set(const FirstSetArgs& a, int num_sms, cudaStream_t st);
-// Order the scored set and emit its certified ranks, n at most; nothing is
+// Order the scored set and emit its certified ranks, n at most, and none from
+// the first row on that missed its interval; nothing is
 // emitted when it holds more than kFirstMax rows (the length is then reported as
 // 2^32 - 1).  The length and the ranks
 // emitted (two words), then the status word, are mirrored to pinned memory.

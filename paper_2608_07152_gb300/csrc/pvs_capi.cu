@@ -222,6 +222,7 @@ void cursor_reset(pvs_cursor* c) {
     c->scanned = false;
     c->bmax_valid = false;
     c->want_mid = c->mid_valid = false;
+    c->pending = PVS_OK;
     c->batch_ws = false;
     c->fresh_ws = false;
     c->horizon = c->horizon_base = 0;
@@ -610,6 +611,7 @@ pvs_status rescan_from_batch(pvs_cursor* c) {
 
 // Make the cursor's working set hold the next n_eff ranks.
 pvs_status prepare_pull(pvs_cursor* c, int64_t n_eff) {
+    if (c->pending != PVS_OK) return (pvs_status)c->pending;
     pvs_status s;
     if (!c->scanned && !c->batch_ws) {
         s = cursor_alloc_rows(c);
@@ -2072,7 +2074,10 @@ static pvs_status next_common(pvs_cursor* c, int32_t n, int32_t* n_out, int64_t*
 
 // The first pull of a cursor through first_pull.cu: the first working set
 // scored and sorted whole, its certified ranks into the pinned buffers and
-// ahead (r at least, 2,048 at most; exactly r unless ahead_ok).  *done stays
+// ahead (r at least, 2,048 at most; exactly r unless ahead_ok).  The set is scored
+// far past the page asked for: where a row below it misses its interval (an
+// imported one: App. A.1), the ranks above that row come out (ahead_ok) and the
+// next pull fails.  *done stays
 // false, with the bounds as they were, when the pull does not qualify (without
 // ahead_ok: r is not all that such a pull delivers), the threshold's values do
 // not fit one CTA, or the set turned out larger than kFirstMax.
@@ -2126,11 +2131,18 @@ static pvs_status first_pull(pvs_cursor* c, int64_t r, bool ahead_ok, bool* done
     if (e != cudaSuccess) return fail(c, cuda_status(e));
     harvest_interval_time(c);
     const int dev_status = *reinterpret_cast<volatile int*>(mirror);
-    if (dev_status != 0) return fail(c, (pvs_status)dev_status);
     const int64_t set = reinterpret_cast<volatile unsigned int*>(len)[0];
     const int64_t got = reinterpret_cast<volatile unsigned int*>(len)[1];
-    if (set > kFirstMax) return PVS_OK;
-    if (got < H) return fail(c, PVS_ERR_INVALID);   // internal invariant
+    if (dev_status != 0) {
+        if (dev_status != PVS_ERR_INTERVAL || !ahead_ok || got == 0)
+            return fail(c, (pvs_status)dev_status);
+        c->pending = dev_status;
+        e = cudaMemsetAsync(c->d_status, 0, sizeof(int), st);
+        if (e != cudaSuccess) return fail(c, cuda_status(e));
+    } else {
+        if (set > kFirstMax) return PVS_OK;
+        if (got < H) return fail(c, PVS_ERR_INVALID);   // internal invariant
+    }
     c->slot_fresh = false;
     c->horizon = got;   // the set is used up
     c->horizon_base = 0;

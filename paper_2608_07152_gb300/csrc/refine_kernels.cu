@@ -9,6 +9,18 @@
 
 namespace pvs {
 
+// A row's score failed: the cursor's status, and the largest key whose ranks
+// (and all below) are void: the row's own where it missed its interval, any
+// where there is no score.
+__device__ inline void note_violation(int* status, DevCounters* ctr, float s, int32_t id) {
+    set_status(status, PVS_ERR_INTERVAL);
+    atomicMax(&ctr->bad_key, rank_key(s, (uint32_t)id));
+}
+__device__ inline void note_failure(int* status, DevCounters* ctr, int code) {
+    set_status(status, code);
+    atomicMax(&ctr->bad_key, ~0ull);
+}
+
 // Warps warp0, warp0 + nwarps, ... of the launch score candidates of one
 // cursor.  lo / hi (bounds of every row) may be null for a cursor that only
 // holds a working set.  A warp fetches the metadata of its next 32
@@ -48,8 +60,8 @@ __device__ inline void refine_warps(const int32_t* __restrict__ cand, const unsi
             if (lane == 0) {
                 ++refined;
                 fallbacks += fb;
-                if (!isfinite(s)) set_status(status, PVS_ERR_OVERFLOW);
-                else if (s < lj || s > hj) set_status(status, PVS_ERR_INTERVAL);
+                if (!isfinite(s)) note_failure(status, ctr, PVS_ERR_OVERFLOW);
+                else if (s < lj || s > hj) note_violation(status, ctr, s, idj);
                 w_lo[wj] = s;
                 w_hi[wj] = s;
                 if (lo) {
@@ -221,8 +233,8 @@ __device__ inline void refine_ring(const RingRefs& a, int stages, int64_t warp0,
         if (lane == 0) {
             ++refined;
             fallbacks += fb;
-            if (!isfinite(s)) set_status(a.status, PVS_ERR_OVERFLOW);
-            else if (s < lj || s > hj) set_status(a.status, PVS_ERR_INTERVAL);
+            if (!isfinite(s)) note_failure(a.status, a.ctr, PVS_ERR_OVERFLOW);
+            else if (s < lj || s > hj) note_violation(a.status, a.ctr, s, md.w);
             a.w_lo[md.x] = s;
             a.w_hi[md.x] = s;
             if (a.lo) {
@@ -234,7 +246,7 @@ __device__ inline void refine_ring(const RingRefs& a, int stages, int64_t warp0,
         if (issue(st)) ++issued;
     }
     if (k < issued) {   // a copy did not arrive in time: record it, drain every copy in flight
-        if (lane == 0) set_status(a.status, PVS_ERR_TIMEOUT);
+        if (lane == 0) note_failure(a.status, a.ctr, PVS_ERR_TIMEOUT);
         for (int k2 = k; k2 < issued; ++k2)
             mbar_wait(&bars[k2 % stages], (uint32_t)((k2 / stages) & 1));
     }

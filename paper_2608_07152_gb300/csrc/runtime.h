@@ -119,6 +119,9 @@ struct pvs_cursor {
     // its arrays and the pull scratch are parts of ws_slab
     int64_t cap_w = 0;                // capacity of the working-set arrays
     void* ws_slab = nullptr;
+    // a pull scored a row that missed its interval below the ranks it computed:
+    // the status of the next pull (the list fails there)
+    int pending = PVS_OK;
     bool batch_ws = false;            // working set came from a batched pass (no full bounds)
     bool fresh_ws = false;            // no pull since the working set was built (many candidates)
     int32_t* w_id = nullptr;
