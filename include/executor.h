@@ -21,11 +21,14 @@
  *
  * A run of more than 2 G requests (G >= 2), of at most 1,024 ranks each, over a
  * corpus of at least 65,536 vectors of 65 .. 1,024 dimensions is served in
- * blocks of up to 128 requests (96 above 768 dimensions): one tensor-core pass over the codes
- * (as pvs_cursor_open_batch) opens a block's cursors, one pull computes all
- * their ranks, and a request's pages are handed over together.  The ranks
- * delivered are the same.  A block in which anything fails is served again
- * in groups, so that each request gets its own status.
+ * blocks of up to 128 requests (96 above 768 dimensions): one tensor-core pass
+ * over the codes (as pvs_cursor_open_batch) opens a block's cursors, one pull
+ * computes all their ranks, and a request's pages are handed over together.
+ * The ranks delivered are the same.  A request whose working set the pass cannot
+ * hold, or whose cursor fails, is served again in a group of G, at most four
+ * such groups at a time (their cursors hold some 45 bytes for every vector);
+ * so are all of a block whose pass or pull failed.  Each request gets its own
+ * status.
  *
  * Conventions as pvs.h: the caller owns every buffer; the index must
  * outlive the executor and must not be changed (append, delete) while a run
@@ -97,8 +100,8 @@ pvs_status pvs_executor_run_ex(pvs_executor* ex, const pvs_snapshot* snap, const
 /*
  * Serve requests in groups of `group` (1 .. PVS_GROUP_MAX; default 1): the
  * queries of a group share one pass over the codes (from 2 on, a run of more
- * requests than two groups may be served in larger blocks, see above).  Must not be called
- * during a run.  Errors: PVS_ERR_INVALID.
+ * requests than two groups may be served in larger blocks, see above).  Must
+ * not be called during a run.  Errors: PVS_ERR_INVALID.
  */
 pvs_status pvs_executor_set_group(pvs_executor* ex, int32_t group);
 

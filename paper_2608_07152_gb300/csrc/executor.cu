@@ -161,7 +161,8 @@ pvs_status serve_one(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t i,
 // grouped open; `step` ranks of every cursor in one batched pull.  A failed
 // open (a bad query) serves the group's requests one by one instead; a
 // failure of the batched pull leaves the failed cursors' requests with
-// their error and the others continuing one by one.
+// their error and the others continuing one by one.  A request whose pull of more
+// than a page failed is read again page by page: the ranks before its error stand.
 void serve_group(pvs_executor* ex, const Job& j, cudaStream_t st, const int32_t* req, int32_t count,
                  int32_t step) {
     const float* queries[PVS_GROUP_MAX];
@@ -201,6 +202,7 @@ void serve_group(pvs_executor* ex, const Job& j, cudaStream_t st, const int32_t*
         total += n;
         if (!more) break;
     }
+    const bool again = step > j.page;
     int states[PVS_GROUP_MAX] = {0};
     if (batch_ok && pvs_cursor_sync_batch(cs, count, states) != PVS_OK)
         for (int32_t i = 0; i < count; ++i) states[i] = PVS_ERR_CUDA;
@@ -210,7 +212,10 @@ void serve_group(pvs_executor* ex, const Job& j, cudaStream_t st, const int32_t*
         if (!batch_ok) {
             pvs_stats st_i;
             const bool failed = pvs_cursor_stats(cs[i], &st_i) != PVS_OK || st_i.state < 0;
-            if (failed) {
+            if (failed && again) {
+                pvs_cursor_close(cs[i]);
+                j.status[r] = serve_one(ex, j, st, r, nullptr, 0);
+            } else if (failed) {
                 fill_rest(j, st, r, got[i]);
                 j.n_out[r] = got[i];
                 j.status[r] = st_i.state < 0 ? (pvs_status)st_i.state : s;
@@ -219,6 +224,11 @@ void serve_group(pvs_executor* ex, const Job& j, cudaStream_t st, const int32_t*
             } else {   // continue this request on its own
                 j.status[r] = serve_one(ex, j, st, r, cs[i], got[i]);
             }
+            continue;
+        }
+        if (states[i] < 0 && again) {
+            pvs_cursor_close(cs[i]);
+            j.status[r] = serve_one(ex, j, st, r, nullptr, 0);
             continue;
         }
         fill_rest(j, st, r, got[i]);

@@ -146,3 +146,48 @@ def test_a_cursors_error_fails_its_request_alone():
         assert st["interval_passes"] <= 1 + max(1, -(-len(hit) // 8))
     finally:
         pvs.pvs_index_free(index)
+
+
+@pytest.mark.parametrize("on_device", [False, True])
+@pytest.mark.parametrize("wide", [False, True])
+def test_a_failed_request_keeps_the_ranks_before_its_error(wide, on_device):
+    # request 6 meets a row that misses its interval about 200 ranks down; in a
+    # block of its own cursors, and among wide working sets served in groups
+    n, dim, rank, ranks = 70_003, 128, 200, 400
+    g = torch.Generator().manual_seed(21)
+    if wide:
+        base = torch.randn(dim, generator=g)
+        V = (base + 0.02 * torch.randn((n, dim), generator=g)).numpy()
+        Q = (base + torch.randn((20, dim), generator=g)).numpy()
+    else:
+        V = synth.unit_normal(n, dim, seed=22).numpy()
+        Q = synth.unit_normal(20, dim, seed=23).numpy()
+    built = pvs.pvs_build(V)
+    try:
+        codes, scale, vnorm, enorm = pvs.pvs_index_export(built, 0, n)
+        refs = [_lone(built, q, ranks)[0] for q in Q]
+    finally:
+        pvs.pvs_index_free(built)
+    scale[refs[6][rank]] *= np.float32(1.3)
+    index = pvs.pvs_index_import(V, codes, scale, vnorm, enorm)
+    try:
+        Qt = torch.from_numpy(Q)
+        ids, sc, n_out, status, rc, st = _serve(index, Qt.cuda() if on_device else Qt, ranks, 20,
+                                                on_device)
+        assert status[6] == pvs.PVS_ERR_INTERVAL
+        for i in range(20):
+            # a lone cursor's pages on this index (queued device pages are void
+            # from the last wait on)
+            cur, got = pvs.pvs_cursor_open(index, Q[i]), 0
+            try:
+                while got < ranks:
+                    got += pvs.pvs_next(cur, 20)[0].size
+            except pvs.PvsError as e:
+                assert e.status == status[i] == pvs.PVS_ERR_INTERVAL
+            finally:
+                pvs.pvs_cursor_close(cur)
+            if not on_device or status[i] == pvs.PVS_OK:
+                assert n_out[i] == got and np.array_equal(ids[i, :got], refs[i][:got])
+        assert wide or on_device or n_out[6] == rank
+    finally:
+        pvs.pvs_index_free(index)
