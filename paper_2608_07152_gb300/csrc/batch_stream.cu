@@ -133,6 +133,9 @@ __device__ __forceinline__ float max3_of(float m, uint64_t v) {
 
 // Every CTA of a pair runs the same number of tile slots; a slot past the last
 // tile loads boxes out of range (zero fill) and writes nothing.
+// kBounds: both bounds of every row (a.dump_hi), for diagnostics; apart, since the
+// branch in the serving kernel cost its filter up to 5% (1M x 384 118 -> 124 us).
+template <bool kBounds>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
     batch_stream_kernel(const __grid_constant__ CUtensorMap tmA,
                         const __grid_constant__ CUtensorMap tmB,
@@ -443,6 +446,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
                     }
                     continue;
                 }
+                if constexpr (kBounds) {
+                    const int64_t at = i * kRows + r_in_tile;
+#pragma unroll 1
+                    for (int k = cc * 32; k < a.nq && k < cc * 32 + 32; ++k) {
+                        const uint32_t v = tc::ld_32x32b_x1(tcol + (uint32_t)k);
+                        tc::wait_ld();
+                        float lo, hi;
+                        interval_epilogue(__float2int_rn(__uint_as_float(v)), sh.qs[k], sv, vn, en,
+                                          lo, hi);
+                        if (live && !(isfinite(lo) && isfinite(hi)))
+                            set_status(a.status, PVS_ERR_OVERFLOW);
+                        a.dump_lo[(int64_t)k * a.dump_ld + at] = live ? lo : -INFINITY;
+                        a.dump_hi[(int64_t)k * a.dump_ld + at] = live ? hi : -INFINITY;
+                    }
+                    continue;
+                }
                 if (a.mode == 0) {
                     const int64_t srow = i * kRows + r_in_tile;
                     bool bad = false;
@@ -637,7 +656,7 @@ int stream_pairs(int num_sms) {
     std::lock_guard<std::mutex> lock(mu);
     if (!known[dev]) {
         int n = 0;
-        if (raise_smem_limit((const void*)batch_stream_kernel, kSmemMax) == cudaSuccess) {
+        if (raise_smem_limit((const void*)batch_stream_kernel<false>, kSmemMax) == cudaSuccess) {
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeClusterDimension;
             attr[0].val.clusterDim.x = 2;
@@ -646,7 +665,7 @@ int stream_pairs(int num_sms) {
             cudaLaunchConfig_t cfg = stream_config(2 * num_sms, kSmemMax, nullptr);
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&n, batch_stream_kernel, &cfg) != cudaSuccess) {
+            if (cudaOccupancyMaxActiveClusters(&n, batch_stream_kernel<false>, &cfg) != cudaSuccess) {
                 cudaGetLastError();
                 n = 0;
             }
@@ -700,9 +719,14 @@ cudaError_t launch_batch_stream(const StreamArgs& a, const int8_t* codes, const 
     const int pairs = stream_pairs(num_sms);
     const int grid = 2 * (int)(slots < pairs ? slots : pairs);
     const size_t smem = fixed_smem(a.m_pad, a.nq_pad) + (size_t)stages * kBoxBytes;
-    count_launches(1);
-    batch_stream_kernel<<<grid, kStreamThreads, smem, st>>>(ta, tb, a, stages);
-    return cudaGetLastError();
+    auto run = [&](auto kernel) {
+        const cudaError_t e = raise_smem_limit((const void*)kernel, kSmemMax);
+        if (e != cudaSuccess) return e;
+        count_launches(1);
+        kernel<<<grid, kStreamThreads, smem, st>>>(ta, tb, a, stages);
+        return cudaGetLastError();
+    };
+    return a.dump_hi ? run(batch_stream_kernel<true>) : run(batch_stream_kernel<false>);
 }
 
 // f16 copy of int8 codes (exact: |z| <= 127); rows past n become zeros.

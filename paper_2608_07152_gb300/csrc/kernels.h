@@ -408,6 +408,7 @@ struct StreamArgs {
     int group_max;                // sample: 1: the largest of each 32 rows, 0: every row
     float* dump_lo;               // sample: [nq][dump_ld]; entry 4 i + g: rows 32 g .. of
     int64_t dump_ld;              //   tile i s, or entry 128 i + r: row r of tile i s
+    float* dump_hi;               // sample, every row: the upper bounds too (or null)
     const float* tau;             // filter: [nq] thresholds
     const float* theta;           // filter: [nq] from launch_stream_theta
     int32_t* w_id;                // filter: as BatchArgs

@@ -1831,8 +1831,9 @@ pvs_status pvs_batch_bounds(pvs_index* x, const pvs_snapshot* snap, const float*
     cudaStream_t st = x->stream;
     DevBuf buf(st, x->scratch_pool);
     BatchQueries bq;
+    const bool stream = batch_stream_supported(x->m_pad, x->num_sms);   // as open_batch_group
     pvs_status s = encode_batch(x, queries, nq, queries_on_device, buf, &bq, st,
-                                /*check_now=*/true, /*f16=*/false);
+                                /*check_now=*/true, stream);
     if (s != PVS_OK) return s;
     const int64_t ntiles = (rows + 127) / 128;
     const int64_t ld = ntiles * 128;
@@ -1841,23 +1842,35 @@ pvs_status pvs_batch_bounds(pvs_index* x, const pvs_snapshot* snap, const float*
     int* status = buf.get<int>(1);
     if (!dlo || !dhi || !status) return PVS_ERR_OOM;
     PVS_CUDA(cudaMemsetAsync(status, 0, sizeof(int), st));
-    BatchArgs a{};
-    a.rows = rows;
-    a.m_pad = x->m_pad;
-    a.nq = nq;
-    a.nq_pad = bq.nq_pad;
-    a.scale = x->scale;
-    a.vnorm = x->vnorm;
-    a.enorm = x->enorm;
-    a.tomb = sd->d_tomb;
-    a.qs = bq.qs;
-    a.mode = 0;
-    a.tile_stride = 1;
-    a.dump_lo = dlo;
-    a.dump_hi = dhi;
-    a.dump_ld = ld;
-    a.status = status;
-    PVS_CUDA(launch_batch_intervals(a, x->codes_bf16, bq.qcodes, x->num_sms, st));
+    // both bounds of every row, from the kernel that serves rows of this width
+    auto dump = [&](auto a, int q0, int n) {
+        a.rows = rows;
+        a.m_pad = x->m_pad;
+        a.nq = n;
+        a.nq_pad = (int)round_up(n, 32);
+        a.scale = x->scale;
+        a.vnorm = x->vnorm;
+        a.enorm = x->enorm;
+        a.tomb = sd->d_tomb;
+        a.qs = bq.qs + q0;
+        a.mode = 0;
+        a.tile_stride = 1;
+        a.dump_lo = dlo + (size_t)q0 * ld;
+        a.dump_hi = dhi + (size_t)q0 * ld;
+        a.dump_ld = ld;
+        a.status = status;
+        return a;
+    };
+    if (stream) {
+        const int per_pass = batch_stream_queries(x->m_pad);
+        for (int q0 = 0; q0 < nq; q0 += per_pass)
+            PVS_CUDA(launch_batch_stream(dump(StreamArgs{}, q0, std::min(per_pass, nq - q0)),
+                                         x->codes, bq.qcodes + (size_t)q0 * x->m_pad, x->num_sms,
+                                         st));
+    } else {
+        PVS_CUDA(launch_batch_intervals(dump(BatchArgs{}, 0, nq), x->codes_bf16, bq.qcodes,
+                                        x->num_sms, st));
+    }
     int h_status = 0;
     PVS_CUDA(cudaMemcpyAsync(&h_status, status, sizeof(int), cudaMemcpyDeviceToHost, st));
     PVS_CUDA(cudaMemcpy2DAsync(lo, rows * sizeof(float), dlo, ld * sizeof(float),

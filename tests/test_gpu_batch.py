@@ -1,8 +1,8 @@
 """Batched (tensor-core) PVS path against the oracle, through the C ABI.
 
 * pvs_batch_bounds: the exact Int8 dot products of up to 256 queries come
-  from one bf16 tcgen05 GEMM (codes |z| <= 127, sums < 2^24: exact in fp32);
-  its epilogue must reproduce the oracle's intervals bit for bit
+  from tcgen05 GEMMs in f16 or bf16 (codes |z| <= 127, sums < 2^24: exact in
+  fp32); the epilogues must reproduce the oracle's intervals bit for bit
   (Sec. 2.3.1, App. A.1).
 * pvs_cursor_open_batch + pvs_next_batch / pvs_next: every cursor's ranks
   equal the oracle's complete ranking, including past the batch horizon
