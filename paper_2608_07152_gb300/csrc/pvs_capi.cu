@@ -356,6 +356,8 @@ pvs_status cursor_alloc_rows(pvs_cursor* c) {
 
 pvs_status cursor_out_reserve(pvs_cursor* c, int64_t n) {
     if (n <= c->out_cap) return PVS_OK;
+    // copies that pvs_next_device queued may still read the old buffers
+    if (c->out_cap > 0) PVS_CUDA(cudaStreamSynchronize(c->stream));
     dev_free(c->d_ids), dev_free(c->d_scores);
     if (c->h_ids) cudaFreeHost(c->h_ids);
     if (c->h_scores) cudaFreeHost(c->h_scores);
