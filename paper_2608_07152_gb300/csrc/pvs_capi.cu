@@ -677,14 +677,18 @@ pvs_status pull(pvs_cursor* c, int64_t n_eff, int64_t* d_ids, float* d_scores,
     cudaStream_t st = c->stream;
     pvs_status s = prepare_pull(c, n_eff);
     if (s != PVS_OK) return fail(c, s);
+    // bounds of every row, kept in step, where the cursor has them: a batched open's
+    // cursor may hold buffers that another snapshot's rows once filled
+    float* const lo = c->scanned ? c->lo : nullptr;
+    float* const hi = c->scanned ? c->hi : nullptr;
     if (n_eff <= kPullFusedMax) {
         // one launch, no host round trip; failures surface at the next sync
         PullArgs a;
         a.w_id = c->w_id;
         a.w_lo = c->w_lo;
         a.w_hi = c->w_hi;
-        a.lo = c->lo;
-        a.hi = c->hi;
+        a.lo = lo;
+        a.hi = hi;
         a.qraw = c->qraw;
         a.raw = x->raw;
         a.m_raw = x->m_raw;
@@ -717,7 +721,7 @@ pvs_status pull(pvs_cursor* c, int64_t n_eff, int64_t* d_ids, float* d_scores,
         e = launch_candidates(c->w_lo, c->w_hi, &c->ctr->w_len, c->sel, c->cand, &c->ctr->cand,
                               grid_w, st);
     if (e == cudaSuccess)
-        e = launch_refine(c->cand, &c->ctr->cand, c->w_id, c->w_lo, c->w_hi, c->lo, c->hi, c->qraw,
+        e = launch_refine(c->cand, &c->ctr->cand, c->w_id, c->w_lo, c->w_hi, lo, hi, c->qraw,
                           x->raw, x->m_raw, c->d_status, c->ctr, 2 * x->num_sms, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->h_small + 1, &c->ctr->cand, sizeof(unsigned int),
@@ -747,12 +751,12 @@ pvs_status pull(pvs_cursor* c, int64_t n_eff, int64_t* d_ids, float* d_scores,
     if (cand < n_eff || top < n_eff) return fail(c, PVS_ERR_INVALID);   // internal invariants
     c->candidates += cand;
     if (top <= kCountEmitMax) {
-        e = launch_count_emit(c->keys, (int)top, (int)n_eff, c->w_id, c->w_lo, c->w_hi, c->lo,
-                              c->hi, d_ids, d_scores, st);
+        e = launch_count_emit(c->keys, (int)top, (int)n_eff, c->w_id, c->w_lo, c->w_hi, lo, hi,
+                              d_ids, d_scores, st);
     } else {
         e = launch_radix_sort_desc(c->keys, c->keys_tmp, top, c->sort_scratch, st);
         if (e == cudaSuccess)
-            e = launch_emit(c->keys, (int)n_eff, c->w_id, c->w_lo, c->w_hi, c->lo, c->hi, d_ids,
+            e = launch_emit(c->keys, (int)n_eff, c->w_id, c->w_lo, c->w_hi, lo, hi, d_ids,
                             d_scores, st);
     }
     if (e != cudaSuccess) return fail(c, cuda_status(e));
