@@ -3,9 +3,8 @@
 // the PVS cursors of Sec. 2.3.
 //
 // A fixed pool of worker threads, each bound to the index's device with its
-// own non-blocking stream.  A run publishes one job and bumps a generation
-// counter; the workers take request indexes from an atomic counter.  For a
-// request a worker opens the cursor on its own stream, reads the pages one
+// own non-blocking stream.  A run publishes one job; the workers take request
+// indexes from it.  For a request a worker opens the cursor on its own stream, reads the pages one
 // after another through pvs_next straight into the request's rows of the
 // caller's buffers, and closes the cursor.  With a group size G >= 2 a
 // worker takes G requests at a time: one grouped open (one pass over the
@@ -51,22 +50,18 @@ struct pvs_executor {
     pvs_index* index = nullptr;
     std::vector<std::thread> threads;
     std::vector<cudaStream_t> streams;
-    std::mutex m;                       // job, generation, busy, stop
+    std::mutex m;                       // guards what follows, up to stop
     std::condition_variable work_cv, done_cv;
     Job job;
-    uint64_t generation = 0;
-    int busy = 0;                       // workers not yet done with the job
-    bool stop = false;
-    std::atomic<int32_t> next{0};       // next request index to hand out
-    std::mutex run_mutex;               // one run at a time
-    int32_t group = 1;                  // requests per grouped open
+    int32_t next = 0;                   // next request index to hand out
+    int32_t open = 0;                   // requests of the job not yet served
     // a run in blocks: the requests that finished blocks left, served in groups
     // by whichever worker is free
-    std::mutex left_mutex;
-    std::condition_variable left_cv;
     std::vector<int32_t> left;
-    int32_t blocks_done = 0;
     int32_t left_groups = 0;            // groups of them being served
+    bool stop = false;
+    std::mutex run_mutex;               // one run at a time
+    int32_t group = 1;                  // requests per grouped open
     std::atomic<int64_t> requests{0}, failed{0}, pages{0}, ranks{0};
     std::atomic<int64_t> passes{0}, refined{0};
     std::mutex ms_mutex;
@@ -366,68 +361,54 @@ void serve_block(pvs_executor* ex, const Job& j, cudaStream_t st, int32_t first,
     for (int32_t r : refused) j.status[r] = serve_one(ex, j, st, r, nullptr, 0);
 }
 
+// A worker takes the job's next block or group, or a group of what finished
+// blocks left, and serves it.  The run is over with its last request, whether or
+// not the workers that found nothing to do have woken up (waiting for them took
+// 20 us of a run of one block).
 void worker_main(pvs_executor* ex, int w) {
     cudaSetDevice(ex->index->device);
     const cudaStream_t st = ex->streams[(size_t)w];
-    uint64_t seen = 0;
+    std::vector<int32_t> req;   // the requests taken
+    std::unique_lock<std::mutex> lk(ex->m);
     for (;;) {
-        Job j;
-        {
-            std::unique_lock<std::mutex> lk(ex->m);
-            ex->work_cv.wait(lk, [&] { return ex->stop || ex->generation != seen; });
-            if (ex->stop) return;
-            seen = ex->generation;
-            j = ex->job;
-        }
+        const auto left_ready = [&] { return !ex->left.empty() && ex->left_groups < kLeftGroups; };
+        ex->work_cv.wait(lk, [&] { return ex->stop || ex->next < ex->job.nq || left_ready(); });
+        if (ex->stop) return;
+        const Job j = ex->job;
         const int32_t G = ex->group;
-        // one group's requests, `ranks` of each at a time
-        auto serve = [&](const std::vector<int32_t>& req, int32_t ranks) {
-            if (req.size() == 1)
+        const bool left = ex->next >= j.nq;
+        const int32_t first = ex->next;
+        int32_t count;
+        if (left) {
+            count = (int32_t)std::min<size_t>((size_t)G, ex->left.size());
+            req.assign(ex->left.end() - count, ex->left.end());
+            ex->left.resize(ex->left.size() - (size_t)count);
+            ++ex->left_groups;
+        } else {
+            count = std::min(j.block ? j.block : G, j.nq - first);
+            ex->next += count;
+            req.resize((size_t)count);
+            for (int32_t k = 0; k < count; ++k) req[(size_t)k] = first + k;
+        }
+        lk.unlock();
+        if (!left && j.block && count > G) {
+            serve_block(ex, j, st, first, count, req);   // req: what it leaves
+        } else {
+            // (a block's requests are at most one batched pull deep)
+            if (count == 1)
                 j.status[req[0]] = serve_one(ex, j, st, req[0], nullptr, 0);
             else
-                serve_group(ex, j, st, req.data(), (int32_t)req.size(), ranks);
-        };
-        std::vector<int32_t> req;
-        const int32_t step = j.block ? j.block : G;
-        const int32_t blocks = j.block ? (j.nq + j.block - 1) / j.block : 0;
-        for (;;) {
-            const int32_t i = ex->next.fetch_add(step, std::memory_order_relaxed);
-            if (i >= j.nq) break;
-            const int32_t count = std::min(step, j.nq - i);
-            if (j.block && count > G) {
-                serve_block(ex, j, st, i, count, req);
-            } else {
-                req.resize((size_t)count);
-                for (int32_t k = 0; k < count; ++k) req[(size_t)k] = i + k;
-            }
-            if (!j.block) {
-                serve(req, j.page);
-                continue;
-            }
-            std::lock_guard<std::mutex> lk(ex->left_mutex);
+                serve_group(ex, j, st, req.data(), count, left ? j.ranks : j.page);
+            req.clear();
+        }
+        lk.lock();
+        if (left) --ex->left_groups;
+        ex->open -= count - (int32_t)req.size();
+        if (!req.empty()) {
             ex->left.insert(ex->left.end(), req.begin(), req.end());
-            ++ex->blocks_done;
-            ex->left_cv.notify_all();
+            ex->work_cv.notify_all();
         }
-        while (j.block) {   // what the blocks left, a group at a time
-            std::unique_lock<std::mutex> lk(ex->left_mutex);
-            ex->left_cv.wait(lk, [&] {
-                return ex->left.empty() ? ex->blocks_done == blocks
-                                        : ex->left_groups < kLeftGroups;
-            });
-            if (ex->left.empty()) break;
-            const size_t n = std::min<size_t>((size_t)G, ex->left.size());
-            req.assign(ex->left.end() - (ptrdiff_t)n, ex->left.end());
-            ex->left.resize(ex->left.size() - n);
-            ++ex->left_groups;
-            lk.unlock();
-            serve(req, j.ranks);   // (a block's requests are at most one batched pull deep)
-            lk.lock();
-            --ex->left_groups;
-            ex->left_cv.notify_all();
-        }
-        std::lock_guard<std::mutex> lk(ex->m);
-        if (--ex->busy == 0) ex->done_cv.notify_all();
+        if (ex->open == 0) ex->done_cv.notify_all();
     }
 }
 
@@ -514,17 +495,13 @@ pvs_status pvs_executor_run_ex(pvs_executor* ex, const pvs_snapshot* snap, const
         ex->job = Job{snap, queries, nq, ranks, page, buffers_on_device ? 1 : 0, ids, scores,
                       n_out, status, 0};
         ex->job.block = batch_block(ex, ex->job);
-        ex->next.store(0, std::memory_order_relaxed);
-        ex->left.clear();
-        ex->blocks_done = 0;
-        ex->left_groups = 0;
-        ex->busy = (int)ex->threads.size();
-        ++ex->generation;
+        ex->next = 0;
+        ex->open = nq;
     }
     ex->work_cv.notify_all();
     {
         std::unique_lock<std::mutex> lk(ex->m);
-        ex->done_cv.wait(lk, [&] { return ex->busy == 0; });
+        ex->done_cv.wait(lk, [&] { return ex->open == 0; });
     }
     for (int32_t i = 0; i < nq; ++i)
         if (status[i] < 0) return (pvs_status)status[i];

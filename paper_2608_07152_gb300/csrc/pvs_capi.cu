@@ -930,12 +930,11 @@ pvs_status encode_batch(pvs_index* x, const float* queries, int nq, bool on_devi
     return PVS_OK;
 }
 
-// A closed cursor to be opened again (null: none): one without row state, or,
-// with `rows`, one with it where there is one.
+// A closed cursor to be opened again (null: none), of a batched open or, with
+// `rows`, of the others.
 pvs_cursor* pooled_cursor(pvs_index* x, bool rows) {
     std::lock_guard<std::mutex> lock(x->pool_mutex);
-    std::vector<pvs_cursor*>& pool =
-        rows && !x->row_cursor_pool.empty() ? x->row_cursor_pool : x->cursor_pool;
+    std::vector<pvs_cursor*>& pool = rows ? x->row_cursor_pool : x->cursor_pool;
     if (pool.empty()) return nullptr;
     pvs_cursor* c = pool.back();
     pool.pop_back();
@@ -2530,7 +2529,8 @@ static void release_cursor(pvs_cursor* c) {
             x->pool_bytes + bytes <= x->pool_limit) {   // keep the buffers for the next cursor
             x->pool_bytes += bytes;
             cursor_reset(c);
-            (c->cap_rows > 0 ? x->row_cursor_pool : x->cursor_pool).push_back(c);
+            const bool batched = c->w_id && c->cap_rows == 0;   // a working set, no bounds
+            (batched ? x->cursor_pool : x->row_cursor_pool).push_back(c);
             return;
         }
     }

@@ -46,9 +46,10 @@ struct pvs_index {
     int* d_status = nullptr;
     float* d_stage = nullptr;         // host-input staging
     size_t stage_floats = 0;
-    // closed cursors whose buffers are reused: those without row state, which
-    // batched opens take, and those with it, which the others take first (mixed, a
-    // batch's hundreds of cursors would all come to hold row state in time)
+    // closed cursors whose buffers are reused, those of batched opens (a working set,
+    // no bounds of every row) apart from the others: mixed, a batch's hundreds of
+    // cursors would all come to hold row state in time, and a lone open would free a
+    // batch's working set for its own (cudaFree waits for the whole device)
     std::vector<pvs_cursor*> cursor_pool, row_cursor_pool;
     size_t pool_bytes = 0;                  // device bytes held by pooled cursors
     size_t pool_limit = 0;                  // at most this many (a quarter of the device)
