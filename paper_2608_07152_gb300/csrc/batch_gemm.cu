@@ -39,12 +39,13 @@
 //           bound reaches tau_q are counted (they fix the horizon).  A cheap
 //           upper bound c + rmax_q < tau_q rejects most pairs before the full
 //           interval is computed.
-#include <cuda.h>
 #include <mutex>
 
+#include "f32x2.cuh"
 #include "kernels.h"
 #include "pvs_common.cuh"
 #include "tc.cuh"
+#include "tensor_map.h"
 
 namespace pvs {
 
@@ -103,27 +104,6 @@ __device__ __forceinline__ void interval_of(float fdot, const QueryScalars& q, f
     const float r = __fadd_ru(E, G);
     lo = __fsub_rd(c, r);
     hi = __fadd_ru(c, r);
-}
-
-// Two fp32 lanes per instruction (f32x2), each lane rounded as its scalar
-// counterpart.
-__device__ __forceinline__ uint64_t pack2(float x, float y) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& x, float& y) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-}
-__device__ __forceinline__ uint64_t mul2_rn(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t add2_ru(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rp.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
 }
 
 // kCta = 2: the two CTAs of each cluster form a pair (cluster rank 0 is the
@@ -369,22 +349,22 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
                     uint32_t r[32];
                     tc::ld_32x32b_x32(tcol + (uint32_t)(cc * 32), r);
                     tc::wait_ld();
-                    const uint64_t sv2 = pack2(sv, sv);
+                    const uint64_t sv2 = f2_pack(sv, sv);
 #pragma unroll
                     for (int k = 0; k < 32; k += 4) {
                         const int q = cc * 32 + k;
                         const float4 s4 = *reinterpret_cast<const float4*>(&sh.fs[q]);
                         const float4 m4 = *reinterpret_cast<const float4*>(&sh.frm[q]);
                         const float4 t4 = *reinterpret_cast<const float4*>(&sh.ftau[q]);
-                        const uint64_t c01 = mul2_rn(mul2_rn(pack2(s4.x, s4.y), sv2),
-                                                     pack2(__uint_as_float(r[k]),
+                        const uint64_t c01 = f2_mul(f2_mul(f2_pack(s4.x, s4.y), sv2),
+                                                     f2_pack(__uint_as_float(r[k]),
                                                            __uint_as_float(r[k + 1])));
-                        const uint64_t c23 = mul2_rn(mul2_rn(pack2(s4.z, s4.w), sv2),
-                                                     pack2(__uint_as_float(r[k + 2]),
+                        const uint64_t c23 = f2_mul(f2_mul(f2_pack(s4.z, s4.w), sv2),
+                                                     f2_pack(__uint_as_float(r[k + 2]),
                                                            __uint_as_float(r[k + 3])));
                         float u0, u1, u2, u3;
-                        unpack2(add2_ru(c01, pack2(m4.x, m4.y)), u0, u1);
-                        unpack2(add2_ru(c23, pack2(m4.z, m4.w)), u2, u3);
+                        f2_unpack(f2_add_ru(c01, f2_pack(m4.x, m4.y)), u0, u1);
+                        f2_unpack(f2_add_ru(c23, f2_pack(m4.z, m4.w)), u2, u3);
                         cand |= ((uint32_t)!(u0 < t4.x) << k) | ((uint32_t)!(u1 < t4.y) << (k + 1)) |
                                 ((uint32_t)!(u2 < t4.z) << (k + 2)) |
                                 ((uint32_t)!(u3 < t4.w) << (k + 3));
@@ -471,45 +451,41 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
 }
 
 // ---- host side ---------------------------------------------------------------
-void* tensor_map_encoder() {
+bool tensor_map_2d(CUtensorMap* m, CUtensorMapDataType type, int elem, const void* base,
+                   uint64_t rows, uint64_t cols, uint32_t box_cols, uint32_t box_rows) {
+    typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
+                                      const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                      const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                      CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
     static std::once_flag once;
-    static void* fn = nullptr;
+    static EncodeTiledFn fn = nullptr;
     std::call_once(once, [] {
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000,
                                              cudaEnableDefault, &q) == cudaSuccess &&
             q == cudaDriverEntryPointSuccess)
-            fn = p;
+            fn = reinterpret_cast<EncodeTiledFn>(p);
         else
             cudaGetLastError();
     });
-    return fn;
-}
-
-namespace {
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() { return reinterpret_cast<EncodeTiledFn>(tensor_map_encoder()); }
-
-// bf16 matrix [rows][cols] (row stride cols), box = [64 cols x box_rows], 128B swizzle.
-bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
-    EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {cols, rows};
-    const cuuint64_t strides[1] = {cols * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kBK, box_rows};
+    const cuuint64_t strides[1] = {cols * (uint64_t)elem};
+    const cuuint32_t box[2] = {box_cols, box_rows};
     const cuuint32_t estr[2] = {1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
-              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+    return fn(m, type, 2, const_cast<void*>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
            CUDA_SUCCESS;
 }
 
+namespace {
+
+// bf16 matrix [rows][cols] (row stride cols), box = [64 cols x box_rows], 128B swizzle.
+bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+    return tensor_map_2d(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, rows, cols, kBK, box_rows);
+}
 
 cudaLaunchConfig_t pair_config(int grid, cudaStream_t st, cudaLaunchAttribute* attr) {
     cudaLaunchConfig_t cfg{};

@@ -44,13 +44,14 @@
 //           warp's buffer; 32 records at a time, one per lane, get their interval and
 //           their place (reserving places chunk by chunk waited out an atomic's
 //           round trip for each).
-#include <cuda.h>
 #include <mutex>
 
+#include "f32x2.cuh"
 #include "kernels.h"
 #include "pvs_common.cuh"
 #include "ring_turns.h"
 #include "tc.cuh"
+#include "tensor_map.h"
 
 namespace pvs {
 namespace {
@@ -95,39 +96,17 @@ __device__ __forceinline__ void give_up(StreamShared& sh, int* status) {
     *reinterpret_cast<volatile int*>(&sh.abort) = 1;
 }
 
-// Four signed Int8 codes -> two f16x2, exact: with the sign bit flipped the
-// byte is the code + 128; under the f16 exponent byte 0x64 it reads 1024 +
-// code + 128, and subtracting 1152 leaves the code.
-__device__ __forceinline__ void widen4(uint32_t w, uint32_t& lo, uint32_t& hi) {
-    const uint32_t x = w ^ 0x80808080u;
-    const uint32_t l = __byte_perm(x, 0x64646464u, 0x4140);
-    const uint32_t h = __byte_perm(x, 0x64646464u, 0x4342);
-    const uint32_t bias = 0x64806480u;   // (1152, 1152) in f16
-    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(lo) : "r"(l), "r"(bias));
-    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(hi) : "r"(h), "r"(bias));
-}
-
 // The 16 codes of a 16-byte piece -> 8 registers, in order.
 __device__ __forceinline__ void widen16(const uint4& v, uint32_t* f) {
-    widen4(v.x, f[0], f[1]);
-    widen4(v.y, f[2], f[3]);
-    widen4(v.z, f[4], f[5]);
-    widen4(v.w, f[6], f[7]);
+    codes_to_f16x2(v.x, f[0], f[1]);
+    codes_to_f16x2(v.y, f[2], f[3]);
+    codes_to_f16x2(v.z, f[4], f[5]);
+    codes_to_f16x2(v.w, f[6], f[7]);
 }
 
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t pack2(float x, float y) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
 __device__ __forceinline__ float max3_of(float m, uint64_t v) {
     float x, y;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+    f2_unpack(v, x, y);
     return fmaxf(fmaxf(m, x), y);
 }
 
@@ -413,7 +392,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
                     // 18 bits, the last lane's), whose own lower bound the 32
                     // rows leave; then a query in every lane.  (Every row's
                     // bound made the epilogue's instructions the sample's
-                    // time: 553k x 768 x 64 queries 190 us, 113 so.)
+                    // time: 553k x 768 x 128 queries 190 us, 113 so.)
                     int m[32];
 #pragma unroll
                     for (int k = 0; k < 32; ++k) {   // (branch-free: the 32 chains overlap)
@@ -483,7 +462,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
                 }
                 // any pair of the chunk that may reach its threshold?  One
                 // maximum per eight queries
-                const uint64_t sv2 = pack2(sv, sv);
+                const uint64_t sv2 = f2_pack(sv, sv);
                 float mx[4];
 #pragma unroll
                 for (int o = 0; o < 4; ++o) {
@@ -491,11 +470,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kStreamThreads, 1)
 #pragma unroll
                     for (int k = 8 * o; k < 8 * o + 8; k += 4) {
                         const float4 nt = *reinterpret_cast<const float4*>(&sh.ntheta[cc * 32 + k]);
-                        m = max3_of(m, fma2(pack2(__uint_as_float(d[k]), __uint_as_float(d[k + 1])),
-                                            sv2, pack2(nt.x, nt.y)));
-                        m = max3_of(m, fma2(pack2(__uint_as_float(d[k + 2]),
+                        m = max3_of(m, f2_fma(f2_pack(__uint_as_float(d[k]), __uint_as_float(d[k + 1])),
+                                            sv2, f2_pack(nt.x, nt.y)));
+                        m = max3_of(m, f2_fma(f2_pack(__uint_as_float(d[k + 2]),
                                                   __uint_as_float(d[k + 3])),
-                                            sv2, pack2(nt.z, nt.w)));
+                                            sv2, f2_pack(nt.z, nt.w)));
                     }
                     mx[o] = live ? m : -INFINITY;   // (the maximum passes over a NaN: none here,
                 }                                   //  dot and s_v are finite)
@@ -604,26 +583,6 @@ __global__ void stream_theta_kernel(const QueryScalars* qs, int nq, const unsign
     theta[q] = th == th ? th : -INFINITY;   // (a NaN rejects nothing)
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// Row-major matrix of `elem`-byte elements, boxes of box_cols x box_rows, 128-byte swizzle.
-bool make_map2d(CUtensorMap* m, CUtensorMapDataType type, int elem, const void* base, uint64_t rows,
-                uint64_t cols, uint32_t box_cols, uint32_t box_rows) {
-    EncodeTiledFn fn = reinterpret_cast<EncodeTiledFn>(tensor_map_encoder());
-    if (!fn) return false;
-    const cuuint64_t dims[2] = {cols, rows};
-    const cuuint64_t strides[1] = {cols * (uint64_t)elem};
-    const cuuint32_t box[2] = {box_cols, box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return fn(m, type, 2, const_cast<void*>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
-           CUDA_SUCCESS;
-}
-
 size_t fixed_smem(int m_pad, int nq_pad) {
     return 1024 + (size_t)(m_pad / 64) * (nq_pad / 2) * 128 + sizeof(StreamShared);
 }
@@ -708,9 +667,9 @@ cudaError_t launch_batch_stream(const StreamArgs& a, const int8_t* codes, const 
     const int stages = stream_stages(a.m_pad, a.nq_pad);
     if (stages < 2) return cudaErrorInvalidValue;
     CUtensorMap ta, tb;
-    if (!make_map2d(&ta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, codes, (uint64_t)a.rows,
+    if (!tensor_map_2d(&ta, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, codes, (uint64_t)a.rows,
                     (uint64_t)a.m_pad, kBox, kRows) ||
-        !make_map2d(&tb, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, qcodes, (uint64_t)a.nq_pad,
+        !tensor_map_2d(&tb, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, qcodes, (uint64_t)a.nq_pad,
                     (uint64_t)a.m_pad, 64, (uint32_t)(a.nq_pad / 2)))
         return cudaErrorInvalidValue;
     const int64_t ntiles = (a.rows + kRows - 1) / kRows;

@@ -427,8 +427,6 @@ cudaError_t launch_stream_theta(const QueryScalars* qs, int nq, const unsigned i
 // dst[0 .. count) = the codes as f16, dst[count .. padded) = 0.
 cudaError_t launch_codes_to_f16(const int8_t* src, uint16_t* dst, int64_t count, int64_t padded,
                                 cudaStream_t st);
-// The driver's cuTensorMapEncodeTiled (null if unavailable).
-void* tensor_map_encoder();
 // status_out[i] = *refs[i].status; ctr_out[i] = *refs[i].ctr (ctr_out may be null).
 cudaError_t launch_gather_state(const CursorRef* refs, int n, int* status_out,
                                 DevCounters* ctr_out, cudaStream_t st);

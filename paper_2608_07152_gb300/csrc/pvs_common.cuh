@@ -91,6 +91,19 @@ __device__ __forceinline__ int fine_digit(float e, float inv) {
     return (int)fminf(fmaxf(rintf(__fmul_rn(e, inv)), -127.0f), 127.0f);
 }
 
+// Four signed Int8 codes -> two f16x2 (bytes 0,1 and bytes 2,3), exact:
+// x = w ^ 0x80808080 holds the codes + 128 as unsigned bytes u; the byte
+// u placed under the f16 exponent byte 0x64 reads as 1024 + u, and
+// subtracting 1152 leaves u - 128, the code.
+__device__ __forceinline__ void codes_to_f16x2(uint32_t w, uint32_t& lo, uint32_t& hi) {
+    const uint32_t x = w ^ 0x80808080u;
+    const uint32_t l = __byte_perm(x, 0x64646464u, 0x4140);
+    const uint32_t h = __byte_perm(x, 0x64646464u, 0x4342);
+    const uint32_t bias = 0x64806480u;   // (1152, 1152) in f16
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(lo) : "r"(l), "r"(bias));
+    asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(hi) : "r"(h), "r"(bias));
+}
+
 __device__ __forceinline__ bool tombstoned(const uint32_t* tomb, int64_t row) {
     return tomb != nullptr && ((__ldg(tomb + (row >> 5)) >> (row & 31)) & 1u);
 }
