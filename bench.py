@@ -9,18 +9,19 @@ in chunks of 20 (open, 50 pulls, close).  The corpus codes (6.9 GB per
 interval pass) are far larger than the 129 MB L2, so no L2 flush is needed.
 
 Both legs run through the library's native request executor
-(pvs_executor_run_ex): WORKERS native threads, each serving GROUP queries
-at a time from one grouped interval pass over the codes
-(pvs_cursor_open_group) and pulling every 20-rank page of the group's
-cursors in one batched launch; every query still gets its own pages.
+(pvs_executor_run_ex): native threads, each serving a block of up to 128
+queries at a time from one streaming pass over the codes and computing the
+block's ranks in one batched pull; every query still gets its own pages.
+(Runs of at most two groups are served by grouped passes.)
 `value` (exact dense ranks/s) has the queries resident in HBM and the ranks
 written to device buffers, timed with CUDA events; `e2e` is the same
-through host buffers (pinned queries in, every page on the host before the
-next is requested), the copies inside the timed region.
-`roofline` reports the grouped interval pass (the dominant kernel):
-algorithmic bytes N * (m_pad + 12) read plus 8 * N * GROUP bytes of bounds
-written per pass, over its CUDA-event duration (the library's events on the
-pass's stream), against the measured HBM copy bandwidth.
+through host buffers (pinned queries in, pages out), the copies inside the
+timed region.
+`roofline` reports the pass over the codes that the executor used: for
+blocks N * (m_pad + 4) algorithmic bytes read, for grouped passes
+N * (m_pad + 12) plus 8 bytes of bounds for every vector and query, over its
+CUDA-event duration (the library's events on the pass's stream), against
+the measured HBM copy bandwidth.
 
 `--impl reference` times the oracle (a plain CPU implementation, run as it
 stands) on a bounded sample of the same workload.  Under torchrun every rank
@@ -1412,8 +1413,8 @@ def eahr_record(args, pvs, synth, torch, np, index, centres, n, rank, dev):
 
 def main_passage(args, pvs, synth, torch, np, rank, world, local, dev, pg):
     """The passage workload (the default): the queries of a step served by
-    the native executor, GROUP at a time from one grouped pass over the
-    codes, every 20-rank page of a group's cursors in one batched pull."""
+    the native executor in blocks that share a streaming pass over the codes
+    (two groups of requests or fewer: in groups that share a grouped pass)."""
     stream = torch.cuda.Stream(device=dev)
     n = args.n
     group = max(1, min(args.group, pvs.PVS_GROUP_MAX))
@@ -1494,7 +1495,8 @@ def main_passage(args, pvs, synth, torch, np, rank, world, local, dev, pg):
     pass_ms = (st1["interval_ms"] - st0["interval_ms"]) / max(passes, 1)
     per_pass = n_timed / max(passes, 1)
     blocks = per_pass > group   # blocks on the tensor cores: working sets only, no bounds
-    read_bytes = n * (m_pad + 12)
+    # (a block reads the norm bounds of the rows that it keeps only)
+    read_bytes = n * (m_pad + (4 if blocks else 12))
     # bounds (lo, hi) of every row per query, and with groups the largest
     # upper bound of each 16-row block per query
     write_bytes = 0 if blocks else (
@@ -1504,7 +1506,7 @@ def main_passage(args, pvs, synth, torch, np, rank, world, local, dev, pg):
     peak, peak_kind = measured_peaks()
     kernel = ("batch_stream_kernel" if blocks else
               "interval_group_kernel" if group > 1 else "interval_pass_kernel")
-    traffic = (None if blocks else
+    traffic = (interval_traffic(n, "batch_stream_kernel_traffic.json") if blocks else
                interval_traffic(n, "interval_group_kernel_passage_traffic.json") if group > 1
                else interval_traffic(n))
 
