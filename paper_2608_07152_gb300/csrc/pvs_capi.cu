@@ -243,7 +243,8 @@ void cursor_reset(pvs_cursor* c) {
     c->scan_ready = false;
 }
 
-// Closed cursors kept per index for reuse: at most kCursorPool of them and
+// Closed cursors kept per index for reuse: at most kCursorPool of each kind (1,024
+// of a batched open's would leave no place for a lone one) and
 // a quarter of the device's memory (at least kCursorPoolBytes) in device
 // buffers.  Batched opens reuse hundreds of small cursors; single-query
 // cursors hold buffers for every row (~460 MB at 8.8M rows), and grouped
@@ -2525,12 +2526,13 @@ static void release_cursor(pvs_cursor* c) {
     if (x) {
         std::lock_guard<std::mutex> lock(x->pool_mutex);
         const size_t bytes = cursor_device_bytes(c);
-        if (x->cursor_pool.size() + x->row_cursor_pool.size() < kCursorPool &&
+        const bool batched = c->w_id && c->cap_rows == 0;   // a working set, no bounds
+        std::vector<pvs_cursor*>& pool = batched ? x->cursor_pool : x->row_cursor_pool;
+        if (pool.size() < kCursorPool &&
             x->pool_bytes + bytes <= x->pool_limit) {   // keep the buffers for the next cursor
             x->pool_bytes += bytes;
             cursor_reset(c);
-            const bool batched = c->w_id && c->cap_rows == 0;   // a working set, no bounds
-            (batched ? x->cursor_pool : x->row_cursor_pool).push_back(c);
+            pool.push_back(c);
             return;
         }
     }

@@ -52,3 +52,31 @@ def test_batched_cursors_after_lone_cursors_of_a_smaller_index(first, device):
                 pvs.pvs_cursor_close(c)
     finally:
         pvs.pvs_index_free(index)
+
+
+def test_a_full_pool_of_batched_cursors_leaves_room_for_lone_ones():
+    """After 1,024 batched cursors a lone cursor's buffers are still kept: a second
+    one takes no more device memory, and its open waits for no cudaFree."""
+    import torch
+    n, m = 400_000, 128
+    V = synth.unit_normal(n, m, seed=11).numpy()
+    Q = synth.unit_normal(256, m, seed=12).numpy()
+    index = pvs.pvs_build(V)
+    try:
+        batches = [pvs.pvs_cursor_open_batch(index, Q, 100) for _ in range(4)]
+        for b in batches:
+            pvs.pvs_cursor_close_batch(b)
+
+        def free_after_a_lone_cursor():
+            c = pvs.pvs_cursor_open(index, Q[0])
+            pvs.pvs_next(c, 20)
+            pvs.pvs_cursor_close(c)
+            torch.cuda.synchronize()
+            return torch.cuda.mem_get_info()[0]
+
+        before = torch.cuda.mem_get_info()[0]
+        first, second = free_after_a_lone_cursor(), free_after_a_lone_cursor()
+        # kept: the bounds of every row (lo, hi), at least
+        assert before - first >= 8 * n and second == first
+    finally:
+        pvs.pvs_index_free(index)
